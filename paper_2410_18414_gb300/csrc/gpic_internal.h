@@ -186,29 +186,24 @@ struct ParticleGeom {
     double lx, ly, inv_dx, inv_dy, dt;
 };
 
-// sp/spp (optional): each particle's species index and the table; the contributions are
-// then multiplied by q_s w_s.
-template <typename T>
-cudaError_t launch_move_deposit(int p, const ParticleGeom& g, T* x, T* y, const T* vx,
-                                const T* vy, int64_t n, double2* j, unsigned int* err,
-                                cudaStream_t s, const int32_t* sp = nullptr,
-                                const SpeciesParams* spp = nullptr);
-template <typename T>
-cudaError_t launch_deposit_charge(int p, const ParticleGeom& g, const T* x, const T* y, int64_t n,
-                                  double2* j, unsigned int* err, cudaStream_t s,
-                                  const int32_t* sp = nullptr, const SpeciesParams* spp = nullptr);
-// Fixed-point current (int64 per component, contribution = round(value * scale)).
-template <typename T>
-cudaError_t launch_move_deposit_fix(int p, const ParticleGeom& g, T* x, T* y, const T* vx,
-                                    const T* vy, int64_t n, longlong2* j, float scale,
-                                    unsigned int* err, cudaStream_t s, const int32_t* sp = nullptr,
+// Move + deposit of the current and deposit of the charge.  sp/spp (optional): each
+// particle's species index and the table; the contributions are then multiplied by q_s w_s.
+// FP64 atomics into double2 sums (the allocation-free pass):
+cudaError_t launch_move_deposit(int p, const ParticleGeom& g, double* x, double* y,
+                                const double* vx, const double* vy, int64_t n, double2* j,
+                                unsigned int* err, cudaStream_t s);
+// FP32 form: int64 per component, contribution = round(value * scale).
+cudaError_t launch_move_deposit_fix(int p, const ParticleGeom& g, float* x, float* y,
+                                    const float* vx, const float* vy, int64_t n, longlong2* j,
+                                    float scale, unsigned int* err, cudaStream_t s,
+                                    const int32_t* sp = nullptr,
                                     const SpeciesParams* spp = nullptr);
-template <typename T>
-cudaError_t launch_deposit_charge_fix(int p, const ParticleGeom& g, const T* x, const T* y,
-                                      int64_t n, longlong2* j, float scale, unsigned int* err,
-                                      cudaStream_t s, const int32_t* sp = nullptr,
+cudaError_t launch_deposit_charge_fix(int p, const ParticleGeom& g, const float* x,
+                                      const float* y, int64_t n, longlong2* j, float scale,
+                                      unsigned int* err, cudaStream_t s,
+                                      const int32_t* sp = nullptr,
                                       const SpeciesParams* spp = nullptr);
-// FP64 path, deterministic: contribution = round(value * scale) summed exactly as 128-bit
+// FP64 path, deterministic: contributions in units of 1/scale summed exactly as 128-bit
 // integers; j holds 2 ng longlong2, the low words (x, y) of each node, then the high words.
 cudaError_t launch_move_deposit_fix128(int p, const ParticleGeom& g, double* x, double* y,
                                        const double* vx, const double* vy, int64_t n,

@@ -113,7 +113,7 @@ extern "C" pic_status pic_move_deposit_noalloc(const pic_config* cfg, int64_t n,
     cudaError_t e = cudaMemsetAsync(s->j, 0, (size_t)nodes * sizeof(double2), stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->err, 0, sizeof(unsigned int), stream);
     if (e == cudaSuccess)
-        e = launch_move_deposit<double>(cfg->spline_order, g, x, y, vx, vy, n, s->j, s->err, stream);
+        e = launch_move_deposit(cfg->spline_order, g, x, y, vx, vy, n, s->j, s->err, stream);
     if (e == cudaSuccess) {
         k_noalloc_finish<<<(nodes + 255) / 256, 256, 0, stream>>>(s->j, cfg->weight * cfg->q / (dx * dy),
                                                                  jx, jy, nodes);

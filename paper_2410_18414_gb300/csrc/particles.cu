@@ -114,35 +114,12 @@ __device__ __forceinline__ bool in_domain(T xi, int n) {
     return xi >= (T)0 && xi <= (T)n;
 }
 
-// Current accumulation policies.  AccF64: FP64 atomics (plain path).  AccFix: each
-// contribution is rounded to an integer multiple of 1/scale and summed with int64
-// atomics, so the grid total does not depend on the order of the additions.
-struct AccF64 {
-    double2* J;
-    template <typename T>
-    __device__ __forceinline__ T pre(T v) const { return v; }
-    // (tx wy, ty wy) to node: the two current components of one stencil node
-    template <typename T>
-    __device__ __forceinline__ void add2(size_t node, T tx, T ty, T wy) const {
-        atomicAdd(&J[node].x, (double)rmul(tx, wy));
-        atomicAdd(&J[node].y, (double)rmul(ty, wy));
-    }
-    template <typename T>
-    __device__ __forceinline__ void add1f(size_t node, T t, T w) const {
-        atomicAdd(&J[node].x, (double)rmul(t, w));
-    }
-    template <typename T>
-    __device__ __forceinline__ void add1(size_t node, T a) const {
-        atomicAdd(&J[node].x, (double)a);
-    }
-};
-
+// FP32 form: each contribution is rounded to an integer multiple of 1/scale and summed with
+// int64 atomics, so the grid total does not depend on the order of the additions.
 struct AccFix {
     longlong2* J;
     float scale;     // 1 / quantum, a power of two
     float s_hi;      // scale 2^-19
-    template <typename T>
-    __device__ __forceinline__ T pre(T v) const { return v; }
     static AccFix make(void* j, float scale) {
         return AccFix{(longlong2*)j, scale, scale * (1.0f / 524288.0f)};
     }
@@ -191,49 +168,6 @@ struct AccFix {
         split2((float)t, wh, ws, h, l);
         atomicAdd(reinterpret_cast<unsigned long long*>(&J[node].x), join(h, l));
     }
-    template <typename T>
-    __device__ __forceinline__ void add1(size_t node, T a) const {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&J[node].x), (unsigned long long)q((float)a, scale));
-    }
-};
-
-// FP64 path: each contribution is rounded once to an integer multiple of the quantum
-// 1/scale (|x| <= 2^60 by the choice of scale, a power of two) and summed exactly as a
-// 128-bit integer per node and component: a low word (unsigned, modulo 2^64) and a high
-// word.  The atomic on the low word returns the word it added to, so the carry out of
-// each addition is known exactly; the carry and the sign extension of x go to the high
-// word, which changes only when the low word wraps.  Integer sums do not depend on the
-// order of the additions, so the deposit is bit-for-bit deterministic.
-struct AccFix128 {
-    longlong2* J;  // [node]: the low words (x, y); [ng + node]: the high words
-    size_t ng;
-    double scale;
-    // the velocity factor carries the scale (exact: a power of two), so each contribution
-    // is rounded to an integer once
-    template <typename T>
-    __device__ __forceinline__ T pre(T v) const { return v * (T)scale; }
-    __device__ __forceinline__ void add_word(size_t node, int comp, long long x) const {
-        unsigned long long* lo = reinterpret_cast<unsigned long long*>(J + node) + comp;
-        const unsigned long long ux = (unsigned long long)x;
-        const unsigned long long old = atomicAdd(lo, ux);
-        const long long dh = (x < 0 ? -1ll : 0ll) + (old + ux < old ? 1ll : 0ll);
-        if (dh != 0)
-            atomicAdd(reinterpret_cast<unsigned long long*>(J + ng + node) + comp,
-                      (unsigned long long)dh);
-    }
-    template <typename T>
-    __device__ __forceinline__ void add2(size_t node, T tx, T ty, T wy) const {
-        add_word(node, 0, __double2ll_rn((double)rmul(tx, wy)));
-        add_word(node, 1, __double2ll_rn((double)rmul(ty, wy)));
-    }
-    template <typename T>
-    __device__ __forceinline__ void add1f(size_t node, T t, T w) const {
-        add_word(node, 0, __double2ll_rn((double)rmul(t, w)));
-    }
-    template <typename T>
-    __device__ __forceinline__ void add1(size_t node, T a) const {
-        add_word(node, 0, __double2ll_rn((double)a * scale));
-    }
 };
 
 // hi 2^64 + lo (two's complement over 128 bits) times unscale, rounded to FP64: the
@@ -249,75 +183,312 @@ __device__ __forceinline__ double fix128_value(long long hi, unsigned long long 
     return (neg ? -m : m) * unscale;
 }
 
-template <typename T, int P, typename Acc>
-__global__ void __launch_bounds__(kThreads)
-k_move_deposit(GeomT<T> g, T* __restrict__ x, T* __restrict__ y, const T* __restrict__ vx,
-               const T* __restrict__ vy, int64_t n, Acc acc, unsigned int* __restrict__ err,
-               const int32_t* __restrict__ sp, SpeciesT<T> spt) {
-    const T dt = g.dt, lx = g.lx, ly = g.ly, idx_ = g.inv_dx, idy = g.inv_dy;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        T vxi = vx[p], vyi = vy[p];
-        T xp = move_pos(x[p], vxi, dt, lx);
-        T yp = move_pos(y[p], vyi, dt, ly);
-        x[p] = xp;
-        y[p] = yp;
-        const T xi = rmul(xp, idx_), yj = rmul(yp, idy);
-        T fq;
-        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny) || !species_factor(sp, spt, p, fq)) {
-            atomicOr(err, (unsigned)ERR_NONFINITE);
-            continue;
-        }
-        if (sp) {  // each contribution carries the particle's q_s w_s
-            vxi = rmul(vxi, fq);
-            vyi = rmul(vyi, fq);
-        }
-        vxi = acc.pre(vxi);
-        vyi = acc.pre(vyi);
-        T wx[P + 1], wy[P + 1];
-        const int ix = Shape<P, T>::weights(xi, wx);
-        const int iy = Shape<P, T>::weights(yj, wy);
-#pragma unroll
-        for (int a = 0; a <= P; ++a) {
-            const int gi = wrap_idx(ix + a, g.nx);
-            const T tx = rmul(vxi, wx[a]), ty = rmul(vyi, wx[a]);
-            const size_t row = (size_t)gi * g.ny;
-#pragma unroll
-            for (int b = 0; b <= P; ++b) acc.add2(row + wrap_idx(iy + b, g.ny), tx, ty, wy[b]);
-        }
+// ------------------------------------------------------------ row deposit --------
+//
+// Deposits over particles in any order.  A warp takes 32 particles, one a lane: move, weights
+// and the factors t = v W_x of each stencil row go to a shared record a particle.  Then the
+// warp's lanes are the words of ONE particle's stencil (node x component; (p+1)^2 2 words of
+// 8 bytes: 32 for cubic shapes, two passes for quartic) and the warp walks its 32 particles:
+// the lanes of an atomic touch the p+1 rows of neighbouring nodes, 2-3 sectors a row, instead
+// of 32 sectors of 32 particles.  L2 takes atomics by the sector: a lane per particle reached
+// 126 (returning) to 158 G words/s on 2^20 cubic particles of a 128 x 128 grid, a lane per
+// word 424 to 468.  With fewer than 17 words a stencil (one component), two or three particles
+// go at once.  Four particles are in flight together, so that the round trips of returning
+// atomics overlap, and neighbours among them with the same stencil base (sorted particles)
+// are added first: one atomic instead of up to four on the same words.
+//
+// Move + deposit, a lane per particle before: FP64, 2^20 particles, 128 x 128, cubic 320 ->
+// 108 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
+// 256 x 192, quartic 353 -> 149 us (bound by L2's atomics still: 17.5 sectors a particle).
+constexpr int kRowThreads = 128;
+
+// FP64 shapes in fixed point: positions X = x/dx 2^sh (one FP64 multiply and conversion),
+// weights in units of 2^-62 by 64-bit multiply-highs.  GB300 issues 2 FP64 operations per
+// clock and SM but 32 32x32+64-bit multiply-adds, and the rounding of every step is 2^-62 of
+// the largest weight, finer than FP64's.
+constexpr long long kOne62 = 1ll << 62;
+__device__ __forceinline__ long long mul62(long long a, long long b) {  // a, b in [0, 2^62]
+    return (long long)__umul64hi((unsigned long long)a << 1, (unsigned long long)b << 1);
+}
+template <int P>
+__device__ __forceinline__ int fix_weights(long long X, int sh, long long* w) {
+    if (P % 2 == 0) X += 1ll << (sh - 1);
+    const int i = (int)(X >> sh);
+    // u: the offset within the cell (odd P) or from the midpoint before it (even P), in [0, 1)
+    const long long u = (X & ((1ll << sh) - 1)) << (62 - sh), v = kOne62 - u;
+    const long long u2 = mul62(u, u), v2 = mul62(v, v);
+    if constexpr (P == 2) {  // ((1-u)^2/2, the rest, u^2/2)
+        w[0] = v2 >> 1;
+        w[2] = u2 >> 1;
+        w[1] = kOne62 - w[0] - w[2];
+        return i - 1;
+    } else if constexpr (P == 3) {  // ((1-u)^3/6, 2/3 - u^2 + u^3/2, the rest, u^3/6)
+        constexpr unsigned long long sixth = 0x2AAAAAAAAAAAAAABull;  // 2^64 / 6
+        const long long u3 = mul62(u2, u), v3 = mul62(v2, v);
+        w[0] = (long long)__umul64hi((unsigned long long)v3, sixth);
+        w[3] = (long long)__umul64hi((unsigned long long)u3, sixth);
+        w[1] = 0x2AAAAAAAAAAAAAABll - u2 + (u3 >> 1);  // 2/3 in units of 2^-62
+        w[2] = kOne62 - w[0] - w[1] - w[3];
+        return i - 1;
+    } else {  // ((1-u)^4, 11 - 12u - 6u^2 + 12u^3 - 4u^4, the rest, 1 + 4u + 6u^2 + 4u^3 - 4u^4,
+              //  u^4) / 24; the polynomials in units of 2^-58
+        constexpr unsigned long long inv24 = 0x0AAAAAAAAAAAAAABull, two3 = 0xAAAAAAAAAAAAAAABull;
+        const long long u3 = mul62(u2, u), u4 = mul62(u2, u2), v4 = mul62(v2, v2);
+        const long long a = u >> 4, a2 = u2 >> 4, a3 = u3 >> 4, a4 = u4 >> 4, one = kOne62 >> 4;
+        const long long n1 = 11 * one - 12 * a - 6 * a2 + 12 * a3 - 4 * a4;
+        const long long n3 = one + 4 * (a + a3 - a4) + 6 * a2;
+        w[0] = (long long)__umul64hi((unsigned long long)v4, inv24);
+        w[1] = (long long)__umul64hi((unsigned long long)n1, two3);  // 16/24
+        w[3] = (long long)__umul64hi((unsigned long long)n3, two3);
+        w[4] = (long long)__umul64hi((unsigned long long)u4, inv24);
+        w[2] = kOne62 - w[0] - w[1] - w[3] - w[4];
+        return i - 2;
     }
 }
+// Fixed-point positions: x/dx 2^sh with nx, ny <= 2^(62 - sh).
+struct FixGeom {
+    double sx, sy;  // 2^sh / dx, 2^sh / dy
+    int sh;
+};
+inline FixGeom fix_geom(const ParticleGeom& g) {
+    int b = 0;
+    while ((1 << b) < (g.nx > g.ny ? g.nx : g.ny)) ++b;
+    const double s = (double)(1ull << (62 - b));
+    return FixGeom{g.inv_dx * s, g.inv_dy * s, 62 - b};
+}
 
-template <typename T, int P, typename Acc>
-__global__ void __launch_bounds__(kThreads)
-k_deposit_charge(ParticleGeom g, const T* __restrict__ x, const T* __restrict__ y, int64_t n,
-                 Acc acc, unsigned int* __restrict__ err, const int32_t* __restrict__ sp,
-                 SpeciesT<T> spt) {
-    const T idx_ = (T)g.inv_dx, idy = (T)g.inv_dy;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const T xi = rmul(x[p], idx_), yj = rmul(y[p], idy);
-        T fq;
-        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny) || !species_factor(sp, spt, p, fq)) {
-            atomicOr(err, (unsigned)ERR_NONFINITE);
-            continue;
-        }
-        T wx[P + 1], wy[P + 1];
-        const int ix = Shape<P, T>::weights(xi, wx);
-        const int iy = Shape<P, T>::weights(yj, wy);
+// A policy says what a particle's record holds (per component the row factors t[a], then
+// W_y[b]), a contribution's value from it and how it is added to word `c` of a node.
+//
+// RowFix: the FP32 form's current.  t = v W_x in FP32; int64 atomics without return.
+struct RowFix {
+    using T = float;
+    using W = float;
+    using V = unsigned long long;
+    AccFix acc;
+    static constexpr bool kExtra = false;
+    __device__ __forceinline__ V value(const float* r, int t, int wy, int) const {
+        float wh, ws;
+        acc.scaled(r[wy], wh, ws);
+        int h, l;
+        AccFix::split2(r[t], wh, ws, h, l);
+        return AccFix::join(h, l);
+    }
+    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+        atomicAdd(reinterpret_cast<V*>(acc.J + node) + c, x);
+        return 0;
+    }
+    __device__ __forceinline__ void finish(size_t, int, V, V) const {}
+    template <int P>
+    __device__ __forceinline__ bool shape(const GeomT<float>& g, float x, float y, int& ix,
+                                          int& iy, float* wx, float* wy) const {
+        const float xi = rmul(x, g.inv_dx), yj = rmul(y, g.inv_dy);
+        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny)) return false;
+        ix = Shape<P, float>::weights(xi, wx);
+        iy = Shape<P, float>::weights(yj, wy);
+        return true;
+    }
+    __device__ __forceinline__ float factor(float v) const { return v; }
+    __device__ __forceinline__ float row(float v, float w) const { return rmul(v, w); }
+    __device__ __forceinline__ float col(float w) const { return w; }
+};
+
+// The FP32 form's charge: round(W_x W_y q_s w_s scale), the factor in the record's last slot.
+struct RowFixCharge : RowFix {
+    static constexpr bool kExtra = true;
+    __device__ __forceinline__ V value(const float* r, int t, int wy, int extra) const {
+        return (V)AccFix::q(rmul(rmul(r[t], r[wy]), r[extra]), acc.scale);
+    }
+    __device__ __forceinline__ float row(float, float w) const { return w; }
+};
+
+// RowFix128: the FP64 path.  Contributions in units of the quantum 1/scale (|x| <= 2^60 by
+// the choice of scale, a power of two) are summed exactly as a 128-bit integer per node and
+// component: a low word (unsigned, modulo 2^64) and a high word.  The atomic on the low word
+// returns the word it added to, so the carry out of each addition is known exactly; the carry
+// and the sign extension of x go to the high word, which changes only when the low word wraps.
+// Integer sums do not depend on the order of the additions, so the deposit is bit-for-bit
+// deterministic.  The factors are integers: v in units of 2^-2 quanta, t = v W_x in half
+// quanta, x = t W_y in quanta, each rounded down once (2^-60 of the bound c; FP64 rounds
+// each product at 2^-53 of its value).
+struct RowFix128 {
+    using T = double;
+    using W = long long;
+    using V = unsigned long long;
+    longlong2* J;  // [node]: the low words (x, y); [ng + node]: the high words
+    size_t ng;
+    double scale4;  // 4 scale
+    FixGeom fg;
+    static constexpr bool kExtra = false;
+    __device__ __forceinline__ V value(const long long* r, int t, int wy, int) const {
+        return (V)__mul64hi(r[t], r[wy]);
+    }
+    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+        return atomicAdd(reinterpret_cast<V*>(J + node) + c, x);
+    }
+    __device__ __forceinline__ void finish(size_t node, int c, V x, V old) const {
+        const long long dh = ((long long)x < 0 ? -1ll : 0ll) + (old + x < old ? 1ll : 0ll);
+        if (dh != 0) atomicAdd(reinterpret_cast<V*>(J + ng + node) + c, (V)dh);
+    }
+    template <int P>
+    __device__ __forceinline__ bool shape(const GeomT<double>& g, double x, double y, int& ix,
+                                          int& iy, long long* wx, long long* wy) const {
+        // NaN and out-of-range values convert to the ends of the int64 range
+        const long long X = __double2ll_rn(rmul(x, fg.sx)), Y = __double2ll_rn(rmul(y, fg.sy));
+        if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh))
+            return false;
+        ix = fix_weights<P>(X, fg.sh, wx);
+        iy = fix_weights<P>(Y, fg.sh, wy);
+        return true;
+    }
+    __device__ __forceinline__ long long factor(double v) const {
+        return __double2ll_rn(rmul(v, scale4));
+    }
+    __device__ __forceinline__ long long row(long long v, long long w) const {
+        return __mul64hi(v, w << 1);
+    }
+    __device__ __forceinline__ long long col(long long w) const { return w << 1; }
+};
+
+// RowF64: FP64 atomics (the allocation-free pass).
+struct RowF64 {
+    using T = double;
+    using W = double;
+    using V = double;
+    double2* J;
+    static constexpr bool kExtra = false;
+    __device__ __forceinline__ V value(const double* r, int t, int wy, int) const {
+        return rmul(r[t], r[wy]);
+    }
+    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+        atomicAdd(reinterpret_cast<double*>(J + node) + c, x);
+        return 0.0;
+    }
+    __device__ __forceinline__ void finish(size_t, int, V, V) const {}
+    template <int P>
+    __device__ __forceinline__ bool shape(const GeomT<double>& g, double x, double y, int& ix,
+                                          int& iy, double* wx, double* wy) const {
+        const double xi = rmul(x, g.inv_dx), yj = rmul(y, g.inv_dy);
+        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny)) return false;
+        ix = Shape<P, double>::weights(xi, wx);
+        iy = Shape<P, double>::weights(yj, wy);
+        return true;
+    }
+    __device__ __forceinline__ double factor(double v) const { return v; }
+    __device__ __forceinline__ double row(double v, double w) const { return rmul(v, w); }
+    __device__ __forceinline__ double col(double w) const { return w; }
+};
+
+// kMove: x, y move by (u0, u1) dt first (the position update); u0, u1: the deposited
+// components (kNC = 1: u0 alone, or 1 for every particle when u0 is NULL, the charge).
+template <typename Pol, int P, int kNC, bool kMove>
+__global__ void __launch_bounds__(kRowThreads)
+k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
+               typename Pol::T* __restrict__ y, const typename Pol::T* __restrict__ u0,
+               const typename Pol::T* __restrict__ u1, int64_t n, Pol pol,
+               unsigned int* __restrict__ err, const int32_t* __restrict__ sp,
+               SpeciesT<typename Pol::T> spt) {
+    using T = typename Pol::T;
+    using W = typename Pol::W;
+    using V = typename Pol::V;
+    constexpr int S1 = P + 1, kWords = S1 * S1 * kNC;
+    constexpr int kGroups = kWords <= 32 ? 32 / kWords : 1;     // particles at once
+    constexpr int kPasses = (kWords + 31) / 32;                 // words a lane of one particle
+    constexpr int kFields = (kNC + 1) * S1 + (Pol::kExtra ? 1 : 0);
+    constexpr int kStride = kFields | 1;  // odd: conflict-free across the lanes' records
+    constexpr int kAhead = 4;
+    __shared__ W rec[kRowThreads * kStride];
+    __shared__ int rbase[kRowThreads];
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    W* mine = rec + threadIdx.x * kStride;
+    // this lane's words: group, stencil row a and column b, component
+    const int group = lane / kWords, lw = lane - group * kWords;
+    int wa[kPasses], wb[kPasses], wc[kPasses];
+    bool on[kPasses];
 #pragma unroll
-        for (int a = 0; a <= P; ++a) {
-            const int gi = wrap_idx(ix + a, g.nx);
+    for (int q = 0; q < kPasses; ++q) {
+        const int word = lw + 32 * q;
+        on[q] = word < kWords && group < kGroups;
+        wa[q] = word / (S1 * kNC);
+        const int r = word - wa[q] * (S1 * kNC);
+        wb[q] = r / kNC;
+        wc[q] = r - wb[q] * kNC;
+    }
+    for (int64_t p0 = (blockIdx.x * (int64_t)kRowThreads + w0); p0 < n;
+         p0 += (int64_t)gridDim.x * kRowThreads) {
+        const int64_t p = p0 + lane;
+        int base = -1;
+        if (p < n) {
+            T xp = x[p], yp = y[p];
+            T v[2] = {(T)1, (T)0};
+            if (u0) v[0] = u0[p];
+            if constexpr (kNC == 2) v[1] = u1[p];
+            if constexpr (kMove) {
+                xp = move_pos(xp, v[0], g.dt, g.lx);
+                yp = move_pos(yp, v[1], g.dt, g.ly);
+                x[p] = xp;
+                y[p] = yp;
+            }
+            W wx[S1], wy[S1];
+            int ix, iy;
+            T fq;
+            if (!pol.template shape<P>(g, xp, yp, ix, iy, wx, wy) ||
+                !species_factor(sp, spt, p, fq)) {
+                atomicOr(err, (unsigned)ERR_NONFINITE);
+            } else {
+                base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
 #pragma unroll
-            for (int b = 0; b <= P; ++b) {
-                const int gj = wrap_idx(iy + b, g.ny);
-                const T wab = rmul(wx[a], wy[b]);
-                acc.add1((size_t)gi * g.ny + gj, sp ? rmul(wab, fq) : wab);
+                for (int c = 0; c < kNC; ++c) {
+                    // with a table each contribution carries the particle's q_s w_s
+                    if (sp && !Pol::kExtra) v[c] = rmul(v[c], fq);
+                    const W f = pol.factor(v[c]);
+#pragma unroll
+                    for (int a = 0; a < S1; ++a) mine[c * S1 + a] = pol.row(f, wx[a]);
+                }
+#pragma unroll
+                for (int b = 0; b < S1; ++b) mine[kNC * S1 + b] = pol.col(wy[b]);
+                if constexpr (Pol::kExtra) mine[kFields - 1] = (W)fq;
             }
         }
+        rbase[threadIdx.x] = base;
+        __syncwarp();
+#pragma unroll 1
+        for (int i0 = 0; i0 * kGroups < 32; i0 += kAhead) {
+#pragma unroll
+            for (int q = 0; q < kPasses; ++q) {
+                int bs[kAhead];
+                V val[kAhead], old[kAhead];
+                size_t node[kAhead];
+#pragma unroll
+                for (int j = 0; j < kAhead; ++j) {
+                    const int k = (i0 + j) * kGroups + group;
+                    bs[j] = on[q] && k < 32 ? rbase[w0 + k] : -1;
+                    val[j] = 0;
+                    node[j] = 0;
+                    if (bs[j] >= 0) {
+                        val[j] = pol.value(rec + (w0 + k) * kStride, wc[q] * S1 + wa[q],
+                                           kNC * S1 + wb[q], kFields - 1);
+                        int gi = (bs[j] >> 16) + wa[q], gj = (bs[j] & 0xFFFF) + wb[q];
+                        if (gi >= g.nx) gi -= g.nx;
+                        if (gj >= g.ny) gj -= g.ny;
+                        node[j] = (size_t)gi * g.ny + gj;
+                        if (j > 0 && bs[j] == bs[j - 1]) {  // the same words: one atomic
+                            val[j] += val[j - 1];
+                            bs[j - 1] = -1;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kAhead; ++j)
+                    if (bs[j] >= 0) old[j] = pol.issue(node[j], wc[q], val[j]);
+#pragma unroll
+                for (int j = 0; j < kAhead; ++j)
+                    if (bs[j] >= 0) pol.finish(node[j], wc[q], val[j], old[j]);
+            }
+        }
+        __syncwarp();  // the records are rewritten
     }
 }
-
 
 // The binned FP32 pass keeps its 32-bit region sums in two parts of a contribution:
 // node totals are hi 2^kLoBits + lo (see AccFix::split2).
@@ -1195,35 +1366,6 @@ k_replay_step(GeomT<T> g, const T* __restrict__ s0, T* __restrict__ s1,
 // gathered with its in-plane gradient, (grad A . v*)_l gains d_l A_z v*_z for l = x, y,
 // P_z is constant, and u = P - q A has three components.
 
-// J_z of the moved particles (after the move of k_move_deposit): x^{n+1}, v_z^n.
-template <typename T, int P, typename Acc>
-__global__ void __launch_bounds__(kThreads)
-k_deposit_z(GeomT<T> g, const T* __restrict__ x, const T* __restrict__ y,
-            const T* __restrict__ vz, int64_t n, const int32_t* __restrict__ sp, SpeciesT<T> spt,
-            Acc acc, unsigned int* __restrict__ err) {
-    const T idx_ = g.inv_dx, idy = g.inv_dy;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const T xi = rmul(x[p], idx_), yj = rmul(y[p], idy);
-        T fq;
-        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny) || !species_factor(sp, spt, p, fq)) {
-            atomicOr(err, (unsigned)ERR_NONFINITE);
-            continue;
-        }
-        T wx[P + 1], wy[P + 1];
-        const int ix = Shape<P, T>::weights(xi, wx);
-        const int iy = Shape<P, T>::weights(yj, wy);
-        const T vzi = acc.pre(sp ? rmul(vz[p], fq) : vz[p]);
-#pragma unroll
-        for (int a = 0; a <= P; ++a) {
-            const size_t row = (size_t)wrap_idx(ix + a, g.nx) * g.ny;
-            const T tz = rmul(vzi, wx[a]);
-#pragma unroll
-            for (int b = 0; b <= P; ++b) acc.add1f(row + wrap_idx(iy + b, g.ny), tz, wy[b]);
-        }
-    }
-}
-
 // Species constants of particle p in the storage precision (the table's, or the single
 // species' q, m, weight).
 template <typename T>
@@ -1404,22 +1546,47 @@ __global__ void k_extract(const cplx_t<T>* __restrict__ src, int stride, int com
         default: return cudaErrorInvalidValue;                             \
     }
 
-#define GPIC_DISPATCH_PA(p, KERNEL, ACC, ...)                                               \
-    switch (p) {                                                                           \
-        case 2: KERNEL<T, 2, ACC><<<blocks_for(n), kThreads, 0, s>>>(__VA_ARGS__); break; \
-        case 3: KERNEL<T, 3, ACC><<<blocks_for(n), kThreads, 0, s>>>(__VA_ARGS__); break; \
-        case 4: KERNEL<T, 4, ACC><<<blocks_for(n), kThreads, 0, s>>>(__VA_ARGS__); break; \
-        default: return cudaErrorInvalidValue;                                             \
-    }
-
-template <typename T>
-cudaError_t launch_move_deposit(int p, const ParticleGeom& g, T* x, T* y, const T* vx,
-                                const T* vy, int64_t n, double2* j, unsigned int* err,
-                                cudaStream_t s, const int32_t* sp, const SpeciesParams* spp) {
+template <typename Pol, int kNC, bool kMove>
+cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typename Pol::T* y,
+                         const typename Pol::T* u0, const typename Pol::T* u1, int64_t n,
+                         const Pol& pol, unsigned int* err, cudaStream_t s, const int32_t* sp,
+                         const SpeciesParams* spp) {
+    using T = typename Pol::T;
     if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_move_deposit, AccF64, typed<T>(g), x, y, vx, vy, n, AccF64{j}, err,
-                     sp, typed_species<T>(spp))
+    const unsigned blocks = (unsigned)((n + kRowThreads - 1) / kRowThreads);
+    const GeomT<T> gt = typed<T>(g);
+    const SpeciesT<T> st = typed_species<T>(spp);
+    switch (p) {
+        case 2: k_deposit_rows<Pol, 2, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
+        case 3: k_deposit_rows<Pol, 3, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
+        case 4: k_deposit_rows<Pol, 4, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
+}
+
+cudaError_t launch_move_deposit(int p, const ParticleGeom& g, double* x, double* y,
+                                const double* vx, const double* vy, int64_t n, double2* j,
+                                unsigned int* err, cudaStream_t s) {
+    return deposit_rows<RowF64, 2, true>(p, g, x, y, vx, vy, n, RowF64{j}, err, s, nullptr,
+                                         nullptr);
+}
+
+cudaError_t launch_move_deposit_fix(int p, const ParticleGeom& g, float* x, float* y,
+                                    const float* vx, const float* vy, int64_t n, longlong2* j,
+                                    float scale, unsigned int* err, cudaStream_t s,
+                                    const int32_t* sp, const SpeciesParams* spp) {
+    return deposit_rows<RowFix, 2, true>(p, g, x, y, vx, vy, n, RowFix{AccFix::make(j, scale)},
+                                         err, s, sp, spp);
+}
+
+cudaError_t launch_deposit_charge_fix(int p, const ParticleGeom& g, const float* x,
+                                      const float* y, int64_t n, longlong2* j, float scale,
+                                      unsigned int* err, cudaStream_t s, const int32_t* sp,
+                                      const SpeciesParams* spp) {
+    return deposit_rows<RowFixCharge, 1, false>(
+        p, g, const_cast<float*>(x), const_cast<float*>(y), nullptr, nullptr, n,
+        RowFixCharge{{AccFix::make(j, scale)}}, err, s, sp, spp);
 }
 
 cudaError_t launch_move_deposit_fix128(int p, const ParticleGeom& g, double* x, double* y,
@@ -1427,58 +1594,38 @@ cudaError_t launch_move_deposit_fix128(int p, const ParticleGeom& g, double* x, 
                                        longlong2* j, size_t ng, double scale, unsigned int* err,
                                        cudaStream_t s, const int32_t* sp,
                                        const SpeciesParams* spp) {
-    using T = double;
-    if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_move_deposit, AccFix128, typed<T>(g), x, y, vx, vy, n,
-                     (AccFix128{j, ng, scale}), err, sp, typed_species<T>(spp))
-    return cudaGetLastError();
+    return deposit_rows<RowFix128, 2, true>(p, g, x, y, vx, vy, n,
+                                            RowFix128{j, ng, 4.0 * scale, fix_geom(g)}, err, s,
+                                            sp, spp);
 }
 
 cudaError_t launch_deposit_charge_fix128(int p, const ParticleGeom& g, const double* x,
                                          const double* y, int64_t n, longlong2* j, size_t ng,
                                          double scale, unsigned int* err, cudaStream_t s,
                                          const int32_t* sp, const SpeciesParams* spp) {
-    using T = double;
-    if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_deposit_charge, AccFix128, g, x, y, n, (AccFix128{j, ng, scale}), err,
-                     sp, typed_species<T>(spp))
-    return cudaGetLastError();
+    return deposit_rows<RowFix128, 1, false>(
+        p, g, const_cast<double*>(x), const_cast<double*>(y), nullptr, nullptr, n,
+        RowFix128{j, ng, 4.0 * scale, fix_geom(g)}, err, s, sp, spp);
+}
+
+template <typename T>
+cudaError_t launch_deposit_z(int p, const ParticleGeom& g, const T* x, const T* y, const T* vz,
+                             int64_t n, const int32_t* sp, const SpeciesParams& spp, void* jz,
+                             size_t ng, double scale, unsigned int* err, cudaStream_t s) {
+    const int32_t* spi = spp.n > 0 ? sp : nullptr;
+    if constexpr (sizeof(T) == 4)
+        return deposit_rows<RowFix, 1, false>(p, g, const_cast<T*>(x), const_cast<T*>(y), vz,
+                                              nullptr, n, RowFix{AccFix::make(jz, (float)scale)},
+                                              err, s, spi, &spp);
+    else
+        return deposit_rows<RowFix128, 1, false>(
+            p, g, const_cast<T*>(x), const_cast<T*>(y), vz, nullptr, n,
+            RowFix128{(longlong2*)jz, ng, 4.0 * scale, fix_geom(g)}, err, s, spi, &spp);
 }
 
 cudaError_t launch_fix128_to_cplx(const longlong2* j, size_t ng, double unscale, double2* out,
                                   cudaStream_t s) {
     k_fix128_to_cplx<<<blocks_for((int64_t)ng), kThreads, 0, s>>>(j, ng, unscale, out);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_deposit_charge(int p, const ParticleGeom& g, const T* x, const T* y, int64_t n,
-                                  double2* j, unsigned int* err, cudaStream_t s,
-                                  const int32_t* sp, const SpeciesParams* spp) {
-    if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_deposit_charge, AccF64, g, x, y, n, AccF64{j}, err, sp,
-                     typed_species<T>(spp))
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_move_deposit_fix(int p, const ParticleGeom& g, T* x, T* y, const T* vx,
-                                    const T* vy, int64_t n, longlong2* j, float scale,
-                                    unsigned int* err, cudaStream_t s, const int32_t* sp,
-                                    const SpeciesParams* spp) {
-    if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_move_deposit, AccFix, typed<T>(g), x, y, vx, vy, n, (AccFix::make(j, scale)),
-                     err, sp, typed_species<T>(spp))
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_deposit_charge_fix(int p, const ParticleGeom& g, const T* x, const T* y,
-                                      int64_t n, longlong2* j, float scale, unsigned int* err,
-                                      cudaStream_t s, const int32_t* sp, const SpeciesParams* spp) {
-    if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_PA(p, k_deposit_charge, AccFix, g, x, y, n, (AccFix::make(j, scale)), err, sp,
-                     typed_species<T>(spp))
     return cudaGetLastError();
 }
 
@@ -1493,22 +1640,6 @@ template cudaError_t launch_replay_step<double>(const ParticleGeom&, const doubl
                                                 const double*, int64_t, cudaStream_t);
 template cudaError_t launch_replay_step<float>(const ParticleGeom&, const float*, float*,
                                                const double*, int64_t, cudaStream_t);
-
-template <typename T>
-cudaError_t launch_deposit_z(int p, const ParticleGeom& g, const T* x, const T* y, const T* vz,
-                             int64_t n, const int32_t* sp, const SpeciesParams& spp, void* jz,
-                             size_t ng, double scale, unsigned int* err, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    const int32_t* spi = spp.n > 0 ? sp : nullptr;
-    if constexpr (sizeof(T) == 4) {
-        GPIC_DISPATCH_PA(p, k_deposit_z, AccFix, typed<T>(g), x, y, vz, n, spi,
-                         typed_species<T>(&spp), (AccFix::make(jz, (float)scale)), err)
-    } else {
-        GPIC_DISPATCH_PA(p, k_deposit_z, AccFix128, typed<T>(g), x, y, vz, n, spi,
-                         typed_species<T>(&spp), (AccFix128{(longlong2*)jz, ng, scale}), err)
-    }
-    return cudaGetLastError();
-}
 
 template <typename T>
 cudaError_t launch_gather_push3(int p, const ParticleGeom& g, const PushParams& pp, const T* x,
@@ -1750,14 +1881,6 @@ cudaError_t launch_extract(const void* src, int stride, int comp, double scale, 
 }
 
 #define GPIC_INST(T)                                                                            \
-    template cudaError_t launch_move_deposit<T>(int, const ParticleGeom&, T*, T*, const T*,     \
-                                                const T*, int64_t, double2*, unsigned int*,     \
-                                                cudaStream_t, const int32_t*,                   \
-                                                const SpeciesParams*);                          \
-    template cudaError_t launch_deposit_charge<T>(int, const ParticleGeom&, const T*, const T*, \
-                                                  int64_t, double2*, unsigned int*,             \
-                                                  cudaStream_t, const int32_t*,                 \
-                                                  const SpeciesParams*);                        \
     template cudaError_t launch_deposit_z<T>(int, const ParticleGeom&, const T*, const T*,      \
                                              const T*, int64_t, const int32_t*,                 \
                                              const SpeciesParams&, void*, size_t, double,       \
@@ -1786,14 +1909,6 @@ cudaError_t launch_extract(const void* src, int stride, int comp, double scale, 
     template cudaError_t launch_extract<T>(const void*, int, int, double, double*, int64_t,     \
                                            cudaStream_t);                                       \
     template cudaError_t launch_wrap_positions<T>(T*, T*, int64_t, double, double, cudaStream_t); \
-    template cudaError_t launch_move_deposit_fix<T>(int, const ParticleGeom&, T*, T*, const T*,   \
-                                                    const T*, int64_t, longlong2*, float,         \
-                                                    unsigned int*, cudaStream_t, const int32_t*,  \
-                                                    const SpeciesParams*);                        \
-    template cudaError_t launch_deposit_charge_fix<T>(int, const ParticleGeom&, const T*,         \
-                                                      const T*, int64_t, longlong2*, float,       \
-                                                      unsigned int*, cudaStream_t,                \
-                                                      const int32_t*, const SpeciesParams*);      \
     template cudaError_t launch_fix_to_cplx<T>(const longlong2*, double, void*, int64_t,          \
                                                cudaStream_t);
 GPIC_INST(double)

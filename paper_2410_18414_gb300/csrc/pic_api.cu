@@ -445,8 +445,8 @@ pic_status setup(pic_handle* h, const pic_particles_in* in) {
         cudaError_t r = launch_wrap_positions<T>((T*)h->x, (T*)h->y, n, c.lx, c.ly, h->s);
         if (r != cudaSuccess) return r;
         if (h->fp32) {
-            r = launch_deposit_charge_fix<T>(h->p, h->geom, (const T*)h->x, (const T*)h->y, n,
-                                             (longlong2*)h->J, h->fix_scale_q, h->err, h->s, sp,
+            r = launch_deposit_charge_fix(h->p, h->geom, (const float*)h->x,
+                                          (const float*)h->y, n, (longlong2*)h->J, h->fix_scale_q, h->err, h->s, sp,
                                              &h->spp);
             if (r != cudaSuccess) return r;
             r = launch_fix_to_cplx<T>((const longlong2*)h->J, h->fix_unscale_q, h->tmp, h->ng, h->s);
@@ -794,7 +794,7 @@ pic_status pic_deposit(pic_handle* h) {
         }
         const int32_t* sp = h->spp.n > 0 ? h->species : nullptr;
         if constexpr (sizeof(T) == 4) {
-            return launch_move_deposit_fix<T>(h->p, h->geom, (T*)h->x, (T*)h->y,
+            return launch_move_deposit_fix(h->p, h->geom, (T*)h->x, (T*)h->y,
                                               (const T*)h->v[h->vcur][0], (const T*)h->v[h->vcur][1],
                                               h->n, (longlong2*)h->J, h->fix_scale_j, h->err, h->s,
                                               sp, &h->spp);
@@ -853,8 +853,8 @@ pic_status pic_field_solve(pic_handle* h) {
             using T = decltype(t);
             cudaError_t r;
             if (h->fp32) {
-                r = launch_deposit_charge_fix<T>(h->p, h->geom, (const T*)h->x, (const T*)h->y,
-                                                 h->n, (longlong2*)h->rhoq, h->fix_scale_q,
+                r = launch_deposit_charge_fix(h->p, h->geom, (const float*)h->x,
+                                              (const float*)h->y, h->n, (longlong2*)h->rhoq, h->fix_scale_q,
                                                  h->err, h->s, sp, &h->spp);
                 if (r == cudaSuccess)
                     r = launch_fix_to_cplx<T>((const longlong2*)h->rhoq, h->fix_unscale_q, h->tmp,
