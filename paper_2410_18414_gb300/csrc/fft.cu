@@ -23,12 +23,35 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// The largest magnitudes of four lines of m complex values (rows of the four arrays, array
+// after array), as high words, into fmax[8] (re, im of each array).
+__device__ __forceinline__ void collect_max(const double2* res, int m, unsigned* fmax) {
+    const int b = threadIdx.x & 3;
+    unsigned re = 0, im = 0;
+    for (int e = threadIdx.x >> 2; e < m; e += blockDim.x >> 2) {
+        const double2 v = res[b * m + e];
+        re = max(re, (unsigned)__double2hiint(v.x) & 0x7fffffffu);
+        im = max(im, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+    }
+    for (int o = 16; o >= 4; o >>= 1) {
+        re = max(re, __shfl_xor_sync(0xffffffffu, re, o));
+        im = max(im, __shfl_xor_sync(0xffffffffu, im, o));
+    }
+    // most CTAs find a value as large already there and leave the word alone
+    if ((threadIdx.x & 31) < 4) {
+        volatile const unsigned* seen = fmax;
+        if (re > seen[2 * b]) atomicMax(fmax + 2 * b, re);
+        if (im > seen[2 * b + 1]) atomicMax(fmax + 2 * b + 1, im);
+    }
+}
+
 // Transforms along y (contiguous): CTA = `rows` consecutive x-indices of all nb arrays.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, int ny, int nb,
         int rows, FftDesc d, const cplx_t<T>* __restrict__ tw, int sign, int interleave,
-        const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear) {
+        const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear,
+        unsigned* __restrict__ fmax) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* b0 = reinterpret_cast<C*>(smem_raw);
@@ -55,6 +78,9 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     __syncthreads();
     C* res = run_passes(b0, b1, d, lines, (const C*)tws, sign);
     if (interleave) {
+        if constexpr (sizeof(T) == 8) {  // a thread's outputs are all of array threadIdx.x % 4
+            if (fmax) collect_max(res, rows * ny, fmax);
+        }
         for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
             int b = e % nb, t = e / nb;
             int jj = t % ny, r = t / ny;
@@ -115,7 +141,8 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 template <typename T>
 static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                               const void* tw, int sign, int interleave, const longlong2* fix_in,
-                              double unscale, longlong2* clear, cudaStream_t s) {
+                              double unscale, longlong2* clear, cudaStream_t s,
+                              unsigned* fmax = nullptr) {
     using C = cplx_t<T>;
     const size_t per_line = 2 * (size_t)ny * sizeof(C);
     const size_t tw_bytes = (size_t)ny * sizeof(C);
@@ -128,13 +155,16 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
     cudaError_t e = set_smem(k_fft_y<T>, smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_fft_y<T>, dim3(nx / rows), dim3(kThreads), smem, s, (const C*)in, (C*)out,
-                      nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear);
+                      nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear,
+                      fmax);
 }
 
 template <typename T>
 cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
-                         const void* tw, int sign, int interleave, cudaStream_t s) {
-    return fft_y_impl<T>(in, out, nx, ny, nb, d, tw, sign, interleave, nullptr, 0.0, nullptr, s);
+                         const void* tw, int sign, int interleave, cudaStream_t s,
+                         unsigned* fmax) {
+    return fft_y_impl<T>(in, out, nx, ny, nb, d, tw, sign, interleave, nullptr, 0.0, nullptr, s,
+                         fmax);
 }
 
 template <typename T>
@@ -169,9 +199,9 @@ cudaError_t launch_twiddles(void* tw, int n, cudaStream_t s) {
 }
 
 template cudaError_t launch_fft_y<double>(const void*, void*, int, int, int, const FftDesc&,
-                                          const void*, int, int, cudaStream_t);
+                                          const void*, int, int, cudaStream_t, unsigned*);
 template cudaError_t launch_fft_y<float>(const void*, void*, int, int, int, const FftDesc&,
-                                         const void*, int, int, cudaStream_t);
+                                         const void*, int, int, cudaStream_t, unsigned*);
 template cudaError_t launch_fft_x<double>(const void*, void*, int, int, int, const FftDesc&,
                                           const void*, int, cudaStream_t);
 template cudaError_t launch_fft_x<float>(const void*, void*, int, int, int, const FftDesc&,

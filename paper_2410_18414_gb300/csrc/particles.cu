@@ -505,9 +505,11 @@ __global__ void k_fix_to_cplx(const longlong2* __restrict__ J, double unscale,
     }
 }
 
-// FP64 path: the 128-bit sums of AccFix128 to complex FP64 values, times `unscale`.
+// FP64 path: the 128-bit sums of RowFix128 to complex FP64 values, times `unscale`; fmax
+// (optional): the eight field maxima that this step's transform collects, set to 0.
 __global__ void k_fix128_to_cplx(const longlong2* __restrict__ J, size_t ng, double unscale,
-                                 double2* __restrict__ out) {
+                                 double2* __restrict__ out, unsigned* __restrict__ fmax) {
+    if (fmax && blockIdx.x == 0 && threadIdx.x < 8) fmax[threadIdx.x] = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < (int64_t)ng;
          k += (int64_t)gridDim.x * blockDim.x) {
         const longlong2 lo = J[k], hi = J[ng + k];
@@ -605,6 +607,42 @@ __device__ __forceinline__ void push_finish(const PushT<T>& pp, unsigned bad, do
     }
 }
 
+// The adjoint's record of one particle's push (see launch_gather_push).
+template <typename T>
+__device__ __forceinline__ void record_push(double* __restrict__ gout, int gout_short, int64_t n,
+                                            int64_t p, T Px, T Py, T vx, T vy, const T* f) {
+    gout[p] = (double)Px;
+    gout[(size_t)n + p] = (double)Py;
+    gout[2 * (size_t)n + p] = (double)vx;
+    gout[3 * (size_t)n + p] = (double)vy;
+    if (!gout_short) {
+#pragma unroll
+        for (int k = 2; k < 8; ++k) gout[(size_t)(k + 2) * n + p] = (double)f[k];
+    }
+}
+
+// Fixed-point fields: fmax holds the high word of the largest |f| on the mesh, which gives
+// the exponent e with |f| < 2^e (bounded below so that the scales stay finite).  A field that
+// is not finite somewhere has no scale: its gathered values are NaN.
+__device__ __forceinline__ int field_exponent(unsigned fmax) {
+    return max((int)(fmax >> 20) - 1022, -900);
+}
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+__device__ __forceinline__ double field_unit(unsigned fmax) {
+    return fmax >= 0x7ff00000u ? __hiloint2double(0x7ff80000, 0) : pow2(field_exponent(fmax) - 58);
+}
+// v in [-2^58, 2^58] as (v.x 2^29 + v.y), |v.y| <= 2^28
+__device__ __forceinline__ int2 limbs58(long long v) {
+    const int lo = (int)((unsigned)v << 3) >> 3;
+    return make_int2((int)((v - lo) >> 29), lo);
+}
+__device__ __forceinline__ int2 field_fix(double f, unsigned fmax) {
+    if (fmax >= 0x7ff00000u) return make_int2(0, 0);
+    return limbs58(__double2ll_rn(rmul(f, pow2(58 - field_exponent(fmax)))));
+}
+
+// FP64 arithmetic, a lane per particle: for runs with so few particles on the mesh that
+// converting its fields (k_fields_to_fix) would cost more than it saves.
 template <typename T, int P>
 __global__ void __launch_bounds__(kThreads)
 k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restrict__ y,
@@ -641,18 +679,223 @@ k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restr
         }
         T vxn1, vyn1;
         push_one(pp, f, p, px, py, vx, vy, vxo, vyo, bad, kin, vxn1, vyn1);
-        if (gout) {  // the adjoint's record of this step (see launcher)
-            gout[p] = (double)px[p];
-            gout[(size_t)n + p] = (double)py[p];
-            gout[2 * (size_t)n + p] = (double)vxn1;
-            gout[3 * (size_t)n + p] = (double)vyn1;
-            if (!gout_short) {
+        if (gout) record_push(gout, gout_short, n, p, px[p], py[p], vxn1, vyn1, f);
+    }
+    push_finish(pp, bad, kin, diag, err);
+}
+
+// ------------------------------------------------------------ row gather ---------
+//
+// Gather + push over particles in any order.  With a lane per particle every 16-byte load of
+// a field node touches 32 lines; here neighbouring lanes share a particle and read one node's
+// values side by side, so a load touches 16 (FP32, two lanes a particle) or 8 lines (FP64,
+// four lanes).  A warp's 32 particles leave their weights in shared memory a lane each, are
+// gathered 16 or 8 at a time, and the gathered fields go back through the same records to
+// the lane that pushes the particle.  Gather + push, a lane per particle before: FP32, 1.5 M
+// particles, 256 x 192, quartic 192 -> 121 us; FP64, 2^20 particles, 128 x 128, cubic
+// 394 -> 127 us (and 4 us for k_fields_to_fix).
+constexpr int kRowGatherThreads = 128;
+
+// FP32: the node order and roundings of every other gather, so the same bits.
+template <int P>
+__global__ void __launch_bounds__(kRowGatherThreads)
+k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
+                   const float* __restrict__ y, float* __restrict__ px, float* __restrict__ py,
+                   const float* __restrict__ vx, const float* __restrict__ vy,
+                   float* __restrict__ vxo, float* __restrict__ vyo, int64_t n,
+                   const float4* __restrict__ F, double* __restrict__ gout, int gout_short,
+                   double* __restrict__ diag, unsigned int* __restrict__ err) {
+    constexpr int S1 = P + 1;
+    constexpr int kStride = (2 * S1 > 8 ? 2 * S1 : 8) | 1;
+    __shared__ float rec[kRowGatherThreads * kStride];
+    __shared__ int rbase[kRowGatherThreads];
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    const int64_t p = blockIdx.x * (int64_t)kRowGatherThreads + threadIdx.x;
+    float* mine = rec + threadIdx.x * kStride;
+    double kin = 0.0;
+    unsigned bad = 0;
+    int base = -1;
+    if (p < n) {
+        const float xi = rmul(x[p], g.inv_dx), yj = rmul(y[p], g.inv_dy);
+        if (!in_domain(xi, g.nx) || !in_domain(yj, g.ny)) {
+            bad |= ERR_NONFINITE;
+        } else {
+            float wx[S1], wy[S1];
+            const int ix = Shape<P, float>::weights(xi, wx);
+            const int iy = Shape<P, float>::weights(yj, wy);
+            base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
 #pragma unroll
-                for (int k = 2; k < 8; ++k) gout[(size_t)(k + 2) * n + p] = (double)f[k];
+            for (int a = 0; a < S1; ++a) {
+                mine[a] = wx[a];
+                mine[S1 + a] = wy[a];
             }
         }
     }
+    rbase[threadIdx.x] = base;
+    __syncwarp();
+#pragma unroll 1
+    for (int t = 0; t < 2; ++t) {
+        const int k = w0 + 16 * t + (lane >> 1), q = lane & 1;
+        float* r = rec + k * kStride;
+        const int kb = rbase[k];
+        float f[4] = {0, 0, 0, 0};
+        if (kb >= 0) {
+            float wy[S1];
+            int col[S1];
+#pragma unroll
+            for (int b = 0; b < S1; ++b) {
+                wy[b] = r[S1 + b];
+                int gj = (kb & 0xFFFF) + b;
+                if (gj >= g.ny) gj -= g.ny;
+                col[b] = 2 * gj + q;
+            }
+#pragma unroll
+            for (int a = 0; a < S1; ++a) {
+                int gi = (kb >> 16) + a;
+                if (gi >= g.nx) gi -= g.nx;
+                const float4* row = F + (size_t)gi * g.ny * 2;
+                const float wxa = r[a];
+#pragma unroll
+                for (int b = 0; b < S1; ++b) {
+                    const float4 v = __ldg(row + col[b]);
+                    const float w = rmul(wxa, wy[b]);
+                    f[0] = rfma(w, v.x, f[0]);
+                    f[1] = rfma(w, v.y, f[1]);
+                    f[2] = rfma(w, v.z, f[2]);
+                    f[3] = rfma(w, v.w, f[3]);
+                }
+            }
+        }
+        __syncwarp();  // both lanes have read the particle's weights
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r[4 * q + i] = f[i];
+    }
+    __syncwarp();
+    if (base >= 0) {
+        float f[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) f[i] = mine[i];
+        float vxn1, vyn1;
+        push_one(pp, f, p, px, py, vx, vy, vxo, vyo, bad, kin, vxn1, vyn1);
+        if (gout) record_push(gout, gout_short, n, p, px[p], py[p], vxn1, vyn1, f);
+    }
     push_finish(pp, bad, kin, diag, err);
+}
+
+// FP64: the fields and the weights in fixed point.  GB300 issues 2 FP64 operations per clock
+// and SM, so the 128 FP64 multiply-adds of a cubic gather (and the weights) held the pipe for
+// 0.39 ms per 2^20 particles; 32x32+64-bit integer multiply-adds issue at 32 (28 measured).
+//   - A field f with |f| < 2^e (e from the largest value on the mesh, found as the transform
+//     writes it) becomes F = rint(f 2^(58-e)), kept as fh 2^29 + fl, |fl| <= 2^28; a weight
+//     W = rint(w 2^58) = wh 2^29 + wl alike.
+//   - sum W F = (sum wh fh) 2^58 + (sum wh fl + wl fh) 2^29 + sum wl fl: three multiply-adds
+//     a node and field.  The sums are exact: the weights add up to 1, so |sum wh fh| <= 2^58,
+//     and |sum wl fh| <= 25 2^28 2^29 < 2^62.  The last sum is below 25 2^56 of 2^116 and is
+//     dropped.
+//   - The roundings (2^-59 of the field's bound in F, as much in W, the dropped sum 2^-55 at
+//     the very most, 2^-58 typically) are finer than the 2^-53 that FP64 rounds each of its
+//     products and sums to, and than the transform's own error in f, 2^-53 of the largest
+//     value.
+// Integer sums do not depend on their order, and the same bits come out on every path.
+template <int P>
+__global__ void __launch_bounds__(kRowGatherThreads)
+k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* __restrict__ x,
+                  const double* __restrict__ y, double* __restrict__ px,
+                  double* __restrict__ py, const double* __restrict__ vx,
+                  const double* __restrict__ vy, double* __restrict__ vxo,
+                  double* __restrict__ vyo, int64_t n, const int4* __restrict__ F,
+                  const unsigned* __restrict__ fmax, double* __restrict__ gout, int gout_short,
+                  double* __restrict__ diag, unsigned int* __restrict__ err) {
+    constexpr int S1 = P + 1, S2 = S1 * S1;
+    constexpr int kStride = S2 | 1;  // at least the 8 gathered values
+    __shared__ int2 rec[kRowGatherThreads * kStride];
+    __shared__ int rbase[kRowGatherThreads];
+    __shared__ double unit[8];
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    const int64_t p = blockIdx.x * (int64_t)kRowGatherThreads + threadIdx.x;
+    int2* mine = rec + threadIdx.x * kStride;
+    if (threadIdx.x < 8) unit[threadIdx.x] = field_unit(fmax[threadIdx.x]);
+    double kin = 0.0;
+    unsigned bad = 0;
+    int base = -1;
+    if (p < n) {
+        const long long X = __double2ll_rn(rmul(x[p], fg.sx)), Y = __double2ll_rn(rmul(y[p], fg.sy));
+        if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh)) {
+            bad |= ERR_NONFINITE;
+        } else {
+            long long wx[S1], wy[S1];
+            const int ix = fix_weights<P>(X, fg.sh, wx);
+            const int iy = fix_weights<P>(Y, fg.sh, wy);
+            base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
+#pragma unroll
+            for (int a = 0; a < S1; ++a)
+#pragma unroll
+                for (int b = 0; b < S1; ++b)
+                    mine[a * S1 + b] = limbs58((mul62(wx[a], wy[b]) + 8) >> 4);
+        }
+    }
+    rbase[threadIdx.x] = base;
+    __syncthreads();
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+        const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
+        const int2* r = rec + k * kStride;
+        const int kb = rbase[k];
+        long long h0 = 0, m0 = 0, h1 = 0, m1 = 0;
+        if (kb >= 0) {
+            int col[S1];
+#pragma unroll
+            for (int b = 0; b < S1; ++b) {
+                int gj = (kb & 0xFFFF) + b;
+                if (gj >= g.ny) gj -= g.ny;
+                col[b] = 4 * gj + q;
+            }
+#pragma unroll
+            for (int a = 0; a < S1; ++a) {
+                int gi = (kb >> 16) + a;
+                if (gi >= g.nx) gi -= g.nx;
+                const int4* row = F + (size_t)gi * g.ny * 4;
+#pragma unroll
+                for (int b = 0; b < S1; ++b) {
+                    const int4 v = __ldg(row + col[b]);
+                    const int2 w = r[a * S1 + b];
+                    h0 += (long long)w.x * v.x;
+                    m0 += (long long)w.x * v.y;
+                    m0 += (long long)w.y * v.x;
+                    h1 += (long long)w.x * v.z;
+                    m1 += (long long)w.x * v.w;
+                    m1 += (long long)w.y * v.z;
+                }
+            }
+        }
+        __syncwarp();  // the four lanes have read the particle's weights
+        long long* out = reinterpret_cast<long long*>(rec + k * kStride);
+        out[2 * q] = h0 + ((m0 + (1ll << 28)) >> 29);
+        out[2 * q + 1] = h1 + ((m1 + (1ll << 28)) >> 29);
+    }
+    __syncwarp();
+    if (base >= 0) {
+        const long long* got = reinterpret_cast<const long long*>(mine);
+        double f[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) f[i] = rmul((double)got[i], unit[i]);
+        double vxn1, vyn1;
+        push_one(pp, f, p, px, py, vx, vy, vxo, vyo, bad, kin, vxn1, vyn1);
+        if (gout) record_push(gout, gout_short, n, p, px[p], py[p], vxn1, vyn1, f);
+    }
+    push_finish(pp, bad, kin, diag, err);
+}
+
+// The fixed-point fields of k_gather_push_fix from the mesh fields (4 complex a node).
+__global__ void k_fields_to_fix(const double2* __restrict__ G, const unsigned* __restrict__ fmax,
+                                int4* __restrict__ F, int64_t n) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int q = (int)(k & 3);
+        const double2 v = G[k];
+        const int2 a = field_fix(v.x, fmax[2 * q]), b = field_fix(v.y, fmax[2 * q + 1]);
+        F[k] = make_int4(a.x, a.y, b.x, b.y);
+    }
 }
 
 // Gather + push over particles sorted by tile and cell (see sort.cu), FP32 form.
@@ -1624,8 +1867,8 @@ cudaError_t launch_deposit_z(int p, const ParticleGeom& g, const T* x, const T* 
 }
 
 cudaError_t launch_fix128_to_cplx(const longlong2* j, size_t ng, double unscale, double2* out,
-                                  cudaStream_t s) {
-    k_fix128_to_cplx<<<blocks_for((int64_t)ng), kThreads, 0, s>>>(j, ng, unscale, out);
+                                  cudaStream_t s, unsigned* fmax) {
+    k_fix128_to_cplx<<<blocks_for((int64_t)ng), kThreads, 0, s>>>(j, ng, unscale, out, fmax);
     return cudaGetLastError();
 }
 
@@ -1697,14 +1940,56 @@ cudaError_t launch_extract_fix(const longlong2* j, int comp, double scale, doubl
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp, const T* x,
-                               const T* y, T* px, T* py, const T* vx, const T* vy, T* vxo,
-                               T* vyo, int64_t n, const void* f, double* gout, double* diag,
-                               unsigned int* err, cudaStream_t s, bool gout_short) {
+cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp,
+                               const float* x, const float* y, float* px, float* py,
+                               const float* vx, const float* vy, float* vxo, float* vyo,
+                               int64_t n, const void* f, double* gout, double* diag,
+                               unsigned int* err, cudaStream_t s, bool gout_short,
+                               const FixFields*) {
     if (n == 0) return cudaSuccess;
-    GPIC_DISPATCH_P(p, k_gather_push, typed<T>(g), typed<T>(pp), x, y, px, py, vx, vy, vxo, vyo, n,
-                    (const cplx_t<T>*)f, gout, gout_short ? 1 : 0, diag, err)
+    const unsigned blocks = (unsigned)((n + kRowGatherThreads - 1) / kRowGatherThreads);
+#define GPIC_GPAIR(PP)                                                                          \
+    k_gather_push_pair<PP><<<blocks, kRowGatherThreads, 0, s>>>(                                \
+        typed<float>(g), typed<float>(pp), x, y, px, py, vx, vy, vxo, vyo, n, (const float4*)f, \
+        gout, gout_short ? 1 : 0, diag, err)
+    switch (p) {
+        case 2: GPIC_GPAIR(2); break;
+        case 3: GPIC_GPAIR(3); break;
+        case 4: GPIC_GPAIR(4); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef GPIC_GPAIR
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp,
+                               const double* x, const double* y, double* px, double* py,
+                               const double* vx, const double* vy, double* vxo, double* vyo,
+                               int64_t n, const void* f, double* gout, double* diag,
+                               unsigned int* err, cudaStream_t s, bool gout_short,
+                               const FixFields* fix) {
+    using T = double;
+    if (n == 0) return cudaSuccess;
+    if (!fix) {
+        GPIC_DISPATCH_P(p, k_gather_push, typed<T>(g), typed<T>(pp), x, y, px, py, vx, vy, vxo,
+                        vyo, n, (const double2*)f, gout, gout_short ? 1 : 0, diag, err)
+        return cudaGetLastError();
+    }
+    const int64_t nc = 4 * (int64_t)g.nx * g.ny;
+    k_fields_to_fix<<<blocks_for(nc), kThreads, 0, s>>>((const double2*)f, fix->fmax,
+                                                        (int4*)fix->f, nc);
+    const unsigned blocks = (unsigned)((n + kRowGatherThreads - 1) / kRowGatherThreads);
+#define GPIC_GFIX(PP)                                                                      \
+    k_gather_push_fix<PP><<<blocks, kRowGatherThreads, 0, s>>>(                            \
+        typed<T>(g), fix_geom(g), typed<T>(pp), x, y, px, py, vx, vy, vxo, vyo, n,         \
+        (const int4*)fix->f, fix->fmax, gout, gout_short ? 1 : 0, diag, err)
+    switch (p) {
+        case 2: GPIC_GFIX(2); break;
+        case 3: GPIC_GFIX(3); break;
+        case 4: GPIC_GFIX(4); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef GPIC_GFIX
     return cudaGetLastError();
 }
 
@@ -1896,10 +2181,6 @@ cudaError_t launch_extract(const void* src, int stride, int comp, double scale, 
                                                    const T*, T*, T*, T*, const int32_t*,        \
                                                    const SpeciesParams&, int64_t, const void*,  \
                                                    unsigned int*, cudaStream_t);                \
-    template cudaError_t launch_gather_push<T>(int, const ParticleGeom&, const PushParams&,     \
-                                               const T*, const T*, T*, T*, const T*, const T*,  \
-                                               T*, T*, int64_t, const void*, double*, double*,  \
-                                               unsigned int*, cudaStream_t, bool);                    \
     template cudaError_t launch_init_particles<T>(int, const ParticleGeom&, const PushParams&,  \
                                                   T*, T*, T*, T*, const T*, const T*, T*, T*,   \
                                                   int64_t, const void*, unsigned int*,          \

@@ -300,6 +300,12 @@ pic_status alloc_state(pic_handle* h) {
     }
     CK(dalloc(h, &h->F4, 4 * h->ng * cs));
     CK(dalloc(h, &h->G, 4 * h->ng * cs));
+    // The FP64 gather in fixed point, where converting the mesh fields (16 FP64 operations a
+    // node) is small beside what it saves (about 200 a particle).
+    if (!h->fp32 && h->vdim == 2 && h->spp.n == 0 && h->n >= (int64_t)(h->ng / 8)) {
+        CK(dalloc(h, &h->fixf.f, 4 * h->ng * cs));
+        CK(dalloc(h, (void**)&h->fixf.fmax, 8 * sizeof(unsigned)));
+    }
     CK(dalloc(h, &h->E, h->ng * cs));
     CK(dalloc(h, &h->tmp, h->ng * cs));
     CK(dalloc(h, (void**)&h->tmpd, h->ng * sizeof(double)));
@@ -835,7 +841,7 @@ pic_status pic_field_solve(pic_handle* h) {
                                         h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s));
     } else {  // the 128-bit sums to FP64, then the transform
         CK(launch_fix128_to_cplx((const longlong2*)h->J, h->ng, h->fix64_unscale_j,
-                                 (double2*)h->tmp, h->s));
+                                 (double2*)h->tmp, h->s, h->fixf.fmax));
         CK(launch_fft_y<double>(h->tmp, h->Z, h->nx, h->ny, 1, h->fy, h->twy, -1, 0, h->s));
         h->launches_now += 1;
     }
@@ -930,7 +936,8 @@ pic_status pic_field_solve(pic_handle* h) {
         cudaError_t r = cudaSuccess;
         if (!fused) r = launch_fft_x<T>(h->F4, h->F4, h->nx, h->ny, 4, h->fx, h->twx, +1, h->s);
         if (r != cudaSuccess) return r;
-        return launch_fft_y<T>(h->F4, h->G, h->nx, h->ny, 4, h->fy, h->twy, +1, 1, h->s);
+        return launch_fft_y<T>(h->F4, h->G, h->nx, h->ny, 4, h->fy, h->twy, +1, 1, h->s,
+                               h->fixf.fmax);
     }));
     h->launches_now += fused ? 3 : 5;
 
@@ -1045,12 +1052,14 @@ pic_status gather_push_step(pic_handle* h, bool fuse, bool defer) {
         TimedScope ts(h, PIC_KT_GATHER);
         CK(by_prec(h, [&](auto t) {
             using T = decltype(t);
-            return launch_gather_push<T>(h->p, h->geom, pp, (const T*)h->x, (const T*)h->y,
-                                         (T*)h->px, (T*)h->py, (const T*)h->v[h->vcur][0],
-                                         (const T*)h->v[h->vcur][1], (T*)h->v[vo][0],
-                                         (T*)h->v[vo][1], h->n, h->G, h->gather_out, h->diag,
-                                         h->err, h->s, h->gather_out_short);
+            return launch_gather_push(h->p, h->geom, pp, (const T*)h->x, (const T*)h->y,
+                                      (T*)h->px, (T*)h->py, (const T*)h->v[h->vcur][0],
+                                      (const T*)h->v[h->vcur][1], (T*)h->v[vo][0],
+                                      (T*)h->v[vo][1], h->n, h->G, h->gather_out, h->diag,
+                                      h->err, h->s, h->gather_out_short,
+                                      h->fixf.f ? &h->fixf : nullptr);
         }));
+        if (h->fixf.f) h->launches_now += 1;
     }
     h->vcur = vo;
     h->launches_now += 1;

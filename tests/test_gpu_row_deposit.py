@@ -74,3 +74,63 @@ def test_row_deposit(p, nx, ny, n, one_cell):
             for have, q in zip(j, (ix, iy)):
                 want = np.asarray(q, dtype=np.float64) * (1.0 / scale * (weight * -1.0 / area))
                 assert np.array_equal(have, want)
+
+
+def _gather(x, y, grid, lx, ly, p):
+    nx, ny = grid.shape
+    ix, wx = _weights((x * (1.0 / (lx / nx))).astype(np.longdouble), p)
+    iy, wy = _weights((y * (1.0 / (ly / ny))).astype(np.longdouble), p)
+    return sum(grid.astype(np.longdouble)[(ix - a) % nx, (iy - b) % ny] * wx[a] * wy[b]
+               for a in range(p + 1) for b in range(p + 1))
+
+
+@pytest.mark.parametrize("nx,ny,n", [(8, 8, 7), (8, 8, 8), (16, 12, 33), (8, 1024, 1025),
+                                     (54, 36, 4099)])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_row_gather_fp64(p, nx, ny, n):
+    """The momentum update of one step from the mesh fields the library reports, against the
+    gather in extended precision; counts on both sides of the fixed-point form's rule (n below
+    nx ny / 8 takes the FP64 arithmetic).  A gathered value is within 2^-51 of the field's
+    largest: at most 25 weights off by 2^-58, 2^-58 of the bound (up to twice the largest) for
+    the fields' rounding and as much for the result's, 25 2^-60 of it for the dropped sum, and
+    2^-53 from the conversion; FP64's own roundings are of that size too.  The force's three
+    terms (|v*| < 3 c) and the update add 2^-53 of each."""
+    rng = np.random.default_rng(77 * p + n)
+    lx, ly = 1.0, ny / nx
+    dt = 0.3 * min(lx / nx, ly / ny)
+    x, y = rng.uniform(0, lx, n), rng.uniform(0, ly, n)
+    vx, vy = rng.uniform(-0.6, 0.6, n), rng.uniform(-0.6, 0.6, n)
+    cfg = pic.make_config(nx, ny, lx, ly, dt, p=p, weight=lx * ly / n)
+    with pic.Simulation(cfg, x, y, vx, vy) as sim:
+        sim.step(1)
+        before = sim.particles()
+        sim.step(1)
+        after = sim.particles()
+        names = ("dphidx", "dphidy", "daxdx", "daxdy", "daydx", "daydy")
+        f = {k: sim.field(k) for k in names}
+    g = {k: _gather(after["x"], after["y"], f[k], lx, ly, p) for k in names}
+    vs = [2 * before[k].astype(np.longdouble) - before[k + "_old"] for k in ("vx", "vy")]
+    for c, key in (("x", "px"), ("y", "py")):
+        terms = (g["dphid" + c], g["daxd" + c] * vs[0], g["dayd" + c] * vs[1])
+        want = before[key] - dt * (-terms[0] + terms[1] + terms[2])
+        peak = sum(np.max(np.abs(f[k])) for k in ("dphid" + c, "daxd" + c, "dayd" + c))
+        bound = dt * (3 * 2.0 ** -51 * peak + 2.0 ** -51 * sum(np.abs(t) for t in terms))
+        assert np.all(np.abs(after[key] - want) <= bound + 2.0 ** -52 * np.abs(want))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 1000])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_row_gather_fp32_is_the_sorted_gather(p, n):
+    """The FP32 gather's lane pairs against the tiled gather of the sorted form: same bits."""
+    rng = np.random.default_rng(7 * p + n)
+    x, y = rng.uniform(0, 1.0, n), rng.uniform(0, 0.75, n)
+    vx, vy = rng.uniform(-0.6, 0.6, n), rng.uniform(-0.6, 0.6, n)
+    out = []
+    for sort in (0, 1):
+        cfg = pic.make_config(32, 24, 1.0, 0.75, 0.01, p=p, weight=0.75 / n,
+                              precision=pic.FP32_FIX64, sort_interval=sort)
+        with pic.Simulation(cfg, x, y, vx, vy) as sim:
+            sim.step(3)
+            out.append(sim.particles())
+    for k in out[0]:
+        assert np.array_equal(out[0][k], out[1][k]), k
