@@ -291,12 +291,16 @@ template <typename T>
 cudaError_t launch_wrap_positions(T* x, T* y, int64_t n, double lx, double ly, cudaStream_t s);
 template <typename Tsrc, typename Tdst>
 cudaError_t launch_convert(const Tsrc* src, Tdst* dst, int64_t n, cudaStream_t s);
-template <typename T>
-cudaError_t launch_scatter_by_id(const T* src, const int32_t* id, double* dst, int64_t n,
-                                 cudaStream_t s);
-// dst[id[k]] = src[k] for int32 values (the species indices of a sorted handle).
-cudaError_t launch_scatter_by_id_i32(const int32_t* src, const int32_t* id, int32_t* dst,
-                                     int64_t n, cudaStream_t s);
+// Read-back: inv[id[k]] = k, and dst[j][i] = src[j][inv[i]] (inv NULL: src[j][i]).
+constexpr int kReadArrays = 8;
+struct ReadArrays {
+    const void* src[kReadArrays];
+    void* dst[kReadArrays];
+    int count;
+};
+cudaError_t launch_invert_ids(const int32_t* id, int32_t* inv, int64_t n, cudaStream_t s);
+template <typename Ts, typename Td>
+cudaError_t launch_read_arrays(const ReadArrays& r, const int32_t* inv, int64_t n, cudaStream_t s);
 
 // Tiles for the particle sort and the shared-memory deposit: t x t cells per tile,
 // ntx x nty tiles; a CTA accumulates into an rx x ry node region starting `halo` nodes

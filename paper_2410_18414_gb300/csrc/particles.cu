@@ -1570,13 +1570,31 @@ __global__ void k_convert(const Ts* __restrict__ s, Td* __restrict__ d, int64_t 
         d[p] = (Td)s[p];
 }
 
-template <typename T>
-__global__ void k_scatter_by_id(const T* __restrict__ s, const int32_t* __restrict__ id,
-                                double* __restrict__ d, int64_t n) {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        int32_t k = id[p];
-        if (k >= 0 && k < n) d[k] = (double)s[p];
+// The read-back of sorted particles in the caller's order.  inv[id[k]] = k, then particle i
+// of the caller is at k = inv[i]: the 4-byte random accesses are reads of arrays that L2
+// mostly holds and the FP64 writes coalesce (scattering the values instead wrote one 8-byte
+// piece of a sector at a time: 0.75 ms per array of 26 M particles).
+__global__ void k_invert_ids(const int32_t* __restrict__ id, int32_t* __restrict__ inv, int64_t n) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = id[k];
+        if (i >= 0 && i < n) inv[i] = (int32_t)k;
+    }
+}
+// dst[j][i] = src[j][inv[i]] (inv NULL: src[j][i]) for the `count` arrays of r.
+template <typename Ts, typename Td>
+__global__ void k_read_arrays(ReadArrays r, const int32_t* __restrict__ inv, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = inv ? (int64_t)__ldcs(inv + i) : i;
+        if ((uint64_t)k >= (uint64_t)n) continue;
+        Ts v[kReadArrays];
+#pragma unroll
+        for (int j = 0; j < kReadArrays; ++j)
+            if (j < r.count) v[j] = __ldg((const Ts*)r.src[j] + k);
+#pragma unroll
+        for (int j = 0; j < kReadArrays; ++j)
+            if (j < r.count) __stcs((Td*)r.dst[j] + i, (Td)v[j]);
     }
 }
 
@@ -2135,27 +2153,35 @@ cudaError_t launch_convert(const Ts* src, Td* dst, int64_t n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_scatter_by_id(const T* src, const int32_t* id, double* dst, int64_t n,
-                                 cudaStream_t s) {
+cudaError_t launch_invert_ids(const int32_t* id, int32_t* inv, int64_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    k_scatter_by_id<T><<<blocks_for(n), kThreads, 0, s>>>(src, id, dst, n);
+    k_invert_ids<<<blocks_for(n), kThreads, 0, s>>>(id, inv, n);
     return cudaGetLastError();
 }
 
-__global__ void k_scatter_by_id_i32(const int32_t* __restrict__ src, const int32_t* __restrict__ id,
-                                    int32_t* __restrict__ dst, int64_t n) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x)
-        dst[id[k]] = src[k];
-}
-
-cudaError_t launch_scatter_by_id_i32(const int32_t* src, const int32_t* id, int32_t* dst,
-                                     int64_t n, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    k_scatter_by_id_i32<<<blocks_for(n), kThreads, 0, s>>>(src, id, dst, n);
+template <typename Ts, typename Td>
+cudaError_t launch_read_arrays(const ReadArrays& r, const int32_t* inv, int64_t n, cudaStream_t s) {
+    if (n == 0 || r.count == 0) return cudaSuccess;
+    // all arrays in one pass while L2 (129 MB) can hold what is read at random, else one at a
+    // time: 26 M particles' arrays are 105 MB each
+    const int each = inv && (int64_t)r.count * n * (int64_t)sizeof(Ts) > (64ll << 20) ? 1 : r.count;
+    for (int j = 0; j < r.count; j += each) {
+        ReadArrays q{};
+        q.count = each;
+        for (int i = 0; i < each; ++i) {
+            q.src[i] = r.src[j + i];
+            q.dst[i] = r.dst[j + i];
+        }
+        k_read_arrays<Ts, Td><<<blocks_for(n), kThreads, 0, s>>>(q, inv, n);
+    }
     return cudaGetLastError();
 }
+template cudaError_t launch_read_arrays<float, double>(const ReadArrays&, const int32_t*, int64_t,
+                                                       cudaStream_t);
+template cudaError_t launch_read_arrays<double, double>(const ReadArrays&, const int32_t*, int64_t,
+                                                        cudaStream_t);
+template cudaError_t launch_read_arrays<int32_t, int32_t>(const ReadArrays&, const int32_t*,
+                                                          int64_t, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_extract(const void* src, int stride, int comp, double scale, double* dst,
@@ -2185,8 +2211,6 @@ cudaError_t launch_extract(const void* src, int stride, int comp, double scale, 
                                                   T*, T*, T*, T*, const T*, const T*, T*, T*,   \
                                                   int64_t, const void*, unsigned int*,          \
                                                   cudaStream_t);                                \
-    template cudaError_t launch_scatter_by_id<T>(const T*, const int32_t*, double*, int64_t,    \
-                                                 cudaStream_t);                                 \
     template cudaError_t launch_extract<T>(const void*, int, int, double, double*, int64_t,     \
                                            cudaStream_t);                                       \
     template cudaError_t launch_wrap_positions<T>(T*, T*, int64_t, double, double, cudaStream_t); \

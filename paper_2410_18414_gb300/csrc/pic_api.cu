@@ -1419,34 +1419,69 @@ pic_status pic_get_field(pic_handle* h, int32_t which, double* dst) {
     return check_device_error(h);
 }
 
+}  // extern "C"
+
+namespace {
+
+// Whether a kernel of the handle's device may write FP64 (or int32) values straight to dst.
+bool writable_in_place(const pic_handle* h, const void* dst) {
+    if (reinterpret_cast<uintptr_t>(dst) % sizeof(double) != 0) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+        cudaGetLastError();  // a host pointer is not an error of the context
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
+// Copies m particle arrays (Ts on the device) to dst (Td, device or host) in the caller's
+// order: one kernel for the destinations on this device, the others through the staging
+// buffer one after another (ordered by the stream).
+template <typename Ts, typename Td>
+pic_status read_arrays(pic_handle* h, const void* const* src, void* const* dst, int m) {
+    if (h->n == 0) return PIC_OK;
+    const int32_t* inv = nullptr;
+    if (h->sorting) {  // the order given to pic_init; the sort's keys are not needed now
+        CK(launch_invert_ids(h->id, h->keys, h->n, h->s));
+        inv = h->keys;
+    }
+    ReadArrays direct{};
+    for (int i = 0; i < m; ++i) {
+        if (!dst[i]) continue;
+        if (writable_in_place(h, dst[i])) {
+            direct.src[direct.count] = src[i];
+            direct.dst[direct.count++] = dst[i];
+            continue;
+        }
+        const void* from = src[i];
+        if (inv || sizeof(Ts) != sizeof(Td)) {
+            ReadArrays one{};
+            one.src[0] = src[i];
+            one.dst[0] = h->stage;
+            one.count = 1;
+            CK((launch_read_arrays<Ts, Td>(one, inv, h->n, h->s)));
+            from = h->stage;
+        }
+        CK(cudaMemcpyAsync(dst[i], from, (size_t)h->n * sizeof(Td), cudaMemcpyDefault, h->s));
+    }
+    CK((launch_read_arrays<Ts, Td>(direct, inv, h->n, h->s)));
+    return PIC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 pic_status pic_read_particles(pic_handle* h, double* x, double* y, double* px, double* py,
                               double* vx, double* vy, double* vx_old, double* vy_old) {
     if (!h) return fail(nullptr, PIC_ERR_INVALID_ARG, "NULL handle");
     if (h->phase != 0) return fail(h, PIC_ERR_STATE, "pic_read_particles inside a step");
     const void* src[8] = {h->x, h->y, h->px, h->py, h->v[h->vcur][0], h->v[h->vcur][1],
                           h->v[1 - h->vcur][0], h->v[1 - h->vcur][1]};
-    double* dst[8] = {x, y, px, py, vx, vy, vx_old, vy_old};
-    const size_t nb = (size_t)h->n * sizeof(double);
-    for (int i = 0; i < 8; ++i) {
-        if (!dst[i] || h->n == 0) continue;
-        if (h->sorting) {  // restore the order given to pic_init
-            CK(by_prec(h, [&](auto t) {
-                using T = decltype(t);
-                return launch_scatter_by_id<T>((const T*)src[i], h->id, h->stage, h->n, h->s);
-            }));
-            CK(cudaMemcpyAsync(dst[i], h->stage, nb, cudaMemcpyDefault, h->s));
-            CK(cudaStreamSynchronize(h->s));
-            continue;
-        }
-        if (h->fp32) {
-            CK(launch_convert<float, double>((const float*)src[i], h->stage, h->n, h->s));
-            CK(cudaMemcpyAsync(dst[i], h->stage, nb, cudaMemcpyDefault, h->s));
-            CK(cudaStreamSynchronize(h->s));  // the staging buffer is reused
-        } else {
-            CK(cudaMemcpyAsync(dst[i], src[i], nb, cudaMemcpyDefault, h->s));
-        }
-    }
-    return check_device_error(h);
+    void* dst[8] = {x, y, px, py, vx, vy, vx_old, vy_old};
+    const pic_status st = h->fp32 ? read_arrays<float, double>(h, src, dst, 8)
+                                  : read_arrays<double, double>(h, src, dst, 8);
+    return st != PIC_OK ? st : check_device_error(h);
 }
 
 pic_status pic_read_particles_z(pic_handle* h, double* pz, double* vz, double* vz_old,
@@ -1456,38 +1491,16 @@ pic_status pic_read_particles_z(pic_handle* h, double* pz, double* vz, double* v
     if ((pz || vz || vz_old) && h->vdim != 3)
         return fail(h, PIC_ERR_STATE, "no z components: the handle is 2D-2V");
     if (species && h->spp.n == 0) return fail(h, PIC_ERR_STATE, "the handle has no species table");
-    const size_t nb = (size_t)h->n * sizeof(double);
     const void* src[3] = {h->pz, h->vz[h->vcur], h->vz[1 - h->vcur]};
-    double* dst[3] = {pz, vz, vz_old};
-    for (int i = 0; i < 3 && h->n > 0; ++i) {
-        if (!dst[i]) continue;
-        if (h->sorting) {  // restore the order given to pic_init
-            CK(by_prec(h, [&](auto t) {
-                using T = decltype(t);
-                return launch_scatter_by_id<T>((const T*)src[i], h->id, h->stage, h->n, h->s);
-            }));
-            CK(cudaMemcpyAsync(dst[i], h->stage, nb, cudaMemcpyDefault, h->s));
-            CK(cudaStreamSynchronize(h->s));
-            continue;
-        }
-        if (h->fp32) {
-            CK(launch_convert<float, double>((const float*)src[i], h->stage, h->n, h->s));
-            CK(cudaMemcpyAsync(dst[i], h->stage, nb, cudaMemcpyDefault, h->s));
-            CK(cudaStreamSynchronize(h->s));  // the staging buffer is reused
-        } else {
-            CK(cudaMemcpyAsync(dst[i], src[i], nb, cudaMemcpyDefault, h->s));
-        }
-    }
-    if (species && h->n > 0) {
-        const int32_t* from = h->species;
-        if (h->sorting) {  // restore the order given to pic_init (in the staging buffer)
-            CK(launch_scatter_by_id_i32(h->species, h->id, (int32_t*)h->stage, h->n, h->s));
-            from = (const int32_t*)h->stage;
-        }
-        CK(cudaMemcpyAsync(species, from, (size_t)h->n * sizeof(int32_t), cudaMemcpyDefault,
-                           h->s));
-    }
-    return check_device_error(h);
+    void* dst[3] = {pz, vz, vz_old};
+    pic_status st = PIC_OK;
+    if (pz || vz || vz_old)
+        st = h->fp32 ? read_arrays<float, double>(h, src, dst, 3)
+                     : read_arrays<double, double>(h, src, dst, 3);
+    const void* ssrc[1] = {h->species};
+    void* sdst[1] = {species};
+    if (st == PIC_OK && species) st = read_arrays<int32_t, int32_t>(h, ssrc, sdst, 1);
+    return st != PIC_OK ? st : check_device_error(h);
 }
 
 pic_status pic_sync(pic_handle* h) {
