@@ -23,9 +23,9 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// The largest magnitudes of four lines of m complex values (rows of the four arrays, array
-// after array), as high words, into fmax[8] (re, im of each array).
-__device__ __forceinline__ void collect_max(const double2* res, int m, unsigned* fmax) {
+// The largest magnitudes of four lines of m complex values as high words into top[8] (shared,
+// zeroed; re, im of each line).
+__device__ __forceinline__ void collect_max(const double2* res, int m, unsigned* top) {
     const int b = threadIdx.x & 3;
     unsigned re = 0, im = 0;
     for (int e = threadIdx.x >> 2; e < m; e += blockDim.x >> 2) {
@@ -37,11 +37,9 @@ __device__ __forceinline__ void collect_max(const double2* res, int m, unsigned*
         re = max(re, __shfl_xor_sync(0xffffffffu, re, o));
         im = max(im, __shfl_xor_sync(0xffffffffu, im, o));
     }
-    // most CTAs find a value as large already there and leave the word alone
     if ((threadIdx.x & 31) < 4) {
-        volatile const unsigned* seen = fmax;
-        if (re > seen[2 * b]) atomicMax(fmax + 2 * b, re);
-        if (im > seen[2 * b + 1]) atomicMax(fmax + 2 * b + 1, im);
+        atomicMax(top + 2 * b, re);
+        atomicMax(top + 2 * b + 1, im);
     }
 }
 
@@ -51,7 +49,7 @@ __global__ void __launch_bounds__(kThreads)
 k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, int ny, int nb,
         int rows, FftDesc d, const cplx_t<T>* __restrict__ tw, int sign, int interleave,
         const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear,
-        unsigned* __restrict__ fmax) {
+        int4* __restrict__ ffix, unsigned* __restrict__ ftop) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* b0 = reinterpret_cast<C*>(smem_raw);
@@ -59,6 +57,8 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     C* b1 = b0 + lines * ny;
     C* tws = b1 + lines * ny;  // twiddles, staged before the wait (they are constant)
     stage_twiddles(tw, tws, ny);
+    __shared__ unsigned top[8];
+    if (threadIdx.x < 8) top[threadIdx.x] = 0;
     const int i0 = blockIdx.x * rows;
     const size_t plane = (size_t)nx * ny;
     griddep_wait();  // the input is the previous kernel's output
@@ -70,7 +70,14 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
         if (fix_in) {  // fixed-point current sums, converted on load
             const longlong2 v = fix_in[src];
             if (clear) clear[src] = longlong2{0, 0};  // the other buffer, for the next deposit
-            b0[e] = mk<C>((double)v.x * unscale, (double)v.y * unscale);
+            if constexpr (sizeof(T) == 4) {
+                b0[e] = mk<C>((double)v.x * unscale, (double)v.y * unscale);
+            } else {  // 128-bit sums: the high words follow the low ones
+                const longlong2 hi = fix_in[plane + src];
+                if (clear) clear[plane + src] = longlong2{0, 0};
+                b0[e] = make_double2(fix128_value(hi.x, (unsigned long long)v.x, unscale),
+                                     fix128_value(hi.y, (unsigned long long)v.y, unscale));
+            }
         } else {
             b0[e] = in[src];
         }
@@ -78,8 +85,22 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     __syncthreads();
     C* res = run_passes(b0, b1, d, lines, (const C*)tws, sign);
     if (interleave) {
-        if constexpr (sizeof(T) == 8) {  // a thread's outputs are all of array threadIdx.x % 4
-            if (fmax) collect_max(res, rows * ny, fmax);
+        if constexpr (sizeof(T) == 8) {
+            if (ffix) {  // nb = 4, one row: the fixed-point fields of the row beside the FP64 ones
+                collect_max(res, ny, top);
+                __syncthreads();
+                if (threadIdx.x < 8) ftop[8 * i0 + threadIdx.x] = top[threadIdx.x];
+                const int b = threadIdx.x & 3;
+                const int er = row_exponent(top[2 * b]), ei = row_exponent(top[2 * b + 1]);
+                for (int e = threadIdx.x; e < 4 * ny; e += blockDim.x) {
+                    const double2 v = res[b * ny + (e >> 2)];
+                    const int2 re = field_fix(v.x, er), im = field_fix(v.y, ei);
+                    const size_t o = (size_t)i0 * ny * 4 + e;
+                    out[o] = v;
+                    ffix[o] = make_int4(re.x, re.y, im.x, im.y);
+                }
+                return;
+            }
         }
         for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
             int b = e % nb, t = e / nb;
@@ -142,7 +163,7 @@ template <typename T>
 static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                               const void* tw, int sign, int interleave, const longlong2* fix_in,
                               double unscale, longlong2* clear, cudaStream_t s,
-                              unsigned* fmax = nullptr) {
+                              const FixFields* fix = nullptr) {
     using C = cplx_t<T>;
     const size_t per_line = 2 * (size_t)ny * sizeof(C);
     const size_t tw_bytes = (size_t)ny * sizeof(C);
@@ -156,15 +177,16 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
     if (e != cudaSuccess) return e;
     return launch_pdl(k_fft_y<T>, dim3(nx / rows), dim3(kThreads), smem, s, (const C*)in, (C*)out,
                       nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear,
-                      fmax);
+                      fix ? (int4*)fix->f : nullptr, fix ? fix->top : nullptr);
 }
 
 template <typename T>
 cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                          const void* tw, int sign, int interleave, cudaStream_t s,
-                         unsigned* fmax) {
+                         const FixFields* fix) {
+    if (fix && (sizeof(T) != 8 || nb != 4 || !interleave)) return cudaErrorInvalidValue;
     return fft_y_impl<T>(in, out, nx, ny, nb, d, tw, sign, interleave, nullptr, 0.0, nullptr, s,
-                         fmax);
+                         fix);
 }
 
 template <typename T>
@@ -199,9 +221,9 @@ cudaError_t launch_twiddles(void* tw, int n, cudaStream_t s) {
 }
 
 template cudaError_t launch_fft_y<double>(const void*, void*, int, int, int, const FftDesc&,
-                                          const void*, int, int, cudaStream_t, unsigned*);
+                                          const void*, int, int, cudaStream_t, const FixFields*);
 template cudaError_t launch_fft_y<float>(const void*, void*, int, int, int, const FftDesc&,
-                                         const void*, int, int, cudaStream_t, unsigned*);
+                                         const void*, int, int, cudaStream_t, const FixFields*);
 template cudaError_t launch_fft_x<double>(const void*, void*, int, int, int, const FftDesc&,
                                           const void*, int, cudaStream_t);
 template cudaError_t launch_fft_x<float>(const void*, void*, int, int, int, const FftDesc&,

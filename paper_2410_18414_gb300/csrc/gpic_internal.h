@@ -112,13 +112,18 @@ enum StepperKind { K_BDF = 0, K_CDF2 = 1, K_DIRK = 2 };
 // ---------------------------------------------------------------- launchers
 
 // In-place or out-of-place 1-D transforms of nb arrays of shape (nx, ny).
-// Along y (contiguous); out_interleave != 0 writes out[(i*ny + j)*nb + b].  fmax (FP64,
-// interleaved with nb = 4; may be NULL) gathers the largest magnitude of each of the eight
-// real outputs, as the high word of its value.
+// The FP64 path's gather fields in fixed point: per node four int4 (the limbs of two fields
+// each), and per mesh row the high words of the eight fields' largest magnitudes.
+struct FixFields {
+    void* f;
+    unsigned* top;
+};
+// Along y (contiguous); out_interleave != 0 writes out[(i*ny + j)*nb + b].  fix (FP64,
+// interleaved with nb = 4; may be NULL): the outputs in fixed point as well.
 template <typename T>
 cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                          const void* twiddle, int sign, int out_interleave, cudaStream_t s,
-                         unsigned* fmax = nullptr);
+                         const FixFields* fix = nullptr);
 // Forward transform along y of the fixed-point current (converted on load); zeroes
 // `clear` (same shape, may be NULL) on the way, the buffer the next deposit sums into.
 template <typename T>
@@ -218,10 +223,9 @@ cudaError_t launch_deposit_charge_fix128(int p, const ParticleGeom& g, const dou
                                          double scale, unsigned int* err, cudaStream_t s,
                                          const int32_t* sp = nullptr,
                                          const SpeciesParams* spp = nullptr);
-// out[k] = the 128-bit sums (x, y) of node k times unscale, as complex FP64; fmax (may be
-// NULL): eight words set to 0 for launch_fft_y.
+// out[k] = the 128-bit sums (x, y) of node k times unscale, as complex FP64.
 cudaError_t launch_fix128_to_cplx(const longlong2* j, size_t ng, double unscale, double2* out,
-                                  cudaStream_t s, unsigned* fmax = nullptr);
+                                  cudaStream_t s);
 // 2D-3V: J_z of the moved particles (x^{n+1}, v_z^n) into the .x parts of jz: int64 sums
 // (FP32 form, float `scale`) or 128-bit sums (FP64, layout of launch_move_deposit_fix128).
 template <typename T>
@@ -245,13 +249,6 @@ struct PushParams {
     int diag;
 };
 
-// The fixed-point gather fields of the FP64 path and the largest magnitude of each (the high
-// word of its FP64 value).
-struct FixFields {
-    void* f;
-    unsigned* fmax;
-};
-
 // gout (FP64, may be NULL): the adjoint's record of the step, ten arrays of n: P^{n+1}
 // (x, y), v^{n+1} (x, y), then the gathered Ax, Ay, dAx/dx, dAx/dy, dAy/dx, dAy/dy.
 cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp,
@@ -260,8 +257,7 @@ cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& p
                                int64_t n, const void* fields4, double* gout, double* diag,
                                unsigned int* err, cudaStream_t s, bool gout_short,
                                const FixFields* fix);
-// FP64: with fix, the gather runs in fixed point on fix->f (nx ny 4 int4, written here from
-// fields4 and the maxima fix->fmax that launch_fft_y left).
+// FP64: with fix, the gather runs in fixed point on the fields that launch_fft_y left there.
 cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp,
                                const double* x, const double* y, double* px, double* py,
                                const double* vx, const double* vy, double* vx_old,

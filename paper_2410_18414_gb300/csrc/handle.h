@@ -47,7 +47,7 @@ struct pic_handle {
     // grid buffers
     double2* J = nullptr;    // deposit accumulator (sum_p v W): 128-bit sums (FP64 path:
                              // longlong2 low words, then high words), or int64 pairs (FP32 form)
-    double2* Jalt = nullptr; // FP32 form: the other int64 buffer, zeroed by the row transform
+    double2* Jalt = nullptr; // the other such buffer, zeroed by the row transform
     // FP32 form: a contribution a is summed as round(a * fix_scale_*) in int64
     float fix_scale_j = 0.f, fix_scale_q = 0.f;
     double fix_unscale_j = 0.0, fix_unscale_q = 0.0;

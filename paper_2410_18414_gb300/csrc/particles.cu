@@ -170,19 +170,6 @@ struct AccFix {
     }
 };
 
-// hi 2^64 + lo (two's complement over 128 bits) times unscale, rounded to FP64: the
-// magnitude is exact below 2^64 before its one rounding, and rounded twice above.
-__device__ __forceinline__ double fix128_value(long long hi, unsigned long long lo,
-                                               double unscale) {
-    const bool neg = hi < 0;
-    if (neg) {
-        lo = ~lo + 1ull;
-        hi = ~hi + (lo == 0ull ? 1ll : 0ll);
-    }
-    const double m = fma((double)hi, 18446744073709551616.0, (double)lo);
-    return (neg ? -m : m) * unscale;
-}
-
 // ------------------------------------------------------------ row deposit --------
 //
 // Deposits over particles in any order.  A warp takes 32 particles, one a lane: move, weights
@@ -414,6 +401,8 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
         wb[q] = r / kNC;
         wc[q] = r - wb[q] * kNC;
     }
+    griddep_wait();
+    griddep_launch();
     for (int64_t p0 = (blockIdx.x * (int64_t)kRowThreads + w0); p0 < n;
          p0 += (int64_t)gridDim.x * kRowThreads) {
         const int64_t p = p0 + lane;
@@ -505,11 +494,9 @@ __global__ void k_fix_to_cplx(const longlong2* __restrict__ J, double unscale,
     }
 }
 
-// FP64 path: the 128-bit sums of RowFix128 to complex FP64 values, times `unscale`; fmax
-// (optional): the eight field maxima that this step's transform collects, set to 0.
+// FP64 path: the 128-bit sums of RowFix128 to complex FP64 values, times `unscale`.
 __global__ void k_fix128_to_cplx(const longlong2* __restrict__ J, size_t ng, double unscale,
-                                 double2* __restrict__ out, unsigned* __restrict__ fmax) {
-    if (fmax && blockIdx.x == 0 && threadIdx.x < 8) fmax[threadIdx.x] = 0;
+                                 double2* __restrict__ out) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < (int64_t)ng;
          k += (int64_t)gridDim.x * blockDim.x) {
         const longlong2 lo = J[k], hi = J[ng + k];
@@ -621,28 +608,8 @@ __device__ __forceinline__ void record_push(double* __restrict__ gout, int gout_
     }
 }
 
-// Fixed-point fields: fmax holds the high word of the largest |f| on the mesh, which gives
-// the exponent e with |f| < 2^e (bounded below so that the scales stay finite).  A field that
-// is not finite somewhere has no scale: its gathered values are NaN.
-__device__ __forceinline__ int field_exponent(unsigned fmax) {
-    return max((int)(fmax >> 20) - 1022, -900);
-}
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-__device__ __forceinline__ double field_unit(unsigned fmax) {
-    return fmax >= 0x7ff00000u ? __hiloint2double(0x7ff80000, 0) : pow2(field_exponent(fmax) - 58);
-}
-// v in [-2^58, 2^58] as (v.x 2^29 + v.y), |v.y| <= 2^28
-__device__ __forceinline__ int2 limbs58(long long v) {
-    const int lo = (int)((unsigned)v << 3) >> 3;
-    return make_int2((int)((v - lo) >> 29), lo);
-}
-__device__ __forceinline__ int2 field_fix(double f, unsigned fmax) {
-    if (fmax >= 0x7ff00000u) return make_int2(0, 0);
-    return limbs58(__double2ll_rn(rmul(f, pow2(58 - field_exponent(fmax)))));
-}
-
 // FP64 arithmetic, a lane per particle: for runs with so few particles on the mesh that
-// converting its fields (k_fields_to_fix) would cost more than it saves.
+// converting its fields would cost more than it saves.
 template <typename T, int P>
 __global__ void __launch_bounds__(kThreads)
 k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restrict__ y,
@@ -693,7 +660,7 @@ k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restr
 // gathered 16 or 8 at a time, and the gathered fields go back through the same records to
 // the lane that pushes the particle.  Gather + push, a lane per particle before: FP32, 1.5 M
 // particles, 256 x 192, quartic 192 -> 121 us; FP64, 2^20 particles, 128 x 128, cubic
-// 394 -> 127 us (and 4 us for k_fields_to_fix).
+// 394 -> 127 us.
 constexpr int kRowGatherThreads = 128;
 
 // FP32: the node order and roundings of every other gather, so the same bits.
@@ -712,6 +679,8 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
     const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
     const int64_t p = blockIdx.x * (int64_t)kRowGatherThreads + threadIdx.x;
     float* mine = rec + threadIdx.x * kStride;
+    griddep_wait();
+    griddep_launch();
     double kin = 0.0;
     unsigned bad = 0;
     int base = -1;
@@ -785,18 +754,28 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
 // FP64: the fields and the weights in fixed point.  GB300 issues 2 FP64 operations per clock
 // and SM, so the 128 FP64 multiply-adds of a cubic gather (and the weights) held the pipe for
 // 0.39 ms per 2^20 particles; 32x32+64-bit integer multiply-adds issue at 32 (28 measured).
-//   - A field f with |f| < 2^e (e from the largest value on the mesh, found as the transform
-//     writes it) becomes F = rint(f 2^(58-e)), kept as fh 2^29 + fl, |fl| <= 2^28; a weight
-//     W = rint(w 2^58) = wh 2^29 + wl alike.
-//   - sum W F = (sum wh fh) 2^58 + (sum wh fl + wl fh) 2^29 + sum wl fl: three multiply-adds
-//     a node and field.  The sums are exact: the weights add up to 1, so |sum wh fh| <= 2^58,
+//   - A field f of a mesh row with |f| < 2^e on the row becomes F = rint(f 2^(58-e)), kept as
+//     fh 2^29 + fl, |fl| <= 2^28 (written by the row's inverse transform, with the row's eight
+//     exponents); a weight W = rint(w 2^58) = wh 2^29 + wl alike.
+//   - Along a row sum W F = (sum wh fh) 2^58 + (sum wh fl + wl fh) 2^29 + sum wl fl: three
+//     multiply-adds a node and field; the rows' sums are shifted to the largest exponent of
+//     the particle's rows and added.  The sums are exact: the weights add up to 1, so |sum wh fh| <= 2^58,
 //     and |sum wl fh| <= 25 2^28 2^29 < 2^62.  The last sum is below 25 2^56 of 2^116 and is
 //     dropped.
-//   - The roundings (2^-59 of the field's bound in F, as much in W, the dropped sum 2^-55 at
+//   - The roundings (2^-59 of the rows' bound in F, as much in W, the dropped sum 2^-55 at
 //     the very most, 2^-58 typically) are finer than the 2^-53 that FP64 rounds each of its
 //     products and sums to, and than the transform's own error in f, 2^-53 of the largest
 //     value.
 // Integer sums do not depend on their order, and the same bits come out on every path.
+//
+// v / 2^d rounded, d >= 0
+__device__ __forceinline__ long long shift_round(long long v, int d) {
+    d = min(d, 62);
+    return (v + ((1ll << d) >> 1)) >> d;
+}
+__device__ __forceinline__ double field_unit(int e) {
+    return e > 1024 ? __hiloint2double(0x7ff80000, 0) : pow2(e - 58);
+}
 template <int P>
 __global__ void __launch_bounds__(kRowGatherThreads)
 k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* __restrict__ x,
@@ -804,17 +783,17 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
                   double* __restrict__ py, const double* __restrict__ vx,
                   const double* __restrict__ vy, double* __restrict__ vxo,
                   double* __restrict__ vyo, int64_t n, const int4* __restrict__ F,
-                  const unsigned* __restrict__ fmax, double* __restrict__ gout, int gout_short,
+                  const unsigned* __restrict__ top, double* __restrict__ gout, int gout_short,
                   double* __restrict__ diag, unsigned int* __restrict__ err) {
     constexpr int S1 = P + 1, S2 = S1 * S1;
     constexpr int kStride = S2 | 1;  // at least the 8 gathered values
     __shared__ int2 rec[kRowGatherThreads * kStride];
     __shared__ int rbase[kRowGatherThreads];
-    __shared__ double unit[8];
     const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
     const int64_t p = blockIdx.x * (int64_t)kRowGatherThreads + threadIdx.x;
     int2* mine = rec + threadIdx.x * kStride;
-    if (threadIdx.x < 8) unit[threadIdx.x] = field_unit(fmax[threadIdx.x]);
+    griddep_wait();
+    griddep_launch();
     double kin = 0.0;
     unsigned bad = 0;
     int base = -1;
@@ -835,29 +814,36 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
         }
     }
     rbase[threadIdx.x] = base;
-    __syncthreads();
+    __syncwarp();
 #pragma unroll 1
     for (int t = 0; t < 4; ++t) {
         const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
         const int2* r = rec + k * kStride;
         const int kb = rbase[k];
-        long long h0 = 0, m0 = 0, h1 = 0, m1 = 0;
+        double f0 = 0.0, f1 = 0.0;
         if (kb >= 0) {
-            int col[S1];
-#pragma unroll
-            for (int b = 0; b < S1; ++b) {
-                int gj = (kb & 0xFFFF) + b;
-                if (gj >= g.ny) gj -= g.ny;
-                col[b] = 4 * gj + q;
-            }
+            int col[S1], row[S1], e0[S1], e1[S1], top0 = -900, top1 = -900;
 #pragma unroll
             for (int a = 0; a < S1; ++a) {
-                int gi = (kb >> 16) + a;
+                int gj = (kb & 0xFFFF) + a, gi = (kb >> 16) + a;
+                if (gj >= g.ny) gj -= g.ny;
                 if (gi >= g.nx) gi -= g.nx;
-                const int4* row = F + (size_t)gi * g.ny * 4;
+                col[a] = 4 * gj + q;
+                row[a] = gi;
+                const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + 4 * gi + q);
+                e0[a] = row_exponent(u.x);
+                e1[a] = row_exponent(u.y);
+                top0 = max(top0, e0[a]);
+                top1 = max(top1, e1[a]);
+            }
+            long long s0 = 0, s1 = 0;
+#pragma unroll
+            for (int a = 0; a < S1; ++a) {
+                const int4* F0 = F + (size_t)row[a] * g.ny * 4;
+                long long h0 = 0, m0 = 1ll << 28, h1 = 0, m1 = 1ll << 28;
 #pragma unroll
                 for (int b = 0; b < S1; ++b) {
-                    const int4 v = __ldg(row + col[b]);
+                    const int4 v = __ldg(F0 + col[b]);
                     const int2 w = r[a * S1 + b];
                     h0 += (long long)w.x * v.x;
                     m0 += (long long)w.x * v.y;
@@ -866,36 +852,25 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
                     m1 += (long long)w.x * v.w;
                     m1 += (long long)w.y * v.z;
                 }
+                s0 += shift_round(h0 + (m0 >> 29), top0 - e0[a]);
+                s1 += shift_round(h1 + (m1 >> 29), top1 - e1[a]);
             }
+            f0 = rmul((double)s0, field_unit(top0));
+            f1 = rmul((double)s1, field_unit(top1));
         }
         __syncwarp();  // the four lanes have read the particle's weights
-        long long* out = reinterpret_cast<long long*>(rec + k * kStride);
-        out[2 * q] = h0 + ((m0 + (1ll << 28)) >> 29);
-        out[2 * q + 1] = h1 + ((m1 + (1ll << 28)) >> 29);
+        double* out = reinterpret_cast<double*>(rec + k * kStride);
+        out[2 * q] = f0;
+        out[2 * q + 1] = f1;
     }
     __syncwarp();
     if (base >= 0) {
-        const long long* got = reinterpret_cast<const long long*>(mine);
-        double f[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) f[i] = rmul((double)got[i], unit[i]);
+        const double* f = reinterpret_cast<const double*>(mine);
         double vxn1, vyn1;
         push_one(pp, f, p, px, py, vx, vy, vxo, vyo, bad, kin, vxn1, vyn1);
         if (gout) record_push(gout, gout_short, n, p, px[p], py[p], vxn1, vyn1, f);
     }
     push_finish(pp, bad, kin, diag, err);
-}
-
-// The fixed-point fields of k_gather_push_fix from the mesh fields (4 complex a node).
-__global__ void k_fields_to_fix(const double2* __restrict__ G, const unsigned* __restrict__ fmax,
-                                int4* __restrict__ F, int64_t n) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int q = (int)(k & 3);
-        const double2 v = G[k];
-        const int2 a = field_fix(v.x, fmax[2 * q]), b = field_fix(v.y, fmax[2 * q + 1]);
-        F[k] = make_int4(a.x, a.y, b.x, b.y);
-    }
 }
 
 // Gather + push over particles sorted by tile and cell (see sort.cu), FP32 form.
@@ -1817,13 +1792,16 @@ cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typen
     const unsigned blocks = (unsigned)((n + kRowThreads - 1) / kRowThreads);
     const GeomT<T> gt = typed<T>(g);
     const SpeciesT<T> st = typed_species<T>(spp);
+#define GPIC_ROWS(PP)                                                                        \
+    launch_pdl(k_deposit_rows<Pol, PP, kNC, kMove>, dim3(blocks), dim3(kRowThreads), 0, s, gt, x, \
+               y, u0, u1, n, pol, err, sp, st)
     switch (p) {
-        case 2: k_deposit_rows<Pol, 2, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
-        case 3: k_deposit_rows<Pol, 3, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
-        case 4: k_deposit_rows<Pol, 4, kNC, kMove><<<blocks, kRowThreads, 0, s>>>(gt, x, y, u0, u1, n, pol, err, sp, st); break;
+        case 2: return GPIC_ROWS(2);
+        case 3: return GPIC_ROWS(3);
+        case 4: return GPIC_ROWS(4);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+#undef GPIC_ROWS
 }
 
 cudaError_t launch_move_deposit(int p, const ParticleGeom& g, double* x, double* y,
@@ -1885,8 +1863,8 @@ cudaError_t launch_deposit_z(int p, const ParticleGeom& g, const T* x, const T* 
 }
 
 cudaError_t launch_fix128_to_cplx(const longlong2* j, size_t ng, double unscale, double2* out,
-                                  cudaStream_t s, unsigned* fmax) {
-    k_fix128_to_cplx<<<blocks_for((int64_t)ng), kThreads, 0, s>>>(j, ng, unscale, out, fmax);
+                                  cudaStream_t s) {
+    k_fix128_to_cplx<<<blocks_for((int64_t)ng), kThreads, 0, s>>>(j, ng, unscale, out);
     return cudaGetLastError();
 }
 
@@ -1966,18 +1944,17 @@ cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& p
                                const FixFields*) {
     if (n == 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((n + kRowGatherThreads - 1) / kRowGatherThreads);
-#define GPIC_GPAIR(PP)                                                                          \
-    k_gather_push_pair<PP><<<blocks, kRowGatherThreads, 0, s>>>(                                \
-        typed<float>(g), typed<float>(pp), x, y, px, py, vx, vy, vxo, vyo, n, (const float4*)f, \
-        gout, gout_short ? 1 : 0, diag, err)
+#define GPIC_GPAIR(PP)                                                                         \
+    launch_pdl(k_gather_push_pair<PP>, dim3(blocks), dim3(kRowGatherThreads), 0, s,            \
+               typed<float>(g), typed<float>(pp), x, y, px, py, vx, vy, vxo, vyo, n,           \
+               (const float4*)f, gout, gout_short ? 1 : 0, diag, err)
     switch (p) {
-        case 2: GPIC_GPAIR(2); break;
-        case 3: GPIC_GPAIR(3); break;
-        case 4: GPIC_GPAIR(4); break;
+        case 2: return GPIC_GPAIR(2);
+        case 3: return GPIC_GPAIR(3);
+        case 4: return GPIC_GPAIR(4);
         default: return cudaErrorInvalidValue;
     }
 #undef GPIC_GPAIR
-    return cudaGetLastError();
 }
 
 cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& pp,
@@ -1993,22 +1970,18 @@ cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& p
                         vyo, n, (const double2*)f, gout, gout_short ? 1 : 0, diag, err)
         return cudaGetLastError();
     }
-    const int64_t nc = 4 * (int64_t)g.nx * g.ny;
-    k_fields_to_fix<<<blocks_for(nc), kThreads, 0, s>>>((const double2*)f, fix->fmax,
-                                                        (int4*)fix->f, nc);
     const unsigned blocks = (unsigned)((n + kRowGatherThreads - 1) / kRowGatherThreads);
-#define GPIC_GFIX(PP)                                                                      \
-    k_gather_push_fix<PP><<<blocks, kRowGatherThreads, 0, s>>>(                            \
-        typed<T>(g), fix_geom(g), typed<T>(pp), x, y, px, py, vx, vy, vxo, vyo, n,         \
-        (const int4*)fix->f, fix->fmax, gout, gout_short ? 1 : 0, diag, err)
+#define GPIC_GFIX(PP)                                                                        \
+    launch_pdl(k_gather_push_fix<PP>, dim3(blocks), dim3(kRowGatherThreads), 0, s, typed<T>(g), \
+               fix_geom(g), typed<T>(pp), x, y, px, py, vx, vy, vxo, vyo, n,                 \
+               (const int4*)fix->f, (const unsigned*)fix->top, gout, gout_short ? 1 : 0, diag, err)
     switch (p) {
-        case 2: GPIC_GFIX(2); break;
-        case 3: GPIC_GFIX(3); break;
-        case 4: GPIC_GFIX(4); break;
+        case 2: return GPIC_GFIX(2);
+        case 3: return GPIC_GFIX(3);
+        case 4: return GPIC_GFIX(4);
         default: return cudaErrorInvalidValue;
     }
 #undef GPIC_GFIX
-    return cudaGetLastError();
 }
 
 cudaError_t launch_gather_push_tiled(int p, const ParticleGeom& g, const PushParams& pp,

@@ -82,7 +82,7 @@ cudaError_t inverse_fft(pic_handle* h, void* buf, void* out, int nb) {
 cudaError_t drop_pending(pic_handle* h) {
     if (!h->pending) return cudaSuccess;
     h->pending = false;
-    return cudaMemsetAsync(h->Jalt, 0, h->ng * sizeof(double2), h->s);
+    return cudaMemsetAsync(h->Jalt, 0, h->jbytes, h->s);
 }
 
 pic_status check_device_error(pic_handle* h) {
@@ -288,10 +288,8 @@ pic_status alloc_state(pic_handle* h) {
     if (h->sorting && h->vdim == 3)
         for (int a = 0; a < 3; ++a) CK(dalloc(h, &h->z_alt[a], pn));
     CK(dalloc(h, (void**)&h->J, h->jbytes));
-    if (h->fp32) {
-        CK(dalloc(h, (void**)&h->Jalt, h->ng * sizeof(double2)));
-        CK(cudaMemsetAsync(h->Jalt, 0, h->ng * sizeof(double2), h->s));
-    }
+    CK(dalloc(h, (void**)&h->Jalt, h->jbytes));
+    CK(cudaMemsetAsync(h->Jalt, 0, h->jbytes, h->s));
     CK(dalloc(h, &h->Z, h->ng * cs));
     if (h->cfg.charge == PIC_CHARGE_DEPOSIT) {
         CK(dalloc(h, &h->rhoq, h->jbytes));
@@ -304,7 +302,7 @@ pic_status alloc_state(pic_handle* h) {
     // node) is small beside what it saves (about 200 a particle).
     if (!h->fp32 && h->vdim == 2 && h->spp.n == 0 && h->n >= (int64_t)(h->ng / 8)) {
         CK(dalloc(h, &h->fixf.f, 4 * h->ng * cs));
-        CK(dalloc(h, (void**)&h->fixf.fmax, 8 * sizeof(unsigned)));
+        CK(dalloc(h, (void**)&h->fixf.top, (size_t)c.nx * 8 * sizeof(unsigned)));
     }
     CK(dalloc(h, &h->E, h->ng * cs));
     CK(dalloc(h, &h->tmp, h->ng * cs));
@@ -771,13 +769,9 @@ pic_status pic_deposit(pic_handle* h) {
         pic_status st = sort_particles(h, false);
         if (st != PIC_OK) return st;
     }
-    if (h->fp32) {
-        // the buffer the previous field solve zeroed (a memset here would break the chain
-        // of dependent launches); J^n stays readable until then
-        std::swap(h->J, h->Jalt);
-    } else {
-        CK(cudaMemsetAsync(h->J, 0, h->jbytes, h->s));
-    }
+    // the buffer the previous field solve zeroed (a memset here would break the chain of
+    // dependent launches); J^n stays readable until then
+    std::swap(h->J, h->Jalt);
     if (h->vdim == 3 && binned_deposit(h))  // the binned pass adds J_z to it
         CK(cudaMemsetAsync(h->Jz, 0, h->jbytes, h->s));
     h->launches_now += 1;
@@ -835,16 +829,13 @@ pic_status pic_field_solve(pic_handle* h) {
     const bool fused = field_columns_smem(h->nx, 2 * h->rsz) <= kFieldColumnsSmemMax;
     TimedScope ts(h, PIC_KT_FIELD);
 
-    // forward transform along y (the FP32 form converts the fixed-point sums on load)
-    if (h->fp32) {
+    // forward transform along y, the fixed-point sums converted on load
+    if (h->fp32)
         CK(launch_fft_y_from_fix<float>((const longlong2*)h->J, h->fix_unscale_j, h->Z, h->nx,
                                         h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s));
-    } else {  // the 128-bit sums to FP64, then the transform
-        CK(launch_fix128_to_cplx((const longlong2*)h->J, h->ng, h->fix64_unscale_j,
-                                 (double2*)h->tmp, h->s, h->fixf.fmax));
-        CK(launch_fft_y<double>(h->tmp, h->Z, h->nx, h->ny, 1, h->fy, h->twy, -1, 0, h->s));
-        h->launches_now += 1;
-    }
+    else
+        CK(launch_fft_y_from_fix<double>((const longlong2*)h->J, h->fix64_unscale_j, h->Z, h->nx,
+                                         h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s));
     if (!fused) CK(by_prec(h, [&](auto t) {
         using T = decltype(t);
         return launch_fft_x<T>(h->Z, h->Z, h->nx, h->ny, 1, h->fx, h->twx, -1, h->s);
@@ -937,7 +928,7 @@ pic_status pic_field_solve(pic_handle* h) {
         if (!fused) r = launch_fft_x<T>(h->F4, h->F4, h->nx, h->ny, 4, h->fx, h->twx, +1, h->s);
         if (r != cudaSuccess) return r;
         return launch_fft_y<T>(h->F4, h->G, h->nx, h->ny, 4, h->fy, h->twy, +1, 1, h->s,
-                               h->fixf.fmax);
+                               h->fixf.f ? &h->fixf : nullptr);
     }));
     h->launches_now += fused ? 3 : 5;
 
@@ -1059,7 +1050,6 @@ pic_status gather_push_step(pic_handle* h, bool fuse, bool defer) {
                                       h->err, h->s, h->gather_out_short,
                                       h->fixf.f ? &h->fixf : nullptr);
         }));
-        if (h->fixf.f) h->launches_now += 1;
     }
     h->vcur = vo;
     h->launches_now += 1;
