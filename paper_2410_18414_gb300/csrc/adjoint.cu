@@ -26,19 +26,22 @@
 //     x^{n+1} = x^n + dt v^n:  x^n b = x^{n+1} b,  v^n b += dt x^{n+1} b
 //   t = 0 (k_adj_init): P^0 = gamma m v^0 and the Taylor start v^{-1}(v^0, E^0).
 //
-// One thread per particle or per mode.  The particle kernels run in the storage type T of
+// One thread per particle or per mode (the stencil passes share a particle among lanes, see
+// k_adj_push_gather).  The particle kernels run in the storage type T of
 // the forward they reverse: FP64 for the plain path, FP32 for the FP32 form (the adjoint
 // of the step in exact arithmetic, evaluated along the FP32 form's trajectory; the
 // fixed-point rounding of its current, piecewise constant, is differentiated as the
 // identity).  The field adjoints they deposit are summed in FP64 (FP32 form: in FP32, the
-// eight values of a node in two vector atomics, then converted), and the reverse field
-// solve is FP64 in both forms, as the forward's per-mode update is.  Shape weights come
+// eight values of a node in two vector atomics), eight values a node side by side, and the
+// reverse field solve is FP64 in both forms, as the forward's per-mode update is.  Shape weights come
 // from Shape<P, T> (the forward's), their derivatives from the closed forms below.
 #include <algorithm>
 
 #include "common.cuh"
 #include "fft_device.cuh"
+#include "fixed.cuh"
 #include "gpic_internal.h"
+#include "launch.cuh"
 
 namespace gpic {
 
@@ -95,124 +98,312 @@ template <typename T> struct DShape<4, T> {
 template <typename T>
 __device__ __forceinline__ bool inside(T xi, int n) { return xi >= (T)0 && xi <= (T)n; }
 
+constexpr int kAdjThreads = 128;
+
+// The field adjoints of a warp's 32 particles, each left in shared memory by its lane (rec:
+// the S2 products W_x W_y, then gb[8]; base: its first node): the warp's lanes become the
+// doubles of ONE particle's stencil nodes (eight a node, side by side), so an atomic touches
+// the p+1 rows of neighbouring nodes instead of 32 particles' nodes.
+template <int P>
+__device__ __forceinline__ void deposit_adjoints(const ParticleGeom& g, const double* rec,
+                                                 int stride, const int* rbase,
+                                                 double* __restrict__ Fb) {
+    constexpr int S1 = P + 1, S2 = S1 * S1;
+    constexpr int kWords = 8 * S2, kPasses = (kWords + 31) / 32;
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+#pragma unroll 2
+    for (int k = 0; k < 32; ++k) {
+        const int base = rbase[w0 + k];
+        if (base < 0) continue;  // uniform for the warp
+        const double* r = rec + (w0 + k) * stride;
+        const double gb = r[S2 + (lane & 7)];
+#pragma unroll
+        for (int q = 0; q < kPasses; ++q) {
+            const int word = lane + 32 * q;
+            if (word >= kWords) break;
+            const int node = word >> 3;
+            const int a = node / S1, b = node - a * S1;
+            int gi = (base >> 16) + a, gj = (base & 0xFFFF) + b;
+            if (gi >= g.nx) gi -= g.nx;
+            if (gj >= g.ny) gj -= g.ny;
+            atomicAdd(Fb + 8 * ((size_t)gi * g.ny + gj) + (lane & 7), r[node] * gb);
+        }
+    }
+}
+
+// The adjoints of one particle's push: f[2..7] the gathered A, grad A; adds to Pb, sets gb,
+// rotates the velocity adjoints.
+template <typename T>
+__device__ __forceinline__ void reverse_push(const PushParams& pp, const T* f, T px1, T py1, T vx,
+                                             T vy, T vxo, T vyo, const AdjParticlesT<T>& ab,
+                                             int64_t p, T* gb) {
+    const T q = (T)pp.q, qdt = (T)(pp.q * pp.dt), c2 = (T)(pp.c * pp.c),
+            mc2 = (T)(pp.m * pp.c * pp.c);
+    // velocity: v = c^2 u / D
+    const T ux = px1 - q * f[2], uy = py1 - q * f[3];
+    const T D = sqrt(c2 * (ux * ux + uy * uy) + mc2 * mc2);
+    const T id = (T)1 / D;
+    const T vbx = ab.vx[p], vby = ab.vy[p];
+    const T cd = c2 * id, udv = (ux * vbx + uy * vby) * cd * id;
+    const T ubx = cd * (vbx - ux * udv), uby = cd * (vby - uy * udv);
+    const T pbx = ab.px[p] + ubx, pby = ab.py[p] + uby;
+    // momentum: P^{n+1} = P^n + q dt (-grad phi + (grad A) . v*)
+    const T vsx = (T)2 * vx - vxo, vsy = (T)2 * vy - vyo;
+    gb[0] = -qdt * pbx;
+    gb[1] = -qdt * pby;
+    gb[2] = -q * ubx;
+    gb[3] = -q * uby;
+    gb[4] = qdt * pbx * vsx;
+    gb[5] = qdt * pby * vsx;
+    gb[6] = qdt * pbx * vsy;
+    gb[7] = qdt * pby * vsy;
+    const T vsbx = qdt * (pbx * f[4] + pby * f[5]);
+    const T vsby = qdt * (pbx * f[6] + pby * f[7]);
+    ab.px[p] = pbx;
+    ab.py[p] = pby;
+    ab.vx[p] = ab.vxo[p] + (T)2 * vsbx;
+    ab.vy[p] = ab.vyo[p] + (T)2 * vsby;
+    ab.vxo[p] = -vsbx;
+    ab.vyo[p] = -vsby;
+}
+
+// FP32, and FP64 for runs with few particles on the mesh (no fixed-point fields): a lane per
+// particle.  (FP32 with the deposit of deposit_adjoints, a float4 a lane: 40 steps of 65,536
+// particles on 64 x 64 took 3.48 ms against 3.31 ms; the atomics then wait for the whole
+// gather instead of running beside it.)
 template <typename T, int P>
-__global__ void __launch_bounds__(kThreads, 3)
+__global__ void __launch_bounds__(kAdjThreads, 6)
 k_adj_push_gather(ParticleGeom g, PushParams pp, const T* __restrict__ x1,
                   const T* __restrict__ y1, const T* __restrict__ px1,
                   const T* __restrict__ py1, const T* __restrict__ vx,
                   const T* __restrict__ vy, const T* __restrict__ vxo,
                   const T* __restrict__ vyo, const double* __restrict__ gfa,
-                  const cplx_t<T>* __restrict__ F, AdjParticlesT<T> ab, double2* __restrict__ Fb,
-                  float4* __restrict__ Fb32, int64_t n, unsigned int* __restrict__ err) {
+                  const cplx_t<T>* __restrict__ F, AdjParticlesT<T> ab, T* __restrict__ Fb,
+                  int64_t n, unsigned int* __restrict__ err) {
     using C = cplx_t<T>;
-    const size_t ng = (size_t)g.nx * g.ny;
-    const T q = (T)pp.q, qdt = (T)(pp.q * pp.dt), c2 = (T)(pp.c * pp.c),
-            mc2 = (T)(pp.m * pp.c * pp.c);
     const T idx_ = (T)g.inv_dx, idy = (T)g.inv_dy;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t p = blockIdx.x * (int64_t)kAdjThreads + threadIdx.x;
+    griddep_wait();
+    griddep_launch();
+    if (p < n) {
         const T xi = rmul(x1[p], idx_), yj = rmul(y1[p], idy);
         if (!inside(xi, g.nx) || !inside(yj, g.ny)) {
             atomicOr(err, (unsigned)ERR_NONFINITE);
-            continue;
-        }
-        T wx[P + 1], wy[P + 1], dwx[P + 1], dwy[P + 1];
-        const int ix = Shape<P, T>::weights(xi, wx);
-        const int iy = Shape<P, T>::weights(yj, wy);
-        // the fields the forward push gathered at x^{n+1} (dphi/dx, dphi/dy, Ax, Ay,
-        // dAx/dx, dAx/dy, dAy/dx, dAy/dy): from the record, or (gfa == NULL, the lean
-        // record) gathered again from the step's fields F in the forward gather's node
-        // order and roundings, which gives the same bits
-        T f[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // f[0], f[1] (grad phi) are not needed here
-        if (gfa) {
-#pragma unroll
-            for (int k = 2; k < 8; ++k) f[k] = (T)gfa[(size_t)(k - 2) * n + p];
         } else {
+            T wx[P + 1], wy[P + 1], dwx[P + 1], dwy[P + 1];
+            const int ix = Shape<P, T>::weights(xi, wx);
+            const int iy = Shape<P, T>::weights(yj, wy);
+            // the fields the forward push gathered at x^{n+1} (dphi/dx, dphi/dy, Ax, Ay,
+            // dAx/dx, dAx/dy, dAy/dx, dAy/dy): from the record, or (gfa == NULL, the lean
+            // record) gathered again from the step's fields F in the forward gather's node
+            // order and roundings, which gives the same bits
+            T f[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // f[0], f[1] (grad phi) are not needed here
+            if (gfa) {
+#pragma unroll
+                for (int k = 2; k < 8; ++k) f[k] = (T)gfa[(size_t)(k - 2) * n + p];
+            } else {
+#pragma unroll 1
+                for (int a = 0; a <= P; ++a) {
+                    const C* row = F + (size_t)wrap_idx(ix + a, g.nx) * g.ny * 4;
+#pragma unroll
+                    for (int b = 0; b <= P; ++b) {
+                        const C* node = row + (size_t)wrap_idx(iy + b, g.ny) * 4;
+                        const T w = rmul(wx[a], wy[b]);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const C v = __ldg(node + k);
+                            f[2 * k] = rfma(w, v.x, f[2 * k]);
+                            f[2 * k + 1] = rfma(w, v.y, f[2 * k + 1]);
+                        }
+                    }
+                }
+            }
+            T gb[8];
+            reverse_push(pp, f, px1[p], py1[p], vx[p], vy[p], vxo[p], vyo[p], ab, p, gb);
+            DShape<P, T>::dweights(xi, dwx);
+            DShape<P, T>::dweights(yj, dwy);
+            // one pass over the stencil: s = sum_f gb_f F_f at each node gives the position
+            // gradient (separable: along y in the row, then across rows), and gb is deposited
+            T xg = 0, yg = 0;
 #pragma unroll 1
             for (int a = 0; a <= P; ++a) {
-                const C* row = F + (size_t)wrap_idx(ix + a, g.nx) * g.ny * 4;
+                const size_t row = (size_t)wrap_idx(ix + a, g.nx) * g.ny;
+                const T wxa = wx[a];
+                T sx = 0, sy = 0;
 #pragma unroll
                 for (int b = 0; b <= P; ++b) {
-                    const C* node = row + (size_t)wrap_idx(iy + b, g.ny) * 4;
-                    const T w = rmul(wx[a], wy[b]);
+                    const size_t nd = row + wrap_idx(iy + b, g.ny);
+                    const C* node = F + nd * 4;
+                    T sn = 0;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const C v = __ldg(node + k);
-                        f[2 * k] = rfma(w, v.x, f[2 * k]);
-                        f[2 * k + 1] = rfma(w, v.y, f[2 * k + 1]);
+                        sn += gb[2 * k] * v.x + gb[2 * k + 1] * v.y;
+                    }
+                    sx += wy[b] * sn;
+                    sy += dwy[b] * sn;
+                    const T w = wxa * wy[b];
+                    if constexpr (sizeof(T) == 4) {  // the node's eight values, four an atomic
+                        float4* fb = reinterpret_cast<float4*>(Fb) + 2 * nd;
+                        atomicAdd(fb, make_float4(w * gb[0], w * gb[1], w * gb[2], w * gb[3]));
+                        atomicAdd(fb + 1, make_float4(w * gb[4], w * gb[5], w * gb[6], w * gb[7]));
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) atomicAdd(Fb + 8 * nd + k, w * gb[k]);
                     }
                 }
+                xg += dwx[a] * sx;
+                yg += wxa * sy;
             }
+            ab.x[p] += idx_ * xg;
+            ab.y[p] += idy * yg;
         }
-        // velocity: v = c^2 u / D
-        const T ux = px1[p] - q * f[2], uy = py1[p] - q * f[3];
-        const T D = sqrt(c2 * (ux * ux + uy * uy) + mc2 * mc2);
-        const T id = (T)1 / D;
-        const T vbx = ab.vx[p], vby = ab.vy[p];
-        const T cd = c2 * id, udv = (ux * vbx + uy * vby) * cd * id;
-        const T ubx = cd * (vbx - ux * udv), uby = cd * (vby - uy * udv);
-        const T pbx = ab.px[p] + ubx, pby = ab.py[p] + uby;
-        // momentum: P^{n+1} = P^n + q dt (-grad phi + (grad A) . v*)
-        const T vsx = (T)2 * vx[p] - vxo[p], vsy = (T)2 * vy[p] - vyo[p];
-        T gb[8];
-        gb[0] = -qdt * pbx;
-        gb[1] = -qdt * pby;
-        gb[2] = -q * ubx;
-        gb[3] = -q * uby;
-        gb[4] = qdt * pbx * vsx;
-        gb[5] = qdt * pby * vsx;
-        gb[6] = qdt * pbx * vsy;
-        gb[7] = qdt * pby * vsy;
-        const T vsbx = qdt * (pbx * f[4] + pby * f[5]);
-        const T vsby = qdt * (pbx * f[6] + pby * f[7]);
-        DShape<P, T>::dweights(xi, dwx);
-        DShape<P, T>::dweights(yj, dwy);
-        // one pass over the stencil: s = sum_f gb_f F_f at each node gives the position
-        // gradient (separable: along y in the row, then across rows), and gb is deposited
-        T xg = 0, yg = 0;
-#pragma unroll 1
-        for (int a = 0; a <= P; ++a) {
-            const size_t row = (size_t)wrap_idx(ix + a, g.nx) * g.ny;
-            const T wxa = wx[a];
-            T sx = 0, sy = 0;
-#pragma unroll
-            for (int b = 0; b <= P; ++b) {
-                const size_t nd = row + wrap_idx(iy + b, g.ny);
-                const C* node = F + nd * 4;
-                T sn = 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const C v = __ldg(node + k);
-                    sn += gb[2 * k] * v.x + gb[2 * k + 1] * v.y;
-                }
-                sx += wy[b] * sn;
-                sy += dwy[b] * sn;
-                const T w = wxa * wy[b];
-                if constexpr (sizeof(T) == 4) {  // the node's eight values, four an atomic
-                    atomicAdd(Fb32 + 2 * nd,
-                              make_float4(w * gb[0], w * gb[1], w * gb[2], w * gb[3]));
-                    atomicAdd(Fb32 + 2 * nd + 1,
-                              make_float4(w * gb[4], w * gb[5], w * gb[6], w * gb[7]));
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        atomicAdd(&Fb[k * ng + nd].x, (double)(w * gb[2 * k]));
-                        atomicAdd(&Fb[k * ng + nd].y, (double)(w * gb[2 * k + 1]));
-                    }
-                }
-            }
-            xg += dwx[a] * sx;
-            yg += wxa * sy;
-        }
-        ab.x[p] += idx_ * xg;
-        ab.y[p] += idy * yg;
-        ab.px[p] = pbx;
-        ab.py[p] = pby;
-        ab.vx[p] = ab.vxo[p] + (T)2 * vsbx;
-        ab.vy[p] = ab.vyo[p] + (T)2 * vsby;
-        ab.vxo[p] = -vsbx;
-        ab.vyo[p] = -vsby;
     }
+}
+
+// FP64 with the forward's fixed-point fields (k_gather_push_fix): the gathers the adjoint
+// needs -- sum_node F_f d(W_x W_y) along x and along y for the position gradient
+// sum_f gb_f grad F_f, and (lean record) A and grad A themselves -- are separable integer
+// sums, four lanes a particle: along a row with W_y and dW_y, then across rows with W_x and
+// dW_x.  The FP64 pipe is left with the push's adjoint and the products the atomics add
+// (about 250 operations a particle instead of 600).  262,144 particles, 128 x 128, cubic: with
+// FP64 gathers and a lane per particle 263 us, now 167 us.
+template <int P, bool kLean>
+__global__ void __launch_bounds__(kAdjThreads)
+k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* __restrict__ x1,
+                      const double* __restrict__ y1, const double* __restrict__ px1,
+                      const double* __restrict__ py1, const double* __restrict__ vx,
+                      const double* __restrict__ vy, const double* __restrict__ vxo,
+                      const double* __restrict__ vyo, const double* __restrict__ gfa,
+                      const int4* __restrict__ F, const unsigned* __restrict__ top,
+                      AdjParticles ab, double* __restrict__ Fb, int64_t n,
+                      unsigned int* __restrict__ err) {
+    constexpr int S1 = P + 1, S2 = S1 * S1, kOut = kLean ? 24 : 16;
+    constexpr int kUse = 4 * S1 + kOut > S2 + 8 ? 4 * S1 + kOut : S2 + 8;
+    constexpr int kStride = kUse | 1;
+    __shared__ double rec[kAdjThreads * kStride];
+    __shared__ int rbase[kAdjThreads];
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    const int64_t p = blockIdx.x * (int64_t)kAdjThreads + threadIdx.x;
+    double* mine = rec + threadIdx.x * kStride;
+    long long X = 0, Y = 0;
+    int base = -1;
+    griddep_wait();
+    griddep_launch();
+    if (p < n) {
+        X = __double2ll_rn(rmul(x1[p], fg.sx));
+        Y = __double2ll_rn(rmul(y1[p], fg.sy));
+        if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh)) {
+            atomicOr(err, (unsigned)ERR_NONFINITE);
+        } else {
+            int2* lim = reinterpret_cast<int2*>(mine);  // W_x, dW_x, W_y, dW_y
+            long long w[S1];
+            const int ix = fix_weights<P>(X, fg.sh, w);
+#pragma unroll
+            for (int a = 0; a < S1; ++a) lim[a] = weight_limbs(w[a]);
+            const int iy = fix_weights<P>(Y, fg.sh, w);
+#pragma unroll
+            for (int a = 0; a < S1; ++a) lim[2 * S1 + a] = weight_limbs(w[a]);
+            fix_dweights<P>(X, fg.sh, w);
+#pragma unroll
+            for (int a = 0; a < S1; ++a) lim[S1 + a] = weight_limbs(w[a]);
+            fix_dweights<P>(Y, fg.sh, w);
+#pragma unroll
+            for (int a = 0; a < S1; ++a) lim[3 * S1 + a] = weight_limbs(w[a]);
+            base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
+        }
+    }
+    rbase[threadIdx.x] = base;
+    __syncwarp();
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+        const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
+        const int kb = rbase[k];
+        if (kb < 0) continue;  // its quad of lanes alone; no warp-wide operation below
+        const int2* lim = reinterpret_cast<const int2*>(rec + k * kStride);
+        int row[S1], e0[S1], e1[S1], top0 = -900, top1 = -900;
+#pragma unroll
+        for (int a = 0; a < S1; ++a) {
+            int gi = (kb >> 16) + a;
+            if (gi >= g.nx) gi -= g.nx;
+            row[a] = gi;
+            const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + 4 * gi + q);
+            e0[a] = row_exponent(u.x);
+            e1[a] = row_exponent(u.y);
+            top0 = max(top0, e0[a]);
+            top1 = max(top1, e1[a]);
+        }
+        long long hx[2] = {0, 0}, mx[2] = {0, 0}, hy[2] = {0, 0}, my[2] = {0, 0};
+        long long hw[2] = {0, 0}, mw[2] = {0, 0};
+#pragma unroll
+        for (int a = 0; a < S1; ++a) {
+            const int4* F0 = F + (size_t)row[a] * g.ny * 4 + q;
+            long long hr[2] = {0, 0}, mr[2] = {0, 0}, hs[2] = {0, 0}, ms[2] = {0, 0};
+#pragma unroll
+            for (int b = 0; b < S1; ++b) {
+                int gj = (kb & 0xFFFF) + b;
+                if (gj >= g.ny) gj -= g.ny;
+                const int4 v = __ldg(F0 + 4 * gj);
+                const int2 wy = lim[2 * S1 + b], dy = lim[3 * S1 + b];
+                mac58(hr[0], mr[0], wy, v.x, v.y);
+                mac58(hr[1], mr[1], wy, v.z, v.w);
+                mac58(hs[0], ms[0], dy, v.x, v.y);
+                mac58(hs[1], ms[1], dy, v.z, v.w);
+            }
+            const int2 wx = lim[a], dx = lim[S1 + a];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int d = c ? top1 - e1[a] : top0 - e0[a];
+                const int2 r = limbs58(shift_round(sum58(hr[c], mr[c]), d));
+                const int2 s = limbs58(shift_round(sum58(hs[c], ms[c]), d));
+                mac58(hx[c], mx[c], dx, r.x, r.y);
+                mac58(hy[c], my[c], wx, s.x, s.y);
+                if (kLean) mac58(hw[c], mw[c], wx, r.x, r.y);
+            }
+        }
+        double* out = rec + k * kStride + 4 * S1 + 2 * q;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const double u = field_unit(c ? top1 : top0);
+            out[c] = (double)sum58(hx[c], mx[c]) * u;
+            out[8 + c] = (double)sum58(hy[c], my[c]) * u;
+            if (kLean) out[16 + c] = (double)sum58(hw[c], mw[c]) * u;
+        }
+    }
+    __syncwarp();
+    if (base >= 0) {
+        const double* got = mine + 4 * S1;
+        double f[8];
+#pragma unroll
+        for (int k = 2; k < 8; ++k) f[k] = kLean ? got[16 + k] : gfa[(size_t)(k - 2) * n + p];
+        double gb[8], xg = 0.0, yg = 0.0;
+        reverse_push(pp, f, px1[p], py1[p], vx[p], vy[p], vxo[p], vyo[p], ab, p, gb);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            xg += gb[k] * got[k];
+            yg += gb[k] * got[8 + k];
+        }
+        ab.x[p] += g.inv_dx * xg;
+        ab.y[p] += g.inv_dy * yg;
+        // the record now holds the products W_x W_y and gb
+        constexpr double unit = 1.0 / 4611686018427387904.0;  // 2^-62
+        long long w[S1];
+        double wy[S1];
+        fix_weights<P>(Y, fg.sh, w);
+#pragma unroll
+        for (int b = 0; b < S1; ++b) wy[b] = (double)w[b] * unit;
+        fix_weights<P>(X, fg.sh, w);
+#pragma unroll
+        for (int a = 0; a < S1; ++a) {
+            const double wx = (double)w[a] * unit;
+#pragma unroll
+            for (int b = 0; b < S1; ++b) mine[a * S1 + b] = wx * wy[b];
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) mine[S2 + k] = gb[k];
+    }
+    __syncwarp();
+    deposit_adjoints<P>(g, rec, kStride, rbase, Fb);
 }
 
 template <typename T, int P>
@@ -222,6 +413,8 @@ k_adj_deposit_move(ParticleGeom g, const T* __restrict__ x1, const T* __restrict
                    const double2* __restrict__ Jb, AdjParticlesT<T> ab, int64_t n,
                    unsigned int* __restrict__ err) {
     const T idx_ = (T)g.inv_dx, idy = (T)g.inv_dy, dt = (T)g.dt;
+    griddep_wait();
+    griddep_launch();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
          p += (int64_t)gridDim.x * blockDim.x) {
         const T xi = rmul(x1[p], idx_), yj = rmul(y1[p], idy);
@@ -264,6 +457,95 @@ k_adj_deposit_move(ParticleGeom g, const T* __restrict__ x1, const T* __restrict
         ab.vx[p] = ab.vx[p] + sx + dt * xb;
         ab.vy[p] = ab.vy[p] + sy + dt * yb;
     }
+}
+
+// The same with the mesh adjoint current in fixed point (an int4 a node, two maxima a row):
+// six separable integer sums, about 35 FP64 operations a particle left of 170.  Measured with
+// FP64 sums 78 us, now 35 us (262,144 particles, cubic).
+template <int P>
+__global__ void __launch_bounds__(kAdjThreads)
+k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1,
+                       const double* __restrict__ y1, const double* __restrict__ vx,
+                       const double* __restrict__ vy, const int4* __restrict__ Jb,
+                       const unsigned* __restrict__ top, AdjParticles ab, int64_t n,
+                       unsigned int* __restrict__ err) {
+    constexpr int S1 = P + 1;
+    const int64_t p = blockIdx.x * (int64_t)kAdjThreads + threadIdx.x;
+    griddep_wait();
+    griddep_launch();
+    if (p >= n) return;
+    const long long X = __double2ll_rn(rmul(x1[p], fg.sx)), Y = __double2ll_rn(rmul(y1[p], fg.sy));
+    if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh)) {
+        atomicOr(err, (unsigned)ERR_NONFINITE);
+        return;
+    }
+    int2 wy[S1], dy[S1];
+    long long wx[S1], dx[S1];
+    const int iy = wrap_idx(fix_weights<P>(Y, fg.sh, wx), g.ny);
+    fix_dweights<P>(Y, fg.sh, dx);
+#pragma unroll
+    for (int b = 0; b < S1; ++b) {
+        wy[b] = weight_limbs(wx[b]);
+        dy[b] = weight_limbs(dx[b]);
+    }
+    const int ix = wrap_idx(fix_weights<P>(X, fg.sh, wx), g.nx);
+    fix_dweights<P>(X, fg.sh, dx);
+    int e[2][S1], tops[2] = {-900, -900};
+#pragma unroll
+    for (int a = 0; a < S1; ++a) {
+        int gi = ix + a;
+        if (gi >= g.nx) gi -= g.nx;
+        const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + gi);
+        e[0][a] = row_exponent(u.x);
+        e[1][a] = row_exponent(u.y);
+        tops[0] = max(tops[0], e[0][a]);
+        tops[1] = max(tops[1], e[1][a]);
+    }
+    // per component: the value, d/dx and d/dy of the gathered current adjoint
+    long long hw[2] = {0, 0}, mw[2] = {0, 0}, hx[2] = {0, 0}, mx[2] = {0, 0};
+    long long hy[2] = {0, 0}, my[2] = {0, 0};
+#pragma unroll
+    for (int a = 0; a < S1; ++a) {
+        int gi = ix + a;
+        if (gi >= g.nx) gi -= g.nx;
+        const int4* row = Jb + (size_t)gi * g.ny;
+        long long hr[2] = {0, 0}, mr[2] = {0, 0}, hs[2] = {0, 0}, ms[2] = {0, 0};
+#pragma unroll
+        for (int b = 0; b < S1; ++b) {
+            int gj = iy + b;
+            if (gj >= g.ny) gj -= g.ny;
+            const int4 v = __ldg(row + gj);
+            mac58(hr[0], mr[0], wy[b], v.x, v.y);
+            mac58(hr[1], mr[1], wy[b], v.z, v.w);
+            mac58(hs[0], ms[0], dy[b], v.x, v.y);
+            mac58(hs[1], ms[1], dy[b], v.z, v.w);
+        }
+        const int2 wa = weight_limbs(wx[a]), da = weight_limbs(dx[a]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int d = tops[c] - e[c][a];
+            const int2 r = limbs58(shift_round(sum58(hr[c], mr[c]), d));
+            const int2 s = limbs58(shift_round(sum58(hs[c], ms[c]), d));
+            mac58(hw[c], mw[c], wa, r.x, r.y);
+            mac58(hx[c], mx[c], da, r.x, r.y);
+            mac58(hy[c], my[c], wa, s.x, s.y);
+        }
+    }
+    double w[2], jx[2], jy[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double u = field_unit(tops[c]);
+        w[c] = (double)sum58(hw[c], mw[c]) * u;
+        jx[c] = (double)sum58(hx[c], mx[c]) * u;
+        jy[c] = (double)sum58(hy[c], my[c]) * u;
+    }
+    const double vxp = vx[p], vyp = vy[p];
+    const double xb = ab.x[p] + g.inv_dx * (vxp * jx[0] + vyp * jx[1]);
+    const double yb = ab.y[p] + g.inv_dy * (vxp * jy[0] + vyp * jy[1]);
+    ab.x[p] = xb;
+    ab.y[p] = yb;
+    ab.vx[p] = ab.vx[p] + w[0] + g.dt * xb;
+    ab.vy[p] = ab.vy[p] + w[1] + g.dt * yb;
 }
 
 constexpr int kModeThreads = 256;
@@ -469,6 +751,8 @@ k_adj_columns(ModeCommon mc, Params ap, const double2* __restrict__ Zb,
     double2* bufB = bufA + 8 * nx;
     double2* tws = bufB + 8 * nx;
     stage_twiddles(tw, tws, nx);
+    griddep_wait();
+    griddep_launch();
     for (int t = threadIdx.x; t < 4 * ncols * nx; t += blockDim.x) {
         const int l = t / nx, i = t - l * nx;
         const int c = l >> 2, k = l & 3;
@@ -603,20 +887,6 @@ k_adj_init(ParticleGeom g, PushParams pp, const T* __restrict__ x0, const T* __r
     }
 }
 
-// The FP32 form's field adjoints, [node][2] float4 (fields 0-3, 4-7), to the four FP64
-// planes of the reverse field solve: plane k holds fields (2k, 2k + 1) of each node.
-__global__ void k_fb32_to_planes(const float4* __restrict__ fb32, double2* __restrict__ Fb,
-                                 int64_t ng) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < ng;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const float4 a = fb32[2 * k], b = fb32[2 * k + 1];
-        Fb[k] = make_double2(a.x, a.y);
-        Fb[ng + k] = make_double2(a.z, a.w);
-        Fb[2 * ng + k] = make_double2(b.x, b.y);
-        Fb[3 * ng + k] = make_double2(b.z, b.w);
-    }
-}
-
 inline int mode_blocks(const ModeCommon& mc) {
     return (mc.nx * mc.ny + kModeThreads - 1) / kModeThreads;
 }
@@ -631,34 +901,79 @@ inline int mode_blocks(const ModeCommon& mc) {
         default: return cudaErrorInvalidValue;                                          \
     }
 
+inline unsigned adj_blocks(int64_t n) { return (unsigned)((n + kAdjThreads - 1) / kAdjThreads); }
+
 template <typename T>
 cudaError_t launch_adj_push_gather(int p, const ParticleGeom& g, const PushParams& pp,
                                    const T* x1, const T* y1, const T* px1, const T* py1,
                                    const T* vx, const T* vy, const T* vxo, const T* vyo,
                                    const double* gf, bool lean, const void* F,
-                                   AdjParticlesT<T> ab, double2* Fb, void* fb32, int64_t n,
+                                   const FixFields* fix, AdjParticlesT<T> ab, T* Fb, int64_t n,
                                    unsigned int* err, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    if (sizeof(T) == 4 && !fb32) return cudaErrorInvalidValue;
     const double* gfa = lean ? nullptr : gf + 4 * n;  // the gathered values of the record
-    GPIC_ADJ_DISPATCH(p, k_adj_push_gather, g, pp, x1, y1, px1, py1, vx, vy, vxo, vyo, gfa,
-                      (const cplx_t<T>*)F, ab, Fb, (float4*)fb32, n, err)
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fb32_to_planes(const void* fb32, double2* Fb, int64_t ng, cudaStream_t s) {
-    k_fb32_to_planes<<<blocks_for(ng), kThreads, 0, s>>>((const float4*)fb32, Fb, ng);
-    return cudaGetLastError();
+    const dim3 grid(adj_blocks(n)), block(kAdjThreads);
+    if constexpr (sizeof(T) == 8) {
+        if (fix) {
+#define GPIC_ADJ_FIX(PP, LEAN)                                                                 \
+    launch_pdl(k_adj_push_gather_fix<PP, LEAN>, grid, block, 0, s, g, fix_geom(g), pp, x1, y1, \
+               px1, py1, vx, vy, vxo, vyo, gfa, (const int4*)fix->f,                           \
+               (const unsigned*)fix->top, ab, Fb, n, err)
+            switch (2 * p + (lean ? 1 : 0)) {
+                case 4: return GPIC_ADJ_FIX(2, false);
+                case 5: return GPIC_ADJ_FIX(2, true);
+                case 6: return GPIC_ADJ_FIX(3, false);
+                case 7: return GPIC_ADJ_FIX(3, true);
+                case 8: return GPIC_ADJ_FIX(4, false);
+                case 9: return GPIC_ADJ_FIX(4, true);
+                default: return cudaErrorInvalidValue;
+            }
+#undef GPIC_ADJ_FIX
+        }
+    }
+#define GPIC_ADJ_PUSH(PP)                                                                       \
+    launch_pdl(k_adj_push_gather<T, PP>, grid, block, 0, s, g, pp, x1, y1, px1, py1, vx, vy, vxo, \
+               vyo, gfa, (const cplx_t<T>*)F, ab, Fb, n, err)
+    switch (p) {
+        case 2: return GPIC_ADJ_PUSH(2);
+        case 3: return GPIC_ADJ_PUSH(3);
+        case 4: return GPIC_ADJ_PUSH(4);
+        default: return cudaErrorInvalidValue;
+    }
+#undef GPIC_ADJ_PUSH
 }
 
 template <typename T>
 cudaError_t launch_adj_deposit_move(int p, const ParticleGeom& g, const T* x1, const T* y1,
                                     const T* vx, const T* vy, const double2* Jb,
-                                    AdjParticlesT<T> ab, int64_t n, unsigned int* err,
-                                    cudaStream_t s) {
+                                    const FixFields* fix, AdjParticlesT<T> ab, int64_t n,
+                                    unsigned int* err, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    GPIC_ADJ_DISPATCH(p, k_adj_deposit_move, g, x1, y1, vx, vy, Jb, ab, n, err)
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        if (fix) {
+#define GPIC_ADJ_MOVE(PP)                                                                       \
+    launch_pdl(k_adj_deposit_move_fix<PP>, dim3(adj_blocks(n)), dim3(kAdjThreads), 0, s, g,     \
+               fix_geom(g), x1, y1, vx, vy, (const int4*)fix->f, (const unsigned*)fix->top, ab, \
+               n, err)
+            switch (p) {
+                case 2: return GPIC_ADJ_MOVE(2);
+                case 3: return GPIC_ADJ_MOVE(3);
+                case 4: return GPIC_ADJ_MOVE(4);
+                default: return cudaErrorInvalidValue;
+            }
+#undef GPIC_ADJ_MOVE
+        }
+    }
+#define GPIC_ADJ_MOVE(PP)                                                                    \
+    launch_pdl(k_adj_deposit_move<T, PP>, dim3(blocks_for(n)), dim3(kThreads), 0, s, g, x1, y1, \
+               vx, vy, Jb, ab, n, err)
+    switch (p) {
+        case 2: return GPIC_ADJ_MOVE(2);
+        case 3: return GPIC_ADJ_MOVE(3);
+        case 4: return GPIC_ADJ_MOVE(4);
+        default: return cudaErrorInvalidValue;
+    }
+#undef GPIC_ADJ_MOVE
 }
 
 template <typename T>
@@ -695,8 +1010,8 @@ cudaError_t adj_columns(const ModeCommon& mc, const Params& ap, const double2* Z
     cudaError_t e = cudaFuncSetAttribute(k_adj_columns<Params>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_adj_columns<Params><<<mc.ny, kModeThreads, sm, s>>>(mc, ap, Zb, Js, fd, tw);
-    return cudaGetLastError();
+    return launch_pdl(k_adj_columns<Params>, dim3(mc.ny), dim3(kModeThreads), sm, s, mc, ap, Zb, Js,
+                      fd, tw);
 }
 
 cudaError_t launch_adj_columns(const ModeCommon& mc, int kind, const AdjModeParams& ap,
@@ -745,11 +1060,12 @@ cudaError_t launch_real_to_cplx(const double* src, double2* dst, int64_t n, cuda
     template cudaError_t launch_adj_push_gather<T>(                                         \
         int, const ParticleGeom&, const PushParams&, const T*, const T*, const T*, const T*, \
         const T*, const T*, const T*, const T*, const double*, bool, const void*,            \
-        AdjParticlesT<T>, double2*, void*, int64_t, unsigned int*, cudaStream_t);           \
+        const FixFields*, AdjParticlesT<T>, T*, int64_t, unsigned int*, cudaStream_t);      \
     template cudaError_t launch_adj_deposit_move<T>(int, const ParticleGeom&, const T*,     \
                                                     const T*, const T*, const T*,           \
-                                                    const double2*, AdjParticlesT<T>,       \
-                                                    int64_t, unsigned int*, cudaStream_t);  \
+                                                    const double2*, const FixFields*,       \
+                                                    AdjParticlesT<T>, int64_t,              \
+                                                    unsigned int*, cudaStream_t);           \
     template cudaError_t launch_adj_init<T>(int, const ParticleGeom&, const PushParams&,    \
                                             const T*, const T*, const T*, const T*,         \
                                             const double2*, AdjParticlesT<T>, double*,      \

@@ -15,7 +15,7 @@
 //             v^{n+1} and the gathered A and grad A of each particle (10 n)
 //   adjoint   particle adjoints (8 n, in T), the history adjoints (BDF: 3 L + k spectra, slot
 //             of time level t = t mod L; CDF-2: 12 by role, each (cur, prev) pair swapped
-//             after every reverse step; DIRK: 9 by role, in place), field-adjoint planes
+//             after every reverse step; DIRK: 9 by role, in place), field-adjoint sums
 //             and transform scratch, and FP64 twiddle tables for the reverse field solve
 //             (an FP32-form handle's own tables are FP32)
 #include <cuda_runtime.h>
@@ -57,10 +57,13 @@ struct pic_adjoint {
     void* ab = nullptr;          // particle adjoints, 8 n
     double2* twx = nullptr;      // FP64 twiddles along x and y
     double2* twy = nullptr;
-    void* fb32 = nullptr;        // FP32 form: the field adjoints as summed, [node][8] float
+    // FP64 with the forward's fixed-point gather: recg holds a step's fixed-point fields and
+    // their row maxima, and the adjoint current on the mesh is kept in fixed point too
+    bool fix = false;
+    FixFields jfix{};
     double2* hb = nullptr;       // history adjoints, nh ng
     double2* role[12] = {};      // CDF-2, DIRK: the history adjoint of each role
-    double2* fb = nullptr;       // field-adjoint planes, 4 ng
+    void* fb = nullptr;          // the field adjoints as summed, [node][8] of T
     double2* zb = nullptr;       // their transforms, 4 ng
     double2* js = nullptr;       // adjoint current spectrum, ng
     double2* jg = nullptr;       // adjoint current on the mesh, ng
@@ -187,6 +190,12 @@ pic_status restore_checkpoint(pic_adjoint* a, const pic_adjoint::Ck& c) {
 // (6); the lean record keeps the first four.
 size_t rec_width(const pic_adjoint* a) { return a->lean ? 4 : 10; }
 
+// Bytes of one step's gather fields in the records: [node][4] complex of T, or the handle's
+// fixed-point fields with their row maxima (one allocation, see FixFields).
+size_t rec_field_bytes(const pic_adjoint* a) {
+    return 4 * a->ng * 2 * a->rsz + (a->fix ? (size_t)a->h->nx * 8 * sizeof(unsigned) : 0);
+}
+
 int seg_begin(const pic_adjoint* a, int c) { return c * a->K; }
 int seg_end(const pic_adjoint* a, int c) { return std::min(a->nsteps, (c + 1) * a->K); }
 
@@ -211,9 +220,9 @@ pic_status step_and_record(pic_adjoint* a, int s, int state_j) {
         st = save_state(a, (char*)a->rec + (size_t)state_j * state_bytes(a));
         if (st != PIC_OK) return st;
     }
-    const size_t gbytes = 4 * a->ng * 2 * a->rsz;
-    CK(cudaMemcpyAsync((char*)a->recg + r * gbytes, h->G, gbytes, cudaMemcpyDeviceToDevice,
-                       h->s));
+    const size_t gbytes = rec_field_bytes(a);
+    CK(cudaMemcpyAsync((char*)a->recg + r * gbytes, a->fix ? h->fixf.f : h->G, gbytes,
+                       cudaMemcpyDeviceToDevice, h->s));
     return PIC_OK;
 }
 
@@ -241,24 +250,22 @@ pic_status backward_step(pic_adjoint* a, int64_t n, const void* s0v, const void*
                          const double* gf, const void* g) {
     pic_handle* h = a->h;
     const size_t np = a->n, ng = a->ng;
-    if (a->f32)
-        CK(cudaMemsetAsync(a->fb32, 0, ng * 8 * sizeof(float), h->s));
-    else
-        CK(cudaMemsetAsync(a->fb, 0, 4 * ng * sizeof(double2), h->s));
     TimedScope tp(h, PIC_KT_ADJ_PUSH);
     CK(by_prec(h, [&](auto t) {
         using T = decltype(t);
         const T* s0 = (const T*)s0v;
         const T* s1 = (const T*)s1v;
+        const FixFields fx{(void*)g, (unsigned*)((char*)g + 4 * ng * sizeof(int4))};
         return launch_adj_push_gather<T>(h->p, h->geom, h->push, s1, s1 + np, s1 + 2 * np,
                                          s1 + 3 * np, s0 + 4 * np, s0 + 5 * np, s0 + 6 * np,
-                                         s0 + 7 * np, gf, a->lean, g, adjoint_arrays<T>(a),
-                                         a->fb, a->fb32, (int64_t)np, h->err, h->s);
+                                         s0 + 7 * np, gf, a->lean, g, a->fix ? &fx : nullptr,
+                                         adjoint_arrays<T>(a), (T*)a->fb, (int64_t)np, h->err,
+                                         h->s);
     }));
-    if (a->f32) CK(launch_fb32_to_planes(a->fb32, a->fb, (int64_t)ng, h->s));
     tp.end();
     TimedScope tf(h, PIC_KT_ADJ_FIELD);
-    CK(launch_fft_y<double>(a->fb, a->zb, h->nx, h->ny, 4, h->fy, a->twy, -1, 0, h->s));
+    // (the transform leaves the sums zeroed for the next step)
+    CK(launch_fft_y_from_sums(a->fb, a->f32, a->zb, h->nx, h->ny, h->fy, a->twy, h->s));
     const bool fused = adj_columns_smem(h->nx) <= kFieldColumnsSmemMax;
     if (!fused) CK(launch_fft_x<double>(a->zb, a->zb, h->nx, h->ny, 4, h->fx, a->twx, -1, h->s));
     AdjModeParams ap{};
@@ -288,11 +295,12 @@ pic_status backward_step(pic_adjoint* a, int64_t n, const void* s0v, const void*
     }
     if (fused) {
         CK(launch_adj_columns(h->mc, a->kind, ap, cp, dp, a->zb, a->js, h->fx, a->twx, h->s));
-        CK(launch_fft_y<double>(a->js, a->jg, h->nx, h->ny, 1, h->fy, a->twy, +1, 0, h->s));
     } else {
         CK(launch_adj_modes(h->mc, a->kind, ap, cp, dp, a->zb, a->js, h->s));
-        CK(fft64_inverse(a, a->js, a->jg));
+        CK(launch_fft_x<double>(a->js, a->js, h->nx, h->ny, 1, h->fx, a->twx, +1, h->s));
     }
+    CK(launch_fft_y<double>(a->js, a->jg, h->nx, h->ny, 1, h->fy, a->twy, +1, 0, h->s,
+                            a->fix ? &a->jfix : nullptr));
     // CDF-2: the adjoints before the step were written into the other buffer of each pair
     if (a->kind == K_CDF2)
         for (int r = 0; r < 12; r += 2) std::swap(a->role[r], a->role[r + 1]);
@@ -303,8 +311,8 @@ pic_status backward_step(pic_adjoint* a, int64_t n, const void* s0v, const void*
         const T* s0 = (const T*)s0v;
         const T* s1 = (const T*)s1v;
         return launch_adj_deposit_move<T>(h->p, h->geom, s1, s1 + np, s0 + 4 * np, s0 + 5 * np,
-                                          a->jg, adjoint_arrays<T>(a), (int64_t)np, h->err,
-                                          h->s);
+                                          a->jg, a->fix ? &a->jfix : nullptr,
+                                          adjoint_arrays<T>(a), (int64_t)np, h->err, h->s);
     }));
     return PIC_OK;
 }
@@ -349,6 +357,7 @@ pic_status pic_adjoint_create_ex(pic_handle* h, int32_t nsteps, int32_t checkpoi
     a->ng = h->ng;
     a->f32 = h->fp32;
     a->rsz = h->rsz;
+    a->fix = h->fixf.f != nullptr;
     const size_t sb = 8 * std::max<size_t>(a->n, 1) * a->rsz;
     const size_t hbytes = (size_t)a->nh * a->ng * sizeof(double2);
     const size_t gb = a->ng * sizeof(double2);
@@ -362,18 +371,20 @@ pic_status pic_adjoint_create_ex(pic_handle* h, int32_t nsteps, int32_t checkpoi
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->final_j, h->jbytes);
     if (e == cudaSuccess) e = aalloc(a, &a->final_g, gfb);
     if (e == cudaSuccess) e = aalloc(a, &a->rec, (size_t)a->K * sb);
-    if (e == cudaSuccess) e = aalloc(a, &a->recg, nrec * gfb);
+    if (e == cudaSuccess) e = aalloc(a, &a->recg, nrec * rec_field_bytes(a));
     if (e == cudaSuccess)
         e = aalloc(a, (void**)&a->recf,
                    nrec * rec_width(a) * std::max<size_t>(a->n, 1) * sizeof(double));
     if (e == cudaSuccess) e = aalloc(a, &a->ab, sb);
-    if (e == cudaSuccess && a->f32) e = aalloc(a, &a->fb32, a->ng * 8 * sizeof(float));
+    if (e == cudaSuccess && a->fix) e = aalloc(a, &a->jfix.f, a->ng * sizeof(int4));
+    if (e == cudaSuccess && a->fix)
+        e = aalloc(a, (void**)&a->jfix.top, (size_t)h->nx * 2 * sizeof(unsigned));
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->twx, (size_t)h->nx * sizeof(double2));
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->twy, (size_t)h->ny * sizeof(double2));
     if (e == cudaSuccess) e = launch_twiddles<double>(a->twx, h->nx, h->s);
     if (e == cudaSuccess) e = launch_twiddles<double>(a->twy, h->ny, h->s);
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->hb, hbytes);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->fb, 4 * gb);
+    if (e == cudaSuccess) e = aalloc(a, &a->fb, a->ng * 8 * a->rsz);
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->zb, 4 * gb);
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->js, gb);
     if (e == cudaSuccess) e = aalloc(a, (void**)&a->jg, gb);
@@ -437,6 +448,7 @@ pic_status pic_adjoint_backward(pic_adjoint* a, const double* bz_bar, const doub
     const size_t hbytes = (size_t)a->nh * ng * sizeof(double2);
     CK(cudaMemsetAsync(a->ab, 0, 8 * std::max<size_t>(np, 1) * a->rsz, h->s));
     CK(cudaMemsetAsync(a->hb, 0, hbytes, h->s));
+    CK(cudaMemsetAsync(a->fb, 0, ng * 8 * a->rsz, h->s));
     if (a->kind != K_BDF)
         for (int r = 0; r < a->nh; ++r) a->role[r] = a->hb + (size_t)r * ng;
     // momentum seeds, converted to the particle storage type (through the FP64 staging
@@ -497,7 +509,7 @@ pic_status pic_adjoint_backward(pic_adjoint* a, const double* bz_bar, const doub
             const void* s1 = (char*)a->rec + (size_t)j * state_bytes(a);
             pic_status st = backward_step(a, s, s0, s1,
                                           a->recf + rec_slot(a, s) * rec_width(a) * np,
-                                          (char*)a->recg + rec_slot(a, s) * 4 * ng * 2 * a->rsz);
+                                          (char*)a->recg + rec_slot(a, s) * rec_field_bytes(a));
             if (st != PIC_OK) return st;
         }
     }

@@ -116,37 +116,6 @@ __device__ __forceinline__ double rdiv(double a, double b) { return __ddiv_rn(a,
 __device__ __forceinline__ float rsqrt_rn(float a) { return __fsqrt_rn(a); }
 __device__ __forceinline__ double rsqrt_rn(double a) { return __dsqrt_rn(a); }
 
-// hi 2^64 + lo (two's complement over 128 bits) times unscale, rounded to FP64: the
-// magnitude is exact below 2^64 before its one rounding, and rounded twice above.
-__device__ __forceinline__ double fix128_value(long long hi, unsigned long long lo,
-                                               double unscale) {
-    const bool neg = hi < 0;
-    if (neg) {
-        lo = ~lo + 1ull;
-        hi = ~hi + (lo == 0ull ? 1ll : 0ll);
-    }
-    const double m = fma((double)hi, 18446744073709551616.0, (double)lo);
-    return (neg ? -m : m) * unscale;
-}
-
-// Fixed-point gather fields (FP64 path): `top` is the high word of the largest |f| of a mesh row,
-// which gives the row's exponent e with |f| < 2^e (bounded below so that the scales stay
-// finite; above 1024 for a row with a value that is not finite, whose gathers are NaN).
-__device__ __forceinline__ int row_exponent(unsigned top) {
-    return top >= 0x7ff00000u ? 2048 : max((int)(top >> 20) - 1022, -900);
-}
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-// v in [-2^58, 2^58] as (v.x 2^29 + v.y), |v.y| <= 2^28
-__device__ __forceinline__ int2 limbs58(long long v) {
-    const int lo = (int)((unsigned)v << 3) >> 3;
-    return make_int2((int)((v - lo) >> 29), lo);
-}
-// f 2^(58 - e), rounded
-__device__ __forceinline__ int2 field_fix(double f, int e) {
-    if (e > 1024) return make_int2(0, 0);
-    return limbs58(__double2ll_rn(rmul(f, pow2(58 - e))));
-}
-
 // x + v dt, wrapped (the IAEM position update)
 template <typename T> __device__ __forceinline__ T move_pos(T x, T v, T dt, T l) {
     return wrap_pos(rfma(v, dt, x), l);

@@ -13,6 +13,7 @@
 //     dst[(j div Ns) Ns R + k + r Ns] = b_r
 // which leaves the transform in natural order after the last pass.
 #include "common.cuh"
+#include "fixed.cuh"
 #include "fft_device.cuh"
 #include "gpic_internal.h"
 #include "launch.cuh"
@@ -23,12 +24,12 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// The largest magnitudes of four lines of m complex values as high words into top[8] (shared,
-// zeroed; re, im of each line).
-__device__ __forceinline__ void collect_max(const double2* res, int m, unsigned* top) {
+// The largest magnitudes of at most four lines of m complex values as high words into top[8]
+// (shared, zeroed; re, im of each line).
+__device__ __forceinline__ void collect_max(const double2* res, int lines, int m, unsigned* top) {
     const int b = threadIdx.x & 3;
     unsigned re = 0, im = 0;
-    for (int e = threadIdx.x >> 2; e < m; e += blockDim.x >> 2) {
+    for (int e = b < lines ? threadIdx.x >> 2 : m; e < m; e += blockDim.x >> 2) {
         const double2 v = res[b * m + e];
         re = max(re, (unsigned)__double2hiint(v.x) & 0x7fffffffu);
         im = max(im, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
@@ -37,7 +38,7 @@ __device__ __forceinline__ void collect_max(const double2* res, int m, unsigned*
         re = max(re, __shfl_xor_sync(0xffffffffu, re, o));
         im = max(im, __shfl_xor_sync(0xffffffffu, im, o));
     }
-    if ((threadIdx.x & 31) < 4) {
+    if ((threadIdx.x & 31) < lines) {
         atomicMax(top + 2 * b, re);
         atomicMax(top + 2 * b + 1, im);
     }
@@ -49,7 +50,7 @@ __global__ void __launch_bounds__(kThreads)
 k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, int ny, int nb,
         int rows, FftDesc d, const cplx_t<T>* __restrict__ tw, int sign, int interleave,
         const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear,
-        int4* __restrict__ ffix, unsigned* __restrict__ ftop) {
+        int4* __restrict__ ffix, unsigned* __restrict__ ftop, void* __restrict__ sums, int sums32) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* b0 = reinterpret_cast<C*>(smem_raw);
@@ -63,7 +64,26 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     const size_t plane = (size_t)nx * ny;
     griddep_wait();  // the input is the previous kernel's output
     griddep_launch();
-    for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
+    if constexpr (sizeof(T) == 8) {
+        if (sums) {  // nb values a node (FP64 or FP32), zeroed for the next sums; one row
+            for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
+                const int jj = e / nb, b = e - jj * nb;
+                const size_t src = (size_t)i0 * ny * nb + e;
+                double2 v;
+                if (sums32) {
+                    float2* q = reinterpret_cast<float2*>(sums) + src;
+                    v = make_double2(q->x, q->y);
+                    *q = make_float2(0.f, 0.f);
+                } else {
+                    double2* q = reinterpret_cast<double2*>(sums) + src;
+                    v = *q;
+                    *q = make_double2(0.0, 0.0);
+                }
+                b0[b * ny + jj] = v;
+            }
+        }
+    }
+    for (int e = sums ? lines * ny : threadIdx.x; e < lines * ny; e += blockDim.x) {
         int l = e / ny, jj = e - l * ny;
         int b = l / rows, r = l - b * rows;
         const size_t src = b * plane + (size_t)(i0 + r) * ny + jj;
@@ -87,7 +107,7 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     if (interleave) {
         if constexpr (sizeof(T) == 8) {
             if (ffix) {  // nb = 4, one row: the fixed-point fields of the row beside the FP64 ones
-                collect_max(res, ny, top);
+                collect_max(res, 4, ny, top);
                 __syncthreads();
                 if (threadIdx.x < 8) ftop[8 * i0 + threadIdx.x] = top[threadIdx.x];
                 const int b = threadIdx.x & 3;
@@ -108,10 +128,25 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
             out[((size_t)(i0 + r) * ny + jj) * nb + b] = res[(b * rows + r) * ny + jj];
         }
     } else {
+        if constexpr (sizeof(T) == 8) {
+            if (ffix) {  // nb = 1: the fixed-point values of the one or two rows as well
+                collect_max(res, rows, ny, top);
+                __syncthreads();
+                if (threadIdx.x < 2 * rows) ftop[2 * i0 + threadIdx.x] = top[threadIdx.x];
+            }
+        }
         for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
             int l = e / ny, jj = e - l * ny;
             int b = l / rows, r = l - b * rows;
-            out[b * plane + (size_t)(i0 + r) * ny + jj] = res[e];
+            const size_t o = b * plane + (size_t)(i0 + r) * ny + jj;
+            out[o] = res[e];
+            if constexpr (sizeof(T) == 8) {
+                if (ffix) {
+                    const int2 re = field_fix(res[e].x, row_exponent(top[2 * l]));
+                    const int2 im = field_fix(res[e].y, row_exponent(top[2 * l + 1]));
+                    ffix[o] = make_int4(re.x, re.y, im.x, im.y);
+                }
+            }
         }
     }
 }
@@ -163,7 +198,8 @@ template <typename T>
 static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                               const void* tw, int sign, int interleave, const longlong2* fix_in,
                               double unscale, longlong2* clear, cudaStream_t s,
-                              const FixFields* fix = nullptr) {
+                              const FixFields* fix = nullptr, void* sums = nullptr,
+                              bool sums32 = false) {
     using C = cplx_t<T>;
     const size_t per_line = 2 * (size_t)ny * sizeof(C);
     const size_t tw_bytes = (size_t)ny * sizeof(C);
@@ -177,16 +213,24 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
     if (e != cudaSuccess) return e;
     return launch_pdl(k_fft_y<T>, dim3(nx / rows), dim3(kThreads), smem, s, (const C*)in, (C*)out,
                       nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear,
-                      fix ? (int4*)fix->f : nullptr, fix ? fix->top : nullptr);
+                      fix ? (int4*)fix->f : nullptr, fix ? fix->top : nullptr, sums,
+                      sums32 ? 1 : 0);
 }
 
 template <typename T>
 cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                          const void* tw, int sign, int interleave, cudaStream_t s,
                          const FixFields* fix) {
-    if (fix && (sizeof(T) != 8 || nb != 4 || !interleave)) return cudaErrorInvalidValue;
+    if (fix && (sizeof(T) != 8 || !(nb == 4 ? interleave : nb == 1 && !interleave)))
+        return cudaErrorInvalidValue;
     return fft_y_impl<T>(in, out, nx, ny, nb, d, tw, sign, interleave, nullptr, 0.0, nullptr, s,
                          fix);
+}
+
+cudaError_t launch_fft_y_from_sums(void* sums, bool f32, void* out, int nx, int ny,
+                                   const FftDesc& d, const void* tw, cudaStream_t s) {
+    return fft_y_impl<double>(nullptr, out, nx, ny, 4, d, tw, -1, 0, nullptr, 0.0, nullptr, s,
+                              nullptr, sums, f32);
 }
 
 template <typename T>

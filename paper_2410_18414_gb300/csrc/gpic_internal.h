@@ -119,11 +119,16 @@ struct FixFields {
     unsigned* top;
 };
 // Along y (contiguous); out_interleave != 0 writes out[(i*ny + j)*nb + b].  fix (FP64,
-// interleaved with nb = 4; may be NULL): the outputs in fixed point as well.
+// interleaved with nb = 4, or nb = 1; may be NULL): the outputs in fixed point as well (nb = 1:
+// one int4 a node, two maxima a row).
 template <typename T>
 cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
                          const void* twiddle, int sign, int out_interleave, cudaStream_t s,
                          const FixFields* fix = nullptr);
+// Forward transform along y of four complex values a node summed by the adjoint's particle
+// kernels (FP64, or FP32 pairs converted on load) into four planes; zeroes the sums.
+cudaError_t launch_fft_y_from_sums(void* sums, bool f32, void* out, int nx, int ny,
+                                   const FftDesc& d, const void* twiddle, cudaStream_t s);
 // Forward transform along y of the fixed-point current (converted on load); zeroes
 // `clear` (same shape, may be NULL) on the way, the buffer the next deposit sums into.
 template <typename T>
@@ -384,25 +389,22 @@ struct AdjModeParams {
 };
 // The reverse particle kernels run in the forward's storage type T (double: the plain
 // path; float: the FP32 form); the current adjoint they read (Jb) is FP64 in both, the
-// field adjoints they add are FP64 (Fb) or, for T = float, FP32 sums (fb32).
+// field adjoints they add (Fb: [node][8], zero before the first step) are sums in T.
 //
 // Reverse push + gather of one step: reads x^{n+1}, P^{n+1} (state n+1), v^n, v^{n-1}
 // (state n), the step's record (gf: the gathered A and grad A at 4 n .. 10 n, FP64, see
-// launch_gather_push; lean: the record stops at 4 n and they are gathered again from F)
-// and the step's gather fields F ([node][4] complex of T); updates the particle adjoints
-// and adds the eight field adjoints into Fb (four planes [k][node] of (f_2k, f_2k+1)).
+// launch_gather_push; lean: the record stops at 4 n and they are gathered again) and the
+// step's gather fields F ([node][4] complex of T) or, FP64, in fixed point (fix); updates
+// the particle adjoints and adds the eight field adjoints into Fb.
 template <typename T>
 cudaError_t launch_adj_push_gather(int p, const ParticleGeom& g, const PushParams& pp,
                                    const T* x1, const T* y1, const T* px1, const T* py1,
                                    const T* vx, const T* vy, const T* vxo, const T* vyo,
                                    const double* gf, bool lean, const void* F,
-                                   AdjParticlesT<T> ab, double2* Fb, void* fb32, int64_t n,
+                                   const FixFields* fix, AdjParticlesT<T> ab, T* Fb, int64_t n,
                                    unsigned int* err, cudaStream_t s);
-// The FP32 form's field adjoints (fb32: [node][2] float4, fields 0-3 and 4-7, summed by
-// launch_adj_push_gather<float>) to the four FP64 planes Fb of the reverse field solve.
-cudaError_t launch_fb32_to_planes(const void* fb32, double2* Fb, int64_t ng, cudaStream_t s);
 // Reverse field solve per mode of the stepper `kind` (a StepperKind: ap, cp or dp used,
-// their pointers the history adjoints): Zb = forward transforms of the four Fb planes;
+// their pointers the history adjoints): Zb = forward transforms of the four planes of Fb;
 // writes the packed adjoint current spectrum Js (unnormalised inverse transform -> mesh).
 // CDF-2 writes the adjoints before the step into the other buffer of each (cur, prev)
 // pair, for the caller to swap; BDF and DIRK update in place.
@@ -416,11 +418,12 @@ cudaError_t launch_adj_columns(const ModeCommon& mc, int kind, const AdjModePara
                                const CdfParams& cp, const DirkParams& dp, const double2* Zb,
                                double2* Js, const FftDesc& fd, const double2* tw,
                                cudaStream_t s);
-// Reverse deposit + move: gathers the mesh current adjoint Jb ([node] (jx, jy)) at x^{n+1}.
+// Reverse deposit + move: gathers the mesh current adjoint Jb ([node] (jx, jy); FP64 with
+// fix: its fixed-point form) at x^{n+1}.
 template <typename T>
 cudaError_t launch_adj_deposit_move(int p, const ParticleGeom& g, const T* x1, const T* y1,
                                     const T* vx, const T* vy, const double2* Jb,
-                                    AdjParticlesT<T> ab, int64_t n, unsigned int* err,
+                                    const FixFields* fix, AdjParticlesT<T> ab, int64_t n, unsigned int* err,
                                     cudaStream_t s);
 // Objective seed sum bzb B_z at the final level, from zs = DFT(bzb).
 cudaError_t launch_adj_seed(const ModeCommon& mc, const double2* zs, double2* ax, double2* ay,

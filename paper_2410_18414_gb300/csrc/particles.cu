@@ -14,6 +14,7 @@
 // position outside [0, L] (including NaN) is never used to index the grid: the
 // particle is skipped and the non-finite bit of the device error word is set.
 #include "common.cuh"
+#include "fixed.cuh"
 #include "gpic_internal.h"
 #include "launch.cuh"
 
@@ -188,61 +189,6 @@ struct AccFix {
 // 108 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
 // 256 x 192, quartic 353 -> 149 us (bound by L2's atomics still: 17.5 sectors a particle).
 constexpr int kRowThreads = 128;
-
-// FP64 shapes in fixed point: positions X = x/dx 2^sh (one FP64 multiply and conversion),
-// weights in units of 2^-62 by 64-bit multiply-highs.  GB300 issues 2 FP64 operations per
-// clock and SM but 32 32x32+64-bit multiply-adds, and the rounding of every step is 2^-62 of
-// the largest weight, finer than FP64's.
-constexpr long long kOne62 = 1ll << 62;
-__device__ __forceinline__ long long mul62(long long a, long long b) {  // a, b in [0, 2^62]
-    return (long long)__umul64hi((unsigned long long)a << 1, (unsigned long long)b << 1);
-}
-template <int P>
-__device__ __forceinline__ int fix_weights(long long X, int sh, long long* w) {
-    if (P % 2 == 0) X += 1ll << (sh - 1);
-    const int i = (int)(X >> sh);
-    // u: the offset within the cell (odd P) or from the midpoint before it (even P), in [0, 1)
-    const long long u = (X & ((1ll << sh) - 1)) << (62 - sh), v = kOne62 - u;
-    const long long u2 = mul62(u, u), v2 = mul62(v, v);
-    if constexpr (P == 2) {  // ((1-u)^2/2, the rest, u^2/2)
-        w[0] = v2 >> 1;
-        w[2] = u2 >> 1;
-        w[1] = kOne62 - w[0] - w[2];
-        return i - 1;
-    } else if constexpr (P == 3) {  // ((1-u)^3/6, 2/3 - u^2 + u^3/2, the rest, u^3/6)
-        constexpr unsigned long long sixth = 0x2AAAAAAAAAAAAAABull;  // 2^64 / 6
-        const long long u3 = mul62(u2, u), v3 = mul62(v2, v);
-        w[0] = (long long)__umul64hi((unsigned long long)v3, sixth);
-        w[3] = (long long)__umul64hi((unsigned long long)u3, sixth);
-        w[1] = 0x2AAAAAAAAAAAAAABll - u2 + (u3 >> 1);  // 2/3 in units of 2^-62
-        w[2] = kOne62 - w[0] - w[1] - w[3];
-        return i - 1;
-    } else {  // ((1-u)^4, 11 - 12u - 6u^2 + 12u^3 - 4u^4, the rest, 1 + 4u + 6u^2 + 4u^3 - 4u^4,
-              //  u^4) / 24; the polynomials in units of 2^-58
-        constexpr unsigned long long inv24 = 0x0AAAAAAAAAAAAAABull, two3 = 0xAAAAAAAAAAAAAAABull;
-        const long long u3 = mul62(u2, u), u4 = mul62(u2, u2), v4 = mul62(v2, v2);
-        const long long a = u >> 4, a2 = u2 >> 4, a3 = u3 >> 4, a4 = u4 >> 4, one = kOne62 >> 4;
-        const long long n1 = 11 * one - 12 * a - 6 * a2 + 12 * a3 - 4 * a4;
-        const long long n3 = one + 4 * (a + a3 - a4) + 6 * a2;
-        w[0] = (long long)__umul64hi((unsigned long long)v4, inv24);
-        w[1] = (long long)__umul64hi((unsigned long long)n1, two3);  // 16/24
-        w[3] = (long long)__umul64hi((unsigned long long)n3, two3);
-        w[4] = (long long)__umul64hi((unsigned long long)u4, inv24);
-        w[2] = kOne62 - w[0] - w[1] - w[3] - w[4];
-        return i - 2;
-    }
-}
-// Fixed-point positions: x/dx 2^sh with nx, ny <= 2^(62 - sh).
-struct FixGeom {
-    double sx, sy;  // 2^sh / dx, 2^sh / dy
-    int sh;
-};
-inline FixGeom fix_geom(const ParticleGeom& g) {
-    int b = 0;
-    while ((1 << b) < (g.nx > g.ny ? g.nx : g.ny)) ++b;
-    const double s = (double)(1ull << (62 - b));
-    return FixGeom{g.inv_dx * s, g.inv_dy * s, 62 - b};
-}
 
 // A policy says what a particle's record holds (per component the row factors t[a], then
 // W_y[b]), a contribution's value from it and how it is added to word `c` of a node.
@@ -767,15 +713,6 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
 //     products and sums to, and than the transform's own error in f, 2^-53 of the largest
 //     value.
 // Integer sums do not depend on their order, and the same bits come out on every path.
-//
-// v / 2^d rounded, d >= 0
-__device__ __forceinline__ long long shift_round(long long v, int d) {
-    d = min(d, 62);
-    return (v + ((1ll << d) >> 1)) >> d;
-}
-__device__ __forceinline__ double field_unit(int e) {
-    return e > 1024 ? __hiloint2double(0x7ff80000, 0) : pow2(e - 58);
-}
 template <int P>
 __global__ void __launch_bounds__(kRowGatherThreads)
 k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* __restrict__ x,

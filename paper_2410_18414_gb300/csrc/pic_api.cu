@@ -301,8 +301,9 @@ pic_status alloc_state(pic_handle* h) {
     // The FP64 gather in fixed point, where converting the mesh fields (16 FP64 operations a
     // node) is small beside what it saves (about 200 a particle).
     if (!h->fp32 && h->vdim == 2 && h->spp.n == 0 && h->n >= (int64_t)(h->ng / 8)) {
-        CK(dalloc(h, &h->fixf.f, 4 * h->ng * cs));
-        CK(dalloc(h, (void**)&h->fixf.top, (size_t)c.nx * 8 * sizeof(unsigned)));
+        const size_t fb = 4 * h->ng * sizeof(int4);  // the maxima follow the fields
+        CK(dalloc(h, &h->fixf.f, fb + (size_t)c.nx * 8 * sizeof(unsigned)));
+        h->fixf.top = (unsigned*)((char*)h->fixf.f + fb);
     }
     CK(dalloc(h, &h->E, h->ng * cs));
     CK(dalloc(h, &h->tmp, h->ng * cs));
