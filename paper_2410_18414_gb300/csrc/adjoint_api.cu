@@ -70,22 +70,10 @@ struct pic_adjoint {
     double2* e0 = nullptr;       // E^0 on the mesh, ng (Ex, Ey)
     double2* tmp = nullptr;      // ng
     bool forward_done = false;
-    std::vector<void*> allocs;
+    BufferArena arena;           // every buffer above
 };
 
 namespace {
-
-cudaError_t aalloc(pic_adjoint* a, void** p, size_t bytes) {
-    *p = nullptr;
-    cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
-    if (e == cudaSuccess) a->allocs.push_back(*p);
-    return e;
-}
-
-void release(pic_adjoint* a) {
-    for (void* p : a->allocs) cudaFree(p);
-    a->allocs.clear();
-}
 
 // The handle's particle arrays in state order (v^n first).
 void handle_arrays(pic_handle* h, void* arr[8]) {
@@ -358,45 +346,52 @@ pic_status pic_adjoint_create_ex(pic_handle* h, int32_t nsteps, int32_t checkpoi
     a->f32 = h->fp32;
     a->rsz = h->rsz;
     a->fix = h->fixf.f != nullptr;
-    const size_t sb = 8 * std::max<size_t>(a->n, 1) * a->rsz;
-    const size_t hbytes = (size_t)a->nh * a->ng * sizeof(double2);
-    const size_t gb = a->ng * sizeof(double2);
-    cudaError_t e = cudaSuccess;
     a->ck.resize(a->nseg + 1);
-    for (auto& c : a->ck) {
-        if (e == cudaSuccess) e = aalloc(a, (void**)&c.state, sb);
-        if (e == cudaSuccess) e = aalloc(a, (void**)&c.hist, hbytes);
-    }
-    const size_t gfb = 4 * a->ng * 2 * a->rsz;  // one step's gather fields
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->final_j, h->jbytes);
-    if (e == cudaSuccess) e = aalloc(a, &a->final_g, gfb);
-    if (e == cudaSuccess) e = aalloc(a, &a->rec, (size_t)a->K * sb);
-    if (e == cudaSuccess) e = aalloc(a, &a->recg, nrec * rec_field_bytes(a));
-    if (e == cudaSuccess)
-        e = aalloc(a, (void**)&a->recf,
-                   nrec * rec_width(a) * std::max<size_t>(a->n, 1) * sizeof(double));
-    if (e == cudaSuccess) e = aalloc(a, &a->ab, sb);
-    if (e == cudaSuccess && a->fix) e = aalloc(a, &a->jfix.f, a->ng * sizeof(int4));
-    if (e == cudaSuccess && a->fix)
-        e = aalloc(a, (void**)&a->jfix.top, (size_t)h->nx * 2 * sizeof(unsigned));
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->twx, (size_t)h->nx * sizeof(double2));
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->twy, (size_t)h->ny * sizeof(double2));
+    auto layout = [&] {  // run twice, see BufferArena
+        const size_t sb = 8 * std::max<size_t>(a->n, 1) * a->rsz;
+        const size_t hbytes = (size_t)a->nh * a->ng * sizeof(double2);
+        const size_t gb = a->ng * sizeof(double2);
+        auto take = [&](auto** p, size_t bytes) {
+            void* v = nullptr;
+            a->arena.take(&v, bytes);
+            *p = static_cast<std::remove_reference_t<decltype(*p)>>(v);
+        };
+        for (auto& c : a->ck) {
+            take(&c.state, sb);
+            take(&c.hist, hbytes);
+        }
+        take(&a->final_j, h->jbytes);
+        take(&a->final_g, 4 * a->ng * 2 * a->rsz);  // one step's gather fields
+        take(&a->rec, (size_t)a->K * sb);
+        take(&a->recg, nrec * rec_field_bytes(a));
+        take(&a->recf, nrec * rec_width(a) * std::max<size_t>(a->n, 1) * sizeof(double));
+        take(&a->ab, sb);
+        if (a->fix) {
+            take(&a->jfix.f, a->ng * sizeof(int4));
+            take(&a->jfix.top, (size_t)h->nx * 2 * sizeof(unsigned));
+        }
+        take(&a->twx, (size_t)h->nx * sizeof(double2));
+        take(&a->twy, (size_t)h->ny * sizeof(double2));
+        take(&a->hb, hbytes);
+        take(&a->fb, a->ng * 8 * a->rsz);
+        take(&a->zb, 4 * gb);
+        take(&a->js, gb);
+        take(&a->jg, gb);
+        take(&a->e0, gb);
+        take(&a->tmp, gb);
+    };
+    layout();
+    cudaError_t e = a->arena.allocate(h->s);
+    layout();
     if (e == cudaSuccess) e = launch_twiddles<double>(a->twx, h->nx, h->s);
     if (e == cudaSuccess) e = launch_twiddles<double>(a->twy, h->ny, h->s);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->hb, hbytes);
-    if (e == cudaSuccess) e = aalloc(a, &a->fb, a->ng * 8 * a->rsz);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->zb, 4 * gb);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->js, gb);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->jg, gb);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->e0, gb);
-    if (e == cudaSuccess) e = aalloc(a, (void**)&a->tmp, gb);
     // E^0 = -grad phi^0 on the mesh (every phi level holds phi^0 at step 0)
     const void* phi0 = a->kind == K_BDF ? h->phi_l[h->head] : a->kind == K_CDF2 ? h->cdf.phi : h->dirk.phi;
     if (e == cudaSuccess) e = launch_adj_e0(h->mc, (const double2*)phi0, a->tmp, h->s);
     if (e == cudaSuccess) e = fft64_inverse(a, a->tmp, a->e0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
     if (e != cudaSuccess) {
-        release(a);
+        a->arena.release();
         delete a;
         return fail(h, PIC_ERR_CUDA, "pic_adjoint_create: %s", cudaGetErrorString(e));
     }
@@ -533,7 +528,7 @@ int32_t pic_adjoint_checkpoint_every(const pic_adjoint* a) { return a ? a->K : 0
 void pic_adjoint_destroy(pic_adjoint* a) {
     if (!a) return;
     if (a->h) cudaStreamSynchronize(a->h->s);
-    release(a);
+    a->arena.release();
     delete a;
 }
 

@@ -5,11 +5,48 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
 #include "gpic_internal.h"
 #include "pic.h"
+
+// One device allocation cut into a handle's (or an adjoint's) buffers: the owner runs its
+// layout twice, first to add up the sizes, then, after allocate(), to take the addresses.  A
+// handle has about 60 buffers, and a cudaMalloc and a cudaFree for each cost more than a short
+// run's steps (set-up, 20 steps of 400,000 particles on 96 x 96, read-back and clean-up:
+// 3.16 ms, with one allocation 1.74 ms).  Buffers asked for as zeroed lie together and are
+// cleared by one memset.
+class BufferArena {
+public:
+    // *p: the buffer's address, or NULL while measuring.
+    void take(void** p, size_t bytes, bool zeroed = false) {
+        const size_t b = (std::max<size_t>(bytes, 16) + 511) & ~(size_t)511;
+        size_t& off = off_[zeroed ? 1 : 0];
+        *p = base_ ? base_ + (zeroed ? size_[0] : 0) + off : nullptr;
+        off += b;
+    }
+    cudaError_t allocate(cudaStream_t s) {
+        size_[0] = off_[0];
+        size_[1] = off_[1];
+        off_[0] = off_[1] = 0;
+        if (size_[0] + size_[1] == 0) return cudaSuccess;
+        void* p = nullptr;
+        cudaError_t e = cudaMalloc(&p, size_[0] + size_[1]);
+        if (e != cudaSuccess) return e;
+        base_ = static_cast<char*>(p);
+        return size_[1] ? cudaMemsetAsync(base_ + size_[0], 0, size_[1], s) : cudaSuccess;
+    }
+    void release() {
+        if (base_) cudaFree(base_);
+        base_ = nullptr;
+    }
+
+private:
+    char* base_ = nullptr;
+    size_t size_[2] = {0, 0}, off_[2] = {0, 0};
+};
 
 struct pic_handle {
     pic_config cfg{};
@@ -112,7 +149,8 @@ struct pic_handle {
     bool pending = false;
     bool no_defer = false;  // set while an ensemble captures the run's steps
     bool stepped = false;
-    std::vector<void*> allocs;
+    BufferArena arena;               // every buffer of the state
+    void* diag_alloc = nullptr;      // diag_ring, allocated when diagnostics are first asked for
     gpic::ModeCommon mc{};
     gpic::ParticleGeom geom{};
     gpic::PushParams push{};

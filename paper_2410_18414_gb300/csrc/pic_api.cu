@@ -202,14 +202,6 @@ pic_status validate(const pic_config* c, const pic_particles_in* in) {
     return PIC_OK;
 }
 
-cudaError_t dalloc(pic_handle* h, void** p, size_t bytes) {
-    *p = nullptr;
-    if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) h->allocs.push_back(*p);
-    return e;
-}
-
 void free_timers(pic_handle* h) {
     for (auto& t : h->kt) {
         for (cudaEvent_t e : t.ev) cudaEventDestroy(e);
@@ -221,8 +213,9 @@ void free_timers(pic_handle* h) {
 
 void free_all(pic_handle* h) {
     free_timers(h);
-    for (void* p : h->allocs) cudaFree(p);
-    h->allocs.clear();
+    h->arena.release();
+    if (h->diag_alloc) cudaFree(h->diag_alloc);
+    h->diag_alloc = nullptr;
 }
 
 // Newest spectral level: 0 phi, 1 Ax, 2 Ay, 3 rho, 4 Az (2D-3V).
@@ -240,103 +233,89 @@ void* newest(pic_handle* h, int which) {
 }
 
 
-pic_status alloc_state(pic_handle* h) {
+// The handle's buffers (run twice, see BufferArena).
+void layout_state(pic_handle* h) {
     const pic_config& c = h->cfg;
+    BufferArena& ar = h->arena;
     const size_t cs = 2 * h->rsz;
-    const size_t pn = (size_t)std::max<int64_t>(h->n, 1) * h->rsz;
+    const size_t np = (size_t)std::max<int64_t>(h->n, 1), pn = np * h->rsz;
+    auto take = [&](auto** p, size_t bytes, bool zeroed = false) {
+        void* v = nullptr;
+        ar.take(&v, bytes, zeroed);
+        *p = static_cast<std::remove_reference_t<decltype(*p)>>(v);
+    };
     if (!h->bound) {  // else the caller's arrays, set by pic_init_bound
-        CK(dalloc(h, &h->x, pn));
-        CK(dalloc(h, &h->y, pn));
-        CK(dalloc(h, &h->px, pn));
-        CK(dalloc(h, &h->py, pn));
+        take(&h->x, pn);
+        take(&h->y, pn);
+        take(&h->px, pn);
+        take(&h->py, pn);
         for (int b = 0; b < 2; ++b)
-            for (int k = 0; k < 2; ++k) CK(dalloc(h, &h->v[b][k], pn));
+            for (int k = 0; k < 2; ++k) take(&h->v[b][k], pn);
     }
-    CK(dalloc(h, (void**)&h->stage, (size_t)std::max<int64_t>(h->n, 1) * sizeof(double)));
+    take(&h->stage, np * sizeof(double));
     if (h->sorting) {
-        const size_t ni = (size_t)std::max<int64_t>(h->n, 1) * sizeof(int);
-        for (int a = 0; a < 8; ++a) CK(dalloc(h, &h->alt[a], pn));
+        const size_t ni = np * sizeof(int);
+        for (int a = 0; a < 8; ++a) take(&h->alt[a], pn);
         if (h->fp32) {  // the moved positions of a pending deposit
-            CK(dalloc(h, &h->xnext, pn));
-            CK(dalloc(h, &h->ynext, pn));
+            take(&h->xnext, pn);
+            take(&h->ynext, pn);
         }
-        CK(dalloc(h, (void**)&h->id, ni));
-        CK(dalloc(h, (void**)&h->id_alt, ni));
-        CK(dalloc(h, (void**)&h->keys, ni));
+        take(&h->id, ni);
+        take(&h->id_alt, ni);
+        take(&h->keys, ni);
         const size_t nt = (size_t)h->tg.nkeys() + 1;
-        CK(dalloc(h, (void**)&h->hist, nt * sizeof(int)));
-        CK(cudaMemsetAsync(h->hist, 0, nt * sizeof(int), h->s));  // kept zero by the sort's scan
-        CK(dalloc(h, (void**)&h->off, nt * sizeof(int)));
-        CK(dalloc(h, (void**)&h->cursor, nt * sizeof(int)));
-        CK(dalloc(h, (void**)&h->bsum, sort_scan_chunks(h->tg.nkeys()) * sizeof(int)));
-        CK(launch_iota(h->id, h->n, h->s));
+        take(&h->hist, nt * sizeof(int), true);  // kept zero by the sort's scan
+        take(&h->off, nt * sizeof(int));
+        take(&h->cursor, nt * sizeof(int));
+        take(&h->bsum, sort_scan_chunks(h->tg.nkeys()) * sizeof(int));
     }
     if (h->vdim == 3) {
-        CK(dalloc(h, &h->pz, pn));
-        CK(dalloc(h, &h->vz[0], pn));
-        CK(dalloc(h, &h->vz[1], pn));
-        CK(dalloc(h, &h->Jz, h->jbytes));
-        CK(dalloc(h, &h->Zz, h->ng * cs));
-        CK(dalloc(h, &h->F2, 2 * h->ng * cs));
-        CK(dalloc(h, &h->Gz, 2 * h->ng * cs));
+        take(&h->pz, pn);
+        take(&h->vz[0], pn);
+        take(&h->vz[1], pn);
+        take(&h->Jz, h->jbytes);
+        take(&h->Zz, h->ng * cs);
+        take(&h->F2, 2 * h->ng * cs);
+        take(&h->Gz, 2 * h->ng * cs);
     }
-    if (h->spp.n > 0)
-        CK(dalloc(h, (void**)&h->species, (size_t)std::max<int64_t>(h->n, 1) * sizeof(int32_t)));
-    if (h->sorting && h->spp.n > 0)  // the sort's second set
-        CK(dalloc(h, (void**)&h->species_alt,
-                  (size_t)std::max<int64_t>(h->n, 1) * sizeof(int32_t)));
+    if (h->spp.n > 0) take(&h->species, np * sizeof(int32_t));
+    if (h->sorting && h->spp.n > 0) take(&h->species_alt, np * sizeof(int32_t));  // the sort's second set
     if (h->sorting && h->vdim == 3)
-        for (int a = 0; a < 3; ++a) CK(dalloc(h, &h->z_alt[a], pn));
-    CK(dalloc(h, (void**)&h->J, h->jbytes));
-    CK(dalloc(h, (void**)&h->Jalt, h->jbytes));
-    CK(cudaMemsetAsync(h->Jalt, 0, h->jbytes, h->s));
-    CK(dalloc(h, &h->Z, h->ng * cs));
+        for (int a = 0; a < 3; ++a) take(&h->z_alt[a], pn);
+    take(&h->J, h->jbytes);
+    take(&h->Jalt, h->jbytes, true);
+    take(&h->Z, h->ng * cs);
     if (h->cfg.charge == PIC_CHARGE_DEPOSIT) {
-        CK(dalloc(h, &h->rhoq, h->jbytes));
-        CK(dalloc(h, &h->ZQ, h->ng * cs));
+        take(&h->rhoq, h->jbytes);
+        take(&h->ZQ, h->ng * cs);
         h->mc.zq = h->ZQ;
     }
-    CK(dalloc(h, &h->F4, 4 * h->ng * cs));
-    CK(dalloc(h, &h->G, 4 * h->ng * cs));
+    take(&h->F4, 4 * h->ng * cs);
+    take(&h->G, 4 * h->ng * cs);
     // The FP64 gather in fixed point, where converting the mesh fields (16 FP64 operations a
     // node) is small beside what it saves (about 200 a particle).
     if (!h->fp32 && h->vdim == 2 && h->spp.n == 0 && h->n >= (int64_t)(h->ng / 8)) {
         const size_t fb = 4 * h->ng * sizeof(int4);  // the maxima follow the fields
-        CK(dalloc(h, &h->fixf.f, fb + (size_t)c.nx * 8 * sizeof(unsigned)));
+        take(&h->fixf.f, fb + (size_t)c.nx * 8 * sizeof(unsigned));
         h->fixf.top = (unsigned*)((char*)h->fixf.f + fb);
     }
-    CK(dalloc(h, &h->E, h->ng * cs));
-    CK(dalloc(h, &h->tmp, h->ng * cs));
-    CK(dalloc(h, (void**)&h->tmpd, h->ng * sizeof(double)));
-    CK(dalloc(h, &h->twx, (size_t)c.nx * cs));
-    CK(dalloc(h, &h->twy, (size_t)c.ny * cs));
-    CK(dalloc(h, (void**)&h->diag, D_NSLOTS * sizeof(double)));
-    {
-        const int stages = c.stepper == PIC_STEPPER_DIRK ? c.dirk_stages : 1;
-        double *kxt = nullptr, *kyt = nullptr, *invd = nullptr;
-        CK(dalloc(h, (void**)&kxt, (size_t)c.nx * sizeof(double)));
-        CK(dalloc(h, (void**)&kyt, (size_t)c.ny * sizeof(double)));
-        CK(dalloc(h, (void**)&invd, (size_t)stages * h->ng * sizeof(double)));
-        h->mc.kxt = kxt;
-        h->mc.kyt = kyt;
-        h->mc.invd = invd;
-        h->mc.dirkm = nullptr;
-        if (c.stepper == PIC_STEPPER_DIRK) {  // the per-mode step matrices
-            double* dirkm = nullptr;
-            CK(dalloc(h, (void**)&dirkm, 8 * h->ng * sizeof(double)));
-            h->mc.dirkm = dirkm;
-        }
-    }
-    CK(dalloc(h, (void**)&h->err, sizeof(unsigned int)));
-    CK(cudaMemsetAsync(h->err, 0, sizeof(unsigned int), h->s));
-    CK(cudaMemsetAsync(h->diag, 0, D_NSLOTS * sizeof(double), h->s));
+    take(&h->E, h->ng * cs);
+    take(&h->tmp, h->ng * cs);
+    take(&h->tmpd, h->ng * sizeof(double));
+    take(&h->twx, (size_t)c.nx * cs);
+    take(&h->twy, (size_t)c.ny * cs);
+    take(&h->diag, D_NSLOTS * sizeof(double), true);
+    const int stages = c.stepper == PIC_STEPPER_DIRK ? c.dirk_stages : 1;
+    take(&h->mc.kxt, (size_t)c.nx * sizeof(double));
+    take(&h->mc.kyt, (size_t)c.ny * sizeof(double));
+    take(&h->mc.invd, (size_t)stages * h->ng * sizeof(double));
+    h->mc.dirkm = nullptr;
+    if (c.stepper == PIC_STEPPER_DIRK)  // the per-mode step matrices
+        take(&h->mc.dirkm, 8 * h->ng * sizeof(double));
+    take(&h->err, sizeof(unsigned int), true);
 
     // time histories are FP64 complex spectra in both precision forms
-    auto spec = [&](void** p) {
-        cudaError_t e = dalloc(h, p, h->ng * sizeof(double2));
-        if (e == cudaSuccess) e = cudaMemsetAsync(*p, 0, h->ng * sizeof(double2), h->s);
-        return e;
-    };
+    auto spec = [&](void** p) { ar.take(p, h->ng * sizeof(double2), true); };
     if (c.stepper == PIC_STEPPER_BDF) {
         const int k = c.bdf_order;
         h->L = 2 * k;
@@ -346,15 +325,39 @@ pic_status alloc_state(pic_handle* h) {
         h->ay_l.assign(h->L, nullptr);
         h->rho_l.assign(h->Lr, nullptr);
         for (int i = 0; i < h->L; ++i) {
-            CK(spec(&h->phi_l[i]));
-            CK(spec(&h->ax_l[i]));
-            CK(spec(&h->ay_l[i]));
+            spec(&h->phi_l[i]);
+            spec(&h->ax_l[i]);
+            spec(&h->ay_l[i]);
         }
-        for (int i = 0; i < h->Lr; ++i) CK(spec(&h->rho_l[i]));
+        for (int i = 0; i < h->Lr; ++i) spec(&h->rho_l[i]);
         if (h->vdim == 3) {
             h->az_l.assign(h->L, nullptr);
-            for (int i = 0; i < h->L; ++i) CK(spec(&h->az_l[i]));
+            for (int i = 0; i < h->L; ++i) spec(&h->az_l[i]);
         }
+    } else if (c.stepper == PIC_STEPPER_CDF2) {
+        void** slots[] = {&h->cdf.phi, &h->cdf.phi_prev, &h->cdf.rho, &h->cdf.rho_prev,
+                          &h->cdf.ax,  &h->cdf.ax_prev,  &h->cdf.ay,  &h->cdf.ay_prev,
+                          &h->cdf.jx,  &h->cdf.jx_prev,  &h->cdf.jy,  &h->cdf.jy_prev};
+        for (void** sl : slots) spec(sl);
+        if (h->vdim == 3)
+            for (void** sl : {&h->az, &h->az_prev, &h->jz, &h->jz_prev}) spec(sl);
+    } else {
+        void** slots[] = {&h->dirk.phi, &h->dirk.vphi, &h->dirk.ax, &h->dirk.vax, &h->dirk.ay,
+                          &h->dirk.vay, &h->dirk.rho,  &h->dirk.jx, &h->dirk.jy};
+        for (void** sl : slots) spec(sl);
+        if (h->vdim == 3)
+            for (void** sl : {&h->az, &h->vaz, &h->jz}) spec(sl);
+    }
+}
+
+pic_status alloc_state(pic_handle* h) {
+    const pic_config& c = h->cfg;
+    layout_state(h);
+    CK(h->arena.allocate(h->s));
+    layout_state(h);
+    if (h->sorting) CK(launch_iota(h->id, h->n, h->s));
+    if (c.stepper == PIC_STEPPER_BDF) {
+        const int k = c.bdf_order;
         // BDF-k with a_0 = 1 (section 3.2) from sum_{j=1..k} (1/j) nabla^j u = dt u'.
         double alpha[kMaxBdf + 1] = {0};
         for (int j = 1; j <= k; ++j) {
@@ -378,19 +381,7 @@ pic_status alloc_state(pic_handle* h) {
         h->bdf.inv_a0 = 1.0 / h->bdf.a[0];
         h->bdf.g = (c.c * beta * c.dt) * (c.c * beta * c.dt);
         h->bdf.g_eps0 = h->bdf.g / c.eps0;
-    } else if (c.stepper == PIC_STEPPER_CDF2) {
-        void** slots[] = {&h->cdf.phi, &h->cdf.phi_prev, &h->cdf.rho, &h->cdf.rho_prev,
-                          &h->cdf.ax,  &h->cdf.ax_prev,  &h->cdf.ay,  &h->cdf.ay_prev,
-                          &h->cdf.jx,  &h->cdf.jx_prev,  &h->cdf.jy,  &h->cdf.jy_prev};
-        for (void** sl : slots) CK(spec(sl));
-        if (h->vdim == 3)
-            for (void** sl : {&h->az, &h->az_prev, &h->jz, &h->jz_prev}) CK(spec(sl));
-    } else {
-        void** slots[] = {&h->dirk.phi, &h->dirk.vphi, &h->dirk.ax, &h->dirk.vax, &h->dirk.ay,
-                          &h->dirk.vay, &h->dirk.rho,  &h->dirk.jx, &h->dirk.jy};
-        for (void** sl : slots) CK(spec(sl));
-        if (h->vdim == 3)
-            for (void** sl : {&h->az, &h->vaz, &h->jz}) CK(spec(sl));
+    } else if (c.stepper == PIC_STEPPER_DIRK) {
         const int s = c.dirk_stages;
         h->dirk.s = s;
         double r0 = 0, r1 = 0;
@@ -1261,9 +1252,8 @@ pic_status pic_set_diagnostics(pic_handle* h, int32_t every) {
     if (!h) return fail(nullptr, PIC_ERR_INVALID_ARG, "NULL handle");
     if (every < 0) return fail(h, PIC_ERR_INVALID_ARG, "every must be >= 0");
     if (every > 0 && !h->diag_ring) {
-        void* p = nullptr;
-        CK(dalloc(h, &p, (size_t)PIC_DIAG_HISTORY * D_NSLOTS * sizeof(double)));
-        h->diag_ring = static_cast<double*>(p);
+        CK(cudaMalloc(&h->diag_alloc, (size_t)PIC_DIAG_HISTORY * D_NSLOTS * sizeof(double)));
+        h->diag_ring = static_cast<double*>(h->diag_alloc);
         h->ring_step.assign(PIC_DIAG_HISTORY, -1);
     }
     h->diag_every = every;
