@@ -44,16 +44,33 @@ __device__ __forceinline__ void collect_max(const double2* res, int lines, int m
     }
 }
 
+// A second set of arrays of the same launch (the CTAs of blockIdx.y = 1).
+template <typename T>
+struct FftSecond {
+    const cplx_t<T>* in;
+    cplx_t<T>* out;
+    int nb;
+    const longlong2* fix_in;
+    longlong2* clear;
+};
+
 // Transforms along y (contiguous): CTA = `rows` consecutive x-indices of all nb arrays.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, int ny, int nb,
         int rows, FftDesc d, const cplx_t<T>* __restrict__ tw, int sign, int interleave,
         const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear,
-        int4* __restrict__ ffix, unsigned* __restrict__ ftop, void* __restrict__ sums, int sums32) {
+        int4* __restrict__ ffix, unsigned* __restrict__ ftop, void* __restrict__ sums, int sums32, FftSecond<T> two) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* b0 = reinterpret_cast<C*>(smem_raw);
+    if (blockIdx.y) {
+        in = two.in;
+        out = two.out;
+        nb = two.nb;
+        fix_in = two.fix_in;
+        clear = two.clear;
+    }
     const int lines = nb * rows;
     C* b1 = b0 + lines * ny;
     C* tws = b1 + lines * ny;  // twiddles, staged before the wait (they are constant)
@@ -199,7 +216,7 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
                               const void* tw, int sign, int interleave, const longlong2* fix_in,
                               double unscale, longlong2* clear, cudaStream_t s,
                               const FixFields* fix = nullptr, void* sums = nullptr,
-                              bool sums32 = false) {
+                              bool sums32 = false, const FftSecond<T>* two = nullptr) {
     using C = cplx_t<T>;
     const size_t per_line = 2 * (size_t)ny * sizeof(C);
     const size_t tw_bytes = (size_t)ny * sizeof(C);
@@ -211,10 +228,11 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
     size_t smem = (size_t)rows * nb * per_line + tw_bytes;
     cudaError_t e = set_smem(k_fft_y<T>, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_fft_y<T>, dim3(nx / rows), dim3(kThreads), smem, s, (const C*)in, (C*)out,
+    return launch_pdl(k_fft_y<T>, dim3(nx / rows, two ? 2 : 1), dim3(kThreads), smem, s,
+                      (const C*)in, (C*)out,
                       nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear,
                       fix ? (int4*)fix->f : nullptr, fix ? fix->top : nullptr, sums,
-                      sums32 ? 1 : 0);
+                      sums32 ? 1 : 0, two ? *two : FftSecond<T>{});
 }
 
 template <typename T>
@@ -236,8 +254,21 @@ cudaError_t launch_fft_y_from_sums(void* sums, bool f32, void* out, int nx, int 
 template <typename T>
 cudaError_t launch_fft_y_from_fix(const longlong2* j, double unscale, void* out, int nx, int ny,
                                   const FftDesc& d, const void* tw, longlong2* clear,
-                                  cudaStream_t s) {
-    return fft_y_impl<T>(nullptr, out, nx, ny, 1, d, tw, -1, 0, j, unscale, clear, s);
+                                  cudaStream_t s, const longlong2* j2, void* out2,
+                                  longlong2* clear2) {
+    const FftSecond<T> two{nullptr, (cplx_t<T>*)out2, 1, j2, clear2};
+    return fft_y_impl<T>(nullptr, out, nx, ny, 1, d, tw, -1, 0, j, unscale, clear, s, nullptr,
+                         nullptr, false, j2 ? &two : nullptr);
+}
+
+template <typename T>
+cudaError_t launch_fft_y_fields(const void* f4, void* g, const void* f2, void* g2, int nx, int ny,
+                                const FftDesc& d, const void* tw, const FixFields* fix,
+                                cudaStream_t s) {
+    if (fix && (sizeof(T) != 8 || f2)) return cudaErrorInvalidValue;
+    const FftSecond<T> two{(const cplx_t<T>*)f2, (cplx_t<T>*)g2, 2, nullptr, nullptr};
+    return fft_y_impl<T>(f4, g, nx, ny, 4, d, tw, +1, 1, nullptr, 0.0, nullptr, s, fix, nullptr,
+                         false, f2 ? &two : nullptr);
 }
 
 template <typename T>
@@ -274,10 +305,18 @@ template cudaError_t launch_fft_x<float>(const void*, void*, int, int, int, cons
                                          const void*, int, cudaStream_t);
 template cudaError_t launch_fft_y_from_fix<double>(const longlong2*, double, void*, int, int,
                                                    const FftDesc&, const void*, longlong2*,
-                                                   cudaStream_t);
+                                                   cudaStream_t, const longlong2*, void*,
+                                                   longlong2*);
+template cudaError_t launch_fft_y_fields<double>(const void*, void*, const void*, void*, int, int,
+                                             const FftDesc&, const void*, const FixFields*,
+                                             cudaStream_t);
 template cudaError_t launch_fft_y_from_fix<float>(const longlong2*, double, void*, int, int,
-                                                  const FftDesc&, const void*, longlong2*,
-                                                  cudaStream_t);
+                                                   const FftDesc&, const void*, longlong2*,
+                                                   cudaStream_t, const longlong2*, void*,
+                                                   longlong2*);
+template cudaError_t launch_fft_y_fields<float>(const void*, void*, const void*, void*, int, int,
+                                             const FftDesc&, const void*, const FixFields*,
+                                             cudaStream_t);
 template cudaError_t launch_twiddles<double>(void*, int, cudaStream_t);
 template cudaError_t launch_twiddles<float>(void*, int, cudaStream_t);
 

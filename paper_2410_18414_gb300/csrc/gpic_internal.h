@@ -130,11 +130,20 @@ cudaError_t launch_fft_y(const void* in, void* out, int nx, int ny, int nb, cons
 cudaError_t launch_fft_y_from_sums(void* sums, bool f32, void* out, int nx, int ny,
                                    const FftDesc& d, const void* twiddle, cudaStream_t s);
 // Forward transform along y of the fixed-point current (converted on load); zeroes
-// `clear` (same shape, may be NULL) on the way, the buffer the next deposit sums into.
+// `clear` (same shape, may be NULL) for the next deposit.  j2 (may be NULL): J_z, transformed
+// to out2 in the same launch.
 template <typename T>
 cudaError_t launch_fft_y_from_fix(const longlong2* j, double unscale, void* out, int nx, int ny,
-                                  const FftDesc& d, const void* tw, longlong2* clear,
-                                  cudaStream_t s);
+                                  const FftDesc& d, const void* twiddle, longlong2* clear,
+                                  cudaStream_t s, const longlong2* j2 = nullptr,
+                                  void* out2 = nullptr, longlong2* clear2 = nullptr);
+// Inverse transforms along y of the gather fields: the four packed spectra f4 to g
+// ([node][4]; with fix, FP64, in fixed point as well) and, with f2, the two of A_z to g2
+// ([node][2]) in the same launch.
+template <typename T>
+cudaError_t launch_fft_y_fields(const void* f4, void* g, const void* f2, void* g2, int nx, int ny,
+                                const FftDesc& d, const void* twiddle, const FixFields* fix,
+                                cudaStream_t s);
 // Along x (stride ny).
 template <typename T>
 cudaError_t launch_fft_x(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
@@ -163,11 +172,6 @@ inline size_t field_columns_smem(int nx, size_t complex_bytes) {
     return 9 * (size_t)nx * complex_bytes;  // two buffers of 4 lines, the twiddles
 }
 constexpr size_t kFieldColumnsSmemMax = 200 * 1024;
-template <typename T>
-cudaError_t launch_field_columns(const ModeCommon& mc, int kind, const BdfParams& bp,
-                                 const CdfParams& cp, const DirkParams& dp, const void* z,
-                                 void* f4, void* e, double* diag, const FftDesc& fd,
-                                 const void* tw, cudaStream_t s);
 // 2D-3V: the A_z wave update of the stepper in use (the same recurrences as A_x with the
 // source mu0 J_z), from zz = FFT(J_z sums); writes the two packed outputs
 // f2 = [(i kx - ky) A_z, A_z] / (nx ny) for the inverse transforms, and adds |E_z|^2 and
@@ -180,10 +184,17 @@ struct ZParams {
     void *jz_n, *jz_prev;    //      J_z^n, J_z^{n-1} (the new current overwrites jz_prev)
     void* vaz;               // DIRK: dA_z/dt; az_n and jz_n hold A_z^n and J_z^n
 };
+// launch_field_columns with zp: the A_z columns (zz transformed along y only, f2 along x only)
+// in the same launch.
 template <typename T>
-cudaError_t launch_zfield(const ModeCommon& mc, const BdfParams& bp, const DirkParams& dp,
-                          const ZParams& zp, const void* zz, void* f2, double* diag,
-                          cudaStream_t s);
+cudaError_t launch_field_columns(const ModeCommon& mc, int kind, const BdfParams& bp,
+                                 const CdfParams& cp, const DirkParams& dp, const void* z,
+                                 void* f4, void* e, double* diag, const FftDesc& fd,
+                                 const void* tw, cudaStream_t s, const ZParams* zp = nullptr,
+                                 const void* zz = nullptr, void* f2 = nullptr);
+template <typename T>
+cudaError_t launch_zfield(const ModeCommon& mc, const BdfParams& bp, const ZParams& zp,
+                          const void* zz, void* f2, double* diag, cudaStream_t s);
 // Fill the wavenumber and inverse-denominator tables of mc (kind: StepperKind).
 cudaError_t launch_mode_tables(const ModeCommon& mc, int kind, const BdfParams& bp,
                                const DirkParams& dp, double* kxt, double* kyt, double* invd,

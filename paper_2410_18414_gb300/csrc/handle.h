@@ -114,7 +114,8 @@ struct pic_handle {
     int32_t* species = nullptr;       // each particle's species index (device)
     void* pz = nullptr;               // P_z (constant: d/dz = 0)
     void* vz[2] = {nullptr, nullptr}; // v_z, rotated with v
-    void* Jz = nullptr;               // J_z sums in the .x parts (double2, or longlong2)
+    void* Jz = nullptr;               // J_z sums in the .x parts (buffers as J and Jalt)
+    void* Jzalt = nullptr;
     void* Zz = nullptr;               // spectrum of J_z
     void* F2 = nullptr;               // the two packed A_z output spectra
     void* Gz = nullptr;               // [node][2] complex: (dAz/dx, dAz/dy), (Az, 0)

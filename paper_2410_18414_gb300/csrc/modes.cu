@@ -507,11 +507,131 @@ __device__ __forceinline__ void prefetch_history(const ModeCommon& mc, const Dir
         for (int a = 0; a < 9; ++a) prefetch_l2(arr[a], i * mc.ny + j);
 }
 
-template <typename C, typename Params>
+// 2D-3V: the A_z update of mode idx from zz = FFT(J_z sums).  With d/dz = 0 the z component of
+// the vector potential obeys its own wave equation with source mu0 J_z, stepped with the same
+// recurrences as A_x; it enters neither the continuity equation nor the gauge.  E_z = -dA_z/dt
+// is the stepper's discrete derivative (BDF: the BDF difference; CDF-2: the centred difference
+// at n+1/2; DIRK: -v_Az), B_x = i ky A_z, B_y = -i kx A_z.  grad, az: the two packed outputs.
+// K: the BDF order where it is known (its loads are then issued together), else 0.
+template <int K>
+__device__ __forceinline__ void z_update(const ModeCommon& mc, const BdfParams& bp,
+                                         const ZParams& zp, int idx, double kx, double ky, zd zz,
+                                         double* acc, zd& grad, zd& az) {
+    const double k2 = kx * kx + ky * ky;
+    const zd jz = zscale(mc.jscale, zz);
+    zd az_new, ez;
+    if (zp.kind == K_BDF) {
+        zd s = zscale(bp.g * mc.mu0, jz);
+        const int k = K > 0 ? K : bp.k;
+        for (int d = 1; d <= 2 * k; ++d) s = zfms(s, bp.C[d], hload(zp.az[d - 1], idx));
+        az_new = zscale(mc.invd[idx], s);
+        zd daz = bp.a[0] * az_new;
+        for (int d = 1; d <= k; ++d) daz = daz + bp.a[d] * hload(zp.az[d - 1], idx);
+        ez = -(1.0 / bp.bdt) * daz;
+        hstore(zp.az_new, idx, az_new);
+    } else if (zp.kind == K_CDF2) {
+        const double dt = mc.dt, inv = mc.invd[idx];
+        const zd azn = hload(zp.az_n, idx), azp = hload(zp.az_prev, idx);
+        if (zp.form == 0) {
+            const double th = 0.5 * mc.c * mc.c * dt * dt;
+            az_new = inv * (2.0 * azn + (th * mc.mu0) * (jz + hload(zp.jz_prev, idx))) - azp;
+        } else {
+            const double h2 = mc.c * mc.c * dt * dt;
+            const zd s = mc.mu0 * hload(zp.jz_n, idx);
+            az_new = (zp.form == 1) ? inv * (2.0 * azn + h2 * s) - azp
+                                    : 2.0 * azn - azp + h2 * (s - k2 * azn);
+        }
+        ez = -(1.0 / dt) * (az_new - azn);
+        hstore(zp.az_prev, idx, az_new);
+        hstore(zp.jz_prev, idx, jz);
+    } else {
+        const zd azn = hload(zp.az_n, idx), vaz = hload(zp.vaz, idx);
+        zd vaz_new;
+        dirk_apply(mc.dirkm + (size_t)idx * 8, azn, vaz, mc.mu0 * hload(zp.jz_n, idx),
+                   mc.mu0 * jz, az_new, vaz_new);
+        ez = -vaz_new;
+        hstore(zp.az_n, idx, az_new);
+        hstore(zp.vaz, idx, vaz_new);
+        hstore(zp.jz_n, idx, jz);
+    }
+    if (mc.diag) {
+        acc[D_WE] += znorm2(ez);
+        acc[D_WB] += k2 * znorm2(az_new);
+    }
+    grad = zscale(mc.inv_n, grad_packed(kx, ky, az_new));
+    az = zscale(mc.inv_n, az_new);
+}
+
+// z_update with one thread per mode over the transformed zz.
+template <typename C>
+__global__ void __launch_bounds__(kModeThreads)
+k_zmode(ModeCommon mc, BdfParams bp, ZParams zp, const C* __restrict__ zz, C* __restrict__ f2,
+        double* __restrict__ diag) {
+    const int nmodes = mc.nx * mc.ny;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    double acc[D_NSLOTS];
+#pragma unroll
+    for (int s = 0; s < D_NSLOTS; ++s) acc[s] = 0.0;
+    if (idx < nmodes) {
+        const int i = idx / mc.ny, j = idx - i * mc.ny;
+        zd grad, az;
+        z_update<0>(mc, bp, zp, idx, mc.kxt[i], mc.kyt[j], zload(zz + idx), acc, grad, az);
+        zstore(f2 + idx, grad);
+        zstore(f2 + (size_t)nmodes + idx, az);
+    }
+    if (mc.diag) reduce_diag(acc, diag);
+}
+
+// The A_z columns of a 2D-3V step in the field columns' launch (blockIdx.y = 1), or none.
+struct NoZColumns {
+    static constexpr bool kOn = false;
+};
+template <typename C>
+struct ZColumns {
+    static constexpr bool kOn = true;
+    BdfParams bp;
+    ZParams zp;
+    const C* zz;
+    C* f2;
+    // the transforms' signs, -1 and +1, as run-time values: with constants the compiler
+    // contracts the inverse's products the other way round and A_z's fields lose the bits
+    // that the separate transforms (k_fft_x) give
+    int forward, inverse;
+};
+template <typename Params> struct OrderOf { static constexpr int value = 0; };
+template <int K> struct OrderOf<BdfOrder<K>> { static constexpr int value = K; };
+template <int K, typename C>
+__device__ void z_column(const ModeCommon& mc, const ZColumns<C>& z, double* __restrict__ diag,
+                         const FftDesc& fd, C* bufA, C* bufB, const C* tws) {
+    const int nx = mc.nx, ny = mc.ny, j = blockIdx.x;
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) bufA[i] = z.zz[(size_t)i * ny + j];
+    __syncthreads();
+    C* zc = run_passes(bufA, bufB, fd, 1, tws, z.forward);
+    C* out = (zc == bufA) ? bufB : bufA;
+    double acc[D_NSLOTS];
+#pragma unroll
+    for (int s = 0; s < D_NSLOTS; ++s) acc[s] = 0.0;
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        zd grad, az;
+        z_update<K>(mc, z.bp, z.zp, i * ny + j, mc.kxt[i], mc.kyt[j], zload(zc + i), acc, grad, az);
+        zstore(out + i, grad);
+        zstore(out + nx + i, az);
+    }
+    __syncthreads();
+    C* res = run_passes(out, zc, fd, 2, tws, z.inverse);
+    const size_t N = (size_t)nx * ny;
+    for (int t = threadIdx.x; t < 2 * nx; t += blockDim.x) {
+        const int f = t / nx, i = t - f * nx;
+        z.f2[f * N + (size_t)i * ny + j] = res[t];
+    }
+    if (mc.diag) reduce_diag(acc, diag);
+}
+
+template <typename C, typename Params, typename Z>
 __global__ void __launch_bounds__(kModeThreads)
 k_field_columns(ModeCommon mc, Params prm, const C* __restrict__ z, C* __restrict__ f4,
                 C* __restrict__ epk, double* __restrict__ diag, FftDesc fd,
-                const C* __restrict__ tw) {
+                const C* __restrict__ tw, Z zcol) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = mc.nx, ny = mc.ny;
     const int j = blockIdx.x;
@@ -521,9 +641,16 @@ k_field_columns(ModeCommon mc, Params prm, const C* __restrict__ z, C* __restric
     C* bufB = bufA + 4 * nx;                   // 4 lines of nx
     C* tws = bufB + 4 * nx;                    // twiddles (constant: staged before the wait)
     stage_twiddles(tw, tws, nx);
-    prefetch_history(mc, prm, j);              // written two or more kernels back
+    if (!Z::kOn || blockIdx.y == 0)
+        prefetch_history(mc, prm, j);          // written two or more kernels back
     griddep_wait();                            // z is the previous kernel's output
     griddep_launch();
+    if constexpr (Z::kOn) {
+        if (blockIdx.y) {
+            z_column<OrderOf<Params>::value>(mc, zcol, diag, fd, bufA, bufB, (const C*)tws);
+            return;
+        }
+    }
     for (int t = threadIdx.x; t < ncols * nx; t += blockDim.x) {
         const int c = t / nx, i = t - c * nx;
         bufA[t] = z[(size_t)i * ny + (c ? jp : j)];
@@ -549,69 +676,6 @@ k_field_columns(ModeCommon mc, Params prm, const C* __restrict__ z, C* __restric
     for (int t = threadIdx.x; t < 4 * nx; t += blockDim.x) {
         const int f = t / nx, i = t - f * nx;
         f4[f * N + (size_t)i * ny + j] = res[t];
-    }
-    if (mc.diag) reduce_diag(acc, diag);
-}
-
-// 2D-3V: the A_z update of mode idx (one thread per mode over zz = FFT(J_z sums)).  With
-// d/dz = 0 the z component of the vector potential obeys its own wave equation with source
-// mu0 J_z, stepped with the same recurrences as A_x; it enters neither the continuity
-// equation nor the gauge.  E_z = -dA_z/dt is the stepper's discrete derivative (BDF: the
-// BDF difference; CDF-2: the centred difference at n+1/2; DIRK: -v_Az), B_x = i ky A_z,
-// B_y = -i kx A_z.
-template <typename C>
-__global__ void __launch_bounds__(kModeThreads)
-k_zmode(ModeCommon mc, BdfParams bp, DirkParams dp, ZParams zp, const C* __restrict__ zz,
-        C* __restrict__ f2, double* __restrict__ diag) {
-    const int nmodes = mc.nx * mc.ny;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    double acc[D_NSLOTS];
-#pragma unroll
-    for (int s = 0; s < D_NSLOTS; ++s) acc[s] = 0.0;
-    if (idx < nmodes) {
-        const int i = idx / mc.ny, j = idx - i * mc.ny;
-        const double kx = mc.kxt[i], ky = mc.kyt[j], K = kx * kx + ky * ky;
-        const zd jz = zscale(mc.jscale, zload(zz + idx));
-        zd az_new, ez;
-        if (zp.kind == K_BDF) {
-            zd s = zscale(bp.g * mc.mu0, jz);
-            for (int d = 1; d <= 2 * bp.k; ++d) s = zfms(s, bp.C[d], hload(zp.az[d - 1], idx));
-            az_new = zscale(mc.invd[idx], s);
-            zd daz = bp.a[0] * az_new;
-            for (int d = 1; d <= bp.k; ++d) daz = daz + bp.a[d] * hload(zp.az[d - 1], idx);
-            ez = -(1.0 / bp.bdt) * daz;
-            hstore(zp.az_new, idx, az_new);
-        } else if (zp.kind == K_CDF2) {
-            const double dt = mc.dt, inv = mc.invd[idx];
-            const zd az = hload(zp.az_n, idx), azp = hload(zp.az_prev, idx);
-            if (zp.form == 0) {
-                const double th = 0.5 * mc.c * mc.c * dt * dt;
-                az_new = inv * (2.0 * az + (th * mc.mu0) * (jz + hload(zp.jz_prev, idx))) - azp;
-            } else {
-                const double h2 = mc.c * mc.c * dt * dt;
-                const zd s = mc.mu0 * hload(zp.jz_n, idx);
-                az_new = (zp.form == 1) ? inv * (2.0 * az + h2 * s) - azp
-                                        : 2.0 * az - azp + h2 * (s - K * az);
-            }
-            ez = -(1.0 / dt) * (az_new - az);
-            hstore(zp.az_prev, idx, az_new);
-            hstore(zp.jz_prev, idx, jz);
-        } else {
-            const zd az = hload(zp.az_n, idx), vaz = hload(zp.vaz, idx);
-            zd vaz_new;
-            dirk_apply(mc.dirkm + (size_t)idx * 8, az, vaz, mc.mu0 * hload(zp.jz_n, idx),
-                       mc.mu0 * jz, az_new, vaz_new);
-            ez = -vaz_new;
-            hstore(zp.az_n, idx, az_new);
-            hstore(zp.vaz, idx, vaz_new);
-            hstore(zp.jz_n, idx, jz);
-        }
-        if (mc.diag) {
-            acc[D_WE] += znorm2(ez);
-            acc[D_WB] += K * znorm2(az_new);
-        }
-        zstore(f2 + idx, zscale(mc.inv_n, grad_packed(kx, ky, az_new)));
-        zstore(f2 + (size_t)nmodes + idx, zscale(mc.inv_n, az_new));
     }
     if (mc.diag) reduce_diag(acc, diag);
 }
@@ -705,13 +769,13 @@ cudaError_t launch_mode_generic(const ModeCommon& mc, const Params& prm, const v
     return cudaGetLastError();
 }
 
-template <typename C, typename Params>
-cudaError_t launch_columns_generic(const ModeCommon& mc, const Params& prm, const void* z,
-                                   void* f4, void* e, double* diag, const FftDesc& fd,
-                                   const void* tw, cudaStream_t s) {
+template <typename C, typename Params, typename Z>
+cudaError_t launch_columns_z(const ModeCommon& mc, const Params& prm, const void* z, void* f4,
+                             void* e, double* diag, const FftDesc& fd, const void* tw,
+                             cudaStream_t s, const Z& zcol) {
     const size_t smem = field_columns_smem(mc.nx, sizeof(C));
     if (smem > kFieldColumnsSmemMax) return cudaErrorInvalidValue;
-    auto kern = k_field_columns<C, Params>;
+    auto kern = k_field_columns<C, Params, Z>;
     if (smem > 48 * 1024) {
         cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem);
@@ -720,8 +784,16 @@ cudaError_t launch_columns_generic(const ModeCommon& mc, const Params& prm, cons
     // one thread per mode of the column: grids up to 128 wide take 128-thread CTAs (one
     // step 1 us shorter at 128 x 128 than with 256, half of whose threads idle)
     const int threads = mc.nx <= 128 ? 128 : kModeThreads;
-    return launch_pdl(kern, dim3(mc.ny), dim3(threads), smem, s, mc, prm, (const C*)z,
-                      (C*)f4, (C*)e, diag, fd, (const C*)tw);
+    return launch_pdl(kern, dim3(mc.ny, Z::kOn ? 2 : 1), dim3(threads), smem, s, mc, prm,
+                      (const C*)z, (C*)f4, (C*)e, diag, fd, (const C*)tw, zcol);
+}
+
+template <typename C, typename Params>
+cudaError_t launch_columns_generic(const ModeCommon& mc, const Params& prm, const void* z,
+                                   void* f4, void* e, double* diag, const FftDesc& fd,
+                                   const void* tw, cudaStream_t s, const ZColumns<C>* zc) {
+    if (zc) return launch_columns_z<C>(mc, prm, z, f4, e, diag, fd, tw, s, *zc);
+    return launch_columns_z<C>(mc, prm, z, f4, e, diag, fd, tw, s, NoZColumns{});
 }
 
 }  // namespace
@@ -745,21 +817,28 @@ template <typename T>
 cudaError_t launch_field_columns(const ModeCommon& mc, int kind, const BdfParams& bp,
                                  const CdfParams& cp, const DirkParams& dp, const void* z,
                                  void* f4, void* e, double* diag, const FftDesc& fd,
-                                 const void* tw, cudaStream_t s) {
+                                 const void* tw, cudaStream_t s, const ZParams* zp,
+                                 const void* zz, void* f2) {
     using C = cplx_t<T>;
+    ZColumns<C> zcols{};
+    const ZColumns<C>* zc = nullptr;
+    if (zp) {
+        zcols = ZColumns<C>{bp, *zp, (const C*)zz, (C*)f2, -1, +1};
+        zc = &zcols;
+    }
     if (kind == K_BDF) {
         static_assert(kMaxBdf == 6, "one column kernel per BDF order");
         switch (bp.k) {
-            case 1: return launch_columns_generic<C>(mc, BdfOrder<1>{bp}, z, f4, e, diag, fd, tw, s);
-            case 2: return launch_columns_generic<C>(mc, BdfOrder<2>{bp}, z, f4, e, diag, fd, tw, s);
-            case 3: return launch_columns_generic<C>(mc, BdfOrder<3>{bp}, z, f4, e, diag, fd, tw, s);
-            case 4: return launch_columns_generic<C>(mc, BdfOrder<4>{bp}, z, f4, e, diag, fd, tw, s);
-            case 5: return launch_columns_generic<C>(mc, BdfOrder<5>{bp}, z, f4, e, diag, fd, tw, s);
-            default: return launch_columns_generic<C>(mc, BdfOrder<6>{bp}, z, f4, e, diag, fd, tw, s);
+            case 1: return launch_columns_generic<C>(mc, BdfOrder<1>{bp}, z, f4, e, diag, fd, tw, s, zc);
+            case 2: return launch_columns_generic<C>(mc, BdfOrder<2>{bp}, z, f4, e, diag, fd, tw, s, zc);
+            case 3: return launch_columns_generic<C>(mc, BdfOrder<3>{bp}, z, f4, e, diag, fd, tw, s, zc);
+            case 4: return launch_columns_generic<C>(mc, BdfOrder<4>{bp}, z, f4, e, diag, fd, tw, s, zc);
+            case 5: return launch_columns_generic<C>(mc, BdfOrder<5>{bp}, z, f4, e, diag, fd, tw, s, zc);
+            default: return launch_columns_generic<C>(mc, BdfOrder<6>{bp}, z, f4, e, diag, fd, tw, s, zc);
         }
     }
-    if (kind == K_CDF2) return launch_columns_generic<C>(mc, cp, z, f4, e, diag, fd, tw, s);
-    return launch_columns_generic<C>(mc, dp, z, f4, e, diag, fd, tw, s);
+    if (kind == K_CDF2) return launch_columns_generic<C>(mc, cp, z, f4, e, diag, fd, tw, s, zc);
+    return launch_columns_generic<C>(mc, dp, z, f4, e, diag, fd, tw, s, zc);
 }
 cudaError_t launch_mode_tables(const ModeCommon& mc, int kind, const BdfParams& bp,
                                const DirkParams& dp, double* kxt, double* kyt, double* invd,
@@ -772,12 +851,10 @@ cudaError_t launch_mode_tables(const ModeCommon& mc, int kind, const BdfParams& 
 }
 
 template <typename T>
-cudaError_t launch_zfield(const ModeCommon& mc, const BdfParams& bp, const DirkParams& dp,
-                          const ZParams& zp, const void* zz, void* f2, double* diag,
-                          cudaStream_t s) {
+cudaError_t launch_zfield(const ModeCommon& mc, const BdfParams& bp, const ZParams& zp,
+                          const void* zz, void* f2, double* diag, cudaStream_t s) {
     using C = cplx_t<T>;
-    k_zmode<C><<<mode_blocks(mc), kModeThreads, 0, s>>>(mc, bp, dp, zp, (const C*)zz, (C*)f2,
-                                                        diag);
+    k_zmode<C><<<mode_blocks(mc), kModeThreads, 0, s>>>(mc, bp, zp, (const C*)zz, (C*)f2, diag);
     return cudaGetLastError();
 }
 
@@ -808,12 +885,12 @@ cudaError_t launch_mode_pack2(const ModeCommon& mc, const void* a, const void* b
     template cudaError_t launch_field_columns<T>(const ModeCommon&, int, const BdfParams&,        \
                                                  const CdfParams&, const DirkParams&, const void*, \
                                                  void*, void*, double*, const FftDesc&,           \
-                                                 const void*, cudaStream_t);                      \
+                                                 const void*, cudaStream_t, const ZParams*,       \
+                                                 const void*, void*);                             \
     template cudaError_t launch_mode_init<T>(const ModeCommon&, const void*, void*, void*, void*, \
                                              cudaStream_t);                                       \
-    template cudaError_t launch_zfield<T>(const ModeCommon&, const BdfParams&, const DirkParams&, \
-                                          const ZParams&, const void*, void*, double*,            \
-                                          cudaStream_t);                                          \
+    template cudaError_t launch_zfield<T>(const ModeCommon&, const BdfParams&, const ZParams&,    \
+                                          const void*, void*, double*, cudaStream_t);             \
     template cudaError_t launch_mode_pack2<T>(const ModeCommon&, const void*, const void*, int,  \
                                               void*, cudaStream_t);
 GPIC_INST(double)

@@ -273,7 +273,8 @@ void layout_state(pic_handle* h) {
         take(&h->pz, pn);
         take(&h->vz[0], pn);
         take(&h->vz[1], pn);
-        take(&h->Jz, h->jbytes);
+        take(&h->Jz, h->jbytes, true);
+        take(&h->Jzalt, h->jbytes, true);
         take(&h->Zz, h->ng * cs);
         take(&h->F2, 2 * h->ng * cs);
         take(&h->Gz, 2 * h->ng * cs);
@@ -764,8 +765,7 @@ pic_status pic_deposit(pic_handle* h) {
     // the buffer the previous field solve zeroed (a memset here would break the chain of
     // dependent launches); J^n stays readable until then
     std::swap(h->J, h->Jalt);
-    if (h->vdim == 3 && binned_deposit(h))  // the binned pass adds J_z to it
-        CK(cudaMemsetAsync(h->Jz, 0, h->jbytes, h->s));
+    if (h->vdim == 3) std::swap(h->Jz, h->Jzalt);
     h->launches_now += 1;
     TimedScope ts(h, PIC_KT_DEPOSIT);
     CK(by_prec(h, [&](auto t) {
@@ -798,7 +798,6 @@ pic_status pic_deposit(pic_handle* h) {
         }
     }));
     if (h->vdim == 3 && !binned_deposit(h)) {  // J_z of the moved particles
-        CK(cudaMemsetAsync(h->Jz, 0, h->jbytes, h->s));
         CK(by_prec(h, [&](auto t) {
             using T = decltype(t);
             return launch_deposit_z<T>(h->p, h->geom, (const T*)h->x, (const T*)h->y,
@@ -821,16 +820,18 @@ pic_status pic_field_solve(pic_handle* h) {
     const bool fused = field_columns_smem(h->nx, 2 * h->rsz) <= kFieldColumnsSmemMax;
     TimedScope ts(h, PIC_KT_FIELD);
 
-    // forward transform along y, the fixed-point sums converted on load
-    if (h->fp32)
-        CK(launch_fft_y_from_fix<float>((const longlong2*)h->J, h->fix_unscale_j, h->Z, h->nx,
-                                        h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s));
-    else
-        CK(launch_fft_y_from_fix<double>((const longlong2*)h->J, h->fix64_unscale_j, h->Z, h->nx,
-                                         h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s));
-    if (!fused) CK(by_prec(h, [&](auto t) {
+    // forward transform along y, the fixed-point sums converted on load (2D-3V: J_z too)
+    const bool z3 = h->vdim == 3;
+    const longlong2* jz = z3 ? (const longlong2*)h->Jz : nullptr;
+    CK(by_prec(h, [&](auto t) {
         using T = decltype(t);
-        return launch_fft_x<T>(h->Z, h->Z, h->nx, h->ny, 1, h->fx, h->twx, -1, h->s);
+        cudaError_t r = launch_fft_y_from_fix<T>(
+            (const longlong2*)h->J, h->fp32 ? h->fix_unscale_j : h->fix64_unscale_j, h->Z, h->nx,
+            h->ny, h->fy, h->twy, (longlong2*)h->Jalt, h->s, jz, h->Zz, (longlong2*)h->Jzalt);
+        if (r != cudaSuccess || fused) return r;
+        r = launch_fft_x<T>(h->Z, h->Z, h->nx, h->ny, 1, h->fx, h->twx, -1, h->s);
+        if (r != cudaSuccess || !z3) return r;
+        return launch_fft_x<T>(h->Zz, h->Zz, h->nx, h->ny, 1, h->fx, h->twx, -1, h->s);
     }));
 
     // the naive update takes rho^{n+1} from the charge deposited at x^{n+1}, transformed
@@ -895,7 +896,12 @@ pic_status pic_field_solve(pic_handle* h) {
         using T = decltype(t);
         if (fused)
             return launch_field_columns<T>(h->mc, kind, bp, h->cdf, h->dirk, h->Z, h->F4, h->E,
-                                           h->diag, h->fx, h->twx, h->s);
+                                           h->diag, h->fx, h->twx, h->s, z3 ? &zp : nullptr,
+                                           h->Zz, h->F2);
+        if (z3) {
+            cudaError_t r = launch_zfield<T>(h->mc, bp, zp, h->Zz, h->F2, h->diag, h->s);
+            if (r != cudaSuccess) return r;
+        }
         if (kind == K_BDF) return launch_mode_bdf<T>(h->mc, bp, h->Z, h->F4, h->E, h->diag, h->s);
         if (kind == K_CDF2) return launch_mode_cdf2<T>(h->mc, h->cdf, h->Z, h->F4, h->E, h->diag, h->s);
         return launch_mode_dirk<T>(h->mc, h->dirk, h->Z, h->F4, h->E, h->diag, h->s);
@@ -912,45 +918,24 @@ pic_status pic_field_solve(pic_handle* h) {
         std::swap(h->cdf.jy, h->cdf.jy_prev);
     }
 
-    // inverse transforms: along x (unless fused above), then along y into the [node][4]
-    // gather layout
+    if (st == PIC_STEPPER_CDF2 && z3) {
+        std::swap(h->az, h->az_prev);
+        std::swap(h->jz, h->jz_prev);
+    }
+
+    // inverse transforms: along x (unless fused above), then along y into the [node][4] gather
+    // layout (2D-3V: and the [node][2] one of A_z)
     CK(by_prec(h, [&](auto t) {
         using T = decltype(t);
         cudaError_t r = cudaSuccess;
         if (!fused) r = launch_fft_x<T>(h->F4, h->F4, h->nx, h->ny, 4, h->fx, h->twx, +1, h->s);
-        if (r != cudaSuccess) return r;
-        return launch_fft_y<T>(h->F4, h->G, h->nx, h->ny, 4, h->fy, h->twy, +1, 1, h->s,
-                               h->fixf.f ? &h->fixf : nullptr);
-    }));
-    h->launches_now += fused ? 3 : 5;
-
-    // 2D-3V: A_z by the same stepper from J_z, and its gather fields (Gz)
-    if (h->vdim == 3) {
-        CK(by_prec(h, [&](auto t) -> cudaError_t {
-            using T = decltype(t);
-            cudaError_t r;
-            if (h->fp32) {
-                r = launch_fix_to_cplx<T>((const longlong2*)h->Jz, h->fix_unscale_j, h->tmp, h->ng,
-                                          h->s);
-                if (r == cudaSuccess) r = forward_fft(h, h->tmp, h->Zz);
-            } else {  // J_z in the real parts
-                r = launch_fix128_to_cplx((const longlong2*)h->Jz, h->ng, h->fix64_unscale_j,
-                                          (double2*)h->tmp, h->s);
-                if (r == cudaSuccess) r = forward_fft(h, h->tmp, h->Zz);
-            }
-            if (r != cudaSuccess) return r;
-            r = launch_zfield<T>(h->mc, bp, h->dirk, zp, h->Zz, h->F2, h->diag, h->s);
-            if (r != cudaSuccess) return r;
+        if (r == cudaSuccess && !fused && z3)
             r = launch_fft_x<T>(h->F2, h->F2, h->nx, h->ny, 2, h->fx, h->twx, +1, h->s);
-            if (r != cudaSuccess) return r;
-            return launch_fft_y<T>(h->F2, h->Gz, h->nx, h->ny, 2, h->fy, h->twy, +1, 1, h->s);
-        }));
-        if (st == PIC_STEPPER_CDF2) {
-            std::swap(h->az, h->az_prev);
-            std::swap(h->jz, h->jz_prev);
-        }
-        h->launches_now += h->fp32 ? 6 : 5;
-    }
+        if (r != cudaSuccess) return r;
+        return launch_fft_y_fields<T>(h->F4, h->G, z3 ? h->F2 : nullptr, h->Gz, h->nx, h->ny,
+                                      h->fy, h->twy, h->fixf.f ? &h->fixf : nullptr, h->s);
+    }));
+    h->launches_now += fused ? 3 : 5 + (z3 ? 3 : 0);
     h->phase = 2;
     return PIC_OK;
 }
@@ -1502,7 +1487,8 @@ int32_t pic_kernels_per_step(const pic_handle* h) {
     // kernels.  Before any step: the count of a step without a sort.
     if (!h->stepped) {
         const bool fused = field_columns_smem(h->nx, 2 * h->rsz) <= kFieldColumnsSmemMax;
-        const int z = h->vdim == 3 ? (h->fp32 ? 7 : 6) : 0;  // J_z deposit and the A_z solve
+        int z = 0;  // 2D-3V: J_z's own deposit, and A_z's own passes where not fused
+        if (h->vdim == 3) z = (binned_deposit(h) ? 0 : 1) + (fused ? 0 : 3);
         return (fused ? 5 : 7) + z;
     }
     return h->launches_last;

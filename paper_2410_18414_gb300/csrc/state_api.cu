@@ -218,6 +218,7 @@ pic_status pic_load_state(pic_handle* h, const void* src, size_t size) {
     h->pending = false;  // a pending deposit of the old state is void
     // the buffer the next deposit sums into starts at zero (the row transform keeps it so)
     CK(cudaMemsetAsync(h->Jalt, 0, h->jbytes, h->s));
+    if (h->vdim == 3) CK(cudaMemsetAsync(h->Jzalt, 0, h->jbytes, h->s));
     CK(cudaStreamSynchronize(h->s));  // src may be released on return
     return check_device_error(h);
 }
