@@ -313,6 +313,15 @@ struct ReadArrays {
 cudaError_t launch_invert_ids(const int32_t* id, int32_t* inv, int64_t n, cudaStream_t s);
 template <typename Ts, typename Td>
 cudaError_t launch_read_arrays(const ReadArrays& r, const int32_t* inv, int64_t n, cudaStream_t s);
+// The same for eight FP64 destinations by records of eight values, with
+// scratch memory for n of them: eight pieces of per = n / 8 records and one for the rest.
+struct RecordSpace {
+    void* piece[9];
+    unsigned per;
+};
+template <typename T>
+cudaError_t launch_read_records(const ReadArrays& r, const int32_t* id, const RecordSpace& sp,
+                                int64_t n, cudaStream_t s);
 
 // Tiles for the particle sort and the shared-memory deposit: t x t cells per tile,
 // ntx x nty tiles; a CTA accumulates into an rx x ry node region starting `halo` nodes

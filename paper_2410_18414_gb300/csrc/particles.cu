@@ -1510,6 +1510,40 @@ __global__ void k_read_arrays(ReadArrays r, const int32_t* __restrict__ inv, int
     }
 }
 
+// The same for eight arrays that L2 does not hold: the sorted particles are written as whole
+// records (32 or 64 bytes, full sectors) to the caller's order, then split.  The records lie
+// in nine pieces of memory, `per` records each (the last: fewer than eight).
+template <typename T>
+struct alignas(8 * sizeof(T)) Record8 {
+    T v[8];
+};
+template <typename T>
+__device__ __forceinline__ Record8<T>* record_at(const RecordSpace& sp, int64_t i) {
+    const unsigned c = min((unsigned)i / sp.per, 8u);
+    return reinterpret_cast<Record8<T>*>(sp.piece[c]) + (i - (int64_t)c * sp.per);
+}
+template <typename T>
+__global__ void k_pack_records(ReadArrays r, const int32_t* __restrict__ id, RecordSpace sp,
+                               int64_t n) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = id[k];
+        Record8<T> rec;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) rec.v[j] = __ldcs((const T*)r.src[j] + k);
+        if ((uint64_t)i < (uint64_t)n) *record_at<T>(sp, i) = rec;
+    }
+}
+template <typename T>
+__global__ void k_split_records(ReadArrays r, RecordSpace sp, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const Record8<T> rec = *record_at<T>(sp, i);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) __stcs((double*)r.dst[j] + i, (double)rec.v[j]);
+    }
+}
+
 // Replay of one FP64 step's particle update from the adjoint's record of that step:
 // state n -> state n+1 with the move of k_move_deposit (the same operations, so the same
 // bits) and the recorded P^{n+1}, v^{n+1}.  States are eight arrays of n in the order x, y,
@@ -2086,6 +2120,17 @@ cudaError_t launch_read_arrays(const ReadArrays& r, const int32_t* inv, int64_t 
     }
     return cudaGetLastError();
 }
+template <typename T>
+cudaError_t launch_read_records(const ReadArrays& r, const int32_t* id, const RecordSpace& sp,
+                                int64_t n, cudaStream_t s) {
+    k_pack_records<T><<<blocks_for(n), kThreads, 0, s>>>(r, id, sp, n);
+    k_split_records<T><<<blocks_for(n), kThreads, 0, s>>>(r, sp, n);
+    return cudaGetLastError();
+}
+template cudaError_t launch_read_records<float>(const ReadArrays&, const int32_t*,
+                                                const RecordSpace&, int64_t, cudaStream_t);
+template cudaError_t launch_read_records<double>(const ReadArrays&, const int32_t*,
+                                                 const RecordSpace&, int64_t, cudaStream_t);
 template cudaError_t launch_read_arrays<float, double>(const ReadArrays&, const int32_t*, int64_t,
                                                        cudaStream_t);
 template cudaError_t launch_read_arrays<double, double>(const ReadArrays&, const int32_t*, int64_t,
