@@ -353,7 +353,12 @@ int sort_scan_chunks(int nkeys);  // chunk totals the scan keeps (size of its bs
 template <typename T>
 cudaError_t launch_tile_sort(const TileGeom& tg, SortArrays<T> src, SortArrays<T> dst, int64_t n,
                              int vidx, int* keys, int* hist, int* off, int* cursor, int* bsum,
-                             cudaStream_t s);
+                             void* map, int map_count, int share, cudaStream_t s);
+// The binned FP32 pass's CTAs (int4 entries: tile, first particle, end, 0; tile -1: none), at
+// most `share` particles each; map_count >= ntiles + n / share.  launch_tile_sort writes it
+// (map may be NULL); launch_cta_map alone, from the offsets of a loaded state.
+cudaError_t launch_cta_map(const TileGeom& tg, const int* off, void* map, int map_count, int share,
+                           cudaStream_t s);
 cudaError_t launch_iota(int32_t* id, int64_t n, cudaStream_t s);
 
 // Binned move + deposit of the FP32 form over tile-sorted particles (x, y, v^n = vx, vy)
@@ -362,18 +367,19 @@ cudaError_t launch_iota(int32_t* id, int64_t n, cudaStream_t s);
 // in registers before its shared atomics.  fused: the gather + push of the step before runs
 // first on each particle (fields4 = that step's gather fields, P and v^{n+1} -> px, py,
 // vxo, vyo; the move and deposit then use v^{n+1}), as launch_gather_push_tiled does it.
-// per_cta: particles per CTA at the mean density.  deposit_binned_fits: whether the tile's
-// regions fit the pass's shared memory.  sp/spp: a species table (each contribution times
+// map, map_count: the CTAs (launch_cta_map).  deposit_binned_fits: whether the tile's regions
+// fit the pass's shared memory; deposit_binned_share: its particles per CTA, one batch.  sp/spp: a species table (each contribution times
 // q_s w_s; the fused push with each species' charge and mass).  vz/jz (2D-3V, not fused):
 // v_z^n of the particles and the int64 J_z sums (.x parts), deposited in the same pass.
 bool deposit_binned_fits(const TileGeom& tg, int p, bool fused, bool z = false);
+int deposit_binned_share(const TileGeom& tg, int p, bool fused, bool z);
 cudaError_t launch_deposit_binned(int p, const ParticleGeom& g, const PushParams& pp,
                                   const TileGeom& tg, const float* x, const float* y, float* xo,
                                   float* yo, float* px, float* py, const float* vx,
                                   const float* vy, float* vxo, float* vyo, int64_t n,
-                                  const int* off, const void* fields4, void* j, float scale,
-                                  double* diag, unsigned int* err, cudaStream_t s, bool fused,
-                                  int per_cta, const int32_t* sp = nullptr,
+                                  const void* map, int map_count, const void* fields4, void* j,
+                                  float scale, double* diag, unsigned int* err, cudaStream_t s,
+                                  bool fused, const int32_t* sp = nullptr,
                                   const SpeciesParams* spp = nullptr, const float* vz = nullptr,
                                   void* jz = nullptr);
 

@@ -80,6 +80,8 @@ struct pic_handle {
     int32_t* species_alt = nullptr;                 // species indices (a species table)
     void* z_alt[3] = {nullptr, nullptr, nullptr};   // 2D-3V: P_z, v_z[0], v_z[1]
     int *keys = nullptr, *hist = nullptr, *off = nullptr, *cursor = nullptr, *bsum = nullptr;
+    void* ctas = nullptr;  // FP32 form: the CTAs of the binned pass, of bin_share particles
+    int ncta = 0, bin_share = 0;
     int launches_now = 0, launches_last = 0;
     // grid buffers
     double2* J = nullptr;    // deposit accumulator (sum_p v W): 128-bit sums (FP64 path:

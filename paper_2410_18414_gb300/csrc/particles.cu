@@ -907,7 +907,7 @@ k_gather_push_tiled(GeomT<float> g, PushT<float> pp, TileGeom tg, const float* _
 // Move + deposit of the FP32 form over tile-sorted particles, and the same pass fused
 // with the gather + push of the step before it (kFused).
 //
-// CTA (tile, split) takes a contiguous share [p0, p1) of one tile's particles and works
+// A CTA takes a contiguous share [p0, p1) of one tile's particles (the sort's map) and works
 // through it in the fewest batches of at most `cap` particles, of equal sizes (a batch
 // costs the same barriers, scan and region flush whatever its size, so a share of
 // cap + 20 runs as two halves, not as cap and 20):
@@ -937,9 +937,9 @@ k_gather_push_tiled(GeomT<float> g, PushT<float> pp, TileGeom tg, const float* _
 // contributions straight to the global grid.  The integer sums make J independent of the
 // order of the particles and of how they are grouped, so the result is the same bits as
 // every other deposit of the FP32 form.
-// Batch capacity: kBinBatchMax where four CTAs per SM still fit (a tile share of about
-// 1024 particles then runs as one batch even when sampling noise puts it a little above
-// 1024), else kBinBatchMin; whether a tiling can use the pass at all is judged at the
+// Batch capacity: kBinBatchMax where as many CTAs per SM still fit as with kBinBatchMin (four
+// on the 128 x 128 workload), else kBinBatchMin; a CTA's share is at most one batch
+// (CtaMap in sort.cu); whether a tiling can use the pass at all is judged at the
 // smaller one.
 constexpr int kBinBatchMin = 1024;
 constexpr int kBinBatchMax = 1152;
@@ -1152,8 +1152,8 @@ k_deposit_binned(GeomT<float> g, PushT<float> pp, TileGeom tg, const float* __re
                  const float* __restrict__ y, float* __restrict__ xo, float* __restrict__ yo,
                  float* __restrict__ px, float* __restrict__ py,
                  const float* __restrict__ vx, const float* __restrict__ vy,
-                 float* __restrict__ vxo, float* __restrict__ vyo, const int* __restrict__ off,
-                 int nsplit, const float2* __restrict__ F, AccFix acc,
+                 float* __restrict__ vxo, float* __restrict__ vyo,
+                 const int4* __restrict__ map, const float2* __restrict__ F, AccFix acc,
                  double* __restrict__ diag, unsigned int* __restrict__ err,
                  const int32_t* __restrict__ sp, BinSpecies bs, const float* __restrict__ vz,
                  AccFix accz, int cap) {
@@ -1172,11 +1172,13 @@ k_deposit_binned(GeomT<float> g, PushT<float> pp, TileGeom tg, const float* __re
     int* cnt = reinterpret_cast<int*>(base + L.cnt);
     float* stz = reinterpret_cast<float*>(base + L.stz);
 
-    const int tt = tg.t * tg.t;
-    const int tile = blockIdx.x / nsplit, split = blockIdx.x - tile * nsplit;
-    const int64_t t0 = off[tile * tt], tcnt = (int64_t)off[(tile + 1) * tt] - t0;
-    const int64_t p0 = t0 + tcnt * split / nsplit, p1 = t0 + tcnt * (split + 1) / nsplit;
-    if (p0 == p1) return;  // uniform for the CTA
+    // (fused, the sort that wrote the map is at least three kernels back; the deposit alone
+    // may come right after it)
+    if (!kFused) griddep_wait();
+    const int4 part = map[blockIdx.x];
+    const int tile = part.x;
+    const int64_t p0 = part.y, p1 = part.z;
+    if (tile < 0) return;  // uniform for the CTA
     const int rx = tg.rx, ry = tg.ry, R = rx * ry;
     if (threadIdx.x < NF) {  // the CTA's particles come to L2 meanwhile
         const float* arr[8] = {x, y, vx, vy, kZ ? vz : px, py, vxo, vyo};
@@ -1997,13 +1999,45 @@ bool deposit_binned_fits(const TileGeom& tg, int p, bool fused, bool z) {
            bin_layout(tg, p, fused, z).bytes <= kBinSmemMax;
 }
 
+// The larger batch capacity where the occupancy calculator still puts as many CTAs on an SM as
+// with the smaller one (shared memory is what limits it), else the smaller one.
+template <int P, bool kFused, bool kSpecies, bool kZ>
+int binned_cap(const TileGeom& tg, cudaError_t* e) {
+    auto kern = k_deposit_binned<P, kFused, kSpecies, kZ>;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBinSmemMax);
+    *e = attr;
+    int per_sm = 0, per_sm_min = 0;
+    const size_t big = (size_t)bin_layout(tg, P, kFused, kZ, kBinBatchMax).bytes;
+    if (*e != cudaSuccess || big > (size_t)kBinSmemMax) return kBinBatchMin;
+    *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, big);
+    if (*e == cudaSuccess)
+        *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm_min, kern, kThreads, (size_t)bin_layout(tg, P, kFused, kZ, kBinBatchMin).bytes);
+    return per_sm > 0 && per_sm >= per_sm_min ? kBinBatchMax : kBinBatchMin;
+}
+
+int deposit_binned_share(const TileGeom& tg, int p, bool fused, bool z) {
+    cudaError_t e = cudaSuccess;
+#define GPIC_SHARE(PP)                                                               \
+    return z ? binned_cap<PP, false, false, true>(tg, &e)                            \
+             : fused ? binned_cap<PP, true, false, false>(tg, &e)                    \
+                     : binned_cap<PP, false, false, false>(tg, &e);
+    switch (p) {
+        case 2: GPIC_SHARE(2)
+        case 3: GPIC_SHARE(3)
+        default: GPIC_SHARE(4)
+    }
+#undef GPIC_SHARE
+}
+
 cudaError_t launch_deposit_binned(int p, const ParticleGeom& g, const PushParams& pp,
                                   const TileGeom& tg, const float* x, const float* y, float* xo,
                                   float* yo, float* px, float* py, const float* vx,
                                   const float* vy, float* vxo, float* vyo, int64_t n,
-                                  const int* off, const void* fields4, void* j, float scale,
-                                  double* diag, unsigned int* err, cudaStream_t s, bool fused,
-                                  int per_cta, const int32_t* sp, const SpeciesParams* spp,
+                                  const void* map, int map_count, const void* fields4, void* j,
+                                  float scale, double* diag, unsigned int* err, cudaStream_t s,
+                                  bool fused, const int32_t* sp, const SpeciesParams* spp,
                                   const float* vz, void* jz) {
     if (n == 0) return cudaSuccess;
     const bool z = vz != nullptr;
@@ -2023,34 +2057,19 @@ cudaError_t launch_deposit_binned(int p, const ParticleGeom& g, const PushParams
         }
         ptyped.weight = 1.0;  // the energy sum carries each particle's w_s already
     }
-    if (!deposit_binned_fits(tg, p, fused, z) || per_cta < 1) return cudaErrorInvalidValue;
-    const int ntiles = tg.ntx * tg.nty;
-    int nsplit = (int)((n + (int64_t)ntiles * per_cta - 1) / ((int64_t)ntiles * per_cta));
-    if (nsplit < 1) nsplit = 1;
-    if (nsplit > 64) nsplit = 64;
-    const int blocks = ntiles * nsplit;
+    if (!deposit_binned_fits(tg, p, fused, z) || !map) return cudaErrorInvalidValue;
+    const int blocks = map_count;
     const AccFix acc = AccFix::make(j, scale);
     const AccFix accz = AccFix::make(jz, scale);
     cudaError_t e = cudaSuccess;
-    // the larger batch capacity where the occupancy calculator still puts four CTAs on an
-    // SM (shared memory is what limits it), else the smaller one
 #define GPIC_BINNED(PP, FF, SS, ZZ)                                                            \
     {                                                                                          \
-        static const cudaError_t attr = cudaFuncSetAttribute(                                  \
-            k_deposit_binned<PP, FF, SS, ZZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-            kBinSmemMax);                                                                      \
-        e = attr;                                                                              \
-        int cap = kBinBatchMin, per_sm = 0;                                                    \
-        const size_t big = (size_t)bin_layout(tg, p, fused, z, kBinBatchMax).bytes;            \
-        if (e == cudaSuccess && big <= (size_t)kBinSmemMax)                                    \
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                 \
-                &per_sm, k_deposit_binned<PP, FF, SS, ZZ>, kThreads, big);                     \
-        if (per_sm >= 4) cap = kBinBatchMax;                                                   \
+        const int cap = binned_cap<PP, FF, SS, ZZ>(tg, &e);                                    \
         const size_t smem = (size_t)bin_layout(tg, p, fused, z, cap).bytes;                    \
         if (e == cudaSuccess)                                                                  \
             e = launch_pdl(k_deposit_binned<PP, FF, SS, ZZ>, dim3(blocks), dim3(kThreads),     \
                            smem, s, typed<float>(g), ptyped, tg, x, y, xo, yo, px, py, vx, vy, \
-                           vxo, vyo, off, nsplit, (const float2*)fields4, acc, diag, err,      \
+                           vxo, vyo, (const int4*)map, (const float2*)fields4, acc, diag, err, \
                            species ? sp : nullptr, bs, vz, accz, cap);                         \
     }
 #define GPIC_BINNED_S(PP, FF)                       \

@@ -233,6 +233,20 @@ void* newest(pic_handle* h, int which) {
 }
 
 
+// Whether the gather + push of the step now finishing may run fused with the next step's
+// move + deposit: the sorted FP32 form (2D-2V, one species) when the tile regions fit the
+// fused kernel's shared memory.  A sort due at the next step then follows its deposit.
+// The sorted FP32 form's deposit runs in the binned pass (with J_z in 2D-3V) when the
+// tiles' regions fit its shared memory.
+bool binned_deposit(const pic_handle* h) {
+    return h->sorting && h->fp32 && deposit_binned_fits(h->tg, h->p, false, h->vdim == 3);
+}
+
+bool fuse_next(const pic_handle* h) {
+    if (!(h->sorting && h->fp32) || h->vdim != 2) return false;
+    return deposit_binned_fits(h->tg, h->p, true);
+}
+
 // The handle's buffers (run twice, see BufferArena).
 void layout_state(pic_handle* h) {
     const pic_config& c = h->cfg;
@@ -265,9 +279,14 @@ void layout_state(pic_handle* h) {
         take(&h->keys, ni);
         const size_t nt = (size_t)h->tg.nkeys() + 1;
         take(&h->hist, nt * sizeof(int), true);  // kept zero by the sort's scan
-        take(&h->off, nt * sizeof(int));
+        take(&h->off, nt * sizeof(int), true);  // (a state saved before the first sort)
         take(&h->cursor, nt * sizeof(int));
         take(&h->bsum, sort_scan_chunks(h->tg.nkeys()) * sizeof(int));
+        if (binned_deposit(h)) {  // the CTAs of the binned pass
+            h->bin_share = deposit_binned_share(h->tg, h->p, fuse_next(h), h->vdim == 3);
+            h->ncta = h->tg.ntx * h->tg.nty + (int)(h->n / h->bin_share);
+            take(&h->ctas, (size_t)h->ncta * sizeof(int4));
+        }
     }
     if (h->vdim == 3) {
         take(&h->pz, pn);
@@ -495,26 +514,6 @@ bool diag_due(const pic_handle* h) {
     return h->diag_every > 0 && ((h->step + 1) % h->diag_every) == 0;
 }
 
-// Particles per CTA of the binned FP32 deposit at the mean density: one batch of its
-// shared-memory binning.  Measured on the 128 x 128 workload (2^20 particles, tiles of
-// about 4096): 1024 a CTA (one batch each) 51 us for the fused kernel, 2048 (two batches)
-// 58 us.
-constexpr int kBinPerCta = 1024;
-
-// Whether the gather + push of the step now finishing may run fused with the next step's
-// move + deposit: the sorted FP32 form (2D-2V, one species) when the tile regions fit the
-// fused kernel's shared memory.  A sort due at the next step then follows its deposit.
-// The sorted FP32 form's deposit runs in the binned pass (with J_z in 2D-3V) when the
-// tiles' regions fit its shared memory.
-bool binned_deposit(const pic_handle* h) {
-    return h->sorting && h->fp32 && deposit_binned_fits(h->tg, h->p, false, h->vdim == 3);
-}
-
-bool fuse_next(const pic_handle* h) {
-    if (!(h->sorting && h->fp32) || h->vdim != 2) return false;
-    return deposit_binned_fits(h->tg, h->p, true);
-}
-
 pic_status gather_push_step(pic_handle* h, bool fuse, bool defer);
 
 // The tile sort.  moved = false: keyed by the positions after this step's move (the sort
@@ -544,7 +543,8 @@ pic_status sort_particles(pic_handle* h, bool moved) {
             }
         // cur[4 + 2 vcur] is v^n_x, the velocity of this step's move
         return launch_tile_sort<T>(h->tg, src, dst, h->n, moved ? -1 : 4 + 2 * h->vcur,
-                                   h->keys, h->hist, h->off, h->cursor, h->bsum, h->s);
+                                   h->keys, h->hist, h->off, h->cursor, h->bsum, h->ctas, h->ncta,
+                                   h->bin_share, h->s);
     }));
     for (int a = 0; a < 8; ++a) std::swap(*cur[a], h->alt[a]);
     std::swap(h->id, h->id_alt);
@@ -778,9 +778,9 @@ pic_status pic_deposit(pic_handle* h) {
                                          (float*)h->px, (float*)h->py,
                                          (const float*)h->v[h->vcur][0],
                                          (const float*)h->v[h->vcur][1], (float*)h->v[vo][0],
-                                         (float*)h->v[vo][1], h->n, h->off, nullptr, h->J,
-                                         h->fix_scale_j, h->diag, h->err, h->s, false,
-                                         kBinPerCta, h->species, &h->spp,
+                                         (float*)h->v[vo][1], h->n, h->ctas, h->ncta, nullptr,
+                                         h->J, h->fix_scale_j, h->diag, h->err, h->s, false,
+                                         h->species, &h->spp,
                                          z3 ? (const float*)h->vz[h->vcur] : nullptr,
                                          z3 ? h->Jz : nullptr);
         }
@@ -993,9 +993,9 @@ pic_status gather_push_step(pic_handle* h, bool fuse, bool defer) {
                                  (const float*)h->y, (float*)xo, (float*)yo, (float*)h->px,
                                  (float*)h->py, (const float*)h->v[h->vcur][0],
                                  (const float*)h->v[h->vcur][1], (float*)h->v[vo][0],
-                                 (float*)h->v[vo][1], h->n, h->off, h->G, h->Jalt,
-                                 h->fix_scale_j, h->diag, h->err, h->s, true, kBinPerCta,
-                                 h->species, &h->spp));
+                                 (float*)h->v[vo][1], h->n, h->ctas, h->ncta, h->G, h->Jalt,
+                                 h->fix_scale_j, h->diag, h->err, h->s, true, h->species,
+                                 &h->spp));
     } else if (h->sorting && h->fp32 && h->vdim == 2 && h->spp.n == 0) {
         TimedScope ts(h, PIC_KT_GATHER);
         CK(launch_gather_push_tiled(h->p, h->geom, pp, h->tg, (const float*)h->x,

@@ -219,6 +219,8 @@ pic_status pic_load_state(pic_handle* h, const void* src, size_t size) {
     // the buffer the next deposit sums into starts at zero (the row transform keeps it so)
     CK(cudaMemsetAsync(h->Jalt, 0, h->jbytes, h->s));
     if (h->vdim == 3) CK(cudaMemsetAsync(h->Jzalt, 0, h->jbytes, h->s));
+    if (h->ctas)  // from the loaded offsets
+        CK(launch_cta_map(h->tg, h->off, h->ctas, h->ncta, h->bin_share, h->s));
     CK(cudaStreamSynchronize(h->s));  // src may be released on return
     return check_device_error(h);
 }
