@@ -476,8 +476,8 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int d = c ? top1 - e1[a] : top0 - e0[a];
-                const int2 r = limbs58(shift_round(sum58(hr[c], mr[c]), d));
-                const int2 s = limbs58(shift_round(sum58(hs[c], ms[c]), d));
+                const int2 r = limbs58(shift_down(sum58(hr[c], mr[c]), d));
+                const int2 s = limbs58(shift_down(sum58(hs[c], ms[c]), d));
                 mac58(hx[c], mx[c], dx, r.x, r.y);
                 mac58(hy[c], my[c], wx, s.x, s.y);
                 if (kLean) mac58(hw[c], mw[c], wx, r.x, r.y);
@@ -486,10 +486,10 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
         double* out = rec + k * kStride + 4 * S1 + 2 * q;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            const double u = field_unit(c ? top1 : top0);
-            out[c] = (double)sum58(hx[c], mx[c]) * u;
-            out[8 + c] = (double)sum58(hy[c], my[c]) * u;
-            if (kLean) out[16 + c] = (double)sum58(hw[c], mw[c]) * u;
+            const int e = c ? top1 : top0;
+            out[c] = fix_value(sum58(hx[c], mx[c]), e);
+            out[8 + c] = fix_value(sum58(hy[c], my[c]), e);
+            if (kLean) out[16 + c] = fix_value(sum58(hw[c], mw[c]), e);
         }
     }
     __syncwarp();
@@ -508,16 +508,16 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
         ab.x[p] += g.inv_dx * xg;
         ab.y[p] += g.inv_dy * yg;
         // the record now holds the products W_x W_y and gb
-        constexpr double unit = 1.0 / 4611686018427387904.0;  // 2^-62
+        // (w 2^-62 = w 2^(-4 - 58))
         long long w[S1];
         double wy[S1];
         fix_weights<P>(Y, fg.sh, w);
 #pragma unroll
-        for (int b = 0; b < S1; ++b) wy[b] = (double)w[b] * unit;
+        for (int b = 0; b < S1; ++b) wy[b] = fix_value(w[b], -4);
         fix_weights<P>(X, fg.sh, w);
 #pragma unroll
         for (int a = 0; a < S1; ++a) {
-            const double wx = (double)w[a] * unit;
+            const double wx = fix_value(w[a], -4);
 #pragma unroll
             for (int b = 0; b < S1; ++b) mine[a * S1 + b] = wx * wy[b];
         }
@@ -646,8 +646,8 @@ k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const int d = tops[c] - e[c][a];
-            const int2 r = limbs58(shift_round(sum58(hr[c], mr[c]), d));
-            const int2 s = limbs58(shift_round(sum58(hs[c], ms[c]), d));
+            const int2 r = limbs58(shift_down(sum58(hr[c], mr[c]), d));
+            const int2 s = limbs58(shift_down(sum58(hs[c], ms[c]), d));
             mac58(hw[c], mw[c], wa, r.x, r.y);
             mac58(hx[c], mx[c], da, r.x, r.y);
             mac58(hy[c], my[c], wa, s.x, s.y);
@@ -656,10 +656,9 @@ k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1
     double w[2], jx[2], jy[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        const double u = field_unit(tops[c]);
-        w[c] = (double)sum58(hw[c], mw[c]) * u;
-        jx[c] = (double)sum58(hx[c], mx[c]) * u;
-        jy[c] = (double)sum58(hy[c], my[c]) * u;
+        w[c] = fix_value(sum58(hw[c], mw[c]), tops[c]);
+        jx[c] = fix_value(sum58(hx[c], mx[c]), tops[c]);
+        jy[c] = fix_value(sum58(hy[c], my[c]), tops[c]);
     }
     const double vxp = vx[p], vyp = vy[p];
     const double xb = ab.x[p] + g.inv_dx * (vxp * jx[0] + vyp * jx[1]);

@@ -52,6 +52,8 @@ struct FftSecond {
     int nb;
     const longlong2* fix_in;
     longlong2* clear;
+    int4* ffix;
+    unsigned* ftop;
 };
 
 // Transforms along y (contiguous): CTA = `rows` consecutive x-indices of all nb arrays.
@@ -70,6 +72,8 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
         nb = two.nb;
         fix_in = two.fix_in;
         clear = two.clear;
+        ffix = two.ffix;
+        ftop = two.ftop;
     }
     const int lines = nb * rows;
     C* b1 = b0 + lines * ny;
@@ -123,16 +127,16 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
     C* res = run_passes(b0, b1, d, lines, (const C*)tws, sign);
     if (interleave) {
         if constexpr (sizeof(T) == 8) {
-            if (ffix) {  // nb = 4, one row: the fixed-point fields of the row beside the FP64 ones
-                collect_max(res, 4, ny, top);
+            if (ffix) {  // one row, nb = 4 or 2: its fixed-point fields beside the FP64 ones
+                collect_max(res, nb, ny, top);
                 __syncthreads();
-                if (threadIdx.x < 8) ftop[8 * i0 + threadIdx.x] = top[threadIdx.x];
-                const int b = threadIdx.x & 3;
+                if (threadIdx.x < 2 * nb) ftop[2 * nb * i0 + threadIdx.x] = top[threadIdx.x];
+                const int b = threadIdx.x & (nb - 1);
                 const int er = row_exponent(top[2 * b]), ei = row_exponent(top[2 * b + 1]);
-                for (int e = threadIdx.x; e < 4 * ny; e += blockDim.x) {
-                    const double2 v = res[b * ny + (e >> 2)];
+                for (int e = threadIdx.x; e < nb * ny; e += blockDim.x) {
+                    const double2 v = res[b * ny + e / nb];
                     const int2 re = field_fix(v.x, er), im = field_fix(v.y, ei);
-                    const size_t o = (size_t)i0 * ny * 4 + e;
+                    const size_t o = (size_t)i0 * ny * nb + e;
                     out[o] = v;
                     ffix[o] = make_int4(re.x, re.y, im.x, im.y);
                 }
@@ -256,7 +260,7 @@ cudaError_t launch_fft_y_from_fix(const longlong2* j, double unscale, void* out,
                                   const FftDesc& d, const void* tw, longlong2* clear,
                                   cudaStream_t s, const longlong2* j2, void* out2,
                                   longlong2* clear2) {
-    const FftSecond<T> two{nullptr, (cplx_t<T>*)out2, 1, j2, clear2};
+    const FftSecond<T> two{nullptr, (cplx_t<T>*)out2, 1, j2, clear2, nullptr, nullptr};
     return fft_y_impl<T>(nullptr, out, nx, ny, 1, d, tw, -1, 0, j, unscale, clear, s, nullptr,
                          nullptr, false, j2 ? &two : nullptr);
 }
@@ -264,9 +268,10 @@ cudaError_t launch_fft_y_from_fix(const longlong2* j, double unscale, void* out,
 template <typename T>
 cudaError_t launch_fft_y_fields(const void* f4, void* g, const void* f2, void* g2, int nx, int ny,
                                 const FftDesc& d, const void* tw, const FixFields* fix,
-                                cudaStream_t s) {
-    if (fix && (sizeof(T) != 8 || f2)) return cudaErrorInvalidValue;
-    const FftSecond<T> two{(const cplx_t<T>*)f2, (cplx_t<T>*)g2, 2, nullptr, nullptr};
+                                const FixFields* fix2, cudaStream_t s) {
+    if ((fix || fix2) && sizeof(T) != 8) return cudaErrorInvalidValue;
+    const FftSecond<T> two{(const cplx_t<T>*)f2, (cplx_t<T>*)g2, 2, nullptr, nullptr,
+                           fix2 ? (int4*)fix2->f : nullptr, fix2 ? fix2->top : nullptr};
     return fft_y_impl<T>(f4, g, nx, ny, 4, d, tw, +1, 1, nullptr, 0.0, nullptr, s, fix, nullptr,
                          false, f2 ? &two : nullptr);
 }
@@ -309,14 +314,14 @@ template cudaError_t launch_fft_y_from_fix<double>(const longlong2*, double, voi
                                                    longlong2*);
 template cudaError_t launch_fft_y_fields<double>(const void*, void*, const void*, void*, int, int,
                                              const FftDesc&, const void*, const FixFields*,
-                                             cudaStream_t);
+                                             const FixFields*, cudaStream_t);
 template cudaError_t launch_fft_y_from_fix<float>(const longlong2*, double, void*, int, int,
                                                    const FftDesc&, const void*, longlong2*,
                                                    cudaStream_t, const longlong2*, void*,
                                                    longlong2*);
 template cudaError_t launch_fft_y_fields<float>(const void*, void*, const void*, void*, int, int,
                                              const FftDesc&, const void*, const FixFields*,
-                                             cudaStream_t);
+                                             const FixFields*, cudaStream_t);
 template cudaError_t launch_twiddles<double>(void*, int, cudaStream_t);
 template cudaError_t launch_twiddles<float>(void*, int, cudaStream_t);
 

@@ -141,12 +141,25 @@ __device__ __forceinline__ long long sum58(long long h, long long m) {
     return h + ((m + (1ll << 28)) >> 29);
 }
 
-// v / 2^d rounded, d >= 0
-__device__ __forceinline__ long long shift_round(long long v, int d) {
-    d = min(d, 62);
-    return (v + ((1ll << d) >> 1)) >> d;
+// v / 2^d rounded down, d >= 0
+__device__ __forceinline__ long long shift_down(long long v, int d) { return v >> min(d, 63); }
+// v 2^(e - 58) rounded to nearest even, by integer operations (an int64 conversion and a
+// multiplication would be two of the FP64 pipe's); NaN for the exponent of a row that is not
+// finite.
+__device__ __forceinline__ double fix_value(long long v, int e) {
+    unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)m);
+    m <<= lz & 63;  // the leading bit to bit 63
+    unsigned long long q = m >> 11;
+    const unsigned r = (unsigned)m & 0x7ffu;
+    q += r + ((unsigned)q & 1u) > 0x400u ? 1u : 0u;
+    // q's leading bit adds 1 to the exponent field (2 when the rounding carried into it)
+    const int field = 1027 + e - lz;
+    q += (unsigned long long)field << 52;
+    if (v < 0) q |= 0x8000000000000000ull;
+    if (v == 0) q = 0;
+    if (e > 1024) q = 0x7ff8000000000000ull;
+    return __longlong_as_double((long long)q);
 }
-__device__ __forceinline__ double field_unit(int e) {
-    return e > 1024 ? __hiloint2double(0x7ff80000, 0) : pow2(e - 58);
-}
+
 }  // namespace gpic

@@ -139,11 +139,11 @@ cudaError_t launch_fft_y_from_fix(const longlong2* j, double unscale, void* out,
                                   void* out2 = nullptr, longlong2* clear2 = nullptr);
 // Inverse transforms along y of the gather fields: the four packed spectra f4 to g
 // ([node][4]; with fix, FP64, in fixed point as well) and, with f2, the two of A_z to g2
-// ([node][2]) in the same launch.
+// ([node][2]; fix2) in the same launch.
 template <typename T>
 cudaError_t launch_fft_y_fields(const void* f4, void* g, const void* f2, void* g2, int nx, int ny,
                                 const FftDesc& d, const void* twiddle, const FixFields* fix,
-                                cudaStream_t s);
+                                const FixFields* fix2, cudaStream_t s);
 // Along x (stride ny).
 template <typename T>
 cudaError_t launch_fft_x(const void* in, void* out, int nx, int ny, int nb, const FftDesc& d,
@@ -282,12 +282,14 @@ cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& p
                                const FixFields* fix);
 // Gather + push with a species table and/or three velocity components (vz == NULL: 2D-2V):
 // fz holds the A_z fields as [node][2] complex ((dAz/dx, dAz/dy), (Az, 0)); P_z is constant.
+// FP64 with fix: the fixed-point fields (fixz: those of A_z) instead.
 template <typename T>
 cudaError_t launch_gather_push3(int p, const ParticleGeom& g, const PushParams& pp, const T* x,
                                 const T* y, T* px, T* py, const T* pz, const T* vx, const T* vy,
                                 const T* vz, T* vx_old, T* vy_old, T* vz_old, const int32_t* sp,
                                 const SpeciesParams& spp, int64_t n, const void* fields4,
-                                const void* fz, double* diag, unsigned int* err, cudaStream_t s);
+                                const void* fz, double* diag, unsigned int* err, cudaStream_t s,
+                                const FixFields* fix, const FixFields* fixz);
 // t = 0 with a species table and/or three velocity components.
 template <typename T>
 cudaError_t launch_init_particles3(int p, const ParticleGeom& g, const PushParams& pp, T* x, T* y,

@@ -97,7 +97,8 @@ struct pic_handle {
     void* Z = nullptr;       // spectrum of J (complex)
     void* F4 = nullptr;      // 4 packed field spectra, inverse-transformed in place
     void* G = nullptr;       // [node][4] complex: the eight real gather fields
-    gpic::FixFields fixf{};  // FP64 path: the gather fields in fixed point (f NULL: not used)
+    // FP64 path: the gather fields in fixed point (f NULL: not used), and those of A_z
+    gpic::FixFields fixf{}, fixz{};
     double* gather_out = nullptr;  // where gather_push also writes the adjoint's record of
                                    // the step (its recording steps), else NULL
     bool gather_out_short = false; // the record without the gathered values (P, v only)

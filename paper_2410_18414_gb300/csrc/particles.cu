@@ -207,11 +207,11 @@ struct RowFix {
         AccFix::split2(r[t], wh, ws, h, l);
         return AccFix::join(h, l);
     }
-    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+    __device__ __forceinline__ V issue(int node, int c, V x) const {
         atomicAdd(reinterpret_cast<V*>(acc.J + node) + c, x);
         return 0;
     }
-    __device__ __forceinline__ void finish(size_t, int, V, V) const {}
+    __device__ __forceinline__ void finish(int, int, V, V) const {}
     template <int P>
     __device__ __forceinline__ bool shape(const GeomT<float>& g, float x, float y, int& ix,
                                           int& iy, float* wx, float* wy) const {
@@ -256,10 +256,10 @@ struct RowFix128 {
     __device__ __forceinline__ V value(const long long* r, int t, int wy, int) const {
         return (V)__mul64hi(r[t], r[wy]);
     }
-    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+    __device__ __forceinline__ V issue(int node, int c, V x) const {
         return atomicAdd(reinterpret_cast<V*>(J + node) + c, x);
     }
-    __device__ __forceinline__ void finish(size_t node, int c, V x, V old) const {
+    __device__ __forceinline__ void finish(int node, int c, V x, V old) const {
         const long long dh = ((long long)x < 0 ? -1ll : 0ll) + (old + x < old ? 1ll : 0ll);
         if (dh != 0) atomicAdd(reinterpret_cast<V*>(J + ng + node) + c, (V)dh);
     }
@@ -293,11 +293,11 @@ struct RowF64 {
     __device__ __forceinline__ V value(const double* r, int t, int wy, int) const {
         return rmul(r[t], r[wy]);
     }
-    __device__ __forceinline__ V issue(size_t node, int c, V x) const {
+    __device__ __forceinline__ V issue(int node, int c, V x) const {
         atomicAdd(reinterpret_cast<double*>(J + node) + c, x);
         return 0.0;
     }
-    __device__ __forceinline__ void finish(size_t, int, V, V) const {}
+    __device__ __forceinline__ void finish(int, int, V, V) const {}
     template <int P>
     __device__ __forceinline__ bool shape(const GeomT<double>& g, double x, double y, int& ix,
                                           int& iy, double* wx, double* wy) const {
@@ -393,7 +393,7 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
             for (int q = 0; q < kPasses; ++q) {
                 int bs[kAhead];
                 V val[kAhead], old[kAhead];
-                size_t node[kAhead];
+                int node[kAhead];
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j) {
                     const int k = (i0 + j) * kGroups + group;
@@ -406,7 +406,7 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                         int gi = (bs[j] >> 16) + wa[q], gj = (bs[j] & 0xFFFF) + wb[q];
                         if (gi >= g.nx) gi -= g.nx;
                         if (gj >= g.ny) gj -= g.ny;
-                        node[j] = (size_t)gi * g.ny + gj;
+                        node[j] = gi * g.ny + gj;  // at most 1024^2 nodes
                         if (j > 0 && bs[j] == bs[j - 1]) {  // the same words: one atomic
                             val[j] += val[j - 1];
                             bs[j - 1] = -1;
@@ -512,6 +512,30 @@ __device__ __forceinline__ void push_core(const PushT<T>& pp, const T* f, T px, 
     vy_new = vyn1;
     if (!isfinite(vxn1) || !isfinite(vyn1)) bad |= ERR_NONFINITE;
     if (pp.diag) kin += kinetic(pp.c2, pp.mc2, pp.c, pp.m, rfma(ux, ux, rmul(uy, uy)));
+}
+
+// 2D-3V: the same with A_z (fz = dAz/dx, dAz/dy, Az) and the z velocities; P_z is constant.
+template <typename T>
+__device__ __forceinline__ void push_core3(const PushT<T>& pp, const T* f, const T* fz, T px, T py,
+                                           T pz, T vx, T vy, T vz, T vxo, T vyo, T vzo,
+                                           unsigned& bad, double& kin, T& Px, T& Py, T& vx_new,
+                                           T& vy_new, T& vz_new) {
+    const T vsx = rfma((T)2, vx, -vxo);
+    const T vsy = rfma((T)2, vy, -vyo);
+    const T vsz = rfma((T)2, vz, -vzo);
+    const T fx = rfma(fz[0], vsz, rfma(f[6], vsy, rfma(f[4], vsx, -f[0])));
+    const T fy = rfma(fz[1], vsz, rfma(f[7], vsy, rfma(f[5], vsx, -f[1])));
+    Px = rfma(pp.qdt, fx, px);
+    Py = rfma(pp.qdt, fy, py);
+    const T ux = rfma(-pp.q, f[2], Px), uy = rfma(-pp.q, f[3], Py), uz = rfma(-pp.q, fz[2], pz);
+    const T u2 = rfma(uz, uz, rfma(ux, ux, rmul(uy, uy)));
+    const T den = rsqrt_rn(rfma(pp.c2, u2, rmul(pp.mc2, pp.mc2)));
+    const T rc = rdiv(pp.c2, den);
+    vx_new = rmul(rc, ux);
+    vy_new = rmul(rc, uy);
+    vz_new = rmul(rc, uz);
+    if (!isfinite(vx_new) || !isfinite(vy_new)) bad |= ERR_NONFINITE;
+    if (pp.diag) kin += kinetic(pp.c2, pp.mc2, pp.c, pp.m, u2);
 }
 
 template <typename T>
@@ -713,6 +737,62 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
 //     products and sums to, and than the transform's own error in f, 2^-53 of the largest
 //     value.
 // Integer sums do not depend on their order, and the same bits come out on every path.
+// Fields 2q and 2q+1 of the `per` int4 a node at one particle (kb: its first node, w: its
+// weights' limbs).
+template <int P>
+__device__ __forceinline__ double2 gather_fix_pair(int nx, int ny, const int4* __restrict__ F,
+                                                   const unsigned* __restrict__ top, int per,
+                                                   int q, int kb, const int2* w) {
+    constexpr int S1 = P + 1;
+    int col[S1], row[S1], e0[S1], e1[S1], top0 = -900, top1 = -900;
+#pragma unroll
+    for (int a = 0; a < S1; ++a) {
+        int gj = (kb & 0xFFFF) + a, gi = (kb >> 16) + a;
+        if (gj >= ny) gj -= ny;
+        if (gi >= nx) gi -= nx;
+        col[a] = per * gj + q;
+        row[a] = gi;
+        const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + per * gi + q);
+        e0[a] = row_exponent(u.x);
+        e1[a] = row_exponent(u.y);
+        top0 = max(top0, e0[a]);
+        top1 = max(top1, e1[a]);
+    }
+    long long s0 = 0, s1 = 0;
+#pragma unroll
+    for (int a = 0; a < S1; ++a) {
+        const int4* F0 = F + (size_t)row[a] * ny * per;
+        long long h0 = 0, m0 = 0, h1 = 0, m1 = 0;
+#pragma unroll
+        for (int b = 0; b < S1; ++b) {
+            const int4 v = __ldg(F0 + col[b]);
+            const int2 wab = w[a * S1 + b];
+            mac58(h0, m0, wab, v.x, v.y);
+            mac58(h1, m1, wab, v.z, v.w);
+        }
+        s0 += shift_down(sum58(h0, m0), top0 - e0[a]);
+        s1 += shift_down(sum58(h1, m1), top1 - e1[a]);
+    }
+    return make_double2(fix_value(s0, top0), fix_value(s1, top1));
+}
+
+// A particle's first node (-1: outside the domain) and the limbs of its (p+1)^2 weights.
+template <int P>
+__device__ __forceinline__ int fix_stencil(const GeomT<double>& g, const FixGeom& fg, double x,
+                                           double y, int2* w) {
+    constexpr int S1 = P + 1;
+    const long long X = __double2ll_rn(rmul(x, fg.sx)), Y = __double2ll_rn(rmul(y, fg.sy));
+    if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh)) return -1;
+    long long wx[S1], wy[S1];
+    const int ix = fix_weights<P>(X, fg.sh, wx);
+    const int iy = fix_weights<P>(Y, fg.sh, wy);
+#pragma unroll
+    for (int a = 0; a < S1; ++a)
+#pragma unroll
+        for (int b = 0; b < S1; ++b) w[a * S1 + b] = weight_limbs(mul62(wx[a], wy[b]));
+    return (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
+}
+
 template <int P>
 __global__ void __launch_bounds__(kRowGatherThreads)
 k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* __restrict__ x,
@@ -722,7 +802,7 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
                   double* __restrict__ vyo, int64_t n, const int4* __restrict__ F,
                   const unsigned* __restrict__ top, double* __restrict__ gout, int gout_short,
                   double* __restrict__ diag, unsigned int* __restrict__ err) {
-    constexpr int S1 = P + 1, S2 = S1 * S1;
+    constexpr int S2 = (P + 1) * (P + 1);
     constexpr int kStride = S2 | 1;  // at least the 8 gathered values
     __shared__ int2 rec[kRowGatherThreads * kStride];
     __shared__ int rbase[kRowGatherThreads];
@@ -735,70 +815,21 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
     unsigned bad = 0;
     int base = -1;
     if (p < n) {
-        const long long X = __double2ll_rn(rmul(x[p], fg.sx)), Y = __double2ll_rn(rmul(y[p], fg.sy));
-        if (X < 0 || X > ((long long)g.nx << fg.sh) || Y < 0 || Y > ((long long)g.ny << fg.sh)) {
-            bad |= ERR_NONFINITE;
-        } else {
-            long long wx[S1], wy[S1];
-            const int ix = fix_weights<P>(X, fg.sh, wx);
-            const int iy = fix_weights<P>(Y, fg.sh, wy);
-            base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
-#pragma unroll
-            for (int a = 0; a < S1; ++a)
-#pragma unroll
-                for (int b = 0; b < S1; ++b)
-                    mine[a * S1 + b] = limbs58((mul62(wx[a], wy[b]) + 8) >> 4);
-        }
+        base = fix_stencil<P>(g, fg, x[p], y[p], mine);
+        if (base < 0) bad |= ERR_NONFINITE;
     }
     rbase[threadIdx.x] = base;
     __syncwarp();
 #pragma unroll 1
     for (int t = 0; t < 4; ++t) {
         const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
-        const int2* r = rec + k * kStride;
         const int kb = rbase[k];
-        double f0 = 0.0, f1 = 0.0;
-        if (kb >= 0) {
-            int col[S1], row[S1], e0[S1], e1[S1], top0 = -900, top1 = -900;
-#pragma unroll
-            for (int a = 0; a < S1; ++a) {
-                int gj = (kb & 0xFFFF) + a, gi = (kb >> 16) + a;
-                if (gj >= g.ny) gj -= g.ny;
-                if (gi >= g.nx) gi -= g.nx;
-                col[a] = 4 * gj + q;
-                row[a] = gi;
-                const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + 4 * gi + q);
-                e0[a] = row_exponent(u.x);
-                e1[a] = row_exponent(u.y);
-                top0 = max(top0, e0[a]);
-                top1 = max(top1, e1[a]);
-            }
-            long long s0 = 0, s1 = 0;
-#pragma unroll
-            for (int a = 0; a < S1; ++a) {
-                const int4* F0 = F + (size_t)row[a] * g.ny * 4;
-                long long h0 = 0, m0 = 1ll << 28, h1 = 0, m1 = 1ll << 28;
-#pragma unroll
-                for (int b = 0; b < S1; ++b) {
-                    const int4 v = __ldg(F0 + col[b]);
-                    const int2 w = r[a * S1 + b];
-                    h0 += (long long)w.x * v.x;
-                    m0 += (long long)w.x * v.y;
-                    m0 += (long long)w.y * v.x;
-                    h1 += (long long)w.x * v.z;
-                    m1 += (long long)w.x * v.w;
-                    m1 += (long long)w.y * v.z;
-                }
-                s0 += shift_round(h0 + (m0 >> 29), top0 - e0[a]);
-                s1 += shift_round(h1 + (m1 >> 29), top1 - e1[a]);
-            }
-            f0 = rmul((double)s0, field_unit(top0));
-            f1 = rmul((double)s1, field_unit(top1));
-        }
+        double2 f = make_double2(0.0, 0.0);
+        if (kb >= 0) f = gather_fix_pair<P>(g.nx, g.ny, F, top, 4, q, kb, rec + k * kStride);
         __syncwarp();  // the four lanes have read the particle's weights
         double* out = reinterpret_cast<double*>(rec + k * kStride);
-        out[2 * q] = f0;
-        out[2 * q + 1] = f1;
+        out[2 * q] = f.x;
+        out[2 * q + 1] = f.y;
     }
     __syncwarp();
     if (base >= 0) {
@@ -1602,6 +1633,11 @@ __device__ __forceinline__ bool push_const(const PushParams& pp, const int32_t* 
     return true;
 }
 
+__device__ __forceinline__ PushT<double> typed_push(const PushParams& pp,
+                                                    const PushConst<double>& c) {
+    return PushT<double>{c.q, c.qdt, pp.c * pp.c, c.mc2, pp.c, c.m, c.w, pp.diag};
+}
+
 template <typename T, int P, bool Z3>
 __global__ void __launch_bounds__(kThreads)
 k_gather_push3(GeomT<T> g, PushParams pp, const T* __restrict__ x, const T* __restrict__ y,
@@ -1681,6 +1717,86 @@ k_gather_push3(GeomT<T> g, PushParams pp, const T* __restrict__ x, const T* __re
         for (int o = 16; o > 0; o >>= 1) kin += __shfl_down_sync(0xffffffffu, kin, o);
         if ((threadIdx.x & 31) == 0 && kin != 0.0) atomicAdd(diag + D_KIN, kin);
     }
+}
+
+// k_gather_push_fix with a species table and/or three velocity components: the A_z fields
+// (fz: two int4 a node) go to the first two of a particle's four lanes.
+// Bound as k_gather_push_fix is; against the FP64 gather, 20 steps and a read-back of 64,000
+// quadratic 2D-3V particles on 192 x 512: 5.25 -> 5.15 ms.
+template <int P, bool Z3>
+__global__ void __launch_bounds__(kRowGatherThreads)
+k_gather_push3_fix(GeomT<double> g, FixGeom fg, PushParams pp, const double* __restrict__ x,
+                   const double* __restrict__ y, double* __restrict__ px,
+                   double* __restrict__ py, const double* __restrict__ pz,
+                   const double* __restrict__ vx, const double* __restrict__ vy,
+                   const double* __restrict__ vz, double* __restrict__ vxo,
+                   double* __restrict__ vyo, double* __restrict__ vzo,
+                   const int32_t* __restrict__ sp, SpeciesParams spp, int64_t n,
+                   const int4* __restrict__ F, const unsigned* __restrict__ top,
+                   const int4* __restrict__ Fz, const unsigned* __restrict__ topz,
+                   double* __restrict__ diag, unsigned int* __restrict__ err) {
+    constexpr int S2 = (P + 1) * (P + 1);
+    constexpr int kStride = (S2 > 12 ? S2 : 12) | 1;  // the weights, then the gathered values
+    __shared__ int2 rec[kRowGatherThreads * kStride];
+    __shared__ int rbase[kRowGatherThreads];
+    const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+    const int64_t p = blockIdx.x * (int64_t)kRowGatherThreads + threadIdx.x;
+    int2* mine = rec + threadIdx.x * kStride;
+    griddep_wait();
+    griddep_launch();
+    double kin = 0.0;
+    unsigned bad = 0;
+    int base = -1;
+    PushConst<double> c;
+    if (p < n) {
+        base = fix_stencil<P>(g, fg, x[p], y[p], mine);
+        if (base >= 0 && !push_const(pp, sp, spp, p, c)) base = -1;
+        if (base < 0) bad |= ERR_NONFINITE;
+    }
+    rbase[threadIdx.x] = base;
+    __syncwarp();
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+        const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
+        const int kb = rbase[k];
+        double2 f = make_double2(0.0, 0.0), fz = f;
+        if (kb >= 0) {
+            f = gather_fix_pair<P>(g.nx, g.ny, F, top, 4, q, kb, rec + k * kStride);
+            if (Z3 && q < 2) fz = gather_fix_pair<P>(g.nx, g.ny, Fz, topz, 2, q, kb, rec + k * kStride);
+        }
+        __syncwarp();  // the four lanes have read the particle's weights
+        double* out = reinterpret_cast<double*>(rec + k * kStride);
+        out[2 * q] = f.x;
+        out[2 * q + 1] = f.y;
+        if (Z3 && q < 2) {
+            out[8 + 2 * q] = fz.x;
+            out[9 + 2 * q] = fz.y;
+        }
+    }
+    __syncwarp();
+    if (base >= 0) {
+        const double* f = reinterpret_cast<const double*>(mine);
+        PushT<double> ps = typed_push(pp, c);
+        double ks = 0.0, Px, Py, vxn1, vyn1;
+        if constexpr (Z3) {
+            double vzn1;
+            push_core3(ps, f, f + 8, px[p], py[p], pz[p], vx[p], vy[p], vz[p], vxo[p], vyo[p],
+                       vzo[p], bad, ks, Px, Py, vxn1, vyn1, vzn1);
+            vzo[p] = vzn1;
+        } else {
+            push_core(ps, f, px[p], py[p], vx[p], vy[p], vxo[p], vyo[p], bad, ks, Px, Py, vxn1,
+                      vyn1);
+        }
+        px[p] = Px;
+        py[p] = Py;
+        vxo[p] = vxn1;
+        vyo[p] = vyn1;
+        kin = c.w * ks;  // w m c^2 (gamma - 1)
+    }
+    PushT<double> sum{};
+    sum.weight = 1.0;
+    sum.diag = pp.diag;
+    push_finish(sum, bad, kin, diag, err);
 }
 
 // t = 0 with species and/or three velocity components: P^0 = gamma m_s v^0 and the Taylor
@@ -1858,11 +1974,33 @@ cudaError_t launch_gather_push3(int p, const ParticleGeom& g, const PushParams& 
                                 const T* y, T* px, T* py, const T* pz, const T* vx, const T* vy,
                                 const T* vz, T* vx_old, T* vy_old, T* vz_old, const int32_t* sp,
                                 const SpeciesParams& spp, int64_t n, const void* fields4,
-                                const void* fz, double* diag, unsigned int* err, cudaStream_t s) {
+                                const void* fz, double* diag, unsigned int* err, cudaStream_t s,
+                                const FixFields* fix, const FixFields* fixz) {
     if (n == 0) return cudaSuccess;
     using C = cplx_t<T>;
     const int32_t* spi = spp.n > 0 ? sp : nullptr;
     const bool z3 = vz != nullptr;
+    if constexpr (sizeof(T) == 8) {
+        if (fix) {
+            const unsigned blocks = (unsigned)((n + kRowGatherThreads - 1) / kRowGatherThreads);
+            const FixFields z = fixz ? *fixz : FixFields{};
+#define GPIC_GFIX3(PP, ZZ)                                                                     \
+    launch_pdl(k_gather_push3_fix<PP, ZZ>, dim3(blocks), dim3(kRowGatherThreads), 0, s,        \
+               typed<T>(g), fix_geom(g), pp, x, y, px, py, pz, vx, vy, vz, vx_old, vy_old,     \
+               vz_old, spi, spp, n, (const int4*)fix->f, (const unsigned*)fix->top,            \
+               (const int4*)z.f, (const unsigned*)z.top, diag, err)
+            switch (2 * p + (z3 ? 1 : 0)) {
+                case 4: return GPIC_GFIX3(2, false);
+                case 5: return GPIC_GFIX3(2, true);
+                case 6: return GPIC_GFIX3(3, false);
+                case 7: return GPIC_GFIX3(3, true);
+                case 8: return GPIC_GFIX3(4, false);
+                case 9: return GPIC_GFIX3(4, true);
+                default: return cudaErrorInvalidValue;
+            }
+#undef GPIC_GFIX3
+        }
+    }
 #define GPIC_GP3(PP)                                                                           \
     if (z3)                                                                                    \
         k_gather_push3<T, PP, true><<<blocks_for(n), kThreads, 0, s>>>(                        \
@@ -2175,7 +2313,8 @@ cudaError_t launch_extract(const void* src, int stride, int comp, double scale, 
                                                 const T*, const T*, T*, T*, T*, const int32_t*, \
                                                 const SpeciesParams&, int64_t, const void*,     \
                                                 const void*, double*, unsigned int*,            \
-                                                cudaStream_t);                                  \
+                                                cudaStream_t, const FixFields*,                 \
+                                                const FixFields*);                              \
     template cudaError_t launch_init_particles3<T>(int, const ParticleGeom&, const PushParams&, \
                                                    T*, T*, T*, T*, T*, const T*, const T*,      \
                                                    const T*, T*, T*, T*, const int32_t*,        \

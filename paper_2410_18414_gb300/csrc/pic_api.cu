@@ -314,10 +314,14 @@ void layout_state(pic_handle* h) {
     take(&h->G, 4 * h->ng * cs);
     // The FP64 gather in fixed point, where converting the mesh fields (16 FP64 operations a
     // node) is small beside what it saves (about 200 a particle).
-    if (!h->fp32 && h->vdim == 2 && h->spp.n == 0 && h->n >= (int64_t)(h->ng / 8)) {
-        const size_t fb = 4 * h->ng * sizeof(int4);  // the maxima follow the fields
-        take(&h->fixf.f, fb + (size_t)c.nx * 8 * sizeof(unsigned));
-        h->fixf.top = (unsigned*)((char*)h->fixf.f + fb);
+    if (!h->fp32 && h->n >= (int64_t)(h->ng / 8)) {
+        auto fix = [&](FixFields& f, int per) {  // the maxima follow the fields
+            const size_t fb = per * h->ng * sizeof(int4);
+            take(&f.f, fb + (size_t)c.nx * 2 * per * sizeof(unsigned));
+            f.top = (unsigned*)((char*)f.f + fb);
+        };
+        fix(h->fixf, 4);
+        if (h->vdim == 3) fix(h->fixz, 2);
     }
     take(&h->E, h->ng * cs);
     take(&h->tmp, h->ng * cs);
@@ -933,7 +937,8 @@ pic_status pic_field_solve(pic_handle* h) {
             r = launch_fft_x<T>(h->F2, h->F2, h->nx, h->ny, 2, h->fx, h->twx, +1, h->s);
         if (r != cudaSuccess) return r;
         return launch_fft_y_fields<T>(h->F4, h->G, z3 ? h->F2 : nullptr, h->Gz, h->nx, h->ny,
-                                      h->fy, h->twy, h->fixf.f ? &h->fixf : nullptr, h->s);
+                                      h->fy, h->twy, h->fixf.f ? &h->fixf : nullptr,
+                                      h->fixz.f ? &h->fixz : nullptr, h->s);
     }));
     h->launches_now += fused ? 3 : 5 + (z3 ? 3 : 0);
     h->phase = 2;
@@ -1014,7 +1019,7 @@ pic_status gather_push_step(pic_handle* h, bool fuse, bool defer) {
                 (const T*)h->pz, (const T*)h->v[h->vcur][0], (const T*)h->v[h->vcur][1],
                 z3 ? (const T*)h->vz[h->vcur] : nullptr, (T*)h->v[vo][0], (T*)h->v[vo][1],
                 z3 ? (T*)h->vz[vo] : nullptr, h->species, h->spp, h->n, h->G, h->Gz, h->diag,
-                h->err, h->s);
+                h->err, h->s, h->fixf.f ? &h->fixf : nullptr, h->fixz.f ? &h->fixz : nullptr);
         }));
     } else {
         TimedScope ts(h, PIC_KT_GATHER);

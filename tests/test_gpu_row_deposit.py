@@ -118,6 +118,52 @@ def test_row_gather_fp64(p, nx, ny, n):
         assert np.all(np.abs(after[key] - want) <= bound + 2.0 ** -52 * np.abs(want))
 
 
+@pytest.mark.parametrize("vdim", [2, 3])
+@pytest.mark.parametrize("nx,ny,n", [(8, 8, 7), (8, 8, 8), (16, 12, 33), (54, 36, 1025)])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_row_gather_fp64_species(p, nx, ny, n, vdim):
+    """As test_row_gather_fp64 with a species table and, at vdim 3, the A_z fields: the
+    momenta, with a fourth term of the force, and the velocities v = u / sqrt(u^2 + m^2) with
+    u = P - q A (c = 1).  A gathered A is within 2^-51 of its peak and u adds 2^-51 of its two
+    terms; |dv/du_c| <= 1 / m for each component, and the root and the quotient add less than
+    2^-50 of v."""
+    rng = np.random.default_rng(177 * p + n)
+    lx, ly = 1.0, ny / nx
+    dt = 0.3 * min(lx / nx, ly / ny)
+    x, y = rng.uniform(0, lx, n), rng.uniform(0, ly, n)
+    vx, vy, vz = (rng.uniform(-0.5, 0.5, n) for _ in range(3))
+    sp = rng.integers(0, 2, n).astype(np.int32)
+    w = lx * ly / n
+    qs, ms = np.array([-1.0, 0.5])[sp], np.array([1.0, 4.0])[sp]
+    cfg = pic.make_config(nx, ny, lx, ly, dt, p=p, vdim=vdim,
+                          species=((-1.0, 1.0, w), (0.5, 4.0, 2 * w)))
+    comps = ("x", "y", "z")[:vdim]
+    with pic.Simulation(cfg, x, y, vx, vy, vz=vz if vdim == 3 else None, species=sp) as sim:
+        sim.step(1)
+        before = sim.particles()
+        sim.step(1)
+        after = sim.particles()
+        f = {k: sim.field(k) for k in ["dphidx", "dphidy"] + [f"a{a}" for a in comps]
+             + [f"da{a}d{c}" for a in comps for c in "xy"]}
+    g = {k: _gather(after["x"], after["y"], f[k], lx, ly, p) for k in f}
+    peak = {k: np.max(np.abs(f[k])) for k in f}
+    vs = {a: 2 * before["v" + a].astype(np.longdouble) - before[f"v{a}_old"] for a in comps}
+    for c in "xy":
+        terms = [-g["dphid" + c]] + [g[f"da{a}d{c}"] * vs[a] for a in comps]
+        want = before["p" + c] + qs * dt * sum(terms)
+        peaks = peak["dphid" + c] + sum(peak[f"da{a}d{c}"] for a in comps)
+        bound = np.abs(qs) * dt * (3 * 2.0 ** -51 * peaks
+                                   + 2.0 ** -51 * sum(np.abs(t) for t in terms))
+        assert np.all(np.abs(after["p" + c] - want) <= bound + 2.0 ** -52 * np.abs(want)), c
+    u = {a: after["p" + a] - qs * g["a" + a] for a in comps}
+    du = sum(np.abs(qs) * 2.0 ** -51 * peak["a" + a]
+             + 2.0 ** -51 * (np.abs(after["p" + a]) + np.abs(qs * g["a" + a])) for a in comps)
+    den = np.sqrt(sum(u[a] ** 2 for a in comps) + (ms * ms).astype(np.longdouble))
+    for a in comps:
+        want = u[a] / den
+        assert np.all(np.abs(after["v" + a] - want) <= du / ms + 2.0 ** -50 * np.abs(want)), a
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 129, 1000])
 @pytest.mark.parametrize("p", [2, 3, 4])
 def test_row_gather_fp32_is_the_sorted_gather(p, n):
