@@ -183,7 +183,12 @@ struct AccFix {
 // word 424 to 468.  With fewer than 17 words a stencil (one component), two or three particles
 // go at once.  Four particles are in flight together, so that the round trips of returning
 // atomics overlap, and neighbours among them with the same stencil base (sorted particles)
-// are added first: one atomic instead of up to four on the same words.
+// are added first: one atomic instead of up to four on the same words.  A stencil that wraps at
+// no edge takes its nodes from one index and the word's constant step; one branch sees to the
+// wrapping ones among the four before their words are formed (a branch for each of the four, or
+// one after their words, parts the loads from the atomics: 40.0 us against 39.7 us a step on
+// 32 x 32).  A step of 1.5 M quartic FP32 particles on 256 x 192 295 -> 272 us, of 2^20
+// quadratic FP64 particles on 128 x 128 230 -> 218 us.
 //
 // Move + deposit, a lane per particle before: FP64, 2^20 particles, 128 x 128, cubic 320 ->
 // 108 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
@@ -336,7 +341,7 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
     W* mine = rec + threadIdx.x * kStride;
     // this lane's words: group, stencil row a and column b, component
     const int group = lane / kWords, lw = lane - group * kWords;
-    int wa[kPasses], wb[kPasses], wc[kPasses];
+    int wa[kPasses], wb[kPasses], wc[kPasses], step[kPasses];
     bool on[kPasses];
 #pragma unroll
     for (int q = 0; q < kPasses; ++q) {
@@ -346,6 +351,7 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
         const int r = word - wa[q] * (S1 * kNC);
         wb[q] = r / kNC;
         wc[q] = r - wb[q] * kNC;
+        step[q] = wa[q] * g.ny + wb[q];
     }
     griddep_wait();
     griddep_launch();
@@ -371,7 +377,11 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                 !species_factor(sp, spt, p, fq)) {
                 atomicOr(err, (unsigned)ERR_NONFINITE);
             } else {
-                base = (wrap_idx(ix, g.nx) << 16) | wrap_idx(iy, g.ny);
+                ix = wrap_idx(ix, g.nx);
+                iy = wrap_idx(iy, g.ny);
+                // the first node's index, or (a stencil that wraps) the complement of its
+                // packed coordinates, below -1
+                base = ix + P < g.nx && iy + P < g.ny ? ix * g.ny + iy : -2 - ((ix << 16) | iy);
 #pragma unroll
                 for (int c = 0; c < kNC; ++c) {
                     // with a table each contribution carries the particle's q_s w_s
@@ -394,19 +404,32 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                 int bs[kAhead];
                 V val[kAhead], old[kAhead];
                 int node[kAhead];
+                bool wraps = false;
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j) {
                     const int k = (i0 + j) * kGroups + group;
                     bs[j] = on[q] && k < 32 ? rbase[w0 + k] : -1;
-                    val[j] = 0;
-                    node[j] = 0;
-                    if (bs[j] >= 0) {
-                        val[j] = pol.value(rec + (w0 + k) * kStride, wc[q] * S1 + wa[q],
-                                           kNC * S1 + wb[q], kFields - 1);
-                        int gi = (bs[j] >> 16) + wa[q], gj = (bs[j] & 0xFFFF) + wb[q];
+                    node[j] = bs[j] + step[q];
+                    wraps |= bs[j] < -1;
+                }
+                if (wraps) {  // one branch for the four, before their words
+#pragma unroll
+                    for (int j = 0; j < kAhead; ++j) {
+                        if (bs[j] >= -1) continue;
+                        const int at = -2 - bs[j];
+                        int gi = (at >> 16) + wa[q], gj = (at & 0xFFFF) + wb[q];
                         if (gi >= g.nx) gi -= g.nx;
                         if (gj >= g.ny) gj -= g.ny;
                         node[j] = gi * g.ny + gj;  // at most 1024^2 nodes
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kAhead; ++j) {
+                    const int k = (i0 + j) * kGroups + group;
+                    val[j] = 0;
+                    if (bs[j] != -1) {
+                        val[j] = pol.value(rec + (w0 + k) * kStride, wc[q] * S1 + wa[q],
+                                           kNC * S1 + wb[q], kFields - 1);
                         if (j > 0 && bs[j] == bs[j - 1]) {  // the same words: one atomic
                             val[j] += val[j - 1];
                             bs[j - 1] = -1;
@@ -415,10 +438,10 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                 }
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j)
-                    if (bs[j] >= 0) old[j] = pol.issue(node[j], wc[q], val[j]);
+                    if (bs[j] != -1) old[j] = pol.issue(node[j], wc[q], val[j]);
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j)
-                    if (bs[j] >= 0) pol.finish(node[j], wc[q], val[j], old[j]);
+                    if (bs[j] != -1) pol.finish(node[j], wc[q], val[j], old[j]);
             }
         }
         __syncwarp();  // the records are rewritten
@@ -1721,8 +1744,8 @@ k_gather_push3(GeomT<T> g, PushParams pp, const T* __restrict__ x, const T* __re
 
 // k_gather_push_fix with a species table and/or three velocity components: the A_z fields
 // (fz: two int4 a node) go to the first two of a particle's four lanes.
-// Bound as k_gather_push_fix is; against the FP64 gather, 20 steps and a read-back of 64,000
-// quadratic 2D-3V particles on 192 x 512: 5.25 -> 5.15 ms.
+// Bound as k_gather_push_fix is.  A step of 2^20 cubic particles on 128 x 128, against the FP64
+// gather: 2D-3V 755 -> 490 us, two species in 2D-2V 547 -> 267 us.
 template <int P, bool Z3>
 __global__ void __launch_bounds__(kRowGatherThreads)
 k_gather_push3_fix(GeomT<double> g, FixGeom fg, PushParams pp, const double* __restrict__ x,
