@@ -1,4 +1,4 @@
-// Particle kernels of one PIC step (Algorithm 1, section 4.2), plain path.
+// Particle kernels of one PIC step (Algorithm 1, section 4.2).
 //
 //   move + deposit : x^{n+1} = x^n + v^n dt (wrapped), then J^{n+1} gets
 //                    q_p v^n W(x^{n+1}/dx - i) W(y^{n+1}/dy - j) / (dx dy) at the
@@ -10,7 +10,9 @@
 //                    v^{n+1} = c^2 (P - qA) / sqrt(c^2 |P - qA|^2 + (m c^2)^2),
 //                    written over v^{n-1} (the caller swaps the velocity buffers).
 //   init           : wrap x^0, P^0 = gamma m v^0, v^{-1} by one Taylor step back in E^0.
-// Particles are SoA arrays; one thread per particle in a grid-stride loop.  A
+// Particles are SoA arrays.  Moves and pushes run a thread a particle; where unsorted or FP64
+// particles meet the mesh, the lanes of a warp share a particle's stencil (row deposit, row
+// gathers), and sorted FP32 particles meet it in shared memory (binned pass).  A
 // position outside [0, L] (including NaN) is never used to index the grid: the
 // particle is skipped and the non-finite bit of the device error word is set.
 #include "common.cuh"
@@ -1601,7 +1603,7 @@ __global__ void k_split_records(ReadArrays r, RecordSpace sp, int64_t n) {
 }
 
 // Replay of one FP64 step's particle update from the adjoint's record of that step:
-// state n -> state n+1 with the move of k_move_deposit (the same operations, so the same
+// state n -> state n+1 with the move of k_deposit_rows (the same operations, so the same
 // bits) and the recorded P^{n+1}, v^{n+1}.  States are eight arrays of n in the order x, y,
 // Px, Py, v^n (x, y), v^{n-1} (x, y); rec is the step's record (P^{n+1}, v^{n+1} first).
 template <typename T>
@@ -2312,6 +2314,8 @@ template cudaError_t launch_read_records<float>(const ReadArrays&, const int32_t
 template cudaError_t launch_read_records<double>(const ReadArrays&, const int32_t*,
                                                  const RecordSpace&, int64_t, cudaStream_t);
 template cudaError_t launch_read_arrays<float, double>(const ReadArrays&, const int32_t*, int64_t,
+                                                       cudaStream_t);
+template cudaError_t launch_read_arrays<double, float>(const ReadArrays&, const int32_t*, int64_t,
                                                        cudaStream_t);
 template cudaError_t launch_read_arrays<double, double>(const ReadArrays&, const int32_t*, int64_t,
                                                         cudaStream_t);

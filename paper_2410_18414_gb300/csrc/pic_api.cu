@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/pic.h: the simulation handle, argument
 // checks, the t = 0 set-up and the three phases of one step (Algorithm 1, section 4.2).
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -18,8 +19,43 @@
 using namespace gpic;
 
 namespace {
+
 thread_local std::string g_init_error;
+
+// Whether a kernel on the handle's device may read or write the `bytes` at p in place: memory of
+// this device, or page-locked host memory from CUDA's own allocator, which is mapped for reads
+// and writes (registered memory may be mapped read-only: it takes the copies, as pageable and
+// managed memory do), aligned, and all of it inside one allocation.
+bool usable_in_place(const pic_handle* h, const void* p, size_t bytes) {
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+    cudaPointerAttributes at{};
+    unsigned flags = 0;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess ||
+        (at.type == cudaMemoryTypeHost &&
+         (at.devicePointer != p || cudaHostGetFlags(&flags, const_cast<void*>(p)) != cudaSuccess ||
+          (flags & cudaHostRegisterReadOnly)))) {
+        cudaGetLastError();  // a pageable pointer is not an error of the context
+        return false;
+    }
+    if (at.type != cudaMemoryTypeHost && (at.type != cudaMemoryTypeDevice || at.device != h->device))
+        return false;
+    static const auto attribute = [] {  // the runtime has no query for an allocation's range
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault,
+                                             &found) != cudaSuccess)
+            cudaGetLastError();
+        return reinterpret_cast<decltype(&cuPointerGetAttribute)>(fn);
+    }();
+    const CUdeviceptr q = reinterpret_cast<CUdeviceptr>(p);
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    return attribute && attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, q) == CUDA_SUCCESS &&
+           attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, q) == CUDA_SUCCESS &&
+           q >= start && q - start <= size && bytes <= size - (q - start);
 }
+
+}  // namespace
 
 
 namespace gpic {
@@ -448,14 +484,22 @@ pic_status setup(pic_handle* h, const pic_particles_in* in) {
         CK(cudaMemcpyAsync(h->species, in->species, (size_t)n * sizeof(int32_t), cudaMemcpyDefault,
                            h->s));
     const int32_t* sp = h->spp.n > 0 ? h->species : nullptr;
+    // arrays that a kernel can read are converted in place by one kernel: set-up with 400,000
+    // FP32 particles from page-locked memory 364 us, with a copy and a conversion an array 398
+    ReadArrays direct{};
     for (int i = 0; i < narr && n > 0 && !h->bound; ++i) {  // bound: in place already
-        if (h->fp32) {
+        if (usable_in_place(h, src[i], nb64)) {
+            direct.src[direct.count] = src[i];
+            direct.dst[direct.count++] = dst[i];
+        } else if (h->fp32) {
             CK(cudaMemcpyAsync(h->stage, src[i], nb64, cudaMemcpyDefault, h->s));
             CK(launch_convert<double, float>(h->stage, (float*)dst[i], n, h->s));
         } else {
             CK(cudaMemcpyAsync(dst[i], src[i], nb64, cudaMemcpyDefault, h->s));
         }
     }
+    CK(h->fp32 ? launch_read_arrays<double, float>(direct, nullptr, n, h->s)
+               : launch_read_arrays<double, double>(direct, nullptr, n, h->s));
 
     void* rho0 = newest(h, 3);
     void* phi0 = newest(h, 0);
@@ -1328,6 +1372,7 @@ pic_status pic_get_field(pic_handle* h, int32_t which, double* dst) {
     if ((which == PIC_FIELD_EX || which == PIC_FIELD_EY) && !h->e_valid)
         return fail(h, PIC_ERR_STATE, "E needs diagnostics on the last step");
     const int64_t n = (int64_t)h->ng;
+    double* const out = usable_in_place(h, dst, h->ng * sizeof(double)) ? dst : h->tmpd;
     cudaError_t e = by_prec(h, [&](auto t) -> cudaError_t {
         using T = decltype(t);
         const size_t cs = sizeof(T) * 2;
@@ -1337,26 +1382,26 @@ pic_status pic_get_field(pic_handle* h, int32_t which, double* dst) {
             case PIC_FIELD_JY:
                 if (h->fp32)
                     return launch_extract_fix((const longlong2*)h->J, which == PIC_FIELD_JY,
-                                              h->fix_unscale_j * h->mc.jscale, h->tmpd, n, h->s);
+                                              h->fix_unscale_j * h->mc.jscale, out, n, h->s);
                 r0 = launch_fix128_to_cplx((const longlong2*)h->J, h->ng, h->fix64_unscale_j,
                                            (double2*)h->tmp, h->s);
                 if (r0 != cudaSuccess) return r0;
                 return launch_extract<double>(h->tmp, 1, which == PIC_FIELD_JY, h->mc.jscale,
-                                              h->tmpd, n, h->s);
+                                              out, n, h->s);
             case PIC_FIELD_JZ:
                 if (h->fp32)
                     return launch_extract_fix((const longlong2*)h->Jz, 0,
-                                              h->fix_unscale_j * h->mc.jscale, h->tmpd, n, h->s);
+                                              h->fix_unscale_j * h->mc.jscale, out, n, h->s);
                 r0 = launch_fix128_to_cplx((const longlong2*)h->Jz, h->ng, h->fix64_unscale_j,
                                            (double2*)h->tmp, h->s);
                 if (r0 != cudaSuccess) return r0;
-                return launch_extract<double>(h->tmp, 1, 0, h->mc.jscale, h->tmpd, n, h->s);
+                return launch_extract<double>(h->tmp, 1, 0, h->mc.jscale, out, n, h->s);
             case PIC_FIELD_DAZDX: case PIC_FIELD_DAZDY:  // Gz: [node][2], (dAz/dx, dAz/dy) first
-                return launch_extract<T>(h->Gz, 2, which == PIC_FIELD_DAZDY, 1.0, h->tmpd, n, h->s);
+                return launch_extract<T>(h->Gz, 2, which == PIC_FIELD_DAZDY, 1.0, out, n, h->s);
             case PIC_FIELD_DPHIDX: case PIC_FIELD_DPHIDY: case PIC_FIELD_GAX: case PIC_FIELD_GAY:
             case PIC_FIELD_DAXDX: case PIC_FIELD_DAXDY: case PIC_FIELD_DAYDX: case PIC_FIELD_DAYDY: {
                 const int f = which - PIC_FIELD_DPHIDX;
-                return launch_extract<T>((const char*)h->G + (f / 2) * cs, 4, f & 1, 1.0, h->tmpd, n, h->s);
+                return launch_extract<T>((const char*)h->G + (f / 2) * cs, 4, f & 1, 1.0, out, n, h->s);
             }
             default: break;
         }
@@ -1383,10 +1428,10 @@ pic_status pic_get_field(pic_handle* h, int32_t which, double* dst) {
         if (r != cudaSuccess) return r;
         r = inverse_fft(h, h->tmp, h->tmp, 1);
         if (r != cudaSuccess) return r;
-        return launch_extract<T>(h->tmp, 1, comp, 1.0, h->tmpd, n, h->s);
+        return launch_extract<T>(h->tmp, 1, comp, 1.0, out, n, h->s);
     });
     CK(e);
-    CK(cudaMemcpyAsync(dst, h->tmpd, h->ng * sizeof(double), cudaMemcpyDefault, h->s));
+    if (out != dst) CK(cudaMemcpyAsync(dst, out, h->ng * sizeof(double), cudaMemcpyDefault, h->s));
     return check_device_error(h);
 }
 
@@ -1394,31 +1439,22 @@ pic_status pic_get_field(pic_handle* h, int32_t which, double* dst) {
 
 namespace {
 
-// Whether a kernel of the handle's device may write FP64 (or int32) values straight to dst.
-bool writable_in_place(const pic_handle* h, const void* dst) {
-    if (reinterpret_cast<uintptr_t>(dst) % sizeof(double) != 0) return false;
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
-        cudaGetLastError();  // a host pointer is not an error of the context
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == h->device;
-}
-
 // Copies m particle arrays (Ts on the device) to dst (Td, device or host) in the caller's
-// order: one kernel for the destinations on this device, the others through the staging
-// buffer one after another (ordered by the stream).
+// order: one kernel for the destinations that it can write in place, on this device or in
+// page-locked host memory (400,000 sorted FP32 particles: 164 us, through the staging buffer
+// and the copy engine 295 us; 26 M: 9.3 against 12.1 ms), the others through the staging buffer
+// one after another (ordered by the stream).
 // (m = 8: the state's arrays, FP64 destinations.)
 template <typename Ts, typename Td>
 pic_status read_arrays(pic_handle* h, const void* const* src, void* const* dst, int m) {
     if (h->n == 0) return PIC_OK;
-    // Sorted runs whose arrays L2 (129 MB) does not hold, read back whole to this device: by
+    // Sorted runs whose arrays L2 (129 MB) does not hold, read back whole and in place: by
     // records, in the sort's second set of arrays, which holds nothing between sorts (26 M
     // particles: 1.4 ms, by the inverse permutation 3.5 ms).
     if constexpr (sizeof(Td) == 8) {
         ReadArrays r{};
         for (int i = 0; i < m && m == 8; ++i) {
-            if (!dst[i] || !writable_in_place(h, dst[i])) break;
+            if (!dst[i] || !usable_in_place(h, dst[i], (size_t)h->n * sizeof(Td))) break;
             r.src[i] = src[i];
             r.dst[i] = dst[i];
             ++r.count;
@@ -1440,7 +1476,7 @@ pic_status read_arrays(pic_handle* h, const void* const* src, void* const* dst, 
     ReadArrays direct{};
     for (int i = 0; i < m; ++i) {
         if (!dst[i]) continue;
-        if (writable_in_place(h, dst[i])) {
+        if (usable_in_place(h, dst[i], (size_t)h->n * sizeof(Td))) {
             direct.src[direct.count] = src[i];
             direct.dst[direct.count++] = dst[i];
             continue;
@@ -1507,7 +1543,7 @@ int32_t pic_velocity_slot(const pic_handle* h) { return h ? h->vcur : -1; }
 
 int32_t pic_kernels_per_step(const pic_handle* h) {
     if (!h) return 0;
-    // Kernels the most recent complete step launched: move_deposit, the row transform,
+    // Kernels the most recent complete step launched: the deposit, the row transform,
     // the fused column pass (or column transforms and the per-mode update on grids too
     // large for it), the inverse row transform, gather_push; a sort step adds its 3
     // kernels.  Before any step: the count of a step without a sort.
