@@ -185,16 +185,17 @@ struct AccFix {
 // word 424 to 468.  With fewer than 17 words a stencil (one component), two or three particles
 // go at once.  Four particles are in flight together, so that the round trips of returning
 // atomics overlap, and neighbours among them with the same stencil base (sorted particles)
-// are added first: one atomic instead of up to four on the same words.  A stencil that wraps at
-// no edge takes its nodes from one index and the word's constant step; one branch sees to the
-// wrapping ones among the four before their words are formed (a branch for each of the four, or
-// one after their words, parts the loads from the atomics: 40.0 us against 39.7 us a step on
-// 32 x 32).  A step of 1.5 M quartic FP32 particles on 256 x 192 295 -> 272 us, of 2^20
+// are added first: one atomic instead of up to four on the same words.
+//
+// Large launches are bound by issue, and of a word's instructions nine were its node's index
+// with two wraps.  kInner: a stencil that wraps at no edge takes its nodes from one index and the
+// word's constant step; one branch sees to the wrapping ones among the four before their words
+// are formed.  A step of 1.5 M quartic FP32 particles on 256 x 192 295 -> 272 us, of 2^20
 // quadratic FP64 particles on 128 x 128 230 -> 218 us.
 //
 // Move + deposit, a lane per particle before: FP64, 2^20 particles, 128 x 128, cubic 320 ->
-// 108 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
-// 256 x 192, quartic 353 -> 149 us (bound by L2's atomics still: 17.5 sectors a particle).
+// 100 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
+// 256 x 192, quartic 353 -> 120 us (bound by L2's atomics still: 17.5 sectors a particle).
 constexpr int kRowThreads = 128;
 
 // A policy says what a particle's record holds (per component the row factors t[a], then
@@ -321,7 +322,7 @@ struct RowF64 {
 
 // kMove: x, y move by (u0, u1) dt first (the position update); u0, u1: the deposited
 // components (kNC = 1: u0 alone, or 1 for every particle when u0 is NULL, the charge).
-template <typename Pol, int P, int kNC, bool kMove>
+template <typename Pol, int P, int kNC, bool kMove, bool kInner>
 __global__ void __launch_bounds__(kRowThreads)
 k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                typename Pol::T* __restrict__ y, const typename Pol::T* __restrict__ u0,
@@ -381,9 +382,10 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
             } else {
                 ix = wrap_idx(ix, g.nx);
                 iy = wrap_idx(iy, g.ny);
-                // the first node's index, or (a stencil that wraps) the complement of its
-                // packed coordinates, below -1
-                base = ix + P < g.nx && iy + P < g.ny ? ix * g.ny + iy : -2 - ((ix << 16) | iy);
+                // packed coordinates; kInner: the first node's index, or (a stencil that
+                // wraps) the complement of the packed coordinates, below -1
+                base = (ix << 16) | iy;
+                if (kInner) base = ix + P < g.nx && iy + P < g.ny ? ix * g.ny + iy : -2 - base;
 #pragma unroll
                 for (int c = 0; c < kNC; ++c) {
                     // with a table each contribution carries the particle's q_s w_s
@@ -406,24 +408,24 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                 int bs[kAhead];
                 V val[kAhead], old[kAhead];
                 int node[kAhead];
+                const auto wrapped = [&](int at) {
+                    int gi = (at >> 16) + wa[q], gj = (at & 0xFFFF) + wb[q];
+                    if (gi >= g.nx) gi -= g.nx;
+                    if (gj >= g.ny) gj -= g.ny;
+                    return gi * g.ny + gj;  // at most 1024^2 nodes
+                };
                 bool wraps = false;
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j) {
                     const int k = (i0 + j) * kGroups + group;
                     bs[j] = on[q] && k < 32 ? rbase[w0 + k] : -1;
-                    node[j] = bs[j] + step[q];
+                    node[j] = kInner ? bs[j] + step[q] : wrapped(bs[j]);
                     wraps |= bs[j] < -1;
                 }
-                if (wraps) {  // one branch for the four, before their words
+                if (kInner && wraps) {  // one branch for the four, before their words
 #pragma unroll
-                    for (int j = 0; j < kAhead; ++j) {
-                        if (bs[j] >= -1) continue;
-                        const int at = -2 - bs[j];
-                        int gi = (at >> 16) + wa[q], gj = (at & 0xFFFF) + wb[q];
-                        if (gi >= g.nx) gi -= g.nx;
-                        if (gj >= g.ny) gj -= g.ny;
-                        node[j] = gi * g.ny + gj;  // at most 1024^2 nodes
-                    }
+                    for (int j = 0; j < kAhead; ++j)
+                        if (bs[j] < -1) node[j] = wrapped(-2 - bs[j]);
                 }
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j) {
@@ -655,7 +657,7 @@ k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restr
 // gathered 16 or 8 at a time, and the gathered fields go back through the same records to
 // the lane that pushes the particle.  Gather + push, a lane per particle before: FP32, 1.5 M
 // particles, 256 x 192, quartic 192 -> 121 us; FP64, 2^20 particles, 128 x 128, cubic
-// 394 -> 127 us.
+// 394 -> 124 us.
 constexpr int kRowGatherThreads = 128;
 
 // FP32: the node order and roundings of every other gather, so the same bits.
@@ -1906,13 +1908,18 @@ cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typen
     const unsigned blocks = (unsigned)((n + kRowThreads - 1) / kRowThreads);
     const GeomT<T> gt = typed<T>(g);
     const SpeciesT<T> st = typed_species<T>(spp);
-#define GPIC_ROWS(PP)                                                                        \
-    launch_pdl(k_deposit_rows<Pol, PP, kNC, kMove>, dim3(blocks), dim3(kRowThreads), 0, s, gt, x, \
-               y, u0, u1, n, pol, err, sp, st)
+    // kInner from three CTAs an SM on: below that the warps wait for their own chains of atomics
+    // and kInner's branch lengthens them (two FP64 quartic steps of 8,700 particles on 256 x 36
+    // 155 us without it, 171 with; 1.5 M FP32 on 256 x 192 294 and 270; 16,384 FP64 on 32 x 32
+    // the same)
+    const bool many = n >= (1 << 16);
+#define GPIC_ROWS(PP, INNER)                                                                 \
+    launch_pdl(k_deposit_rows<Pol, PP, kNC, kMove, INNER>, dim3(blocks), dim3(kRowThreads), 0, s, \
+               gt, x, y, u0, u1, n, pol, err, sp, st)
     switch (p) {
-        case 2: return GPIC_ROWS(2);
-        case 3: return GPIC_ROWS(3);
-        case 4: return GPIC_ROWS(4);
+        case 2: return many ? GPIC_ROWS(2, true) : GPIC_ROWS(2, false);
+        case 3: return many ? GPIC_ROWS(3, true) : GPIC_ROWS(3, false);
+        case 4: return many ? GPIC_ROWS(4, true) : GPIC_ROWS(4, false);
         default: return cudaErrorInvalidValue;
     }
 #undef GPIC_ROWS

@@ -44,7 +44,9 @@ def _deposit(x, y, v, nx, ny, lx, ly, p):
 
 @pytest.mark.parametrize("nx,ny,n,one_cell", [(8, 8, 1, False), (16, 12, 31, False),
                                               (16, 12, 33, True), (32, 8, 129, True),
-                                              (8, 1024, 1000, False), (54, 36, 4099, False)])
+                                              (8, 1024, 1000, False), (54, 36, 4099, False),
+                                              # from 65,536 particles on: one index a stencil
+                                              (8, 8, 65536, False), (54, 36, 65539, True)])
 @pytest.mark.parametrize("p", [2, 3, 4])
 def test_row_deposit(p, nx, ny, n, one_cell):
     rng = np.random.default_rng(1000 * p + n)
