@@ -411,7 +411,8 @@ void pic_destroy(pic_handle *h);
  * `checkpoint_every` steps (K).  The backward pass rebuilds each segment of K steps from
  * its checkpoint -- the particle states (S = 64 n bytes per step of the segment in FP64,
  * 32 n in the FP32 form) and each step's record (see pic_adjoint_mode) -- then runs it
- * backwards.  With G = 64 nx ny bytes of gather fields a step (32 nx ny in the FP32 form):
+ * backwards.  With G = 64 nx ny bytes of gather fields a step (and 32 nx of
+ * their scales; 32 nx ny in the FP32 form):
  * PIC_ADJ_REPLAY (the default) keeps every step's record from the forward pass and replays
  * only the particle move, costing about (nsteps/K + 1 + K) S + nsteps (80 n + G) bytes
  * (PIC_ADJ_REPLAY_LEAN: 32 n in place of 80 n); PIC_ADJ_RECOMPUTE re-runs the segment's
