@@ -390,11 +390,11 @@ k_adj_push_gather(ParticleGeom g, PushParams pp, const double* __restrict__ x1,
 // dW_x.  The FP64 pipe is left with the push's adjoint and the products the atomics add
 // (about 250 operations a particle instead of 600).  262,144 particles, 128 x 128, cubic: with
 // FP64 gathers and a lane per particle 263 us, now 137 us.  Bound by the FP64 pipe (72%) and its
-// latency: five CTAs an SM (96 registers, no spills) instead of four, 148 -> 137 us; six spill.
-// The lean form gains nothing (144.5 -> 146 us) and quartic shapes spill at five: they take the
-// registers they need.
+// latency: five CTAs an SM (96 registers, 24 bytes spilled) instead of four, 148 -> 137 us; six
+// are slower.  The lean form gains nothing at five (144.5 -> 146 us) and quartic shapes spill:
+// they keep the four and three that their registers allow.
 template <int P, bool kLean>
-__global__ void __launch_bounds__(kAdjThreads, kLean || P > 3 ? 1 : 5)
+__global__ void __launch_bounds__(kAdjThreads, P > 3 ? 3 : P == 3 && kLean ? 4 : 5)
 k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* __restrict__ x1,
                       const double* __restrict__ y1, const double* __restrict__ px1,
                       const double* __restrict__ py1, const double* __restrict__ vx,
@@ -587,9 +587,9 @@ k_adj_deposit_move(ParticleGeom g, const T* __restrict__ x1, const T* __restrict
 // The same with the mesh adjoint current in fixed point (an int4 a node, two maxima a row):
 // six separable integer sums, about 35 FP64 operations a particle left of 170.  Measured with
 // FP64 sums 78 us, now 31 us (262,144 particles, cubic; four CTAs an SM of 128 registers, 34 us
-// with three; quartic shapes spill there and keep three).
+// with three; quartic shapes would spill and keep two).
 template <int P>
-__global__ void __launch_bounds__(kAdjThreads, P > 3 ? 1 : 4)
+__global__ void __launch_bounds__(kAdjThreads, P > 3 ? 2 : 4)
 k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1,
                        const double* __restrict__ y1, const double* __restrict__ vx,
                        const double* __restrict__ vy, const int4* __restrict__ Jb,
