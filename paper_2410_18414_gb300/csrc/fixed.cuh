@@ -127,6 +127,23 @@ __device__ __forceinline__ void fix_dweights(long long X, int sh, long long* d) 
         d[2] = -(d[0] + d[1] + d[3] + d[4]);
     }
 }
+// The FP64 deposit's products (RowFix128), each rounded to nearest with v and -v alike: +v and -v
+// at one place cancel exactly and the errors of many particles do not add up on one side
+// (rounded down, every node's current was half a quantum a contribution too small).
+// t = v W_x in units of 2^-3 quanta from v in 2^-2 quanta (|v| <= 2^62): 2^62 2 3/4 < 2^63.
+__device__ __forceinline__ long long deposit_row(long long v, long long w) {
+    const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const unsigned __int128 t = (unsigned __int128)m * (unsigned long long)w;
+    const long long r = (long long)(unsigned long long)((t + ((unsigned __int128)1 << 60)) >> 61);
+    return v < 0 ? -r : r;
+}
+// x = t W_y in quanta.  The weight (units of 2^-62) comes made odd by deposit_col, so that t W_y
+// is never halfway between two quanta for |t| < 2^63 (it would need t = 0 mod 2^64) and
+// floor((floor(2 x) + 1) / 2) is the nearest for either sign.
+__device__ __forceinline__ long long deposit_col(long long w) { return w | 1; }
+__device__ __forceinline__ long long deposit_value(long long t, long long w) {
+    return (__mul64hi(t, w) + 1) >> 1;
+}
 // a weight in units of 2^-62 as limbs in units of 2^-58
 __device__ __forceinline__ int2 weight_limbs(long long w) { return limbs58((w + 8) >> 4); }
 

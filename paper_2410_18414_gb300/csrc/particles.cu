@@ -249,9 +249,9 @@ struct RowFixCharge : RowFix {
 // returns the word it added to, so the carry out of each addition is known exactly; the carry
 // and the sign extension of x go to the high word, which changes only when the low word wraps.
 // Integer sums do not depend on the order of the additions, so the deposit is bit-for-bit
-// deterministic.  The factors are integers: v in units of 2^-2 quanta, t = v W_x in half
-// quanta, x = t W_y in quanta, each rounded down once (2^-60 of the bound c; FP64 rounds
-// each product at 2^-53 of its value).
+// deterministic.  The factors are integers: v in units of 2^-2 quanta, t = v W_x in 2^-3, x =
+// t W_y in quanta, each rounded to nearest once (deposit_row, deposit_value): x is within
+// 0.6 quanta and no one-sided error is left, whatever v is.
 struct RowFix128 {
     using T = double;
     using W = long long;
@@ -262,7 +262,7 @@ struct RowFix128 {
     FixGeom fg;
     static constexpr bool kExtra = false;
     __device__ __forceinline__ V value(const long long* r, int t, int wy, int) const {
-        return (V)__mul64hi(r[t], r[wy]);
+        return (V)deposit_value(r[t], r[wy]);
     }
     __device__ __forceinline__ V issue(int node, int c, V x) const {
         return atomicAdd(reinterpret_cast<V*>(J + node) + c, x);
@@ -286,9 +286,9 @@ struct RowFix128 {
         return __double2ll_rn(rmul(v, scale4));
     }
     __device__ __forceinline__ long long row(long long v, long long w) const {
-        return __mul64hi(v, w << 1);
+        return deposit_row(v, w);
     }
-    __device__ __forceinline__ long long col(long long w) const { return w << 1; }
+    __device__ __forceinline__ long long col(long long w) const { return deposit_col(w); }
 };
 
 // RowF64: FP64 atomics (the allocation-free pass).

@@ -76,6 +76,22 @@ void shape(int sh) {
     }
 }
 
+// deposit P SH: (v, X, Y) -> the (p+1)^2 contributions of v W_x W_y
+template <int P>
+void deposit(int sh) {
+    const std::vector<long long> in = read_all<long long>();
+    for (size_t k = 0; k + 2 < in.size(); k += 3) {
+        long long wx[P + 1], wy[P + 1];
+        fix_weights<P>(in[k + 1], sh, wx);
+        fix_weights<P>(in[k + 2], sh, wy);
+        for (int a = 0; a <= P; ++a)
+            for (int b = 0; b <= P; ++b) {
+                const long long x = deposit_value(deposit_row(in[k], wx[a]), deposit_col(wy[b]));
+                std::fwrite(&x, sizeof x, 1, stdout);
+            }
+    }
+}
+
 template <typename F>
 void by_degree(int p, F&& f) {
     if (p == 2) f(std::integral_constant<int, 2>());
@@ -90,5 +106,6 @@ int main(int argc, char** argv) {
     const std::string what = argv[1];
     const int p = std::atoi(argv[2]), sh = std::atoi(argv[3]);
     if (what == "shape") by_degree(p, [&](auto P) { shape<decltype(P)::value>(sh); });
+    if (what == "deposit") by_degree(p, [&](auto P) { deposit<decltype(P)::value>(sh); });
     return 0;
 }
