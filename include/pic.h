@@ -248,7 +248,9 @@ pic_status pic_ensemble_create(pic_handle *const *runs, int32_t count, void *str
  * already enqueued on the runs' streams, and later work on a run's stream waits for
  * them, so pic_step, pic_read_particles, pic_get_field... on a run see the result.  A
  * run advanced on its own (pic_step) by a number of steps that is not a multiple of P
- * no longer matches the graph: PIC_ERR_STATE.  Errors: PIC_ERR_INVALID_ARG (NULL,
+ * no longer matches the graph: PIC_ERR_STATE.  Where whole periods advanced on its own, or a
+ * loaded state, left a run's buffers in another rotation, the call captures the graph again
+ * first (it then synchronises the runs and the ensemble's stream).  Errors: PIC_ERR_INVALID_ARG (NULL,
  * nsteps < 0 or not a multiple of P), PIC_ERR_CUDA; text in pic_last_error(NULL).
  * Device-side errors latch in each run and are reported by pic_sync on that run. */
 pic_status pic_ensemble_step(pic_ensemble *e, int32_t nsteps);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <numeric>
 #include <cstdarg>
@@ -1111,9 +1112,12 @@ pic_status gather_push_step(pic_handle* h, bool fuse, bool defer) {
 
 // ------------------------------------------------------------ ensembles ----
 
+using Rotation = std::array<const void*, 45>;
+
 struct pic_ensemble {
     std::vector<pic_handle*> runs;
     std::vector<int64_t> step0;  // each run's step count when the graph was captured
+    std::vector<Rotation> at;    // and where its buffers stood (rotation)
     cudaStream_t s = nullptr;
     int period = 0;
     cudaGraph_t graph = nullptr;
@@ -1144,10 +1148,92 @@ void ensemble_release(pic_ensemble* e) {
     delete e;
 }
 
-pic_status efail(pic_ensemble* e, pic_status st, const char* msg, cudaError_t ce = cudaSuccess) {
-    if (e) ensemble_release(e);
+pic_status efail(pic_status st, const char* msg, cudaError_t ce = cudaSuccess) {
     if (ce != cudaSuccess) return fail(nullptr, st, "%s: %s", msg, cudaGetErrorString(ce));
     return fail(nullptr, st, "%s", msg);
+}
+
+// Everything of a run that its steps rotate: the addresses that a captured step has built in.
+// A whole period returns each of them within one pic_step call; calls that start from a pending
+// deposit (x, y change places with xnext, ynext there) and loaded states may leave others.
+Rotation rotation(const pic_handle* h) {
+    const auto at = [](int k) { return reinterpret_cast<const void*>((intptr_t)k); };
+    return Rotation{h->x,       h->y,       h->xnext,       h->ynext,   h->px,       h->py,
+                    h->v[0][0], h->v[0][1], h->v[1][0],     h->v[1][1], h->J,        h->Jalt,
+                    h->Jz,      h->Jzalt,   h->id,          h->id_alt,  h->species,  h->species_alt,
+                    h->pz,      h->vz[0],   h->vz[1],       h->az,      h->az_prev,  h->jz,
+                    h->jz_prev, h->cdf.phi, h->cdf.rho,     h->cdf.ax,  h->cdf.ay,   h->cdf.jx,
+                    h->cdf.jy,  h->alt[0],  h->alt[1],      h->alt[2],  h->alt[3],   h->alt[4],
+                    h->alt[5],  h->alt[6],  h->alt[7],      h->z_alt[0], h->z_alt[1], h->z_alt[2],
+                    at(h->vcur), at(h->head), at(h->head_r)};
+}
+
+// Captures a period of every run into e's graph (in place of the one it has).
+pic_status ensemble_capture(pic_ensemble* e) {
+    const int32_t count = (int32_t)e->runs.size();
+    cudaError_t ce = cudaSuccess;
+    // nothing of the runs may be pending outside the capture (a pending deposit is redone
+    // by the graph's first step)
+    for (pic_handle* h : e->runs) {
+        if ((ce = drop_pending(h)) != cudaSuccess)
+            return efail(PIC_ERR_CUDA, "clearing a pending deposit failed", ce);
+        if ((ce = cudaStreamSynchronize(h->s)) != cudaSuccess)
+            return efail(PIC_ERR_CUDA, "synchronising a run failed", ce);
+    }
+    if ((ce = cudaStreamSynchronize(e->s)) != cudaSuccess)
+        return efail(PIC_ERR_CUDA, "synchronising the ensemble stream failed", ce);
+    // Capturing runs the step functions on the host: their buffer rotations advance by
+    // the period and so end where they started; the step counts are put back.
+    std::vector<pic_handle> saved;
+    saved.reserve(count);
+    for (pic_handle* h : e->runs) saved.push_back(*h);
+    auto restore = [&] {
+        for (int32_t i = 0; i < count; ++i) *e->runs[i] = saved[i];
+    };
+    ce = cudaStreamBeginCapture(e->s, cudaStreamCaptureModeRelaxed);
+    if (ce != cudaSuccess) return efail(PIC_ERR_CUDA, "cudaStreamBeginCapture failed", ce);
+    pic_status st = PIC_OK;
+    int32_t failed = 0;
+    cudaError_t cap = cudaEventRecord(e->ev, e->s);
+    for (int32_t i = 0; i < count && cap == cudaSuccess && st == PIC_OK; ++i) {
+        pic_handle* h = e->runs[i];
+        failed = i;
+        cap = cudaStreamWaitEvent(h->s, e->ev, 0);  // the run's stream joins the capture
+        h->no_defer = true;  // the captured period ends between two steps
+        if (cap == cudaSuccess) st = pic_step(h, e->period);
+        h->no_defer = false;
+        if (cap == cudaSuccess && st == PIC_OK) cap = cudaEventRecord(e->ev_run[i], h->s);
+        if (cap == cudaSuccess && st == PIC_OK) cap = cudaStreamWaitEvent(e->s, e->ev_run[i], 0);
+    }
+    cudaGraph_t g = nullptr;
+    ce = cudaStreamEndCapture(e->s, &g);
+    std::string why = st != PIC_OK ? "capturing the steps of run " + std::to_string(failed) +
+                                         " failed: " + e->runs[failed]->errmsg
+                                   : "";
+    restore();
+    cudaGraphExec_t exec = nullptr;
+    if (st == PIC_OK && cap == cudaSuccess && ce == cudaSuccess && g) {
+        ce = cudaGraphInstantiate(&exec, g, 0);
+        if (ce != cudaSuccess) why = "cudaGraphInstantiate failed";
+    } else if (st == PIC_OK) {
+        why = cap != cudaSuccess ? "capture failed" : "cudaStreamEndCapture failed";
+        if (cap != cudaSuccess) ce = cap;
+    }
+    if (!exec) {
+        if (g) cudaGraphDestroy(g);
+        return efail(st != PIC_OK ? st : PIC_ERR_CUDA, why.c_str(), st != PIC_OK ? cudaSuccess : ce);
+    }
+    if (e->exec) cudaGraphExecDestroy(e->exec);
+    if (e->graph) cudaGraphDestroy(e->graph);
+    e->graph = g;
+    e->exec = exec;
+    e->step0.clear();
+    e->at.clear();
+    for (const pic_handle* h : e->runs) {
+        e->step0.push_back(h->step);
+        e->at.push_back(rotation(h));
+    }
+    return PIC_OK;
 }
 
 }  // namespace
@@ -1184,55 +1270,15 @@ pic_status pic_ensemble_create(pic_handle* const* runs, int32_t count, void* str
         ce = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
         if (ce == cudaSuccess) e->ev_run.push_back(v);
     }
-    if (ce != cudaSuccess) return efail(e, PIC_ERR_CUDA, "event creation failed", ce);
-    // nothing of the runs may be pending outside the capture (a pending deposit is redone
-    // by the graph's first step)
-    for (pic_handle* h : e->runs) {
-        if ((ce = drop_pending(h)) != cudaSuccess)
-            return efail(e, PIC_ERR_CUDA, "clearing a pending deposit failed", ce);
-        if ((ce = cudaStreamSynchronize(h->s)) != cudaSuccess)
-            return efail(e, PIC_ERR_CUDA, "synchronising a run failed", ce);
+    if (ce != cudaSuccess) {
+        ensemble_release(e);
+        return efail(PIC_ERR_CUDA, "event creation failed", ce);
     }
-    if ((ce = cudaStreamSynchronize(e->s)) != cudaSuccess)
-        return efail(e, PIC_ERR_CUDA, "synchronising the ensemble stream failed", ce);
-    // Capturing runs the step functions on the host: their buffer rotations advance by
-    // the period and so end where they started; the step counts are put back.
-    std::vector<pic_handle> saved;
-    saved.reserve(count);
-    for (pic_handle* h : e->runs) {
-        saved.push_back(*h);
-        e->step0.push_back(h->step);
+    const pic_status st = ensemble_capture(e);
+    if (st != PIC_OK) {
+        ensemble_release(e);
+        return st;
     }
-    auto restore = [&] {
-        for (int32_t i = 0; i < count; ++i) *e->runs[i] = saved[i];
-    };
-    ce = cudaStreamBeginCapture(e->s, cudaStreamCaptureModeRelaxed);
-    if (ce != cudaSuccess) return efail(e, PIC_ERR_CUDA, "cudaStreamBeginCapture failed", ce);
-    pic_status st = PIC_OK;
-    int32_t failed = 0;
-    cudaError_t cap = cudaEventRecord(e->ev, e->s);
-    for (int32_t i = 0; i < count && cap == cudaSuccess && st == PIC_OK; ++i) {
-        pic_handle* h = e->runs[i];
-        failed = i;
-        cap = cudaStreamWaitEvent(h->s, e->ev, 0);  // the run's stream joins the capture
-        h->no_defer = true;  // the captured period ends between two steps
-        if (cap == cudaSuccess) st = pic_step(h, e->period);
-        h->no_defer = false;
-        if (cap == cudaSuccess && st == PIC_OK) cap = cudaEventRecord(e->ev_run[i], h->s);
-        if (cap == cudaSuccess && st == PIC_OK) cap = cudaStreamWaitEvent(e->s, e->ev_run[i], 0);
-    }
-    cudaGraph_t g = nullptr;
-    ce = cudaStreamEndCapture(e->s, &g);
-    e->graph = g;
-    std::string why = st != PIC_OK ? "capturing the steps of run " + std::to_string(failed) +
-                                         " failed: " + e->runs[failed]->errmsg
-                                   : "";
-    restore();
-    if (st != PIC_OK) return efail(e, st, why.c_str());
-    if (cap != cudaSuccess) return efail(e, PIC_ERR_CUDA, "capture failed", cap);
-    if (ce != cudaSuccess || !g) return efail(e, PIC_ERR_CUDA, "cudaStreamEndCapture failed", ce);
-    ce = cudaGraphInstantiate(&e->exec, e->graph, 0);
-    if (ce != cudaSuccess) return efail(e, PIC_ERR_CUDA, "cudaGraphInstantiate failed", ce);
     *out = e;
     return PIC_OK;
 }
@@ -1253,6 +1299,12 @@ pic_status pic_ensemble_step(pic_ensemble* e, int32_t nsteps) {
                         "multiple of %d)", (int)i, e->period);
     }
     if (nsteps == 0) return PIC_OK;
+    bool moved = false;
+    for (size_t i = 0; i < n; ++i) moved |= rotation(e->runs[i]) != e->at[i];
+    if (moved) {  // the graph's addresses are not the runs' any more
+        const pic_status st = ensemble_capture(e);
+        if (st != PIC_OK) return st;
+    }
     cudaError_t ce = cudaSuccess;
     // a run stepped alone since may hold a pending deposit: the graph redoes it
     for (size_t i = 0; i < n && ce == cudaSuccess; ++i) ce = drop_pending(e->runs[i]);
