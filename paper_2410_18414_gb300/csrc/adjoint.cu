@@ -390,7 +390,7 @@ k_adj_push_gather(ParticleGeom g, PushParams pp, const double* __restrict__ x1,
 // dW_x.  The FP64 pipe is left with the push's adjoint and the products the atomics add
 // (about 250 operations a particle instead of 600).  262,144 particles, 128 x 128, cubic: with
 // FP64 gathers and a lane per particle 263 us, now 137 us.  Bound by the FP64 pipe (72%) and its
-// latency: five CTAs an SM (96 registers, 24 bytes spilled) instead of four, 148 -> 137 us; six
+// latency: five CTAs an SM (96 registers, 32 bytes spilled) instead of four, 148 -> 137 us; six
 // are slower.  The lean form gains nothing at five (144.5 -> 146 us) and quartic shapes spill:
 // they keep the four and three that their registers allow.
 template <int P, bool kLean>
@@ -400,7 +400,7 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
                       const double* __restrict__ py1, const double* __restrict__ vx,
                       const double* __restrict__ vy, const double* __restrict__ vxo,
                       const double* __restrict__ vyo, const double* __restrict__ gfa,
-                      const int4* __restrict__ F, const unsigned* __restrict__ top,
+                      const int4* __restrict__ F, const int* __restrict__ ex,
                       AdjParticles ab, double* __restrict__ Fb, int64_t n,
                       unsigned int* __restrict__ err) {
     constexpr int S1 = P + 1, S2 = S1 * S1, kOut = kLean ? 24 : 16;
@@ -452,47 +452,46 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
             int gi = (kb >> 16) + a;
             if (gi >= g.nx) gi -= g.nx;
             row[a] = gi;
-            const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + 4 * gi + q);
-            e0[a] = row_exponent(u.x);
-            e1[a] = row_exponent(u.y);
+            const int2 u = __ldg(reinterpret_cast<const int2*>(ex) + 4 * gi + q);
+            e0[a] = u.x;
+            e1[a] = u.y;
             top0 = max(top0, e0[a]);
             top1 = max(top1, e1[a]);
         }
-        long long hx[2] = {0, 0}, mx[2] = {0, 0}, hy[2] = {0, 0}, my[2] = {0, 0};
-        long long hw[2] = {0, 0}, mw[2] = {0, 0};
+        LimbSum sx[2], sy[2], sw[2];
 #pragma unroll
         for (int a = 0; a < S1; ++a) {
             const int4* F0 = F + (size_t)row[a] * g.ny * 4 + q;
-            long long hr[2] = {0, 0}, mr[2] = {0, 0}, hs[2] = {0, 0}, ms[2] = {0, 0};
+            LimbSum rr[2], rs[2];  // along the row with W_y, dW_y
 #pragma unroll
             for (int b = 0; b < S1; ++b) {
                 int gj = (kb & 0xFFFF) + b;
                 if (gj >= g.ny) gj -= g.ny;
                 const int4 v = __ldg(F0 + 4 * gj);
                 const int2 wy = lim[2 * S1 + b], dy = lim[3 * S1 + b];
-                mac58(hr[0], mr[0], wy, v.x, v.y);
-                mac58(hr[1], mr[1], wy, v.z, v.w);
-                mac58(hs[0], ms[0], dy, v.x, v.y);
-                mac58(hs[1], ms[1], dy, v.z, v.w);
+                rr[0].add(wy, v.x, v.y);
+                rr[1].add(wy, v.z, v.w);
+                rs[0].add(dy, v.x, v.y);
+                rs[1].add(dy, v.z, v.w);
             }
             const int2 wx = lim[a], dx = lim[S1 + a];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int d = c ? top1 - e1[a] : top0 - e0[a];
-                const int2 r = limbs58(shift_down(sum58(hr[c], mr[c]), d));
-                const int2 s = limbs58(shift_down(sum58(hs[c], ms[c]), d));
-                mac58(hx[c], mx[c], dx, r.x, r.y);
-                mac58(hy[c], my[c], wx, s.x, s.y);
-                if (kLean) mac58(hw[c], mw[c], wx, r.x, r.y);
+                const int2 r = limbs(rr[c].shifted(d));
+                const int2 s = limbs(rs[c].shifted(d));
+                sx[c].add(dx, r.x, r.y);
+                sy[c].add(wx, s.x, s.y);
+                if (kLean) sw[c].add(wx, r.x, r.y);
             }
         }
         double* out = rec + k * kStride + 4 * S1 + 2 * q;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const int e = c ? top1 : top0;
-            out[c] = fix_value(sum58(hx[c], mx[c]), e);
-            out[8 + c] = fix_value(sum58(hy[c], my[c]), e);
-            if (kLean) out[16 + c] = fix_value(sum58(hw[c], mw[c]), e);
+            out[c] = fix_value(sx[c].value(), e);
+            out[8 + c] = fix_value(sy[c].value(), e);
+            if (kLean) out[16 + c] = fix_value(sw[c].value(), e);
         }
     }
     __syncwarp();
@@ -511,16 +510,16 @@ k_adj_push_gather_fix(ParticleGeom g, FixGeom fg, PushParams pp, const double* _
         ab.x[p] += g.inv_dx * xg;
         ab.y[p] += g.inv_dy * yg;
         // the record now holds the products W_x W_y and gb
-        // (w 2^-62 = w 2^(-4 - 58))
+        // (w 2^-62 = w 2^(-2 - 60))
         long long w[S1];
         double wy[S1];
         fix_weights<P>(Y, fg.sh, w);
 #pragma unroll
-        for (int b = 0; b < S1; ++b) wy[b] = fix_value(w[b], -4);
+        for (int b = 0; b < S1; ++b) wy[b] = fix_value(w[b], -2);
         fix_weights<P>(X, fg.sh, w);
 #pragma unroll
         for (int a = 0; a < S1; ++a) {
-            const double wx = fix_value(w[a], -4);
+            const double wx = fix_value(w[a], -2);
 #pragma unroll
             for (int b = 0; b < S1; ++b) mine[a * S1 + b] = wx * wy[b];
         }
@@ -593,7 +592,7 @@ __global__ void __launch_bounds__(kAdjThreads, P > 3 ? 2 : 4)
 k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1,
                        const double* __restrict__ y1, const double* __restrict__ vx,
                        const double* __restrict__ vy, const int4* __restrict__ Jb,
-                       const unsigned* __restrict__ top, AdjParticles ab, int64_t n,
+                       const int* __restrict__ ex, AdjParticles ab, int64_t n,
                        unsigned int* __restrict__ err) {
     constexpr int S1 = P + 1;
     const int64_t p = blockIdx.x * (int64_t)kAdjThreads + threadIdx.x;
@@ -621,48 +620,47 @@ k_adj_deposit_move_fix(ParticleGeom g, FixGeom fg, const double* __restrict__ x1
     for (int a = 0; a < S1; ++a) {
         int gi = ix + a;
         if (gi >= g.nx) gi -= g.nx;
-        const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + gi);
-        e[0][a] = row_exponent(u.x);
-        e[1][a] = row_exponent(u.y);
+        const int2 u = __ldg(reinterpret_cast<const int2*>(ex) + gi);
+        e[0][a] = u.x;
+        e[1][a] = u.y;
         tops[0] = max(tops[0], e[0][a]);
         tops[1] = max(tops[1], e[1][a]);
     }
     // per component: the value, d/dx and d/dy of the gathered current adjoint
-    long long hw[2] = {0, 0}, mw[2] = {0, 0}, hx[2] = {0, 0}, mx[2] = {0, 0};
-    long long hy[2] = {0, 0}, my[2] = {0, 0};
+    LimbSum sw[2], sx[2], sy[2];
 #pragma unroll
     for (int a = 0; a < S1; ++a) {
         int gi = ix + a;
         if (gi >= g.nx) gi -= g.nx;
         const int4* row = Jb + (size_t)gi * g.ny;
-        long long hr[2] = {0, 0}, mr[2] = {0, 0}, hs[2] = {0, 0}, ms[2] = {0, 0};
+        LimbSum rr[2], rs[2];
 #pragma unroll
         for (int b = 0; b < S1; ++b) {
             int gj = iy + b;
             if (gj >= g.ny) gj -= g.ny;
             const int4 v = __ldg(row + gj);
-            mac58(hr[0], mr[0], wy[b], v.x, v.y);
-            mac58(hr[1], mr[1], wy[b], v.z, v.w);
-            mac58(hs[0], ms[0], dy[b], v.x, v.y);
-            mac58(hs[1], ms[1], dy[b], v.z, v.w);
+            rr[0].add(wy[b], v.x, v.y);
+            rr[1].add(wy[b], v.z, v.w);
+            rs[0].add(dy[b], v.x, v.y);
+            rs[1].add(dy[b], v.z, v.w);
         }
         const int2 wa = weight_limbs(wx[a]), da = weight_limbs(dx[a]);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const int d = tops[c] - e[c][a];
-            const int2 r = limbs58(shift_down(sum58(hr[c], mr[c]), d));
-            const int2 s = limbs58(shift_down(sum58(hs[c], ms[c]), d));
-            mac58(hw[c], mw[c], wa, r.x, r.y);
-            mac58(hx[c], mx[c], da, r.x, r.y);
-            mac58(hy[c], my[c], wa, s.x, s.y);
+            const int2 r = limbs(rr[c].shifted(d));
+            const int2 s = limbs(rs[c].shifted(d));
+            sw[c].add(wa, r.x, r.y);
+            sx[c].add(da, r.x, r.y);
+            sy[c].add(wa, s.x, s.y);
         }
     }
     double w[2], jx[2], jy[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        w[c] = fix_value(sum58(hw[c], mw[c]), tops[c]);
-        jx[c] = fix_value(sum58(hx[c], mx[c]), tops[c]);
-        jy[c] = fix_value(sum58(hy[c], my[c]), tops[c]);
+        w[c] = fix_value(sw[c].value(), tops[c]);
+        jx[c] = fix_value(sx[c].value(), tops[c]);
+        jy[c] = fix_value(sy[c].value(), tops[c]);
     }
     const double vxp = vx[p], vyp = vy[p];
     const double xb = ab.x[p] + g.inv_dx * (vxp * jx[0] + vyp * jx[1]);
@@ -1043,7 +1041,7 @@ cudaError_t launch_adj_push_gather(int p, const ParticleGeom& g, const PushParam
 #define GPIC_ADJ_FIX(PP, LEAN)                                                                 \
     launch_pdl(k_adj_push_gather_fix<PP, LEAN>, grid, block, 0, s, g, fix_geom(g), pp, x1, y1, \
                px1, py1, vx, vy, vxo, vyo, gfa, (const int4*)fix->f,                           \
-               (const unsigned*)fix->top, ab, Fb, n, err)
+               (const int*)fix->exp, ab, Fb, n, err)
             switch (2 * p + (lean ? 1 : 0)) {
                 case 4: return GPIC_ADJ_FIX(2, false);
                 case 5: return GPIC_ADJ_FIX(2, true);
@@ -1087,7 +1085,7 @@ cudaError_t launch_adj_deposit_move(int p, const ParticleGeom& g, const T* x1, c
         if (fix) {
 #define GPIC_ADJ_MOVE(PP)                                                                       \
     launch_pdl(k_adj_deposit_move_fix<PP>, dim3(adj_blocks(n)), dim3(kAdjThreads), 0, s, g,     \
-               fix_geom(g), x1, y1, vx, vy, (const int4*)fix->f, (const unsigned*)fix->top, ab, \
+               fix_geom(g), x1, y1, vx, vy, (const int4*)fix->f, (const int*)fix->exp, ab, \
                n, err)
             switch (p) {
                 case 2: return GPIC_ADJ_MOVE(2);

@@ -181,7 +181,7 @@ size_t rec_width(const pic_adjoint* a) { return a->lean ? 4 : 10; }
 // Bytes of one step's gather fields in the records: [node][4] complex of T, or the handle's
 // fixed-point fields with their row maxima (one allocation, see FixFields).
 size_t rec_field_bytes(const pic_adjoint* a) {
-    return 4 * a->ng * 2 * a->rsz + (a->fix ? (size_t)a->h->nx * 8 * sizeof(unsigned) : 0);
+    return 4 * a->ng * 2 * a->rsz + (a->fix ? (size_t)a->h->nx * 8 * sizeof(int) : 0);
 }
 
 int seg_begin(const pic_adjoint* a, int c) { return c * a->K; }
@@ -243,7 +243,7 @@ pic_status backward_step(pic_adjoint* a, int64_t n, const void* s0v, const void*
         using T = decltype(t);
         const T* s0 = (const T*)s0v;
         const T* s1 = (const T*)s1v;
-        const FixFields fx{(void*)g, (unsigned*)((char*)g + 4 * ng * sizeof(int4))};
+        const FixFields fx{(void*)g, (int*)((char*)g + 4 * ng * sizeof(int4))};
         return launch_adj_push_gather<T>(h->p, h->geom, h->push, s1, s1 + np, s1 + 2 * np,
                                          s1 + 3 * np, s0 + 4 * np, s0 + 5 * np, s0 + 6 * np,
                                          s0 + 7 * np, gf, a->lean, g, a->fix ? &fx : nullptr,
@@ -368,7 +368,7 @@ pic_status pic_adjoint_create_ex(pic_handle* h, int32_t nsteps, int32_t checkpoi
         take(&a->ab, sb);
         if (a->fix) {
             take(&a->jfix.f, a->ng * sizeof(int4));
-            take(&a->jfix.top, (size_t)h->nx * 2 * sizeof(unsigned));
+            take(&a->jfix.exp, (size_t)h->nx * 2 * sizeof(int));
         }
         take(&a->twx, (size_t)h->nx * sizeof(double2));
         take(&a->twy, (size_t)h->ny * sizeof(double2));

@@ -53,7 +53,7 @@ struct FftSecond {
     const longlong2* fix_in;
     longlong2* clear;
     int4* ffix;
-    unsigned* ftop;
+    int* fexp;
 };
 
 // Transforms along y (contiguous): CTA = `rows` consecutive x-indices of all nb arrays.
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads)
 k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, int ny, int nb,
         int rows, FftDesc d, const cplx_t<T>* __restrict__ tw, int sign, int interleave,
         const longlong2* __restrict__ fix_in, double unscale, longlong2* __restrict__ clear,
-        int4* __restrict__ ffix, unsigned* __restrict__ ftop, void* __restrict__ sums, int sums32, FftSecond<T> two) {
+        int4* __restrict__ ffix, int* __restrict__ fexp, void* __restrict__ sums, int sums32, FftSecond<T> two) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* b0 = reinterpret_cast<C*>(smem_raw);
@@ -73,7 +73,7 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
         fix_in = two.fix_in;
         clear = two.clear;
         ffix = two.ffix;
-        ftop = two.ftop;
+        fexp = two.fexp;
     }
     const int lines = nb * rows;
     C* b1 = b0 + lines * ny;
@@ -130,7 +130,7 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
             if (ffix) {  // one row, nb = 4 or 2: its fixed-point fields beside the FP64 ones
                 collect_max(res, nb, ny, top);
                 __syncthreads();
-                if (threadIdx.x < 2 * nb) ftop[2 * nb * i0 + threadIdx.x] = top[threadIdx.x];
+                if (threadIdx.x < 2 * nb) fexp[2 * nb * i0 + threadIdx.x] = row_exponent(top[threadIdx.x]);
                 const int b = threadIdx.x & (nb - 1);
                 const int er = row_exponent(top[2 * b]), ei = row_exponent(top[2 * b + 1]);
                 for (int e = threadIdx.x; e < nb * ny; e += blockDim.x) {
@@ -153,7 +153,7 @@ k_fft_y(const cplx_t<T>* __restrict__ in, cplx_t<T>* __restrict__ out, int nx, i
             if (ffix) {  // nb = 1: the fixed-point values of the one or two rows as well
                 collect_max(res, rows, ny, top);
                 __syncthreads();
-                if (threadIdx.x < 2 * rows) ftop[2 * i0 + threadIdx.x] = top[threadIdx.x];
+                if (threadIdx.x < 2 * rows) fexp[2 * i0 + threadIdx.x] = row_exponent(top[threadIdx.x]);
             }
         }
         for (int e = threadIdx.x; e < lines * ny; e += blockDim.x) {
@@ -235,7 +235,7 @@ static cudaError_t fft_y_impl(const void* in, void* out, int nx, int ny, int nb,
     return launch_pdl(k_fft_y<T>, dim3(nx / rows, two ? 2 : 1), dim3(kThreads), smem, s,
                       (const C*)in, (C*)out,
                       nx, ny, nb, rows, d, (const C*)tw, sign, interleave, fix_in, unscale, clear,
-                      fix ? (int4*)fix->f : nullptr, fix ? fix->top : nullptr, sums,
+                      fix ? (int4*)fix->f : nullptr, fix ? fix->exp : nullptr, sums,
                       sums32 ? 1 : 0, two ? *two : FftSecond<T>{});
 }
 
@@ -271,7 +271,7 @@ cudaError_t launch_fft_y_fields(const void* f4, void* g, const void* f2, void* g
                                 const FixFields* fix2, cudaStream_t s) {
     if ((fix || fix2) && sizeof(T) != 8) return cudaErrorInvalidValue;
     const FftSecond<T> two{(const cplx_t<T>*)f2, (cplx_t<T>*)g2, 2, nullptr, nullptr,
-                           fix2 ? (int4*)fix2->f : nullptr, fix2 ? fix2->top : nullptr};
+                           fix2 ? (int4*)fix2->f : nullptr, fix2 ? fix2->exp : nullptr};
     return fft_y_impl<T>(f4, g, nx, ny, 4, d, tw, +1, 1, nullptr, 0.0, nullptr, s, fix, nullptr,
                          false, f2 ? &two : nullptr);
 }

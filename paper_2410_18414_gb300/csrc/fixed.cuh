@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "gpic_internal.h"
 
@@ -31,15 +33,16 @@ __device__ __forceinline__ int row_exponent(unsigned top) {
     return top >= 0x7ff00000u ? 2048 : max((int)(top >> 20) - 1022, -900);
 }
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-// v in [-2^58, 2^58] as (v.x 2^29 + v.y), |v.y| <= 2^28
-__device__ __forceinline__ int2 limbs58(long long v) {
-    const int lo = (int)((unsigned)v << 3) >> 3;
-    return make_int2((int)((v - lo) >> 29), lo);
+// v in [-2^61, 2^61] as (v.x 2^31 + v.y), |v.y| <= 2^30
+__device__ __forceinline__ int2 limbs(long long v) {
+    const int lo = (int)((unsigned)v << 1) >> 1;
+    return make_int2((int)((v - lo) >> 31), lo);
 }
-// f 2^(58 - e), rounded
+// f 2^(60 - e), rounded: a value keeps its 53 bits down to 2^-7 of its row's bound 2^e, and below
+// that the rounding is 2^-61 of the bound
 __device__ __forceinline__ int2 field_fix(double f, int e) {
     if (e > 1024) return make_int2(0, 0);
-    return limbs58(__double2ll_rn(rmul(f, pow2(58 - e))));
+    return limbs(__double2ll_rn(rmul(f, pow2(60 - e))));
 }
 
 // FP64 shapes in fixed point: positions X = x/dx 2^sh (one FP64 multiply and conversion),
@@ -144,24 +147,35 @@ __device__ __forceinline__ long long deposit_col(long long w) { return w | 1; }
 __device__ __forceinline__ long long deposit_value(long long t, long long w) {
     return (__mul64hi(t, w) + 1) >> 1;
 }
-// a weight in units of 2^-62 as limbs in units of 2^-58
-__device__ __forceinline__ int2 weight_limbs(long long w) { return limbs58((w + 8) >> 4); }
+// a weight (or derivative) in units of 2^-62 as limbs in units of 2^-61
+__device__ __forceinline__ int2 weight_limbs(long long w) { return limbs((w + 1) >> 1); }
 
-// One term of a sum of products of limbs: (h 2^58 + m 2^29) += w f, the product of the low
-// limbs dropped.
-__device__ __forceinline__ void mac58(long long& h, long long& m, int2 w, int fh, int fl) {
-    h += (long long)w.x * fh;
-    m += (long long)w.x * fl;
-    m += (long long)w.y * fh;
-}
-// the sum in units of 2^-58 of its factors' units' product
-__device__ __forceinline__ long long sum58(long long h, long long m) {
-    return h + ((m + (1ll << 28)) >> 29);
-}
+// A sum of products of limbs in units of f: 2 h + m 2^-30, the product of the low limbs (at most
+// half a unit a term) dropped.  Bounds for the two passes of a gather, with sum |w| <= 1 or, for
+// derivatives, 2 (quadratic shapes) and |f| <= 2^60 or, derivatives gathered along the row, 2^61,
+// never both doubled: |h| <= 2^60, |m| <= 1.5 2^62.
+struct LimbSum {
+    long long h = 0, m = 0;
+    __device__ __forceinline__ void add(int2 w, int fh, int fl) {
+        h += (long long)w.x * fh;
+        m += (long long)w.x * fl;
+        m += (long long)w.y * fh;
+    }
+    // rounded to nearest
+    __device__ __forceinline__ long long value() const { return 2 * h + ((m + (1ll << 29)) >> 30); }
+    // divided by 2^d, d >= 0, rounded to nearest: floor((floor(2 sum / 2^d) + 1) / 2)
+    __device__ __forceinline__ long long shifted(int d) const {
+        long long t = 4 * h + (m >> 29);
+#ifdef __CUDA_ARCH__
+        asm("shr.s64 %0, %0, %1;" : "+l"(t) : "r"(d));  // amounts above 63 leave the sign
+#else
+        t >>= std::min(d, 63);
+#endif
+        return (t + 1) >> 1;
+    }
+};
 
-// v / 2^d rounded down, d >= 0
-__device__ __forceinline__ long long shift_down(long long v, int d) { return v >> min(d, 63); }
-// v 2^(e - 58) rounded to nearest even, by integer operations (an int64 conversion and a
+// v 2^(e - 60) rounded to nearest even, by integer operations (an int64 conversion and a
 // multiplication would be two of the FP64 pipe's); NaN for the exponent of a row that is not
 // finite.
 __device__ __forceinline__ double fix_value(long long v, int e) {
@@ -172,7 +186,7 @@ __device__ __forceinline__ double fix_value(long long v, int e) {
     const unsigned r = (unsigned)m & 0x7ffu;
     q += r + ((unsigned)q & 1u) > 0x400u ? 1u : 0u;
     // q's leading bit adds 1 to the exponent field (2 when the rounding carried into it)
-    const int field = 1027 + e - lz;
+    const int field = 1025 + e - lz;
     q += (unsigned long long)field << 52;
     if (v < 0) q |= 0x8000000000000000ull;
     if (v == 0) q = 0;

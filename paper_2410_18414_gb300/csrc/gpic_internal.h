@@ -113,10 +113,10 @@ enum StepperKind { K_BDF = 0, K_CDF2 = 1, K_DIRK = 2 };
 
 // In-place or out-of-place 1-D transforms of nb arrays of shape (nx, ny).
 // The FP64 path's gather fields in fixed point: per node four int4 (the limbs of two fields
-// each), and per mesh row the high words of the eight fields' largest magnitudes.
+// each), and per mesh row the eight fields' exponents (row_exponent).
 struct FixFields {
     void* f;
-    unsigned* top;
+    int* exp;
 };
 // Along y (contiguous); out_interleave != 0 writes out[(i*ny + j)*nb + b].  fix (FP64,
 // interleaved with nb = 4, or nb = 1; may be NULL): the outputs in fixed point as well (nb = 1:

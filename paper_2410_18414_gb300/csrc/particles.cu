@@ -751,24 +751,27 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
 // FP64: the fields and the weights in fixed point.  GB300 issues 2 FP64 operations per clock
 // and SM, so the 128 FP64 multiply-adds of a cubic gather (and the weights) held the pipe for
 // 0.39 ms per 2^20 particles; 32x32+64-bit integer multiply-adds issue at 32 (28 measured).
-//   - A field f of a mesh row with |f| < 2^e on the row becomes F = rint(f 2^(58-e)), kept as
-//     fh 2^29 + fl, |fl| <= 2^28 (written by the row's inverse transform, with the row's eight
-//     exponents); a weight W = rint(w 2^58) = wh 2^29 + wl alike.
-//   - Along a row sum W F = (sum wh fh) 2^58 + (sum wh fl + wl fh) 2^29 + sum wl fl: three
+//   - A field f of a mesh row with |f| < 2^e on the row becomes F = rint(f 2^(60-e)), kept as
+//     fh 2^31 + fl, |fl| <= 2^30 (written by the row's inverse transform, with the row's eight
+//     exponents); a weight W = rint(w 2^61) = wh 2^31 + wl alike.
+//   - Along a row sum W F = (sum wh fh) 2^62 + (sum wh fl + wl fh) 2^31 + sum wl fl: three
 //     multiply-adds a node and field; the rows' sums are shifted to the largest exponent of
-//     the particle's rows and added.  The sums are exact: the weights add up to 1, so |sum wh fh| <= 2^58,
-//     and |sum wl fh| <= 25 2^28 2^29 < 2^62.  The last sum is below 25 2^56 of 2^116 and is
-//     dropped.
-//   - The roundings (2^-59 of the rows' bound in F, as much in W, the dropped sum 2^-55 at
-//     the very most, 2^-58 typically) are finer than the 2^-53 that FP64 rounds each of its
-//     products and sums to, and than the transform's own error in f, 2^-53 of the largest
-//     value.
+//     the particle's rows, rounded to nearest, and added.  The last sum is dropped.
+//   - So where a field is far below its row's largest value it has fewer than FP64's 53 bits, and
+//     so have the weights below 2^-8: the error is absolute, about 2^-61 of the rows' bound.
+//     FP64 rounds each product at 2^-53 of itself, which is more wherever the stencil's own
+//     values reach 2^-8 of the bound; where they do not, the field's own error is larger than
+//     both, 2^-53 of the row's rms from the transform alone, at least 2^-58 of its peak on a row
+//     of 1024.  Gathers of a cubic shape, error of the value with the transform's included, FP64
+//     / fixed point in units of the transform's: smooth fields 1.24-1.70 / 1.05-1.17, noise
+//     1.15-1.27 / 1.02-1.03, rows of a single peak 1.000 / 0.98-1.01 (32^2 to 1024^2; in units
+//     of 2^-58 with the rows rounded down the last was 1.04-1.08, and one-sided).
 // Integer sums do not depend on their order, and the same bits come out on every path.
 // Fields 2q and 2q+1 of the `per` int4 a node at one particle (kb: its first node, w: its
 // weights' limbs).
 template <int P>
 __device__ __forceinline__ double2 gather_fix_pair(int nx, int ny, const int4* __restrict__ F,
-                                                   const unsigned* __restrict__ top, int per,
+                                                   const int* __restrict__ ex, int per,
                                                    int q, int kb, const int2* w) {
     constexpr int S1 = P + 1;
     int col[S1], row[S1], e0[S1], e1[S1], top0 = -900, top1 = -900;
@@ -779,9 +782,9 @@ __device__ __forceinline__ double2 gather_fix_pair(int nx, int ny, const int4* _
         if (gi >= nx) gi -= nx;
         col[a] = per * gj + q;
         row[a] = gi;
-        const uint2 u = __ldg(reinterpret_cast<const uint2*>(top) + per * gi + q);
-        e0[a] = row_exponent(u.x);
-        e1[a] = row_exponent(u.y);
+        const int2 u = __ldg(reinterpret_cast<const int2*>(ex) + per * gi + q);
+        e0[a] = u.x;
+        e1[a] = u.y;
         top0 = max(top0, e0[a]);
         top1 = max(top1, e1[a]);
     }
@@ -789,16 +792,16 @@ __device__ __forceinline__ double2 gather_fix_pair(int nx, int ny, const int4* _
 #pragma unroll
     for (int a = 0; a < S1; ++a) {
         const int4* F0 = F + (size_t)row[a] * ny * per;
-        long long h0 = 0, m0 = 0, h1 = 0, m1 = 0;
+        LimbSum r0, r1;
 #pragma unroll
         for (int b = 0; b < S1; ++b) {
             const int4 v = __ldg(F0 + col[b]);
             const int2 wab = w[a * S1 + b];
-            mac58(h0, m0, wab, v.x, v.y);
-            mac58(h1, m1, wab, v.z, v.w);
+            r0.add(wab, v.x, v.y);
+            r1.add(wab, v.z, v.w);
         }
-        s0 += shift_down(sum58(h0, m0), top0 - e0[a]);
-        s1 += shift_down(sum58(h1, m1), top1 - e1[a]);
+        s0 += r0.shifted(top0 - e0[a]);
+        s1 += r1.shifted(top1 - e1[a]);
     }
     return make_double2(fix_value(s0, top0), fix_value(s1, top1));
 }
@@ -827,7 +830,7 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
                   double* __restrict__ py, const double* __restrict__ vx,
                   const double* __restrict__ vy, double* __restrict__ vxo,
                   double* __restrict__ vyo, int64_t n, const int4* __restrict__ F,
-                  const unsigned* __restrict__ top, double* __restrict__ gout, int gout_short,
+                  const int* __restrict__ ex, double* __restrict__ gout, int gout_short,
                   double* __restrict__ diag, unsigned int* __restrict__ err) {
     constexpr int S2 = (P + 1) * (P + 1);
     constexpr int kStride = S2 | 1;  // at least the 8 gathered values
@@ -852,7 +855,7 @@ k_gather_push_fix(GeomT<double> g, FixGeom fg, PushT<double> pp, const double* _
         const int k = w0 + 8 * t + (lane >> 2), q = lane & 3;
         const int kb = rbase[k];
         double2 f = make_double2(0.0, 0.0);
-        if (kb >= 0) f = gather_fix_pair<P>(g.nx, g.ny, F, top, 4, q, kb, rec + k * kStride);
+        if (kb >= 0) f = gather_fix_pair<P>(g.nx, g.ny, F, ex, 4, q, kb, rec + k * kStride);
         __syncwarp();  // the four lanes have read the particle's weights
         double* out = reinterpret_cast<double*>(rec + k * kStride);
         out[2 * q] = f.x;
@@ -1759,8 +1762,8 @@ k_gather_push3_fix(GeomT<double> g, FixGeom fg, PushParams pp, const double* __r
                    const double* __restrict__ vz, double* __restrict__ vxo,
                    double* __restrict__ vyo, double* __restrict__ vzo,
                    const int32_t* __restrict__ sp, SpeciesParams spp, int64_t n,
-                   const int4* __restrict__ F, const unsigned* __restrict__ top,
-                   const int4* __restrict__ Fz, const unsigned* __restrict__ topz,
+                   const int4* __restrict__ F, const int* __restrict__ ex,
+                   const int4* __restrict__ Fz, const int* __restrict__ exz,
                    double* __restrict__ diag, unsigned int* __restrict__ err) {
     constexpr int S2 = (P + 1) * (P + 1);
     constexpr int kStride = (S2 > 12 ? S2 : 12) | 1;  // the weights, then the gathered values
@@ -1788,8 +1791,8 @@ k_gather_push3_fix(GeomT<double> g, FixGeom fg, PushParams pp, const double* __r
         const int kb = rbase[k];
         double2 f = make_double2(0.0, 0.0), fz = f;
         if (kb >= 0) {
-            f = gather_fix_pair<P>(g.nx, g.ny, F, top, 4, q, kb, rec + k * kStride);
-            if (Z3 && q < 2) fz = gather_fix_pair<P>(g.nx, g.ny, Fz, topz, 2, q, kb, rec + k * kStride);
+            f = gather_fix_pair<P>(g.nx, g.ny, F, ex, 4, q, kb, rec + k * kStride);
+            if (Z3 && q < 2) fz = gather_fix_pair<P>(g.nx, g.ny, Fz, exz, 2, q, kb, rec + k * kStride);
         }
         __syncwarp();  // the four lanes have read the particle's weights
         double* out = reinterpret_cast<double*>(rec + k * kStride);
@@ -2019,8 +2022,8 @@ cudaError_t launch_gather_push3(int p, const ParticleGeom& g, const PushParams& 
 #define GPIC_GFIX3(PP, ZZ)                                                                     \
     launch_pdl(k_gather_push3_fix<PP, ZZ>, dim3(blocks), dim3(kRowGatherThreads), 0, s,        \
                typed<T>(g), fix_geom(g), pp, x, y, px, py, pz, vx, vy, vz, vx_old, vy_old,     \
-               vz_old, spi, spp, n, (const int4*)fix->f, (const unsigned*)fix->top,            \
-               (const int4*)z.f, (const unsigned*)z.top, diag, err)
+               vz_old, spi, spp, n, (const int4*)fix->f, (const int*)fix->exp,            \
+               (const int4*)z.f, (const int*)z.exp, diag, err)
             switch (2 * p + (z3 ? 1 : 0)) {
                 case 4: return GPIC_GFIX3(2, false);
                 case 5: return GPIC_GFIX3(2, true);
@@ -2117,7 +2120,7 @@ cudaError_t launch_gather_push(int p, const ParticleGeom& g, const PushParams& p
 #define GPIC_GFIX(PP)                                                                        \
     launch_pdl(k_gather_push_fix<PP>, dim3(blocks), dim3(kRowGatherThreads), 0, s, typed<T>(g), \
                fix_geom(g), typed<T>(pp), x, y, px, py, vx, vy, vxo, vyo, n,                 \
-               (const int4*)fix->f, (const unsigned*)fix->top, gout, gout_short ? 1 : 0, diag, err)
+               (const int4*)fix->f, (const int*)fix->exp, gout, gout_short ? 1 : 0, diag, err)
     switch (p) {
         case 2: return GPIC_GFIX(2);
         case 3: return GPIC_GFIX(3);

@@ -354,8 +354,8 @@ void layout_state(pic_handle* h) {
     if (!h->fp32 && h->n >= (int64_t)(h->ng / 8)) {
         auto fix = [&](FixFields& f, int per) {  // the maxima follow the fields
             const size_t fb = per * h->ng * sizeof(int4);
-            take(&f.f, fb + (size_t)c.nx * 2 * per * sizeof(unsigned));
-            f.top = (unsigned*)((char*)f.f + fb);
+            take(&f.f, fb + (size_t)c.nx * 2 * per * sizeof(int));
+            f.exp = (int*)((char*)f.f + fb);
         };
         fix(h->fixf, 4);
         if (h->vdim == 3) fix(h->fixz, 2);

@@ -92,6 +92,61 @@ void deposit(int sh) {
     }
 }
 
+// gather P SH: (nx, ny, n, the field [nx][ny], x and y of n particles in cells) -> per particle
+// the value gathered as k_gather_push_fix does, then value, d/dx and d/dy by the separable sums
+// of the reverse kernels (the bits of four doubles)
+template <int P>
+void gather(int sh) {
+    constexpr int S1 = P + 1;
+    const std::vector<double> in = read_all<double>();
+    const int nx = (int)in[0], ny = (int)in[1], n = (int)in[2];
+    const double *f = &in[3], *xs = f + (size_t)nx * ny, *ys = xs + n;
+    std::vector<int2> F((size_t)nx * ny);
+    std::vector<int> e(nx);
+    for (int i = 0; i < nx; ++i) {
+        unsigned top = 0;
+        for (int j = 0; j < ny; ++j) {
+            unsigned long long bits;
+            std::memcpy(&bits, f + (size_t)i * ny + j, sizeof bits);
+            top = max(top, (unsigned)(bits >> 32) & 0x7fffffffu);
+        }
+        e[i] = row_exponent(top);
+        for (int j = 0; j < ny; ++j) F[(size_t)i * ny + j] = field_fix(f[(size_t)i * ny + j], e[i]);
+    }
+    const double scale = std::ldexp(1.0, sh);
+    for (int p = 0; p < n; ++p) {
+        const long long X = __double2ll_rn(xs[p] * scale), Y = __double2ll_rn(ys[p] * scale);
+        long long wx[S1], wy[S1], dx[S1], dy[S1];
+        const int ix = fix_weights<P>(X, sh, wx), iy = fix_weights<P>(Y, sh, wy);
+        fix_dweights<P>(X, sh, dx);
+        fix_dweights<P>(Y, sh, dy);
+        int top = -900;
+        for (int a = 0; a < S1; ++a) top = max(top, e[(ix + a + nx) % nx]);
+        long long s0 = 0;
+        LimbSum sum[3];
+        for (int a = 0; a < S1; ++a) {
+            const int gi = (ix + a + nx) % nx;
+            LimbSum r0, rr, rs;
+            for (int b = 0; b < S1; ++b) {
+                const int2 v = F[(size_t)gi * ny + (iy + b + ny) % ny];
+                r0.add(weight_limbs(mul62(wx[a], wy[b])), v.x, v.y);
+                rr.add(weight_limbs(wy[b]), v.x, v.y);
+                rs.add(weight_limbs(dy[b]), v.x, v.y);
+            }
+            const int d = top - e[gi];
+            s0 += r0.shifted(d);
+            const int2 r = limbs(rr.shifted(d));
+            const int2 s = limbs(rs.shifted(d));
+            sum[0].add(weight_limbs(wx[a]), r.x, r.y);
+            sum[1].add(weight_limbs(dx[a]), r.x, r.y);
+            sum[2].add(weight_limbs(wx[a]), s.x, s.y);
+        }
+        const double out[4] = {fix_value(s0, top), fix_value(sum[0].value(), top),
+                               fix_value(sum[1].value(), top), fix_value(sum[2].value(), top)};
+        std::fwrite(out, sizeof out, 1, stdout);
+    }
+}
+
 template <typename F>
 void by_degree(int p, F&& f) {
     if (p == 2) f(std::integral_constant<int, 2>());
@@ -106,6 +161,7 @@ int main(int argc, char** argv) {
     const std::string what = argv[1];
     const int p = std::atoi(argv[2]), sh = std::atoi(argv[3]);
     if (what == "shape") by_degree(p, [&](auto P) { shape<decltype(P)::value>(sh); });
+    if (what == "gather") by_degree(p, [&](auto P) { gather<decltype(P)::value>(sh); });
     if (what == "deposit") by_degree(p, [&](auto P) { deposit<decltype(P)::value>(sh); });
     return 0;
 }

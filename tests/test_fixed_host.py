@@ -91,3 +91,78 @@ def test_deposit_rounding(host, p):
         assert max(map(abs, errs)) <= 0.5 + 0.75 / 16 + 0.25
         total += sum(errs)
     assert abs(total) <= 6 * 0.8 * math.sqrt(v.size * n2)
+
+
+def _weights(xi, p):
+    """Nodes (base - k), weights and derivatives in extended precision."""
+    s = xi.astype(np.longdouble) + np.longdouble(p + 1) / 2
+    base = np.floor(s)
+    u = s - base
+    w = [np.ones_like(u)]
+    for d in range(1, p + 1):
+        low = w
+        w = [((u + k) * w[k] if k < d else 0) / d + ((d + 1 - u - k) * w[k - 1] if k else 0) / d
+             for k in range(d + 1)]
+    dw = [(low[k] if k < p else 0) - (low[k - 1] if k else 0) for k in range(p + 1)]
+    return base.astype(np.int64), w, dw
+
+
+def _gather(f, x, y, p):
+    """The value, its derivative along x and along y."""
+    nx, ny = f.shape
+    (ix, wx, dx), (iy, wy, dy) = _weights(x, p), _weights(y, p)
+    v = {(a, b): f.astype(np.longdouble)[(ix - a) % nx, (iy - b) % ny]
+         for a in range(p + 1) for b in range(p + 1)}
+    return [sum(q[a] * r[b] * v[a, b] for a, b in v) for q, r in ((wx, wy), (dx, wy), (wx, dy))]
+
+
+def _host_gather(host, f, x, y, p, sh):
+    data = np.concatenate([[f.shape[0], f.shape[1], x.size], f.ravel(), x, y])
+    out = host("gather", p, sh, data).view(np.float64).reshape(-1, 4).T
+    return out[0], out[1:]  # the value with products of weights; value, d/dx, d/dy separably
+
+
+@pytest.mark.parametrize("nx,ny", [(32, 32), (16, 1024)])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_gather_beside_a_peak(host, p, nx, ny):
+    """Rows where one node holds 1 and the others noise of 1e-17 (the size of a transform's error),
+    gathered away from that node.  In units u = 2^-60 of the row's bound 2: the field's rounding,
+    each row's sum and its shift add errors of variance 1/12 (the first and the derivatives' rows
+    weighted, at most by 2), the others vanish with the fields: below 1 u rms and no mean."""
+    rng = np.random.default_rng(p + ny)
+    f = 1e-17 * rng.uniform(-1, 1, (nx, ny))
+    f[5, 7] = 1.0
+    n, sh = 2000, 52
+    x, y = 5 + rng.uniform(-0.9, 0.9, n), rng.uniform(11.0, ny - 3.0, n)
+    x, y = (np.rint(v * 2.0 ** 40) / 2.0 ** 40 for v in (x, y))
+    want = _gather(f, x, y, p)
+    two, sep = _host_gather(host, f, x, y, p, sh)
+    u = 2.0 ** -59
+    for have, ref in zip((two, *sep), (want[0], *want)):
+        err = ((have - ref) / u).astype(np.float64)
+        assert np.sqrt(np.mean(err ** 2)) <= 1.0
+        assert abs(np.mean(err)) <= 6 / np.sqrt(n)
+
+
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_gather_of_uneven_rows(host, p):
+    """Rows of very different size, zeros and powers of two among them: every result within its
+    worst case.  In u (2^-60 of the stencil's largest row bound): half for each rounded field,
+    row sum and shift, half a unit for each dropped product of low limbs, and (p+1)^2 weights off
+    by 64 (p+1) 2^-62 at the very most (see test_weights_and_derivatives), a quarter of a unit
+    of u each, doubled for derivatives; FP64's rounding of the result besides."""
+    rng = np.random.default_rng(90 + p)
+    nx, ny, n, sh = 24, 16, 1500, 57
+    f = rng.standard_normal((nx, ny)) * 10.0 ** rng.integers(-25, 8, (nx, 1))
+    f[3] = 0.0
+    f[8] = 2.0 ** rng.integers(-40, 3, ny)
+    x, y = rng.uniform(0, nx, n), rng.uniform(0, ny, n)
+    x, y = (np.rint(v * 2.0 ** 45) / 2.0 ** 45 for v in (x, y))
+    want = _gather(f, x, y, p)
+    two, sep = _host_gather(host, f, x, y, p, sh)
+    ix = _weights(x, p)[0]
+    top = np.max([np.max(np.abs(f), axis=1)[(ix - a) % nx] for a in range(p + 1)], axis=0)
+    u = 2.0 ** np.floor(np.log2(np.maximum(top, 1e-300)) + 1) * 2.0 ** -60
+    worst = 2 * (0.5 + (p + 2) + 0.5 * (p + 1) ** 2 + 0.25 * (p + 1) ** 2 * 64 * (p + 1))
+    for have, ref in zip((two, *sep), (want[0], *want)):
+        assert np.all(np.abs(have - ref) <= worst * u + 2.0 ** -53 * np.abs(ref))
