@@ -329,7 +329,9 @@ int64_t pic_step_count(const pic_handle *h);
 int32_t pic_kernels_per_step(const pic_handle *h);
 
 /* Kernel timing, a measurement aid.  The library brackets each launch group below with
- * a pair of CUDA events on the handle's stream and sums their elapsed times:
+ * a pair of CUDA events on the handle's stream and sums their elapsed times (the records
+ * keep the groups of a timed step from overlapping as those of an untimed one do, so their
+ * sum is above its time):
  *   PIC_KT_SORT     the particle sort (keys, scan, scatter) of a sorting step
  *   PIC_KT_DEPOSIT  the move + current deposit kernel (not the clearing of J)
  *   PIC_KT_FIELD    all kernels of pic_field_solve

@@ -1133,12 +1133,20 @@ cudaError_t launch_adj_modes(const ModeCommon& mc, int kind, const AdjModeParams
     return adj_modes(mc, ap, Zb, Js, s);
 }
 
+constexpr size_t kSms = 152, kSmemPerSm = 228 * 1024;
+
 size_t adj_columns_smem(int nx) { return 17 * (size_t)nx * sizeof(double2); }
 
 template <typename Params>
 cudaError_t adj_columns(const ModeCommon& mc, const Params& ap, const double2* Zb, double2* Js,
                         const FftDesc& fd, const double2* tw, cudaStream_t s) {
-    const size_t sm = adj_columns_smem(mc.nx);
+    // Shared memory for as many CTAs an SM as spread over the SMs need, not more: started early,
+    // beside the row transform before them, the CTAs (62 registers a thread with BDF, so four an
+    // SM) crowded on the SMs that it leaves free and waited for each other's FP64 pipe.  A reversed
+    // BDF-2 step of 262,144 particles on 128 x 128: FP32 form 129 -> 122 us, FP64 217 -> 210;
+    // with events around the launch group 75 us of it were the field solve, now 44.
+    const size_t per_sm = (mc.ny + kSms - 1) / kSms;
+    const size_t sm = std::max(adj_columns_smem(mc.nx), kSmemPerSm / (per_sm + 1));
     cudaError_t e = cudaFuncSetAttribute(k_adj_columns<Params>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
