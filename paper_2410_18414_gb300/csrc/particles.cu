@@ -15,6 +15,8 @@
 // gathers), and sorted FP32 particles meet it in shared memory (binned pass).  A
 // position outside [0, L] (including NaN) is never used to index the grid: the
 // particle is skipped and the non-finite bit of the device error word is set.
+#include <type_traits>
+
 #include "common.cuh"
 #include "fixed.cuh"
 #include "gpic_internal.h"
@@ -187,8 +189,8 @@ struct AccFix {
 // atomics overlap, and neighbours among them with the same stencil base (sorted particles)
 // are added first: one atomic instead of up to four on the same words.
 //
-// Large launches are bound by issue, and of a word's instructions nine were its node's index
-// with two wraps.  kInner: a stencil that wraps at no edge takes its nodes from one index and the
+// Of a word's instructions nine were its node's index with two wraps.  kInner (see deposit_rows
+// for where): a stencil that wraps at no edge takes its nodes from one index and the
 // word's constant step; one branch sees to the wrapping ones among the four before their words
 // are formed.  A step of 1.5 M quartic FP32 particles on 256 x 192 295 -> 272 us, of 2^20
 // quadratic FP64 particles on 128 x 128 230 -> 218 us.
@@ -1911,21 +1913,30 @@ cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typen
     const unsigned blocks = (unsigned)((n + kRowThreads - 1) / kRowThreads);
     const GeomT<T> gt = typed<T>(g);
     const SpeciesT<T> st = typed_species<T>(spp);
-    // kInner from three CTAs an SM on: below that the warps wait for their own chains of atomics
-    // and kInner's branch lengthens them (two FP64 quartic steps of 8,700 particles on 256 x 36
-    // 155 us without it, 171 with; 1.5 M FP32 on 256 x 192 294 and 270; 16,384 FP64 on 32 x 32
-    // the same)
-    const bool many = n >= (1 << 16);
-#define GPIC_ROWS(PP, INNER)                                                                 \
-    launch_pdl(k_deposit_rows<Pol, PP, kNC, kMove, INNER>, dim3(blocks), dim3(kRowThreads), 0, s, \
-               gt, x, y, u0, u1, n, pol, err, sp, st)
+    // kInner for FP32 and quartic shapes at any count (us a step without / with it, particles in
+    // random order: FP32 quartic 6,000 on 128 x 128 30.5 / 29.9, cubic 20,000 on 256 x 36 27.2 /
+    // 26.9, 49,152 quadratic on 128 x 96 27.4 / 26.0; FP64 quartic 6,000 on 256 x 36 83.2 / 75.1,
+    // 32,768 on 128 x 128 97.9 / 92.6, 80,000 on 512 x 384 312 / 308).  FP64 quadratic and cubic
+    // launches of few CTAs wait for their own chains of atomics, which the branch lengthens, and
+    // cross over between 33,000 and 56,000 particles (128 x 128, cubic: 6,000 56.1 / 56.3, 32,768
+    // 67.3 / 67.4, 56,000 77.3 / 77.0, 80,000 84.6 / 83.6).
+    const auto launch = [&](auto degree) {
+        constexpr int P = decltype(degree)::value;
+        const auto rows = [&](auto inner) {
+            return launch_pdl(k_deposit_rows<Pol, P, kNC, kMove, decltype(inner)::value>,
+                              dim3(blocks), dim3(kRowThreads), 0, s, gt, x, y, u0, u1, n, pol, err,
+                              sp, st);
+        };
+        if constexpr (P < 4 && sizeof(T) == 8)
+            if (n < (1 << 16)) return rows(std::false_type());
+        return rows(std::true_type());
+    };
     switch (p) {
-        case 2: return many ? GPIC_ROWS(2, true) : GPIC_ROWS(2, false);
-        case 3: return many ? GPIC_ROWS(3, true) : GPIC_ROWS(3, false);
-        case 4: return many ? GPIC_ROWS(4, true) : GPIC_ROWS(4, false);
+        case 2: return launch(std::integral_constant<int, 2>());
+        case 3: return launch(std::integral_constant<int, 3>());
+        case 4: return launch(std::integral_constant<int, 4>());
         default: return cudaErrorInvalidValue;
     }
-#undef GPIC_ROWS
 }
 
 cudaError_t launch_move_deposit(int p, const ParticleGeom& g, double* x, double* y,
