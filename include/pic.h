@@ -190,7 +190,9 @@ typedef struct {
  * roles every step: pic_velocity_slot says which pair holds v^n.  Only for unsorted
  * (sort_interval 0), 2D-2V, single-species configurations, else PIC_ERR_UNSUPPORTED;
  * PIC_ERR_INVALID_ARG for NULL arrays (n > 0) or arrays that are not device memory.
- * pic_read_particles, checkpoints, ensembles and the adjoint work as for pic_init. */
+ * A caller that writes the arrays between steps keeps every speed below c (PIC_FP64: from
+ * 1.25 c, rounded up to a power of two, a particle is left out of J and reported as
+ * PIC_ERR_NONFINITE).  pic_read_particles, checkpoints, ensembles and the adjoint work as for pic_init. */
 pic_status pic_init_bound(const pic_config *cfg, const pic_particles_bound *particles,
                           void *cuda_stream, pic_handle **out);
 

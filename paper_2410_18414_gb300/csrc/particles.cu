@@ -232,6 +232,7 @@ struct RowFix {
         return true;
     }
     __device__ __forceinline__ float factor(float v) const { return v; }
+    __device__ __forceinline__ bool fits(float) const { return true; }
     __device__ __forceinline__ float row(float v, float w) const { return rmul(v, w); }
     __device__ __forceinline__ float col(float w) const { return w; }
 };
@@ -287,6 +288,10 @@ struct RowFix128 {
     __device__ __forceinline__ long long factor(double v) const {
         return __double2ll_rn(rmul(v, scale4));
     }
+    // |v| below 1.25 c: the products and the sum of four contributions stay within int64
+    __device__ __forceinline__ bool fits(long long f) const {
+        return (unsigned long long)f + (5ull << 60) <= (10ull << 60);
+    }
     __device__ __forceinline__ long long row(long long v, long long w) const {
         return deposit_row(v, w);
     }
@@ -318,6 +323,7 @@ struct RowF64 {
         return true;
     }
     __device__ __forceinline__ double factor(double v) const { return v; }
+    __device__ __forceinline__ bool fits(double) const { return true; }
     __device__ __forceinline__ double row(double v, double w) const { return rmul(v, w); }
     __device__ __forceinline__ double col(double w) const { return w; }
 };
@@ -393,6 +399,10 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                     // with a table each contribution carries the particle's q_s w_s
                     if (sp && !Pol::kExtra) v[c] = rmul(v[c], fq);
                     const W f = pol.factor(v[c]);
+                    if (!pol.fits(f)) {  // (bound arrays that the caller has written)
+                        base = -1;
+                        atomicOr(err, (unsigned)ERR_NONFINITE);
+                    }
 #pragma unroll
                     for (int a = 0; a < S1; ++a) mine[c * S1 + a] = pol.row(f, wx[a]);
                 }
