@@ -214,6 +214,49 @@ SMEM_WAVEFRONTS = {
 }
 
 
+# Warp instructions per launch of the FP64 path's kernels, by the pipe they issue to (ncu:
+# sm__inst_executed_pipe_fp64.sum, sm__inst_executed_pipe_alu.sum, smsp__inst_executed.sum), from
+# committed captures.  Most of the method's flops run as integer instructions, so it is these
+# that say how full the machine is.
+PIPE_INSTRUCTIONS = {
+    # (kernel, workload): ({pipe: warp instructions}, source file, its SHA-1 prefix, profile)
+}
+# Warp instructions a clock and SM: the FP64 pipe takes one in 16 clocks (2 lanes), the ALU pipe
+# two a clock, the four schedulers issue four.
+PIPE_PEAK = {"fp64": 1 / 16, "alu": 2.0, "issue": 4.0}
+
+
+def pipes_of(kernel, workload, ms, sm_mhz, nsm):
+    """How full each pipe is while the kernel runs: committed instructions per launch over the
+    event-timed launch; the fullest is the bound.  None without a capture of this source."""
+    entry = PIPE_INSTRUCTIONS.get((kernel, workload))
+    if entry is None:
+        return None, "no ncu capture of this kernel on this workload is committed"
+    counts, src, sha, profile = entry
+    if source_sha1(src) != sha:
+        return None, f"{src} changed since the capture in {profile}"
+    clocks = ms * 1e-3 * nsm * sm_mhz * 1e6
+    return ({k: {"warp_instructions": v, "frac": v / clocks / PIPE_PEAK[k]}
+             for k, v in counts.items()}, f"ncu capture: {profile}")
+
+
+def fp64_roofline(kernel, capture, workload, flops, ms, sm_mhz, nsm):
+    """The fullest pipe of an FP64 kernel; beside it the method's flop rate, which is a
+    throughput and no pipe's use (the stencil sums run as integers)."""
+    pk = peaks()
+    pipes, src = pipes_of(capture, workload, ms, sm_mhz, nsm)
+    line = {"kernel": kernel, "bound": None, "achieved": None, "peak": None,
+            "unit": "warp instructions per SM clock", "frac": None, "pipes": pipes,
+            "source": src, "method": {"gflops": flops / (ms * 1e-3) / 1e9,
+                                      "fp64_fma_gflops": pk["fp64_gflops"],
+                                      "peak_source": pk["fp64_src"]}}
+    if pipes:
+        top = max(pipes, key=lambda k: pipes[k]["frac"])
+        line.update(bound=top, frac=pipes[top]["frac"], peak=PIPE_PEAK[top],
+                    achieved=pipes[top]["frac"] * PIPE_PEAK[top])
+    return line
+
+
 def source_sha1(name):
     import hashlib
     path = os.path.join(ROOT, "paper_2410_18414_gb300", "csrc", name)
@@ -844,26 +887,24 @@ def flops_adj_push(p):
 
 
 def adjoint_roofline(p, n, ms, form="fp64"):
-    """The reverse push against the FP64 pipe (its FMA rate measured on this device); in
-    the FP32 form its particle arithmetic is FP32 (the field-adjoint sums stay FP64) and
-    the FP32 peak is the reference."""
+    """The reverse push: in FP64 the fullest pipe (see fp64_roofline) at the maximum SM clock; in
+    the FP32 form its particle arithmetic is FP32 and the FP32 peak is the reference."""
     if not ms:
         return None
-    pk = peaks()
-    achieved = flops_adj_push(p) * n / (ms * 1e-3) / 1e12
-    if form == "fp32":
-        peak, src = fp32_peak_gflops(2070), "FP32 FMA issue rate at the 2070 MHz maximum SM clock"
-        traffic, traffic_src = None, "not captured for the FP32 form"
-    else:
-        peak, src = pk["fp64_gflops"], pk["fp64_src"]
+    flops = flops_adj_push(p) * n
+    if form != "fp32":
+        line = fp64_roofline("k_adj_push_gather_fix", "adj_push_gather", "adjoint128", flops, ms,
+                             2070.0, 152)
         traffic, traffic_src = traffic_of("adj_push_gather", "adjoint128")
-    return {"kernel": "k_adj_push_gather_pair" if form == "fp32" else "k_adj_push_gather_fix",
-            "bound": "alu", "achieved": achieved,
+        line.update(traffic=traffic, traffic_source=traffic_src,
+                    note=f"{flops_adj_push(p)} flops per particle of the method (cubic: 600)")
+        return line
+    achieved, peak = flops / (ms * 1e-3) / 1e12, fp32_peak_gflops(2070)
+    return {"kernel": "k_adj_push_gather_pair", "bound": "alu", "achieved": achieved,
             "peak": peak / 1e3, "unit": "TFLOP/s", "frac": achieved * 1e3 / peak,
-            "traffic": traffic, "traffic_source": traffic_src, "peak_source": src,
-            "note": f"{flops_adj_push(p)} {form.upper()} flops per particle (cubic: 600)"
-                    + ("" if form == "fp32" else
-                       "; the method's count: the gathers run on the integer pipe")}
+            "traffic": None, "traffic_source": "not captured for the FP32 form",
+            "peak_source": "FP32 FMA issue rate at the 2070 MHz maximum SM clock",
+            "note": f"{flops_adj_push(p)} FP32 flops per particle (cubic: 600)"}
 
 
 def main():
@@ -931,8 +972,6 @@ def main():
         k["gflops"] = k["flops"] / (k["ms"] * 1e-3) / 1e9
         k["gbs"] = k["bytes"] / (k["ms"] * 1e-3) / 1e9
         k["frac_hbm"] = k["gbs"] / pk["hbm_gbs"]
-        if not fp32:
-            k["frac_fp64_alu"] = k["gflops"] / pk["fp64_gflops"]
         kern[name] = k
     # the dominant particle kernel: the one with the most time per step
     dom_name = max(kern, key=lambda k: kern[k]["ms"] * kern[k]["launches"])
@@ -956,16 +995,12 @@ def main():
         if smem is not None:
             roofline["smem_pipe"] = smem
     else:
-        roofline = {"kernel": dom_name, "bound": "alu", "achieved": dom["gflops"],
-                    "peak": pk["fp64_gflops"], "unit": "GFLOP/s",
-                    "frac": dom["gflops"] / pk["fp64_gflops"],
-                    "traffic": traffic, "traffic_source": traffic_src,
-                    "peak_source": pk["fp64_src"],
-                    # the method's flops: the stencil work of the FP64 path runs as integer
-                    # multiply-adds, so this fraction may exceed what the FP64 pipe does
-                    "note": "flops of the method; the stencil sums run on the integer pipe",
-                    "hbm": {"achieved_gbs": dom["gbs"], "peak_gbs": pk["hbm_gbs"],
-                            "frac": dom["gbs"] / pk["hbm_gbs"], "peak_source": pk["hbm_src"]}}
+        nsm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+        roofline = fp64_roofline(dom_name, dom_name, a.workload, dom["flops"], dom["ms"],
+                                 clk.get("sm_mhz") or 2070.0, nsm)
+        roofline.update(traffic=traffic, traffic_source=traffic_src,
+                        hbm={"achieved_gbs": dom["gbs"], "peak_gbs": pk["hbm_gbs"],
+                             "frac": dom["gbs"] / pk["hbm_gbs"], "peak_source": pk["hbm_src"]})
 
     # the configuration's whole run (its own step count, whatever --steps says): every
     # step in one pic_step call (the call's steps run back to back, so no L2 flush

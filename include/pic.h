@@ -437,8 +437,11 @@ typedef enum {
                               steps from its checkpoint (least memory) */
     PIC_ADJ_REPLAY_LEAN = 2 /* as PIC_ADJ_REPLAY with per particle only P^{n+1}, v^{n+1}
                               (32 n + G bytes per step): the reverse push gathers A and
-                              grad A again from the recorded fields (the same bits, a second
-                              pass over the stencil) */
+                              grad A again from the recorded fields, a second pass over the
+                              stencil (the FP32 form, and FP64 with fewer than nx ny / 8
+                              particles: the same bits; FP64 otherwise: row by row in place of
+                              the forward's products of weights, apart by less than FP64's
+                              rounding of the largest value on the stencil's rows) */
 } pic_adjoint_mode;
 
 /* Prepare the adjoint of the next `nsteps` steps of h.  h must be fresh from pic_init

@@ -34,7 +34,8 @@
 // identity).  The field adjoints they deposit are summed in FP64 (FP32 form: in FP32, the
 // eight values of a node in two vector atomics), eight values a node side by side, and the
 // reverse field solve is FP64 in both forms, as the forward's per-mode update is.  Shape weights come
-// from Shape<P, T> (the forward's), their derivatives from the closed forms below.
+// from Shape<P, T> (the forward's) and their derivatives from the closed forms below; in the
+// fixed-point kernels (..._fix) from fix_weights and fix_dweights.
 #include <algorithm>
 
 #include "common.cuh"
@@ -389,8 +390,8 @@ k_adj_push_gather(ParticleGeom g, PushParams pp, const double* __restrict__ x1,
 // sums, four lanes a particle: along a row with W_y and dW_y, then across rows with W_x and
 // dW_x.  The FP64 pipe is left with the push's adjoint and the products the atomics add
 // (about 250 operations a particle instead of 600).  262,144 particles, 128 x 128, cubic: with
-// FP64 gathers and a lane per particle 263 us, now 137 us.  Bound by the FP64 pipe (72%) and its
-// latency: five CTAs an SM (96 registers, 32 bytes spilled) instead of four, 148 -> 137 us; six
+// FP64 gathers and a lane per particle 263 us, now 139 us.  Bound by the FP64 pipe (72%) and its
+// latency: five CTAs an SM (96 registers, 32 bytes spilled) instead of four, 148 -> 137 us (with limbs of 29 bits); six
 // are slower.  The lean form gains nothing at five (144.5 -> 146 us) and quartic shapes spill:
 // they keep the four and three that their registers allow.
 template <int P, bool kLean>
@@ -585,7 +586,7 @@ k_adj_deposit_move(ParticleGeom g, const T* __restrict__ x1, const T* __restrict
 
 // The same with the mesh adjoint current in fixed point (an int4 a node, two maxima a row):
 // six separable integer sums, about 35 FP64 operations a particle left of 170.  Measured with
-// FP64 sums 78 us, now 31 us (262,144 particles, cubic; four CTAs an SM of 128 registers, 34 us
+// FP64 sums 78 us, now 32 us (262,144 particles, cubic; four CTAs an SM of 128 registers, 34 us
 // with three; quartic shapes would spill and keep two).
 template <int P>
 __global__ void __launch_bounds__(kAdjThreads, P > 3 ? 2 : 4)

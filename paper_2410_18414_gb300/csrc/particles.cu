@@ -196,7 +196,7 @@ struct AccFix {
 // quadratic FP64 particles on 128 x 128 230 -> 218 us.
 //
 // Move + deposit, a lane per particle before: FP64, 2^20 particles, 128 x 128, cubic 320 ->
-// 100 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
+// 109 us (issue slots 65% busy, the ALU pipe 61%); FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
 // 256 x 192, quartic 353 -> 120 us (bound by L2's atomics still: 17.5 sectors a particle).
 constexpr int kRowThreads = 128;
 
@@ -669,7 +669,7 @@ k_gather_push(GeomT<T> g, PushT<T> pp, const T* __restrict__ x, const T* __restr
 // gathered 16 or 8 at a time, and the gathered fields go back through the same records to
 // the lane that pushes the particle.  Gather + push, a lane per particle before: FP32, 1.5 M
 // particles, 256 x 192, quartic 192 -> 121 us; FP64, 2^20 particles, 128 x 128, cubic
-// 394 -> 124 us.
+// 394 -> 122 us.
 constexpr int kRowGatherThreads = 128;
 
 // FP32: the node order and roundings of every other gather, so the same bits.
@@ -778,7 +778,7 @@ k_gather_push_pair(GeomT<float> g, PushT<float> pp, const float* __restrict__ x,
 //     / fixed point in units of the transform's: smooth fields 1.24-1.70 / 1.05-1.17, noise
 //     1.15-1.27 / 1.02-1.03, rows of a single peak 1.000 / 0.98-1.01 (32^2 to 1024^2; in units
 //     of 2^-58 with the rows rounded down the last was 1.04-1.08, and one-sided).
-// Integer sums do not depend on their order, and the same bits come out on every path.
+// Integer sums do not depend on their order: the forward's paths give the same bits.
 // Fields 2q and 2q+1 of the `per` int4 a node at one particle (kb: its first node, w: its
 // weights' limbs).
 template <int P>

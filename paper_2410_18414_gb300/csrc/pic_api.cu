@@ -755,8 +755,8 @@ static pic_status init_impl(const pic_config* cfg, const pic_particles_in* init,
     } else {
         // FP64 path: |v W_x W_y| < c and |W_x W_y| <= 1 (times max |q_s w_s|), so quanta of
         // 2^-60 of those bounds keep every contribution below 2^60 (one int64 word); the
-        // 128-bit sums have room for any number of them.  The quantum (8.7e-19 c for the
-        // current) is far below FP64 rounding of a node's total.
+        // 128-bit sums have room for any number of them.  The quantum is 8.7e-19 c for the
+        // current; contributions are rounded to the nearest one.
         const int kc = (int)std::ceil(std::log2(cfg->c)) + (int)std::ceil(std::log2(rmax));
         h->fix64_scale_j = std::ldexp(1.0, 60 - kc);
         h->fix64_unscale_j = std::ldexp(1.0, kc - 60);
