@@ -192,12 +192,18 @@ struct AccFix {
 // Of a word's instructions nine were its node's index with two wraps.  kInner (see deposit_rows
 // for where): a stencil that wraps at no edge takes its nodes from one index and the
 // word's constant step; one branch sees to the wrapping ones among the four before their words
-// are formed.  A step of 1.5 M quartic FP32 particles on 256 x 192 295 -> 272 us, of 2^20
-// quadratic FP64 particles on 128 x 128 230 -> 218 us.
+// are formed.  It took a step of 1.5 M quartic FP32 particles on 256 x 192 from 295 to 272 us, of
+// 2^20 quadratic FP64 particles on 128 x 128 from 230 to 218 us.
+//
+// The four particles' values are formed whether or not a lane wants them, from records that are
+// there in any case: with a branch around each, the compiler let them wait for their shared loads
+// one after another in some instances of the kernel (2^20 quartic FP64 particles on 128 x 128:
+// deposit 291 or 231 us by the look of unrelated code, now 219; 20,000 quartic FP32 on 256 x 256
+// 12.3 -> 10.2).
 //
 // Move + deposit, a lane per particle before: FP64, 2^20 particles, 128 x 128, cubic 320 ->
-// 109 us (issue slots 65% busy, the ALU pipe 61%); FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
-// 256 x 192, quartic 353 -> 120 us (bound by L2's atomics still: 17.5 sectors a particle).
+// 108 us; FP64, 16,384 particles, 32 x 32, quadratic 28 -> 13 us; FP32, 1.5 M particles,
+// 256 x 192, quartic 353 -> 116 us (bound by L2's atomics still: 17.5 sectors a particle).
 constexpr int kRowThreads = 128;
 
 // A policy says what a particle's record holds (per component the row factors t[a], then
@@ -254,7 +260,7 @@ struct RowFixCharge : RowFix {
 // Integer sums do not depend on the order of the additions, so the deposit is bit-for-bit
 // deterministic.  The factors are integers: v in units of 2^-2 quanta, t = v W_x in 2^-3, x =
 // t W_y in quanta, each rounded to nearest once (deposit_row, deposit_value): x is within
-// 0.6 quanta and no one-sided error is left, whatever v is.
+// 0.8 quanta (0.6 for slow particles) and no one-sided error is left, whatever v is.
 struct RowFix128 {
     using T = double;
     using W = long long;
@@ -441,15 +447,18 @@ k_deposit_rows(GeomT<typename Pol::T> g, typename Pol::T* __restrict__ x,
                 }
 #pragma unroll
                 for (int j = 0; j < kAhead; ++j) {
-                    const int k = (i0 + j) * kGroups + group;
-                    val[j] = 0;
-                    if (bs[j] != -1) {
-                        val[j] = pol.value(rec + (w0 + k) * kStride, wc[q] * S1 + wa[q],
-                                           kNC * S1 + wb[q], kFields - 1);
-                        if (j > 0 && bs[j] == bs[j - 1]) {  // the same words: one atomic
-                            val[j] += val[j - 1];
-                            bs[j - 1] = -1;
-                        }
+                    // (formed whether or not it is wanted: in a branch each, the four would
+                    // wait for their records one after another)
+                    const int k = min((i0 + j) * kGroups + group, 31);
+                    const V x = pol.value(rec + (w0 + k) * kStride, wc[q] * S1 + wa[q],
+                                          kNC * S1 + wb[q], kFields - 1);
+                    val[j] = bs[j] != -1 ? x : V(0);
+                }
+#pragma unroll
+                for (int j = 1; j < kAhead; ++j) {
+                    if (bs[j] == bs[j - 1]) {  // the same words: one atomic
+                        val[j] += val[j - 1];
+                        bs[j - 1] = -1;
                     }
                 }
 #pragma unroll
@@ -1923,13 +1932,14 @@ cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typen
     const unsigned blocks = (unsigned)((n + kRowThreads - 1) / kRowThreads);
     const GeomT<T> gt = typed<T>(g);
     const SpeciesT<T> st = typed_species<T>(spp);
-    // kInner for FP32 and quartic shapes at any count (us a step without / with it, particles in
-    // random order: FP32 quartic 6,000 on 128 x 128 30.5 / 29.9, cubic 20,000 on 256 x 36 27.2 /
-    // 26.9, 49,152 quadratic on 128 x 96 27.4 / 26.0; FP64 quartic 6,000 on 256 x 36 83.2 / 75.1,
-    // 32,768 on 128 x 128 97.9 / 92.6, 80,000 on 512 x 384 312 / 308).  FP64 quadratic and cubic
-    // launches of few CTAs wait for their own chains of atomics, which the branch lengthens, and
-    // cross over between 33,000 and 56,000 particles (128 x 128, cubic: 6,000 56.1 / 56.3, 32,768
-    // 67.3 / 67.4, 56,000 77.3 / 77.0, 80,000 84.6 / 83.6).
+    // kInner for the FP64 path's quartic shapes at any count, for the others from 65,536 particles:
+    // launches of few CTAs wait for their own chains of atomics, which the branch lengthens (but
+    // the quartic FP64 words, two passes of 25 nodes, gain more from the index).  Both sides
+    // measured from 6,000 to 160,000 particles on 32 x 32, 128 x 128, 256 x 36 and 512 x 384, us a
+    // step without / with it.  FP64 quartic: 6,000 on 256 x 36 80.8 / 73.1, 80,000 on 128 x 128
+    // 107.1 / 100.0.  FP64 cubic on 256 x 36: 6,000 56.5 / 57.0, 40,000 68.8 / 69.1, 56,000 72.6 /
+    // 72.5, 80,000 80.4 / 79.8.  FP32 quartic on 32 x 32: 6,000 21.4 / 22.4, cubic on 128 x 128:
+    // 56,000 30.3 / 31.1, 80,000 34.3 / 31.7.
     const auto launch = [&](auto degree) {
         constexpr int P = decltype(degree)::value;
         const auto rows = [&](auto inner) {
@@ -1937,7 +1947,7 @@ cudaError_t deposit_rows(int p, const ParticleGeom& g, typename Pol::T* x, typen
                               dim3(blocks), dim3(kRowThreads), 0, s, gt, x, y, u0, u1, n, pol, err,
                               sp, st);
         };
-        if constexpr (P < 4 && sizeof(T) == 8)
+        if constexpr (P < 4 || !std::is_same_v<Pol, RowFix128>)
             if (n < (1 << 16)) return rows(std::false_type());
         return rows(std::true_type());
     };
