@@ -197,9 +197,9 @@ def flops_gather_deposit(p):
 # time: when the source has changed since, the bench line reports no traffic.
 TRAFFIC = {
     # (kernel, workload): (bytes per launch, source file, its SHA-1 prefix, profile)
-    ("gather_deposit", "weibel128"): (34.42e6 + 0.029e6, "particles.cu", "f0e455eb0364",
+    ("gather_deposit", "weibel128"): (34.42e6 + 0.027e6, "particles.cu", "5cfe7772d28a",
                                       "profiles/gather_deposit_fused_weibel128.md"),
-    ("gather_deposit", "weibel512"): (852.38e6 + 596.31e6, "particles.cu", "f0e455eb0364",
+    ("gather_deposit", "weibel512"): (852.36e6 + 596.12e6, "particles.cu", "5cfe7772d28a",
                                       "profiles/gather_deposit_fused_weibel512.md"),
 }
 
@@ -209,7 +209,7 @@ TRAFFIC = {
 # wavefront per SM clock is the pipe's peak (128 B a clock).
 SMEM_WAVEFRONTS = {
     # (kernel, workload): (wavefronts per launch, source file, its SHA-1 prefix, profile)
-    ("gather_deposit", "weibel128"): (9.39e6, "particles.cu", "f0e455eb0364",
+    ("gather_deposit", "weibel128"): (9.39e6, "particles.cu", "5cfe7772d28a",
                                       "profiles/gather_deposit_fused_weibel128.md"),
 }
 
@@ -221,9 +221,9 @@ SMEM_WAVEFRONTS = {
 PIPE_INSTRUCTIONS = {
     # (kernel, workload): ({pipe: warp instructions}, source file, its SHA-1 prefix, profile)
     ("gather_push", "weibel128"): ({"fp64": 1.278e6, "alu": 38.37e6, "issue": 87.03e6},
-                                   "particles.cu", "f0e455eb0364", "profiles/fp64_weibel128.md"),
-    ("deposit", "weibel128"): ({"fp64": 0.590e6, "alu": 39.08e6, "issue": 82.69e6},
-                               "particles.cu", "f0e455eb0364", "profiles/fp64_weibel128.md"),
+                                   "particles.cu", "5cfe7772d28a", "profiles/fp64_weibel128.md"),
+    ("deposit", "weibel128"): ({"fp64": 0.590e6, "alu": 39.87e6, "issue": 77.22e6},
+                               "particles.cu", "5cfe7772d28a", "profiles/fp64_weibel128.md"),
     ("adj_push_gather", "adjoint128"): ({"fp64": 1.835e6, "alu": 26.44e6, "issue": 64.80e6},
                                         "adjoint.cu", "094bb1c45dd3",
                                         "profiles/adjoint_weibel_adjoint128_fp64.md"),
